@@ -713,12 +713,12 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
         case MGMLMC_OP_G5: mg::launch_gamma5<double2>(yt, xt, c.lev[l].nsites, c.lev[l].d, nrhs, c.stream); break;
         case MGMLMC_OP_SMOOTH:
             if (c.opt.mg_precision == 64) {
-                mg::apply_smoother_operator<double2>(c, l, yt, xt, nrhs, nullptr);
+                mg::apply_smoother_operator<double2>(c, l, yt, xt, nrhs);
             } else {
                 float2* x32 = c.scratch<float2>("ap_x32", (size_t)nin * nrhs);
                 float2* y32 = c.scratch<float2>("ap_y32", (size_t)nout * nrhs);
                 mg::launch_convert<float2, double2>(x32, xt, nin * nrhs, c.stream);
-                mg::apply_smoother_operator<float2>(c, l, y32, x32, nrhs, nullptr);
+                mg::apply_smoother_operator<float2>(c, l, y32, x32, nrhs);
                 mg::launch_convert<double2, float2>(yt, y32, nout * nrhs, c.stream);
             }
             break;
@@ -887,12 +887,13 @@ extern "C" int mgmlmc_autotune(mgmlmc_ctx* h, size_t hbm_budget, int max_trials,
         s.N = q.N;
         s.m = q.m;
         s.kcycle = q.kc;
+        s.nu = std::max(start.nu_pre, q.nu);
         const size_t b = mg::footprint_bytes(s);
         if (bytes) *bytes = b;
         return b <= budget;
     };
     const uint64_t kSeed = 0x2211153839ull;
-    int trials = 0, last_N = -1, warm_m = 0, warm_kc = -1;
+    int trials = 0, last_N = -1, warm_m = 0, warm_kc = -1, warm_nu = 0;
     double best_rate = -1;
     Cand best{start.max_block_rhs, start.fgmres_restart, start.nu_post, start.kcycle_iters};
     std::vector<Cand> tried;
@@ -919,14 +920,15 @@ extern "C" int mgmlmc_autotune(mgmlmc_ctx* h, size_t hbm_budget, int max_trials,
                            "autotune: a trial solve did not converge");
             }
         };
-        // work space of this width, a longer restart or another coarse-grid correction:
-        // allocated in an untimed run
-        if (q.N != last_N || q.m > warm_m || q.kc != warm_kc) {
+        // work space of this width, a longer restart, more smoothing steps or another
+        // coarse-grid correction: allocated in an untimed run
+        if (q.N != last_N || q.m > warm_m || q.nu > warm_nu || q.kc != warm_kc) {
             if (q.N != last_N) release_scratch(c);
             run_all();
-            if (q.N != last_N) warm_m = 0;
+            if (q.N != last_N) warm_m = warm_nu = 0;
             last_N = q.N;
             warm_m = std::max(warm_m, q.m);
+            warm_nu = std::max(warm_nu, q.nu);
             warm_kc = q.kc;
         }
         cudaEvent_t e0, e1;
@@ -977,7 +979,7 @@ extern "C" int mgmlmc_autotune(mgmlmc_ctx* h, size_t hbm_budget, int max_trials,
         // 3. smoother steps, 4. coarse-grid correction
         for (int nu : {2, 6}) {
             Cand q{best.N, best.m, nu, best.kc};
-            if (trials < max_trials && !was_tried(q)) time_one(q);
+            if (trials < max_trials && !was_tried(q) && fits(q, nullptr)) time_one(q);
         }
         if (c.L >= 4) {
             Cand q{best.N, best.m, best.nu, best.kc > 0 ? 0 : 2};

@@ -163,13 +163,16 @@ struct Ctx {
 };
 
 // ---- solver layer (solver.cu)
-template <typename C> void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, double2* dots);
+// mode 0: y = D x; 1: y = b - D x; 2: y = D x and alpha[j] = <y, x>_j / <y, y>_j (the
+// minimal-residual coefficient); 3: alpha only (y may be null).
+template <typename C> void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* alpha);
 template <typename C> void apply_restrict(Ctx& c, int l, C* xc, const C* x, int N);
-template <typename C> void apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate);
+// xt (may be null): true if the BF16 operand tiles of x were written there as well.
+template <typename C> bool apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate, void* xt = nullptr);
 template <typename C> void mg_cycle(Ctx& c, int l, C* e, const C* r, int N);
 // y = D_l M_l^{-1} x, the operator of the block-Jacobi smoother (coarse levels
-// above the coarsest); dots (2N, may be null) receive conj(y).x and |y|^2 per rhs.
-template <typename C> void apply_smoother_operator(Ctx& c, int l, C* y, const C* x, int N, double2* dots);
+// above the coarsest).
+template <typename C> void apply_smoother_operator(Ctx& c, int l, C* y, const C* x, int N);
 // FGMRES(m) in precision C on level l; x holds the initial guess (zero if x_zero).
 // At most max_cycles restart cycles.  Returns outer iterations; *ok = 1 if the
 // relative residual reached tol (or the cycle budget ended, for inner solves).

@@ -24,7 +24,11 @@ struct Shape {
     int m = 24;                      // FGMRES restart length
     int precision = 64;              // mg_precision
     int kcycle = 0;                  // K-cycle steps per coarse-grid correction
+    int nu = 4;                      // smoothing steps per level (the larger of pre and post)
 };
+
+// Residuals that the smoother keeps at once: those of a group of at most 8 steps.
+inline int smoother_slots(int nu) { return std::min(std::max(nu, 1), 8); }
 
 inline size_t footprint_bytes(const Shape& s) {
     const double N = std::max(1, s.N);
@@ -53,9 +57,11 @@ inline size_t footprint_bytes(const Shape& s) {
         }
         if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * N * 16;            // FP64 Galerkin apply
         if (l + 1 < L) {
-            b += n * N * sz * 3 + 2.0 * (double)s.n[l + 1] * N * sz;         // V-cycle blocks
-            if (bf16 && l > 0) b += 3.0 * st * std::ceil(N / 128) * 8192 + n * N * 8;   // BF16 tiles, rhs
-            if (bf16 && l == 0) b += 2.0 * n * N * 4;                        // fine-level BF16 r and p
+            const double K = smoother_slots(s.nu);
+            const bool tiles = bf16 && l > 0 && s.d[l] == 16;                // smoothed on the tensor cores
+            b += n * N * sz * (tiles ? 3 : K + 1) + 2.0 * (double)s.n[l + 1] * N * sz;   // V-cycle blocks
+            if (tiles) b += (K + 2) * st * std::ceil(N / 128) * 8192 + n * N * 8;        // BF16 tiles, rhs
+            if (bf16 && l == 0) b += (K + 1) * n * N * 4;                    // fine-level BF16 r and p
         }
         if (s.kcycle > 0 && l > 0 && l + 1 < L)
             b += (2.0 * s.kcycle + 1) * n * N * sz + G * (s.kcycle + 1) * N * 16;   // K-cycle bases

@@ -79,23 +79,31 @@ void launch_finalize(double2* out, const double2* part, int groups, int count, c
 void launch_finalize(double* out, const double* part, int groups, int count, cudaStream_t s);
 // Row-major partials (the stencils' minimal-residual dots): out[i] = sum_g part[i * groups + g].
 void launch_finalize_rows(double2* out, const double2* part, int groups, int count, cudaStream_t s);
+// alpha[j] = <y, x>_j / <y, y>_j (0 where <y, y> is 0) from a stencil's partials of its two dots.
+template <typename C>
+void launch_finalize_alpha(C* alpha, const double2* part, int groups, int N, cudaStream_t s);
 
 // --------------------------------------------------------------- stencils
 // Fine Wilson-Schwinger operator (2 spins, U(1) links U[site][mu]).
 //  mode 0: y = D x;  mode 1: y = b - D x;
 //  mode 2: y = D x and part[0][j][g] = <y, x>_j, part[1][j][g] = <y, y>_j (MR smoother;
 //          row-major in the group index g = blockIdx.y, see launch_finalize_rows)
+//  mode 3: the dots of mode 2 without y (which may be null)
 template <typename C>
 void launch_wilson(C* y, const C* x, const C* b, const C* U, double m0, int lx, int lt, int N,
                    int mode, double2* part, int groups, cudaStream_t s);
 // Fine-level smoother in BF16 (one bf16x2 word per complex value, [row][rhs]):
-// y = D x with per-rhs dots conj(y).x, |y|^2 (partials as launch_wilson mode 2; N % 4 == 0),
-// the FP32 -> BF16 conversion, and e (=|+=) alpha r, r -= alpha p (r in place).
+// y = D x (y may be null) with per-rhs dots conj(y).x, |y|^2 (partials as launch_wilson
+// mode 2; N % 4 == 0), the residual b - D x rounded to BF16 (N even), and the smoother's
+// updates: rn = r - alpha p, e (=|+=) sum_{s < K} alpha_s r_s over K <= 8 slots (N % 4 == 0).
 void launch_wilson_bf16(uint32_t* y, const uint32_t* x, const float2* U, double m0, int lx, int lt, int N,
                         double2* part, int groups, cudaStream_t s);
-void launch_pack_bf16(uint32_t* y, const float2* x, long long count, cudaStream_t s);
-void launch_mr_update_fine_bf16(float2* e, uint32_t* r, const uint32_t* p, const double2* dots, long long n, int N,
-                                bool e_is_zero, cudaStream_t s);
+void launch_wilson_residual_bf16(uint32_t* y, const float2* x, const float2* b, const float2* U, double m0, int lx,
+                                 int lt, int N, int groups, cudaStream_t s);
+void launch_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r, const uint32_t* p, const float2* alpha, long long n,
+                                int N, cudaStream_t s);
+void launch_mr_combine_bf16(float2* e, const uint32_t* rs, size_t slot, int K, const float2* alpha, long long n, int N,
+                            bool e_is_zero, cudaStream_t s);
 // Coarse 5-point block stencil y_s = sum_dir A[s][dir] x_nbr(s,dir), d x d complex blocks,
 // dir = 0 self, 1 +x, 2 -x, 3 +t, 4 -t (periodic; boundary signs live in the blocks).
 template <typename C>
@@ -112,13 +120,18 @@ int block_stencil_groups(int nsites, int d, int N);
 template <typename C>
 void launch_restrict(C* xc, const C* x, const C* P, int lx, int lt, int d, int ax, int at, int nvec,
                      int N, cudaStream_t s);
+// xt (may be null): where the kernel can (FP32, d = 16, nvec 2, 4 or 8) it also writes the
+// result's BF16 operand tiles (launch_pack_tiles_bf16) there, and returns true.
 template <typename C>
-void launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax, int at, int nvec,
-                    int N, bool accumulate, cudaStream_t s);
-// MR update: alpha_j = <p,r>/<p,p> from dots[2][N]; e += alpha r; r -= alpha p.
+bool launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax, int at, int nvec,
+                    int N, bool accumulate, cudaStream_t s, void* xt = nullptr);
+// Minimal-residual smoother: rn = r - alpha p, and e (=|+=) sum_{s < K} alpha_s r_s over the
+// K <= 8 residuals r_s in slots of rs (slot: values between them; alpha[K][N]).
 template <typename C>
-void launch_mr_update(C* e, C* r, const C* p, const double2* dots, long long n, int N, bool e_is_zero,
-                      cudaStream_t s);
+void launch_mr_update(C* rn, const C* r, const C* p, const C* alpha, long long n, int N, cudaStream_t s);
+template <typename C>
+void launch_mr_combine(C* e, const C* rs, size_t slot, int K, const C* alpha, long long n, int N, bool e_is_zero,
+                       cudaStream_t s);
 // Gamma5 on a level with d dof per site: +1 on the first d/2 dof, -1 on the rest.
 template <typename C>
 void launch_gamma5(C* y, const C* x, long long nsites, int d, int N, cudaStream_t s);
@@ -186,22 +199,25 @@ void launch_deflation_correction_bf16(double2* smp, const double2* X, const __nv
 // smoother: E holds the blocks of every site and direction as BF16 real 32 x 32
 // operands (launch_embed_stencil_bf16); the input x is given as BF16 tiles
 // (per site and 128-rhs tile, 8 KB in the MMA's K-major layout, written by
-// launch_pack_tiles_bf16 or launch_mr_update_tc).  y = A x in FP32 plus per-rhs
+// launch_pack_tiles_bf16, launch_prolong or launch_mr_update_tiles).  y = A x in FP32 plus per-rhs
 // dots conj(y).x, |y|^2 (partials as launch_block_stencil).  err: device flag set
 // when a bounded wait gave up.
 bool tc_stencil_supported(int d, int N);
 void launch_embed_stencil_bf16(__nv_bfloat16* E, const float2* A, int nsites, cudaStream_t s);
 size_t tc_tiles_bytes(int nsites, int N);
 void launch_pack_tiles_bf16(__nv_bfloat16* rt, const float2* x, int nsites, int N, cudaStream_t s);
-// yh (= or +=) alpha r, r -= alpha p with alpha = dots[j] / dots[N + j]; rt (may be
-// null) receives the BF16 tiles of the new r.  d = 16.
-void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const double2* dots, int nsites, int N, bool first,
+// yh (= or +=) alpha r, r -= alpha p; rt (may be null) receives the BF16 tiles of the new
+// r.  d = 16.
+void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const float2* alpha, int nsites, int N, bool first,
                          __nv_bfloat16* rt, cudaStream_t s);
-// yh (= or +=) alpha r, r -= alpha p with r and p as BF16 tiles (r updated in place).
-void launch_mr_update_bf16(float2* yh, __nv_bfloat16* rt, const __nv_bfloat16* pt, const double2* dots, int nsites,
-                           int N, bool first, cudaStream_t s);
+// rn = r - alpha p as BF16 tiles (rn distinct from r), and e (=|+=) Minv sum_{s < K} alpha_s r_s over
+// K consecutive sets of tiles (tc_tiles_bytes apart).
+void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __nv_bfloat16* p, const float2* alpha,
+                            int nsites, int N, cudaStream_t s);
+void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const float2* alpha, const float2* Minv,
+                             int nsites, int N, bool accumulate, cudaStream_t s);
 int block_stencil_tc_groups(int nsites, int N);
-// Output: y (FP32 rows) or yt (BF16 tiles), exactly one non-null; with b (FP32 rows,
+// Output: y (FP32 rows), yt (BF16 tiles) or neither (the dots only); with b (FP32 rows,
 // yt only) the tiles receive the residual b - A x and no dots are formed.
 void launch_block_stencil_tc(float2* y, __nv_bfloat16* yt, const float2* b, const __nv_bfloat16* xt,
                              const __nv_bfloat16* E, int lx, int lt, int N, double2* part, int groups, int* err,
@@ -237,6 +253,10 @@ void launch_block_diag_inverse(double2* Minv, double2* work, const double2* A, i
                                cudaStream_t s);
 void launch_precondition_blocks(double2* Ahat, const double2* A, const double2* Minv, int lx, int lt, int d,
                                 cudaStream_t s);
+// y[s] (+)= Minv[s] sum_{q < K} alpha_q x_q[s] over K slots of x.
+template <typename C>
+void launch_block_diag_combine(C* y, const C* x, size_t slot, int K, const C* alpha, const C* Minv, int nsites, int d,
+                               int N, bool accumulate, cudaStream_t s);
 // y[s] (+)= Minv[s] x[s] for every site (d x d complex blocks), N rhs.
 template <typename C>
 void launch_block_diag_apply(C* y, const C* x, const C* Minv, int nsites, int d, int N, bool accumulate,

@@ -15,6 +15,13 @@
 
 namespace mg {
 
+// BF16 pairs (one complex value per 32-bit word).
+__device__ __forceinline__ float2 bf2_lo(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+__device__ __forceinline__ uint32_t f2_bf(float2 v) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+    return *reinterpret_cast<const uint32_t*>(&b);
+}
+
 // Threads of the one-rhs-per-thread CTAs: 128, or fewer for narrower blocks so that
 // no lane idles (N = 64: two warps).
 static int cta_threads(int N) { return std::min(128, (N + 31) / 32 * 32); }
@@ -71,16 +78,18 @@ __global__ void __launch_bounds__(256) k_wilson(C* __restrict__ y, const C* __re
                 o0 = csub(b[site * N2 + j], o0);
                 o1 = csub(b[site * N2 + N + j], o1);
             }
-            y[site * N2 + j] = o0;
-            y[site * N2 + N + j] = o1;
-            if (MODE == 2) {
+            if (MODE != 3) {
+                y[site * N2 + j] = o0;
+                y[site * N2 + N + j] = o1;
+            }
+            if (MODE >= 2) {
                 cfmac(dyx, o0, p0);
                 cfmac(dyx, o1, p1);
                 dyy = fma(o0.x, o0.x, fma(o0.y, o0.y, fma(o1.x, o1.x, fma(o1.y, o1.y, dyy))));
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE >= 2) {
         __shared__ double2 sh[2][kRowLanes][kRhsTile + 1];
         sh[0][threadIdx.y][threadIdx.x] = to_d(dyx);
         sh[1][threadIdx.y][threadIdx.x] = make_double2((double)dyy, 0.0);
@@ -137,8 +146,8 @@ __global__ void __launch_bounds__(256) k_block_stencil(C* __restrict__ y, const 
                     const long long idx = ((long long)site * d + c) * N + j;
                     C o = acc[r];
                     if (MODE == 1) o = csub(b[idx], o);
-                    y[idx] = o;
-                    if (MODE == 2) {
+                    if (MODE != 3) y[idx] = o;
+                    if (MODE >= 2) {
                         cfmac(dyx, o, x[idx]);
                         dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
                     }
@@ -146,7 +155,7 @@ __global__ void __launch_bounds__(256) k_block_stencil(C* __restrict__ y, const 
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE >= 2) {
         __syncthreads();
         double2* sh = reinterpret_cast<double2*>(smem_raw);   // reuse: [2][8][33]
         sh[(0 * kRowLanes + threadIdx.y) * (kRhsTile + 1) + threadIdx.x] = to_d(dyx);
@@ -204,15 +213,15 @@ __global__ void __launch_bounds__(128) k_block_stencil_d(C* __restrict__ y, cons
                 const long long idx = ((long long)site * D + c) * N + j;
                 C o = acc[c];
                 if (MODE == 1) o = csub(b[idx], o);
-                y[idx] = o;
-                if (MODE == 2) {
+                if (MODE != 3) y[idx] = o;
+                if (MODE >= 2) {
                     cfmac(dyx, o, x[idx]);
                     dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
                 }
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE >= 2) {
         // per-rhs partials: one thread per rhs, no cross-thread reduction needed
         if (j < N) {
             part[((long long)0 * N + j) * gridDim.y + blockIdx.y] = to_d(dyx);
@@ -277,8 +286,8 @@ __global__ void __launch_bounds__(128) k_block_stencil_f2(float2* __restrict__ y
                     o0 = make_float2(bv.x - o0.x, bv.y - o0.y);
                     o1 = make_float2(bv.z - o1.x, bv.w - o1.y);
                 }
-                *reinterpret_cast<float4*>(y + idx) = make_float4(o0.x, o0.y, o1.x, o1.y);
-                if (MODE == 2) {
+                if (MODE != 3) *reinterpret_cast<float4*>(y + idx) = make_float4(o0.x, o0.y, o1.x, o1.y);
+                if (MODE >= 2) {
                     const float4 xv = *reinterpret_cast<const float4*>(x + idx);
                     cfmac(dyx0, o0, make_float2(xv.x, xv.y));
                     cfmac(dyx1, o1, make_float2(xv.z, xv.w));
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(128) k_block_stencil_f2(float2* __restrict__ y
             }
         }
     }
-    if (MODE == 2 && j < N) {
+    if (MODE >= 2 && j < N) {
         const long long G = gridDim.y;
         part[((long long)0 * N + j) * G + blockIdx.y] = to_d(dyx0);
         part[((long long)0 * N + j + 1) * G + blockIdx.y] = to_d(dyx1);
@@ -302,7 +311,7 @@ __global__ void __launch_bounds__(128) k_block_stencil_f2(float2* __restrict__ y
 // computes rows 8h .. 8h + 7).  Each shared-memory read of a block entry serves four
 // rhs, 16 FMA per 8 bytes read, twice as many as with two rhs per thread, whose FMA pipe
 // waits on the shared-memory reads.  Per output the sums run in the same order as in
-// k_block_stencil_f2, so y is the same; the MODE 2 dots add the two halves last.
+// k_block_stencil_f2, so y is the same; the dots (MODE 2, 3) add the two halves last.
 // Block = 2 T threads with T = blockDim.x / 2 a multiple of 32; N % 4 == 0.
 template <int MODE>
 __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y, const float2* __restrict__ x,
@@ -310,7 +319,7 @@ __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y
                                                           int lx, int lt, int N, double2* __restrict__ part) {
     constexpr int D = 16, H = 8;
     __shared__ float2 At[5 * D * D];
-    __shared__ float red[MODE == 2 ? 64 * 12 : 1];     // half 1's dots, T <= 64
+    __shared__ float red[MODE >= 2 ? 64 * 12 : 1];     // half 1's dots, T <= 64
     const int T = blockDim.x >> 1;
     const int h = threadIdx.x >= T ? 1 : 0;
     const int tq = threadIdx.x - h * T;
@@ -372,9 +381,11 @@ __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y
                     o[2] = make_float2(b1v.x - o[2].x, b1v.y - o[2].y);
                     o[3] = make_float2(b1v.z - o[3].x, b1v.w - o[3].y);
                 }
-                *reinterpret_cast<float4*>(y + idx) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
-                *reinterpret_cast<float4*>(y + idx + 2) = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
-                if (MODE == 2) {
+                if (MODE != 3) {
+                    *reinterpret_cast<float4*>(y + idx) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+                    *reinterpret_cast<float4*>(y + idx + 2) = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
+                }
+                if (MODE >= 2) {
                     const float4 x0v = *reinterpret_cast<const float4*>(x + idx);
                     const float4 x1v = *reinterpret_cast<const float4*>(x + idx + 2);
                     const float2 xs[4] = {make_float2(x0v.x, x0v.y), make_float2(x0v.z, x0v.w),
@@ -388,7 +399,7 @@ __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE >= 2) {
         // half 1 hands its sums to half 0, which writes the per-rhs partials
         if (h == 1)
 #pragma unroll
@@ -440,14 +451,14 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
             }
             const long long idx = ((long long)site * D + c) * N + j;
             if (MODE == 1) acc = csub(b[idx], acc);
-            y[idx] = acc;
-            if (MODE == 2) {
+            if (MODE != 3) y[idx] = acc;
+            if (MODE >= 2) {
                 cfmac(dyx, acc, x[idx]);
                 dyy = fma(acc.x, acc.x, fma(acc.y, acc.y, dyy));
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE >= 2) {
         red[0][c][tx] = to_d(dyx);
         red[1][c][tx] = make_double2((double)dyy, 0.0);
         __syncthreads();
@@ -459,10 +470,21 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
     }
 }
 
-// y[s] (+)= Minv[s] x[s]: block = 128 rhs, one site per iteration, Minv[s] in
-// shared memory; generic d (<= 32).
+// y[s] (+)= Minv[s] sum_q alpha_q x_q[s] over the K residuals x_q of a group of smoother
+// steps (slots of the block x; K = 1 and no alpha: the plain product): block = 128 rhs,
+// one site per iteration, Minv[s] in shared memory; generic d (<= 32).
 template <typename C>
-__global__ void __launch_bounds__(128) k_block_diag_apply(C* __restrict__ y, const C* __restrict__ x,
+__device__ __forceinline__ C step_sum(const C* __restrict__ x, size_t slot, int K, const C* __restrict__ alpha,
+                                      long long idx, int j, int N) {
+    if (!alpha) return x[idx];
+    C acc = czero<C>();
+    for (int q = 0; q < K; ++q) cfma(acc, alpha[q * N + j], x[q * slot + idx]);
+    return acc;
+}
+
+template <typename C>
+__global__ void __launch_bounds__(128) k_block_diag_apply(C* __restrict__ y, const C* __restrict__ x, size_t slot,
+                                                          int K, const C* __restrict__ alpha,
                                                           const C* __restrict__ Minv, int nsites, int d, int N,
                                                           bool accumulate) {
     __shared__ C Ms[32 * 32];
@@ -473,7 +495,7 @@ __global__ void __launch_bounds__(128) k_block_diag_apply(C* __restrict__ y, con
         __syncthreads();
         if (j >= N) continue;
         C xv[32];
-        for (int b = 0; b < d; ++b) xv[b] = x[((long long)site * d + b) * N + j];
+        for (int b = 0; b < d; ++b) xv[b] = step_sum(x, slot, K, alpha, ((long long)site * d + b) * N + j, j, N);
         for (int c = 0; c < d; ++c) {
             C acc = accumulate ? y[((long long)site * d + c) * N + j] : czero<C>();
             for (int b = 0; b < d; ++b) cfma(acc, Ms[c * d + b], xv[b]);
@@ -485,7 +507,8 @@ __global__ void __launch_bounds__(128) k_block_diag_apply(C* __restrict__ y, con
 // The same with the block size fixed at compile time: the input column stays in
 // registers (a runtime d puts it in local memory), all loads issued before the FMAs.
 template <typename C, int D>
-__global__ void __launch_bounds__(128) k_block_diag_apply_d(C* __restrict__ y, const C* __restrict__ x,
+__global__ void __launch_bounds__(128) k_block_diag_apply_d(C* __restrict__ y, const C* __restrict__ x, size_t slot,
+                                                            int K, const C* __restrict__ alpha,
                                                             const C* __restrict__ Minv, int nsites, int N,
                                                             bool accumulate) {
     __shared__ C Ms[D * D];
@@ -496,33 +519,50 @@ __global__ void __launch_bounds__(128) k_block_diag_apply_d(C* __restrict__ y, c
         __syncthreads();
         if (j >= N) continue;
         C xv[D], acc[D];
+        const long long base = (long long)site * D * N + j;
+        if (alpha) {
 #pragma unroll
-        for (int b = 0; b < D; ++b) {
-            xv[b] = x[((long long)site * D + b) * N + j];
-            acc[b] = accumulate ? y[((long long)site * D + b) * N + j] : czero<C>();
+            for (int b = 0; b < D; ++b) xv[b] = czero<C>();
+            for (int q = 0; q < K; ++q) {
+                const C a = alpha[q * N + j];
+#pragma unroll
+                for (int b = 0; b < D; ++b) cfma(xv[b], a, x[q * slot + base + (long long)b * N]);
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < D; ++b) xv[b] = x[base + (long long)b * N];
         }
+#pragma unroll
+        for (int b = 0; b < D; ++b) acc[b] = accumulate ? y[base + (long long)b * N] : czero<C>();
 #pragma unroll
         for (int c = 0; c < D; ++c) {
 #pragma unroll
             for (int b = 0; b < D; ++b) cfma(acc[c], Ms[c * D + b], xv[b]);
-            y[((long long)site * D + c) * N + j] = acc[c];
+            y[base + (long long)c * N] = acc[c];
         }
     }
 }
 
 template <typename C>
-void launch_block_diag_apply(C* y, const C* x, const C* Minv, int nsites, int d, int N, bool accumulate,
-                             cudaStream_t s) {
+void launch_block_diag_combine(C* y, const C* x, size_t slot, int K, const C* alpha, const C* Minv, int nsites, int d,
+                               int N, bool accumulate, cudaStream_t s) {
     MG_REQUIRE(d <= 32, MGMLMC_EINVAL, "block-diagonal apply: d <= 32");
     const int th = cta_threads(N);
     const int tiles = (N + th - 1) / th;
     int G = 16 * kNumSM / tiles;
     if (G > nsites) G = nsites;
     if (G < 1) G = 1;
-    if (d == 16) k_block_diag_apply_d<C, 16><<<dim3(tiles, G), th, 0, s>>>(y, x, Minv, nsites, N, accumulate);
-    else if (d == 8) k_block_diag_apply_d<C, 8><<<dim3(tiles, G), th, 0, s>>>(y, x, Minv, nsites, N, accumulate);
-    else k_block_diag_apply<C><<<dim3(tiles, G), th, 0, s>>>(y, x, Minv, nsites, d, N, accumulate);
+    const dim3 g(tiles, G);
+    if (d == 16) k_block_diag_apply_d<C, 16><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, N, accumulate);
+    else if (d == 8) k_block_diag_apply_d<C, 8><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, N, accumulate);
+    else k_block_diag_apply<C><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, d, N, accumulate);
     MG_LAUNCHED();
+}
+
+template <typename C>
+void launch_block_diag_apply(C* y, const C* x, const C* Minv, int nsites, int d, int N, bool accumulate,
+                             cudaStream_t s) {
+    launch_block_diag_combine<C>(y, x, 0, 1, nullptr, Minv, nsites, d, N, accumulate, s);
 }
 
 // xc[S][o] = sum_{site in S} sum_{a in spin block s(o)} conj(P[site][a][j(o)]) x[site][a]
@@ -659,6 +699,17 @@ __global__ void __launch_bounds__(128) k_prolong_nv(C* __restrict__ x, const C* 
     }
 }
 
+// Row j of a site's BF16 operand tile (128 rhs x 16 complex values, K-major core
+// matrices of 8 rows x 16 bytes: the layout of the tensor-core stencil).
+__device__ __forceinline__ void store_bf16_row(uint8_t* xt, int site, int j, int N, const float2* v) {
+    const int T = (N + 127) / 128, r = j & 127;
+    uint8_t* row = xt + ((size_t)site * T + (j >> 7)) * 8192 + (r >> 3) * 512 + (r & 7) * 16;
+#pragma unroll
+    for (int cg = 0; cg < 4; ++cg)
+        *reinterpret_cast<uint4*>(row + cg * 128) =
+            make_uint4(f2_bf(v[4 * cg]), f2_bf(v[4 * cg + 1]), f2_bf(v[4 * cg + 2]), f2_bf(v[4 * cg + 3]));
+}
+
 // The same two operators with the dofs per fine site (D) fixed at compile time: the
 // loads of QB aggregate sites (QB * D values per thread) are issued together before
 // the FMAs, instead of one load per loop trip.
@@ -709,10 +760,12 @@ __global__ void __launch_bounds__(128) k_restrict_nvd(C* __restrict__ xc, const 
     }
 }
 
+// xt (FP32, D = 16; may be null): the BF16 operand tiles of the result as well (the
+// tensor-core residual reads them), so that no pass over x packs them later.
 template <typename C, int NV, int D, int QB>
 __global__ void __launch_bounds__(128) k_prolong_nvd(C* __restrict__ x, const C* __restrict__ xc,
                                                      const C* __restrict__ P, int lx, int lt, int ax, int at, int N,
-                                                     bool accumulate) {
+                                                     bool accumulate, uint8_t* __restrict__ xt) {
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     constexpr int HD = D / 2;
@@ -754,31 +807,144 @@ __global__ void __launch_bounds__(128) k_prolong_nvd(C* __restrict__ x, const C*
                     for (int jv = 0; jv < NV; ++jv) cfma(ov[qq][a], Pq[a * NV + jv], cv[(a < HD ? 0 : NV) + jv]);
                     x[((long long)site * D + a) * N + j] = ov[qq][a];
                 }
+                if constexpr (sizeof(C) == 8 && D == 16) {
+                    if (xt) store_bf16_row(xt, site, j, N, ov[qq]);
+                }
             }
         }
     }
 }
 
-template <typename C>
-__global__ void k_mr_update(C* __restrict__ e, C* __restrict__ r, const C* __restrict__ p,
-                            const double2* __restrict__ dots, long long n, int N, bool e_is_zero) {
-    using R = re_t<C>;
-    const int j = blockIdx.x * kRhsTile + threadIdx.x;
+// The minimal-residual smoother keeps the residuals r_0 .. r_{K-1} of a group of steps
+// (rs, one slot of n x N each) and adds sum_s alpha_s r_s to the correction once per
+// group, instead of reading and writing the correction in every step: a step moves r and
+// p in and the next r out (3 vectors instead of 5), and the last step of all forms no
+// residual.  The sums run over the steps in order, as the step-by-step updates did.
+// All are bound by HBM (or L2); V values of one row per thread in 16-byte accesses where
+// N allows.  A block is bx x (256 / bx) threads with bx the power of two that covers the
+// N / V columns (at most 32), so that narrow blocks keep every lane busy.
+template <typename T, int V> struct alignas(sizeof(T) * V) VecOf { T v[V]; };
+
+// rn = r - alpha p (rn may be r: every value is read before its place is written)
+template <typename C, int V>
+__global__ void __launch_bounds__(256) k_mr_update(C* rn, const C* r, const C* __restrict__ p,
+                                                   const C* __restrict__ alpha, long long n, int N) {
+    const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
-    const double2 pr = dots[j];
-    const double pp = dots[N + j].x;
-    const double2 al = (pp > 0.0) ? make_double2(pr.x / pp, pr.y / pp) : make_double2(0.0, 0.0);
-    const C a = mk((R)al.x, (R)al.y);
-    for (long long i = (long long)blockIdx.y * kRowLanes + threadIdx.y; i < n;
-         i += (long long)gridDim.y * kRowLanes) {
-        const long long idx = i * N + j;
-        const C rv = r[idx];
-        C ev = e_is_zero ? czero<C>() : e[idx];
-        cfma(ev, a, rv);
-        e[idx] = ev;
-        C rn = rv;
-        C ap = cmul(a, p[idx]);
-        r[idx] = csub(rn, ap);
+    C a[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) a[q] = alpha[j + q];
+    const long long S = (long long)gridDim.y * blockDim.y;
+    for (long long i0 = (long long)blockIdx.y * blockDim.y + threadIdx.y; i0 < n; i0 += 2 * S) {
+        VecOf<C, V> rv[2], pv[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long i = i0 + u * S;
+            if (i < n) {
+                rv[u] = *reinterpret_cast<const VecOf<C, V>*>(r + i * N + j);
+                pv[u] = *reinterpret_cast<const VecOf<C, V>*>(p + i * N + j);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long i = i0 + u * S;
+            if (i < n) {
+#pragma unroll
+                for (int q = 0; q < V; ++q) rv[u].v[q] = csub(rv[u].v[q], cmul(a[q], pv[u].v[q]));
+                *reinterpret_cast<VecOf<C, V>*>(rn + i * N + j) = rv[u];
+            }
+        }
+    }
+}
+
+// e (=|+=) sum_{s < K} alpha_s r_s
+constexpr int kMrGroup = 8;   // as in the solver's group loop
+template <typename C, int V>
+__global__ void __launch_bounds__(256) k_mr_combine(C* __restrict__ e, const C* __restrict__ rs, size_t slot, int K,
+                                                    const C* __restrict__ alpha, long long n, int N, bool e_is_zero) {
+    const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (j >= N) return;
+    for (long long i = (long long)blockIdx.y * blockDim.y + threadIdx.y; i < n;
+         i += (long long)gridDim.y * blockDim.y) {
+        VecOf<C, V> rv[kMrGroup], ev;
+#pragma unroll
+        for (int s = 0; s < kMrGroup; ++s)
+            if (s < K) rv[s] = *reinterpret_cast<const VecOf<C, V>*>(rs + s * slot + i * N + j);
+        if (!e_is_zero) ev = *reinterpret_cast<const VecOf<C, V>*>(e + i * N + j);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            C acc = e_is_zero ? czero<C>() : ev.v[q];
+#pragma unroll
+            for (int s = 0; s < kMrGroup; ++s)
+                if (s < K) cfma(acc, alpha[s * N + j + q], rv[s].v[q]);
+            ev.v[q] = acc;
+        }
+        *reinterpret_cast<VecOf<C, V>*>(e + i * N + j) = ev;
+    }
+}
+
+// The same two with the residuals and the image in BF16 (one bf16x2 word per complex
+// value), four rhs per thread: 16-byte accesses.  N % 4 == 0.
+__global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* __restrict__ rn,
+                                                             const uint32_t* __restrict__ r,
+                                                             const uint32_t* __restrict__ p,
+                                                             const float2* __restrict__ alpha, long long n, int N) {
+    const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (j >= N) return;
+    float2 a[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = alpha[j + q];
+    const long long S = (long long)gridDim.y * blockDim.y;
+    for (long long i0 = (long long)blockIdx.y * blockDim.y + threadIdx.y; i0 < n; i0 += 2 * S) {
+        VecOf<uint32_t, 4> rv[2], pv[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long i = i0 + u * S;
+            if (i < n) {
+                rv[u] = *reinterpret_cast<const VecOf<uint32_t, 4>*>(r + i * N + j);
+                pv[u] = *reinterpret_cast<const VecOf<uint32_t, 4>*>(p + i * N + j);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long i = i0 + u * S;
+            if (i < n) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    rv[u].v[q] = f2_bf(csub(bf2_lo(rv[u].v[q]), cmul(a[q], bf2_lo(pv[u].v[q]))));
+                *reinterpret_cast<VecOf<uint32_t, 4>*>(rn + i * N + j) = rv[u];
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_mr_combine_bf16(float2* __restrict__ e, const uint32_t* __restrict__ rs,
+                                                         size_t slot, int K, const float2* __restrict__ alpha,
+                                                         long long n, int N, bool e_is_zero) {
+    const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (j >= N) return;
+    for (long long i = (long long)blockIdx.y * blockDim.y + threadIdx.y; i < n;
+         i += (long long)gridDim.y * blockDim.y) {
+        VecOf<uint32_t, 4> rv[kMrGroup];
+        VecOf<float2, 2> ev[2];
+        float2* er = e + i * N + j;
+#pragma unroll
+        for (int s = 0; s < kMrGroup; ++s)
+            if (s < K) rv[s] = *reinterpret_cast<const VecOf<uint32_t, 4>*>(rs + s * slot + i * N + j);
+        if (!e_is_zero) {
+            ev[0] = *reinterpret_cast<const VecOf<float2, 2>*>(er);
+            ev[1] = *reinterpret_cast<const VecOf<float2, 2>*>(er + 2);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float2 acc = e_is_zero ? make_float2(0.f, 0.f) : ev[q >> 1].v[q & 1];
+#pragma unroll
+            for (int s = 0; s < kMrGroup; ++s)
+                if (s < K) cfma(acc, alpha[s * N + j + q], bf2_lo(rv[s].v[q]));
+            ev[q >> 1].v[q & 1] = acc;
+        }
+        *reinterpret_cast<VecOf<float2, 2>*>(er) = ev[0];
+        *reinterpret_cast<VecOf<float2, 2>*>(er + 2) = ev[1];
     }
 }
 
@@ -805,8 +971,10 @@ int stencil_groups_bf16(int nsites, int N) {
     return (int)std::max(1LL, std::min(need, 3LL * kNumSM / gx));
 }
 
+
 // FP32 Wilson operator with two rhs per thread: 16-byte loads and stores (a warp
 // moves 512 B per access), half the index arithmetic per rhs.  N even.
+// MODE 4: the residual b - D x rounded to BF16 (one bf16x2 word per complex value).
 template <int MODE>
 __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const float2* __restrict__ x,
                                                    const float2* __restrict__ b, const float2* __restrict__ U,
@@ -869,7 +1037,7 @@ __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const
                     o1[r] = csub(o1[r], ctimesi(u));
                 }
             }
-            if (MODE == 1) {
+            if (MODE == 1 || MODE == 4) {
                 float2 b0[2], b1[2];
                 ld2(b, site * N2 + j, b0[0], b0[1]);
                 ld2(b, site * N2 + N + j, b1[0], b1[1]);
@@ -879,9 +1047,15 @@ __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const
                     o1[r] = csub(b1[r], o1[r]);
                 }
             }
-            *reinterpret_cast<float4*>(y + site * N2 + j) = make_float4(o0[0].x, o0[0].y, o0[1].x, o0[1].y);
-            *reinterpret_cast<float4*>(y + site * N2 + N + j) = make_float4(o1[0].x, o1[0].y, o1[1].x, o1[1].y);
-            if (MODE == 2) {
+            if (MODE == 4) {
+                uint32_t* yb = reinterpret_cast<uint32_t*>(y);
+                *reinterpret_cast<uint2*>(yb + site * N2 + j) = make_uint2(f2_bf(o0[0]), f2_bf(o0[1]));
+                *reinterpret_cast<uint2*>(yb + site * N2 + N + j) = make_uint2(f2_bf(o1[0]), f2_bf(o1[1]));
+            } else if (MODE != 3) {
+                *reinterpret_cast<float4*>(y + site * N2 + j) = make_float4(o0[0].x, o0[0].y, o0[1].x, o0[1].y);
+                *reinterpret_cast<float4*>(y + site * N2 + N + j) = make_float4(o1[0].x, o1[0].y, o1[1].x, o1[1].y);
+            }
+            if (MODE == 2 || MODE == 3) {
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     cfmac(dyx[r], o0[r], p0[r]);
@@ -892,7 +1066,7 @@ __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const
             }
         }
     }
-    if (MODE == 2) {
+    if (MODE == 2 || MODE == 3) {
         __shared__ double2 sh[2][kRowLanes][2 * kRhsTile + 1];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -923,7 +1097,8 @@ bool wilson_f2<float2>(float2* y, const float2* x, const float2* b, const float2
     switch (mode) {
         case 0: k_wilson_f2<0><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
         case 1: k_wilson_f2<1><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        default: k_wilson_f2<2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        case 2: k_wilson_f2<2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        default: k_wilson_f2<3><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
     return true;
@@ -934,17 +1109,13 @@ bool wilson_f2<float2>(float2* y, const float2* x, const float2* b, const float2
 // one bf16x2 per complex value): the operator y = D x with the MR dots
 // conj(y).x, |y|^2 (FP32 arithmetic, two rhs per thread, 8-byte accesses), the
 // FP32 -> BF16 packing and the MR update e (=|+=) alpha r, r -= alpha p.
-__device__ __forceinline__ float2 bf2_lo(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
-__device__ __forceinline__ uint32_t f2_bf(float2 v) {
-    const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
-    return *reinterpret_cast<const uint32_t*>(&b);
-}
 
 // Four rhs per thread: 16-byte accesses (four bf16x2 words), ten loads of a site in
 // flight per thread.  N % 4 == 0.
 // RPT right-hand sides per thread (4: 16-byte accesses, a warp spans 128 rhs; 2: 8-byte
 // accesses, 64 rhs, so that a block of 64 keeps every lane busy).
-template <int RPT>
+// STORE = false: the dots only (the last minimal-residual step needs no image).
+template <int RPT, bool STORE>
 __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y, const uint32_t* __restrict__ x,
                                                         const float2* __restrict__ U, float mass, int lx, int lt,
                                                         int N, double2* __restrict__ part) {
@@ -1023,7 +1194,8 @@ __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y
                 w0[r] = f2_bf(o0);
                 w1[r] = f2_bf(o1);
             }
-            if constexpr (RPT == 4) {
+            if constexpr (!STORE) {
+            } else if constexpr (RPT == 4) {
                 *reinterpret_cast<uint4*>(y + site * N2 + j) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
                 *reinterpret_cast<uint4*>(y + site * N2 + N + j) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
             } else {
@@ -1053,85 +1225,26 @@ __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y
     }
 }
 
-__global__ void k_pack_bf16(uint32_t* __restrict__ y, const float2* __restrict__ x, long long count) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < count) y[i] = f2_bf(x[i]);
-}
-
-// Two rhs per thread: 8-byte BF16 and 16-byte FP32 accesses; two rows per loop trip
-// with all their loads issued first.  N even.
-__global__ void k_mr_update_fine_bf16(float2* __restrict__ e, uint32_t* __restrict__ r, const uint32_t* __restrict__ p,
-                                      const double2* __restrict__ dots, long long n, int N, bool e_is_zero) {
-    const int j = 2 * (blockIdx.x * kRhsTile + threadIdx.x);
-    if (j >= N) return;
-    float2 a[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const double2 pr = dots[j + q];
-        const double pp = dots[N + j + q].x;
-        a[q] = pp > 0.0 ? make_float2((float)(pr.x / pp), (float)(pr.y / pp)) : make_float2(0.f, 0.f);
-    }
-    const long long S = (long long)gridDim.y * kRowLanes;
-    for (long long i0 = (long long)blockIdx.y * kRowLanes + threadIdx.y; i0 < n; i0 += 2 * S) {
-        uint2 rw[2], pw[2];
-        float4 ev[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const long long i = i0 + u * S;
-            const bool in = i < n;
-            const long long idx = i * N + j;
-            rw[u] = in ? *reinterpret_cast<const uint2*>(r + idx) : make_uint2(0u, 0u);
-            pw[u] = in ? *reinterpret_cast<const uint2*>(p + idx) : make_uint2(0u, 0u);
-            ev[u] = (in && !e_is_zero) ? *reinterpret_cast<const float4*>(e + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const long long i = i0 + u * S;
-            if (i >= n) break;
-            const long long idx = i * N + j;
-            const float2 r0 = bf2_lo(rw[u].x), r1 = bf2_lo(rw[u].y), p0 = bf2_lo(pw[u].x), p1 = bf2_lo(pw[u].y);
-            float2 e0 = make_float2(ev[u].x, ev[u].y), e1 = make_float2(ev[u].z, ev[u].w);
-            cfma(e0, a[0], r0);
-            cfma(e1, a[1], r1);
-            *reinterpret_cast<float4*>(e + idx) = make_float4(e0.x, e0.y, e1.x, e1.y);
-            *reinterpret_cast<uint2*>(r + idx) =
-                make_uint2(f2_bf(csub(r0, cmul(a[0], p0))), f2_bf(csub(r1, cmul(a[1], p1))));
-        }
-    }
-}
-
 void launch_wilson_bf16(uint32_t* y, const uint32_t* x, const float2* U, double m0, int lx, int lt, int N,
                         double2* part, int groups, cudaStream_t s) {
     MG_REQUIRE(N % 4 == 0, MGMLMC_EINVAL, "BF16 Wilson operator: N a multiple of 4");
     if (N % 128 == 0) {
         dim3 g(N / 128, groups);
-        k_wilson_bf16<4><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        if (y) k_wilson_bf16<4, true><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        else k_wilson_bf16<4, false><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
     } else {
         dim3 g((N / 2 + kRhsTile - 1) / kRhsTile, groups);
-        k_wilson_bf16<2><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        if (y) k_wilson_bf16<2, true><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        else k_wilson_bf16<2, false><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
     }
     MG_LAUNCHED();
 }
 
-void launch_pack_bf16(uint32_t* y, const float2* x, long long count, cudaStream_t s) {
-    k_pack_bf16<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(y, x, count);
-    MG_LAUNCHED();
-}
-
-void launch_mr_update_fine_bf16(float2* e, uint32_t* r, const uint32_t* p, const double2* dots, long long n, int N,
-                                bool e_is_zero, cudaStream_t s) {
-    MG_REQUIRE(N % 2 == 0, MGMLMC_EINVAL, "BF16 MR update: N even");
-    // N / 64 column blocks (two rhs per thread): row groups for one wave of as many CTAs
-    // per SM as are resident
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mr_update_fine_bf16, kRhsTile * kRowLanes, 0));
-        per_sm = std::max(1, per_sm);
-    }
-    const int gx = (N / 2 + kRhsTile - 1) / kRhsTile;
-    const long long need = (n + kRowLanes - 1) / kRowLanes;
-    const int gy = (int)std::max(1LL, std::min(need, (long long)per_sm * kNumSM / gx));
-    k_mr_update_fine_bf16<<<dim3(gx, gy), blk(), 0, s>>>(e, r, p, dots, n, N, e_is_zero);
+void launch_wilson_residual_bf16(uint32_t* y, const float2* x, const float2* b, const float2* U, double m0, int lx,
+                                 int lt, int N, int groups, cudaStream_t s) {
+    MG_REQUIRE(N % 2 == 0, MGMLMC_EINVAL, "BF16 Wilson residual: N even");
+    dim3 g((N / 2 + kRhsTile - 1) / kRhsTile, groups);
+    k_wilson_f2<4><<<g, blk(), 0, s>>>(reinterpret_cast<float2*>(y), x, b, U, (float)(m0 + 2.0), lx, lt, N, nullptr);
     MG_LAUNCHED();
 }
 
@@ -1145,7 +1258,8 @@ void launch_wilson(C* y, const C* x, const C* b, const C* U, double m0, int lx, 
     switch (mode) {
         case 0: k_wilson<C, 0><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
         case 1: k_wilson<C, 1><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        default: k_wilson<C, 2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        case 2: k_wilson<C, 2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        default: k_wilson<C, 3><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
 }
@@ -1161,11 +1275,13 @@ static void bs_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int lt
         MG_CUDA(cudaFuncSetAttribute(k_block_stencil<C, RPT, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         MG_CUDA(cudaFuncSetAttribute(k_block_stencil<C, RPT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         MG_CUDA(cudaFuncSetAttribute(k_block_stencil<C, RPT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        MG_CUDA(cudaFuncSetAttribute(k_block_stencil<C, RPT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     }
     switch (mode) {
         case 0: k_block_stencil<C, RPT, 0><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
         case 1: k_block_stencil<C, RPT, 1><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
-        default: k_block_stencil<C, RPT, 2><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
+        case 2: k_block_stencil<C, RPT, 2><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
+        default: k_block_stencil<C, RPT, 3><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
     }
     MG_LAUNCHED();
 }
@@ -1181,7 +1297,8 @@ static bool bsd_f2(float2* y, const float2* x, const float2* b, const float2* A,
         switch (mode) {
             case 0: k_block_stencil_f4<0><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
             case 1: k_block_stencil_f4<1><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-            default: k_block_stencil_f4<2><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+            case 2: k_block_stencil_f4<2><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+            default: k_block_stencil_f4<3><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
         }
         MG_LAUNCHED();
         return true;
@@ -1191,7 +1308,8 @@ static bool bsd_f2(float2* y, const float2* x, const float2* b, const float2* A,
     switch (mode) {
         case 0: k_block_stencil_f2<D, 0><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
         case 1: k_block_stencil_f2<D, 1><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        default: k_block_stencil_f2<D, 2><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 2: k_block_stencil_f2<D, 2><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        default: k_block_stencil_f2<D, 3><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
     return true;
@@ -1211,9 +1329,22 @@ static void bsd_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int l
     switch (mode) {
         case 0: k_block_stencil_d<C, D, 0><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
         case 1: k_block_stencil_d<C, D, 1><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        default: k_block_stencil_d<C, D, 2><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 2: k_block_stencil_d<C, D, 2><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        default: k_block_stencil_d<C, D, 3><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
+}
+
+template <typename C, int D>
+static void bsn_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int lt, int N, int mode, double2* part,
+                         int groups, cudaStream_t s) {
+    const dim3 g((N + 7) / 8, groups), th(8, D);
+    switch (mode) {
+        case 0: k_block_stencil_narrow<C, D, 0><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 1: k_block_stencil_narrow<C, D, 1><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 2: k_block_stencil_narrow<C, D, 2><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        default: k_block_stencil_narrow<C, D, 3><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+    }
 }
 
 // The one-rhs-per-thread kernels need wide blocks; narrow blocks (the setup solves
@@ -1241,16 +1372,8 @@ void launch_block_stencil(C* y, const C* x, const C* b, const C* A, int lx, int 
                           double2* part, int groups, cudaStream_t s) {
     MG_REQUIRE(d >= 2 && d <= 64, MGMLMC_EINVAL, "block stencil: 2 <= d <= 64");
     if (use_narrow_kernel(d, N)) {
-        dim3 g((N + 7) / 8, groups);
-        if (d == 16) {
-            if (mode == 0) k_block_stencil_narrow<C, 16, 0><<<g, dim3(8, 16), 0, s>>>(y, x, b, A, lx, lt, N, part);
-            else if (mode == 1) k_block_stencil_narrow<C, 16, 1><<<g, dim3(8, 16), 0, s>>>(y, x, b, A, lx, lt, N, part);
-            else k_block_stencil_narrow<C, 16, 2><<<g, dim3(8, 16), 0, s>>>(y, x, b, A, lx, lt, N, part);
-        } else {
-            if (mode == 0) k_block_stencil_narrow<C, 8, 0><<<g, dim3(8, 8), 0, s>>>(y, x, b, A, lx, lt, N, part);
-            else if (mode == 1) k_block_stencil_narrow<C, 8, 1><<<g, dim3(8, 8), 0, s>>>(y, x, b, A, lx, lt, N, part);
-            else k_block_stencil_narrow<C, 8, 2><<<g, dim3(8, 8), 0, s>>>(y, x, b, A, lx, lt, N, part);
-        }
+        if (d == 16) bsn_dispatch<C, 16>(y, x, b, A, lx, lt, N, mode, part, groups, s);
+        else bsn_dispatch<C, 8>(y, x, b, A, lx, lt, N, mode, part, groups, s);
         MG_LAUNCHED();
         return;
     }
@@ -1264,7 +1387,7 @@ void launch_block_stencil(C* y, const C* x, const C* b, const C* A, int lx, int 
 
 template <typename C, int NV>
 static void rp_launch(bool restrict_op, C* xc_or_x, const C* in, const C* P, int lx, int lt, int d, int ax, int at,
-                      int N, bool accumulate, cudaStream_t s) {
+                      int N, bool accumulate, uint8_t* xt, cudaStream_t s) {
     const int ncs = (lx / ax) * (lt / at);
     const int th = cta_threads(N);
     const int tiles = (N + th - 1) / th;
@@ -1274,13 +1397,13 @@ static void rp_launch(bool restrict_op, C* xc_or_x, const C* in, const C* P, int
     const size_t sm = (size_t)ax * at * d * NV * sizeof(C);
     if (d == 2) {
         if (restrict_op) k_restrict_nvd<C, NV, 2, 4><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N);
-        else k_prolong_nvd<C, NV, 2, 4><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate);
+        else k_prolong_nvd<C, NV, 2, 4><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr);
         MG_LAUNCHED();
         return;
     }
     if (d == 16) {
         if (restrict_op) k_restrict_nvd<C, NV, 16, 1><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N);
-        else k_prolong_nvd<C, NV, 16, 1><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate);
+        else k_prolong_nvd<C, NV, 16, 1><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt);
         MG_LAUNCHED();
         return;
     }
@@ -1293,12 +1416,12 @@ static void rp_launch(bool restrict_op, C* xc_or_x, const C* in, const C* P, int
 
 template <typename C>
 static bool rp_fast(bool restrict_op, C* out, const C* in, const C* P, int lx, int lt, int d, int ax, int at,
-                    int nvec, int N, bool accumulate, cudaStream_t s) {
+                    int nvec, int N, bool accumulate, uint8_t* xt, cudaStream_t s) {
     if ((size_t)ax * at * d * nvec * sizeof(C) > 48 * 1024) return false;
     switch (nvec) {
-        case 2: rp_launch<C, 2>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, s); return true;
-        case 4: rp_launch<C, 4>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, s); return true;
-        case 8: rp_launch<C, 8>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, s); return true;
+        case 2: rp_launch<C, 2>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, xt, s); return true;
+        case 4: rp_launch<C, 4>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, xt, s); return true;
+        case 8: rp_launch<C, 8>(restrict_op, out, in, P, lx, lt, d, ax, at, N, accumulate, xt, s); return true;
         default: return false;
     }
 }
@@ -1306,7 +1429,7 @@ static bool rp_fast(bool restrict_op, C* out, const C* in, const C* P, int lx, i
 template <typename C>
 void launch_restrict(C* xc, const C* x, const C* P, int lx, int lt, int d, int ax, int at, int nvec, int N,
                      cudaStream_t s) {
-    if (rp_fast<C>(true, xc, x, P, lx, lt, d, ax, at, nvec, N, false, s)) return;
+    if (rp_fast<C>(true, xc, x, P, lx, lt, d, ax, at, nvec, N, false, nullptr, s)) return;
     const int ncs = (lx / ax) * (lt / at);
     int G = row_groups((long long)ncs * kRowLanes, N, 4);
     k_restrict<C><<<dim3(rhs_tiles(N), G), blk(), 0, s>>>(xc, x, P, lx, lt, d, ax, at, nvec, N);
@@ -1314,19 +1437,72 @@ void launch_restrict(C* xc, const C* x, const C* P, int lx, int lt, int d, int a
 }
 
 template <typename C>
-void launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax, int at, int nvec, int N,
-                    bool accumulate, cudaStream_t s) {
-    if (rp_fast<C>(false, x, xc, P, lx, lt, d, ax, at, nvec, N, accumulate, s)) return;
+bool launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax, int at, int nvec, int N,
+                    bool accumulate, cudaStream_t s, void* xt) {
+    uint8_t* tiles = (sizeof(C) == 8 && d == 16) ? reinterpret_cast<uint8_t*>(xt) : nullptr;
+    if (rp_fast<C>(false, x, xc, P, lx, lt, d, ax, at, nvec, N, accumulate, tiles, s)) return tiles != nullptr;
     const long long rows = (long long)lx * lt * d;
     k_prolong<C><<<dim3(rhs_tiles(N), row_groups(rows, N)), blk(), 0, s>>>(x, xc, P, lx, lt, d, ax, at, nvec, N,
                                                                              accumulate);
     MG_LAUNCHED();
+    return false;
+}
+
+// Block shape and grid of the row kernels above: V values per thread along the rhs, at
+// most `per_sm` CTAs of 256 threads per SM.
+static void row_shape(long long n, int N, int V, int per_sm, dim3& g, dim3& b) {
+    const int cols = (N + V - 1) / V;
+    int bx = 1;
+    while (bx < cols && bx < 32) bx *= 2;
+    const int by = 256 / bx, gx = (cols + bx - 1) / bx;
+    const long long need = (n + by - 1) / by;
+    g = dim3(gx, (unsigned)std::max(1LL, std::min(need, (long long)per_sm * kNumSM / gx)));
+    b = dim3(bx, by);
 }
 
 template <typename C>
-void launch_mr_update(C* e, C* r, const C* p, const double2* dots, long long n, int N, bool e_is_zero,
-                      cudaStream_t s) {
-    k_mr_update<C><<<dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s>>>(e, r, p, dots, n, N, e_is_zero);
+void launch_mr_update(C* rn, const C* r, const C* p, const C* alpha, long long n, int N, cudaStream_t s) {
+    dim3 g, b;
+    if (sizeof(C) == 8 && N % 2 == 0) {
+        row_shape(n, N, 2, 8, g, b);
+        k_mr_update<C, sizeof(C) == 8 ? 2 : 1><<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+    } else {
+        row_shape(n, N, 1, 8, g, b);
+        k_mr_update<C, 1><<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+    }
+    MG_LAUNCHED();
+}
+
+template <typename C>
+void launch_mr_combine(C* e, const C* rs, size_t slot, int K, const C* alpha, long long n, int N, bool e_is_zero,
+                       cudaStream_t s) {
+    MG_REQUIRE(K >= 1 && K <= kMrGroup, MGMLMC_EINVAL, "smoother: group size");
+    dim3 g, b;
+    if (sizeof(C) == 8 && N % 2 == 0) {
+        row_shape(n, N, 2, 8, g, b);
+        k_mr_combine<C, sizeof(C) == 8 ? 2 : 1><<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
+    } else {
+        row_shape(n, N, 1, 8, g, b);
+        k_mr_combine<C, 1><<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
+    }
+    MG_LAUNCHED();
+}
+
+void launch_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r, const uint32_t* p, const float2* alpha, long long n,
+                                int N, cudaStream_t s) {
+    MG_REQUIRE(N % 4 == 0, MGMLMC_EINVAL, "BF16 MR update: N a multiple of 4");
+    dim3 g, b;
+    row_shape(n, N, 4, 8, g, b);
+    k_mr_update_fine_bf16<<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+    MG_LAUNCHED();
+}
+
+void launch_mr_combine_bf16(float2* e, const uint32_t* rs, size_t slot, int K, const float2* alpha, long long n, int N,
+                            bool e_is_zero, cudaStream_t s) {
+    MG_REQUIRE(N % 4 == 0 && K >= 1 && K <= kMrGroup, MGMLMC_EINVAL, "BF16 MR sum: N a multiple of 4, group size");
+    dim3 g, b;
+    row_shape(n, N, 4, 8, g, b);
+    k_mr_combine_bf16<<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
     MG_LAUNCHED();
 }
 
@@ -1344,10 +1520,13 @@ void launch_gamma5(C* y, const C* x, long long nsites, int d, int N, cudaStream_
                                           double2*, int, cudaStream_t);                                 \
     template void launch_restrict<C>(C*, const C*, const C*, int, int, int, int, int, int, int,         \
                                      cudaStream_t);                                                     \
-    template void launch_prolong<C>(C*, const C*, const C*, int, int, int, int, int, int, int, bool,    \
-                                    cudaStream_t);                                                      \
-    template void launch_mr_update<C>(C*, C*, const C*, const double2*, long long, int, bool,           \
-                                      cudaStream_t);                                                    \
+    template bool launch_prolong<C>(C*, const C*, const C*, int, int, int, int, int, int, int, bool,    \
+                                    cudaStream_t, void*);                                               \
+    template void launch_mr_update<C>(C*, const C*, const C*, const C*, long long, int, cudaStream_t);  \
+    template void launch_mr_combine<C>(C*, const C*, size_t, int, const C*, long long, int, bool,       \
+                                       cudaStream_t);                                                   \
+    template void launch_block_diag_combine<C>(C*, const C*, size_t, int, const C*, const C*, int, int, \
+                                               int, bool, cudaStream_t);                                \
     template void launch_gamma5<C>(C*, const C*, long long, int, int, cudaStream_t);                  \
     template void launch_block_diag_apply<C>(C*, const C*, const C*, int, int, int, bool, cudaStream_t);
 INST(double2)

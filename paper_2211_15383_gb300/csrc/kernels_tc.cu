@@ -536,11 +536,12 @@ namespace tc {
 //
 // The input of the stencil is not the FP32 vector itself but its BF16 copy
 // stored in the MMA's own operand layout: per site and 128-rhs tile, an 8 KB
-// K-major tile whose row j is the 16 complex components of rhs j (pad rows of a
-// partial last tile are zero).  The kernels that produce the smoother's
-// residuals write that copy as they go (k_pack_tiles for the first one,
-// k_mr_update_tc for the next ones), so the stencil moves 8 KB blocks straight
-// into shared memory and never converts.
+// K-major tile whose row j is the 16 complex components of rhs j (the pad rows of a
+// partial last tile hold anything: they only reach the pad rows of the product).  The
+// kernels that produce the smoother's operands write that copy as they go (the
+// prolongation and the residual form of the stencil, k_mr_update_tiles for the next
+// residuals), so the stencil moves 8 KB blocks straight into shared memory and never
+// converts.
 //
 // Warp-specialised and persistent: three CTAs per SM, each over one 128-rhs tile
 // and a strided set of sites; a CTA's work is a sequence of jobs (site,
@@ -595,7 +596,8 @@ __global__ void k_embed_stencil(__nv_bfloat16* __restrict__ E, const float2* __r
     E[sd * (KD * KD) + kmaj32_off(n, k) / 2] = __float2bfloat16(v);
 }
 
-// BF16 tiles of x: rt[(site * T + t) * 4096 + off / 2], zero rows for rhs >= N.
+// BF16 tiles of x: rt[(site * T + t) * 4096 + off / 2], zero rows for rhs >= N (a whole
+// 128-row tile).
 // Thread = (site, component group of 4, rhs): four FP32 loads, one 16-byte store.
 // Grid: x = (site, component group), y = 128-rhs tile.
 __global__ void k_pack_tiles(__nv_bfloat16* __restrict__ rt, const float2* __restrict__ x, int nsites, int N) {
@@ -616,23 +618,19 @@ __global__ void k_pack_tiles(__nv_bfloat16* __restrict__ rt, const float2* __res
     (void)nsites;
 }
 
-// Minimal-residual update of the block-Jacobi smoother (alpha = dots[j] / dots[N + j]):
+// Minimal-residual update of the pre-smoother, whose caller needs the final residual:
 // yh (=|+=) alpha r, r -= alpha p, and (rt != null) the BF16 tiles of the new r.
 // Thread = (site, rhs): the 16 rows of the site, four 16-byte tile pieces.
 __global__ void __launch_bounds__(CH) k_mr_update_tc(float2* __restrict__ yh, float2* __restrict__ r,
-                                                    const float2* __restrict__ p, const double2* __restrict__ dots,
+                                                    const float2* __restrict__ p, const float2* __restrict__ alpha,
                                                     int N, bool first, __nv_bfloat16* __restrict__ rt) {
     const int T = gridDim.y, tt = blockIdx.y;     // grid: x = site, y = 128-rhs tile
     const int j = tt * CH + threadIdx.x;
     const int site = blockIdx.x;
     float ax = 0.f, ay = 0.f;
     if (j < N) {
-        const double2 pr = dots[j];
-        const double pp = dots[N + j].x;
-        if (pp > 0.0) {
-            ax = (float)(pr.x / pp);
-            ay = (float)(pr.y / pp);
-        }
+        ax = alpha[j].x;
+        ay = alpha[j].y;
     }
     uint8_t* tile = rt ? reinterpret_cast<uint8_t*>(rt) + ((size_t)site * T + tt) * TILE_A : nullptr;
     // all loads of the thread first (memory-level parallelism), then the arithmetic
@@ -668,49 +666,95 @@ __global__ void __launch_bounds__(CH) k_mr_update_tc(float2* __restrict__ yh, fl
     }
 }
 
-// Minimal-residual update with r and p held only as BF16 tiles (the smoother's
-// residual needs no more than a few digits): yh (=|+=) alpha r (FP32), r -= alpha p
-// (BF16 tiles, in place).  Thread = (site, rhs): one row of each tile.
-__global__ void __launch_bounds__(CH) k_mr_update_bf16(float2* __restrict__ yh, __nv_bfloat16* __restrict__ rt,
-                                                      const __nv_bfloat16* __restrict__ pt,
-                                                      const double2* __restrict__ dots, int N, bool first) {
-    const int T = gridDim.y, tt = blockIdx.y;     // grid: x = site, y = 128-rhs tile
-    const int jl = threadIdx.x, j = tt * CH + jl;
-    const int site = blockIdx.x;
-    if (j >= N) return;                           // pad rows stay zero
-    const double2 pr = dots[j];
-    const double pp = dots[N + j].x;
-    const float ax = pp > 0.0 ? (float)(pr.x / pp) : 0.f, ay = pp > 0.0 ? (float)(pr.y / pp) : 0.f;
-    const size_t toff = ((size_t)site * T + tt) * TILE_A;
-    uint8_t* rrow = reinterpret_cast<uint8_t*>(rt) + toff;
-    const uint8_t* prow = reinterpret_cast<const uint8_t*>(pt) + toff;
-    uint4 rw[4], pw[4];
+// Minimal-residual update with r and p held only as BF16 tiles (the smoother's residual
+// needs no more than a few digits): rn = r - alpha p.  The correction is not touched: the
+// residuals of a group of steps stay in their own slots, and k_block_diag_tiles adds
+// M^{-1} sum_s alpha_s r_s once per group.  A step moves 12 B per complex value instead of
+// 28, and the last one none.  One warp per 8-row group of a tile (512 contiguous bytes,
+// 16 B per lane: row lane & 7), four groups in flight; only the row groups that hold rhs
+// are touched.  Bound by HBM, or by L2 where the tiles fit it.
+__global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* __restrict__ rn, const uint4* __restrict__ r,
+                                                         const uint4* __restrict__ p,
+                                                         const float2* __restrict__ alpha, int nsites, int N, int T) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+    const int G8 = (N + 7) >> 3;                  // row groups of a site
+    const long long chunks = (long long)nsites * G8;
+    const long long W = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long c0 = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c0 < chunks; c0 += U * W) {
+        uint4 rw[U], pw[U];
+        size_t off[U];
+        float2 a[U];
 #pragma unroll
-    for (int cg = 0; cg < 4; ++cg) {
-        rw[cg] = *reinterpret_cast<const uint4*>(rrow + kmaj32_off(jl, 8 * cg));
-        pw[cg] = *reinterpret_cast<const uint4*>(prow + kmaj32_off(jl, 8 * cg));
-    }
-    const size_t base = (size_t)site * D * N + j;
-    float2 ev[D];
-#pragma unroll
-    for (int c = 0; c < D; ++c) ev[c] = first ? make_float2(0.f, 0.f) : yh[base + (size_t)c * N];
-#pragma unroll
-    for (int cg = 0; cg < 4; ++cg) {
-        uint32_t rr[4] = {rw[cg].x, rw[cg].y, rw[cg].z, rw[cg].w};
-        const uint32_t pq[4] = {pw[cg].x, pw[cg].y, pw[cg].z, pw[cg].w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = 4 * cg + q;
-            const float rx = __uint_as_float(rr[q] << 16), ry = __uint_as_float(rr[q] & 0xFFFF0000u);
-            const float px = __uint_as_float(pq[q] << 16), py = __uint_as_float(pq[q] & 0xFFFF0000u);
-            ev[c].x = fmaf(ax, rx, fmaf(-ay, ry, ev[c].x));
-            ev[c].y = fmaf(ax, ry, fmaf(ay, rx, ev[c].y));
-            rr[q] = pack_bf16(rx - fmaf(ax, px, -ay * py), ry - fmaf(ax, py, ay * px));
+        for (int u = 0; u < U; ++u) {
+            const long long ch = c0 + u * W;
+            if (ch < chunks) {
+                const int site = (int)(ch / G8), g = (int)(ch % G8), j = 8 * g + (lane & 7);
+                off[u] = (((size_t)site * T + (g >> 4)) * 16 + (g & 15)) * 32 + lane;
+                rw[u] = r[off[u]];
+                pw[u] = p[off[u]];
+                a[u] = j < N ? alpha[j] : make_float2(0.f, 0.f);
+            }
         }
-        *reinterpret_cast<uint4*>(rrow + kmaj32_off(jl, 8 * cg)) = make_uint4(rr[0], rr[1], rr[2], rr[3]);
-    }
 #pragma unroll
-    for (int c = 0; c < D; ++c) yh[base + (size_t)c * N] = ev[c];
+        for (int u = 0; u < U; ++u) {
+            if (c0 + u * W >= chunks) break;
+            uint32_t rr[4] = {rw[u].x, rw[u].y, rw[u].z, rw[u].w};
+            const uint32_t pq[4] = {pw[u].x, pw[u].y, pw[u].z, pw[u].w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float rx = __uint_as_float(rr[q] << 16), ry = __uint_as_float(rr[q] & 0xFFFF0000u);
+                const float px = __uint_as_float(pq[q] << 16), py = __uint_as_float(pq[q] & 0xFFFF0000u);
+                rr[q] = pack_bf16(rx - fmaf(a[u].x, px, -a[u].y * py), ry - fmaf(a[u].x, py, a[u].y * px));
+            }
+            rn[off[u]] = make_uint4(rr[0], rr[1], rr[2], rr[3]);
+        }
+    }
+}
+
+// e (=|+=) M^{-1} sum_{s < K} alpha_s r_s with the residuals r_s as BF16 tiles (slots of
+// `slot` bytes): thread = (site, rhs), M^{-1} of the site in shared memory.
+__global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e, const uint8_t* __restrict__ rt,
+                                                         size_t slot, int K, const float2* __restrict__ alpha,
+                                                         const float2* __restrict__ Minv, int nsites, int N, int T,
+                                                         bool accumulate) {
+    __shared__ float2 Ms[D * D];
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int site = blockIdx.y; site < nsites; site += gridDim.y) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < D * D; q += blockDim.x) Ms[q] = Minv[(size_t)site * D * D + q];
+        __syncthreads();
+        if (j >= N) continue;
+        const uint8_t* row = rt + ((size_t)site * T + (j >> 7)) * TILE_A + kmaj32_off(j & 127, 0);
+        const size_t base = (size_t)site * D * N + j;
+        float2 v[D], acc[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+            v[c] = make_float2(0.f, 0.f);
+            acc[c] = accumulate ? e[base + (size_t)c * N] : make_float2(0.f, 0.f);
+        }
+#pragma unroll 2
+        for (int s = 0; s < K; ++s) {
+            const float2 a = alpha[s * N + j];
+            uint4 w[4];
+#pragma unroll
+            for (int cg = 0; cg < 4; ++cg) w[cg] = *reinterpret_cast<const uint4*>(row + s * slot + cg * 128);
+#pragma unroll
+            for (int cg = 0; cg < 4; ++cg) {
+                const uint32_t x[4] = {w[cg].x, w[cg].y, w[cg].z, w[cg].w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    cfma(v[4 * cg + q], a,
+                         make_float2(__uint_as_float(x[q] << 16), __uint_as_float(x[q] & 0xFFFF0000u)));
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+#pragma unroll
+            for (int q = 0; q < D; ++q) cfma(acc[c], Ms[c * D + q], v[q]);
+            e[base + (size_t)c * N] = acc[c];
+        }
+    }
 }
 
 // Bounded wait that also gives up as soon as another role has aborted.
@@ -734,7 +778,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 // FORM 0: y = A x as FP32 rows, with the dots; 1: y as BF16 tiles (yt), with the dots;
-// 2: the residual b - A x as BF16 tiles (yt), b FP32 rows, no dots.
+// 2: the residual b - A x as BF16 tiles (yt), b FP32 rows, no dots; 3: the dots only (the
+// last minimal-residual step).  The pad rows of a partial tile are not written: a row of
+// an MMA operand reaches only the same row of the product, so what they hold meets no rhs.
 template <int FORM>
 __global__ void __launch_bounds__(THREADS, kCtasPerSm)
     k_block_stencil_tc(float2* __restrict__ y, __nv_bfloat16* __restrict__ yt, const float2* __restrict__ b,
@@ -865,13 +911,6 @@ __global__ void __launch_bounds__(THREADS, kCtasPerSm)
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
             if (lane == 0) mbar_arrive(&aempty[as]);      // accumulator may be overwritten
-            if (FORM != 0 && j >= N) {
-                // pad rows of a partial tile stay zero
-                uint8_t* yrow = reinterpret_cast<uint8_t*>(yt) + ((size_t)(blockIdx.x + si * G) * T + t) * TILE_A;
-#pragma unroll
-                for (int cg = 0; cg < 4; ++cg)
-                    *reinterpret_cast<uint4*>(yrow + kmaj32_off(jl, 8 * cg)) = make_uint4(0u, 0u, 0u, 0u);
-            }
             if (j < N) {
                 const int site = blockIdx.x + si * G;
                 float2 ov[D];
@@ -883,7 +922,7 @@ __global__ void __launch_bounds__(THREADS, kCtasPerSm)
                         ov[co] = make_float2(bv.x - ov[co].x, bv.y - ov[co].y);
                     }
                 }
-                if (FORM != 0) {
+                if (FORM == 1 || FORM == 2) {
                     uint8_t* yrow = reinterpret_cast<uint8_t*>(yt) + ((size_t)site * T + t) * TILE_A;
 #pragma unroll
                     for (int cg = 0; cg < 4; ++cg) {
@@ -946,10 +985,10 @@ void launch_pack_tiles_bf16(__nv_bfloat16* rt, const float2* x, int nsites, int 
     MG_LAUNCHED();
 }
 
-void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const double2* dots, int nsites, int N, bool first,
+void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const float2* alpha, int nsites, int N, bool first,
                          __nv_bfloat16* rt, cudaStream_t s) {
     MG_REQUIRE(nsites >= 1 && nsites <= (1 << 30) && tc_tiles(N) <= 65535, MGMLMC_EINVAL, "BF16 tiles: size");
-    tc::tcs::k_mr_update_tc<<<dim3(nsites, tc_tiles(N)), tc::tcs::CH, 0, s>>>(yh, r, p, dots, N, first, rt);
+    tc::tcs::k_mr_update_tc<<<dim3(nsites, tc_tiles(N)), tc::tcs::CH, 0, s>>>(yh, r, p, alpha, N, first, rt);
     MG_LAUNCHED();
 }
 
@@ -976,18 +1015,36 @@ void launch_block_stencil_tc(float2* y, __nv_bfloat16* yt, const float2* b, cons
                              cudaStream_t s) {
     MG_REQUIRE(tc_stencil_supported(16, N), MGMLMC_EINVAL, "tensor-core stencil: d = 16");
     MG_REQUIRE(groups >= 1 && groups <= lx * lt, MGMLMC_EINVAL, "tensor-core stencil: bad grid");
-    MG_REQUIRE((y != nullptr) != (yt != nullptr) && !(b && y), MGMLMC_EINVAL, "tensor-core stencil: one output form");
+    MG_REQUIRE(!(y && yt) && !(b && !yt), MGMLMC_EINVAL, "tensor-core stencil: one output form");
     MG_REQUIRE(((uintptr_t)xt & 15) == 0 && ((uintptr_t)E & 15) == 0 && ((uintptr_t)yt & 15) == 0, MGMLMC_EINVAL,
                "tensor-core stencil: operands must be 16-byte aligned");
     if (y) bstc_launch<0>(y, yt, b, xt, E, lx, lt, N, part, groups, err, s);
+    else if (!yt) bstc_launch<3>(y, yt, b, xt, E, lx, lt, N, part, groups, err, s);
     else if (!b) bstc_launch<1>(y, yt, b, xt, E, lx, lt, N, part, groups, err, s);
     else bstc_launch<2>(y, yt, b, xt, E, lx, lt, N, part, groups, err, s);
 }
 
-void launch_mr_update_bf16(float2* yh, __nv_bfloat16* rt, const __nv_bfloat16* pt, const double2* dots, int nsites,
-                           int N, bool first, cudaStream_t s) {
+void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __nv_bfloat16* p, const float2* alpha,
+                            int nsites, int N, cudaStream_t s) {
     MG_REQUIRE(nsites >= 1 && nsites <= (1 << 30) && tc_tiles(N) <= 65535, MGMLMC_EINVAL, "BF16 tiles: size");
-    tc::tcs::k_mr_update_bf16<<<dim3(nsites, tc_tiles(N)), tc::tcs::CH, 0, s>>>(yh, rt, pt, dots, N, first);
+    const long long chunks = (long long)nsites * ((N + 7) / 8);
+    const long long need = (chunks + 31) / 32;    // 8 warps x 4 chunks per CTA
+    const int g = (int)(need < 6LL * kNumSM ? need : 6LL * kNumSM);
+    tc::tcs::k_mr_update_tiles<<<g, 256, 0, s>>>(reinterpret_cast<uint4*>(rn), reinterpret_cast<const uint4*>(r),
+                                                 reinterpret_cast<const uint4*>(p), alpha, nsites, N, tc_tiles(N));
+    MG_LAUNCHED();
+}
+
+void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const float2* alpha, const float2* Minv,
+                             int nsites, int N, bool accumulate, cudaStream_t s) {
+    const int th = N >= 128 ? 128 : (N + 31) / 32 * 32;
+    const int tiles = (N + th - 1) / th;
+    int G = 16 * kNumSM / tiles;
+    if (G > nsites) G = nsites;
+    if (G < 1) G = 1;
+    tc::tcs::k_block_diag_tiles<<<dim3(tiles, G), th, 0, s>>>(e, reinterpret_cast<const uint8_t*>(rt),
+                                                              tc_tiles_bytes(nsites, N), K, alpha, Minv, nsites, N,
+                                                              tc_tiles(N), accumulate);
     MG_LAUNCHED();
 }
 

@@ -112,6 +112,7 @@ size_t footprint_bytes(const mgmlmc_request& r, const Geometry& g) {
     s.m = r.opt.fgmres_restart;
     s.precision = r.opt.mg_precision;
     s.kcycle = r.opt.kcycle_iters;
+    s.nu = std::max(r.opt.nu_pre, r.opt.nu_post);
     return mg::footprint_bytes(s);
 }
 
@@ -121,7 +122,8 @@ std::string shape_key(const mgmlmc_request& r) {
         s += ":" + std::to_string(r.agg_x[l]) + "," + std::to_string(r.agg_t[l]) + "," + std::to_string(r.nvec[l]);
     s += "/t" + std::to_string(term_levels_of(r));
     s += "/k" + std::to_string(r.k) + "/p" + std::to_string(r.opt.mg_precision) + "/N" +
-         std::to_string(r.opt.max_block_rhs) + "/m" + std::to_string(r.opt.fgmres_restart);
+         std::to_string(r.opt.max_block_rhs) + "/m" + std::to_string(r.opt.fgmres_restart) + "/s" +
+         std::to_string(mg::smoother_slots(r.opt.nu_pre)) + "," + std::to_string(mg::smoother_slots(r.opt.nu_post));
     return s;
 }
 

@@ -6,6 +6,7 @@
 // The smoother S^(nu) is nu steps of minimal residual (GMRES(1)) per rhs: one
 // of the Krylov smoothers Sect. 3.1 lists; FGMRES tolerates its
 // non-linearity.  The coarsest level is solved by its stored dense inverse.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 
@@ -49,7 +50,7 @@ static bool galerkin_form_cheaper(const Ctx& c, int l) {
 
 template <typename C> static bool galerkin_apply(Ctx&, C*, const C*, const C*, int, int) { return false; }
 template <> bool galerkin_apply<double2>(Ctx& c, double2* y, const double2* x, const double2* b, int N, int mode) {
-    if (mode == 2 || !galerkin_form_cheaper(c, 1)) return false;
+    if (mode >= 2 || !galerkin_form_cheaper(c, 1)) return false;
     const Level& F = c.lev[0];
     const Level& Cl = c.lev[1];
     double2* t = c.scratch<double2>("gal64_t", (size_t)F.n * N);
@@ -67,8 +68,15 @@ template <> bool galerkin_apply<double2>(Ctx& c, double2* y, const double2* x, c
     return true;
 }
 
+// The minimal-residual coefficients from a stencil's partial dots.
 template <typename C>
-void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, double2* dots) {
+static void mr_alpha(Ctx& c, C* alpha, const double2* part, int groups, int N) {
+    ProfScope ps(c, "reduce", (double)groups * 2 * N * 16, (double)groups * 2 * N * 2);
+    launch_finalize_alpha<C>(alpha, part, groups, N, c.stream);
+}
+
+template <typename C>
+void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* alpha) {
     if (l == 1 && galerkin_apply<C>(c, y, x, b, N, mode)) return;
     const Level& L = c.lev[l];
     const int groups = (l == 0) ? stencil_groups(L.nsites, N) : block_stencil_groups(L.nsites, L.d, N);
@@ -76,11 +84,11 @@ void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, doubl
     // operator data once; flops: 60 per fine site and rhs, 8 d^2 * 5 per coarse site and rhs
     const double s = sizeof(C);
     const double vec = (double)L.n * N * s;
-    const double bytes = vec * (mode == 1 ? 3 : 2) +
+    const double bytes = vec * (mode == 1 ? 3 : mode == 3 ? 1 : 2) +
                          (l == 0 ? 2.0 * L.nsites * s : 5.0 * L.nsites * L.d * L.d * s);
     const double flops = (l == 0) ? 60.0 * L.nsites * N : 40.0 * L.d * L.d * (double)L.nsites * N;
     double2* part = nullptr;
-    if (mode == 2) part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
+    if (mode >= 2) part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
     {
         ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)), bytes, flops);
         if (l == 0)
@@ -88,10 +96,7 @@ void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, doubl
         else
             launch_block_stencil<C>(y, x, b, blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
-    if (mode == 2) {
-        ProfScope ps(c, "reduce", (double)groups * 2 * N * 16, (double)groups * 2 * N * 2);
-        launch_finalize_rows(dots, part, groups, 2 * N, c.stream);
-    }
+    if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
 }
 
 int* device_error_flag(Ctx& c) {
@@ -108,14 +113,16 @@ int* device_error_flag(Ctx& c) {
 template <typename C> static bool tc_smoother(const Level&, int) { return false; }
 template <> bool tc_smoother<float2>(const Level& L, int N) { return L.Ahat16 && tc_stencil_supported(L.d, N); }
 
-static __nv_bfloat16* tc_tiles(Ctx& c, int l, int N) {
-    return reinterpret_cast<__nv_bfloat16*>(c.scratch_bytes(nm("mr_rt", l, 2), tc_tiles_bytes(c.lev[l].nsites, N)));
+// `slots` consecutive sets of BF16 tiles of one level-l block vector.
+static __nv_bfloat16* tc_tiles(Ctx& c, const char* name, int l, int N, int slots = 1) {
+    return reinterpret_cast<__nv_bfloat16*>(
+        c.scratch_bytes(nm(name, l, 2), slots * tc_tiles_bytes(c.lev[l].nsites, N)));
 }
 
 // y = (D_l M_l^{-1}) x on the tensor cores, x given as its BF16 tiles xt, y as FP32 rows
-// (y) or BF16 tiles (yt); dots as apply_Dhat (against the BF16 x).
+// (y) or BF16 tiles (yt), or only alpha (may be null) = <y, x> / <y, y> (against the BF16 x).
 static void apply_Dhat_tc(Ctx& c, int l, float2* y, __nv_bfloat16* yt, const __nv_bfloat16* xt, int N,
-                          double2* dots) {
+                          float2* alpha) {
     const Level& L = c.lev[l];
     const int groups = block_stencil_tc_groups(L.nsites, N);
     double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
@@ -123,13 +130,12 @@ static void apply_Dhat_tc(Ctx& c, int l, float2* y, __nv_bfloat16* yt, const __n
         // algorithmic traffic: BF16 x (4 B per complex) and y (FP32 8 B or BF16 4 B) once,
         // the BF16 operands once
         ProfScope ps(c, "D" + std::to_string(l + 1) + ".bf16",
-                     (double)L.n * N * (4 + (yt ? 4 : 8)) + 5.0 * L.nsites * 8.0 * L.d * L.d,
+                     (double)L.n * N * (4 + (yt ? 4 : y ? 8 : 0)) + 5.0 * L.nsites * 8.0 * L.d * L.d,
                      40.0 * L.d * L.d * (double)L.nsites * N);
         launch_block_stencil_tc(y, yt, nullptr, xt, L.Ahat16, L.lx, L.lt, N, part, groups, device_error_flag(c),
                                 c.stream);
     }
-    ProfScope ps(c, "reduce", (double)groups * 2 * N * 16, (double)groups * 2 * N * 2);
-    launch_finalize_rows(dots, part, groups, 2 * N, c.stream);
+    if (alpha) mr_alpha<float2>(c, alpha, part, groups, N);
 }
 
 static void pack_tiles(Ctx& c, int l, __nv_bfloat16* xt, const float2* x, int N) {
@@ -138,38 +144,37 @@ static void pack_tiles(Ctx& c, int l, __nv_bfloat16* xt, const float2* x, int N)
     launch_pack_tiles_bf16(xt, x, L.nsites, N, c.stream);
 }
 
-// y = (D_l M_l^{-1}) x with the precomputed block stencil (block-Jacobi smoother).
+// y = (D_l M_l^{-1}) x with the precomputed block stencil (block-Jacobi smoother); mode 0, 2
+// or 3 as apply_D.
 template <typename C>
-static void apply_Dhat(Ctx& c, int l, C* y, const C* x, int N, double2* dots) {
+static void apply_Dhat(Ctx& c, int l, C* y, const C* x, int N, int mode, C* alpha) {
     const Level& L = c.lev[l];
     const int groups = block_stencil_groups(L.nsites, L.d, N);
     const double s = sizeof(C);
-    double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
+    double2* part = mode >= 2 ? c.scratch<double2>("part_st", (size_t)groups * 2 * N) : nullptr;
     {
         ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
-                     (double)L.n * N * s * 2 + 5.0 * L.nsites * L.d * L.d * s,
+                     (double)L.n * N * s * (mode == 3 ? 1 : 2) + 5.0 * L.nsites * L.d * L.d * s,
                      40.0 * L.d * L.d * (double)L.nsites * N);
-        launch_block_stencil<C>(y, x, nullptr, hat_blocks<C>(L), L.lx, L.lt, L.d, N, 2, part, groups, c.stream);
+        launch_block_stencil<C>(y, x, nullptr, hat_blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
-    ProfScope ps(c, "reduce", (double)groups * 2 * N * 16, (double)groups * 2 * N * 2);
-    launch_finalize_rows(dots, part, groups, 2 * N, c.stream);
+    if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
 }
 
-template <typename C> static bool apply_smoother_tc(Ctx&, int, C*, const C*, int, double2*) { return false; }
-template <> bool apply_smoother_tc<float2>(Ctx& c, int l, float2* y, const float2* x, int N, double2* dots) {
+template <typename C> static bool apply_smoother_tc(Ctx&, int, C*, const C*, int) { return false; }
+template <> bool apply_smoother_tc<float2>(Ctx& c, int l, float2* y, const float2* x, int N) {
     if (!tc_smoother<float2>(c.lev[l], N)) return false;
-    __nv_bfloat16* xt = tc_tiles(c, l, N);
+    __nv_bfloat16* xt = tc_tiles(c, "mr_rt", l, N);
     pack_tiles(c, l, xt, x, N);
-    apply_Dhat_tc(c, l, y, nullptr, xt, N, dots);
+    apply_Dhat_tc(c, l, y, nullptr, xt, N, nullptr);
     return true;
 }
 
 template <typename C>
-void apply_smoother_operator(Ctx& c, int l, C* y, const C* x, int N, double2* dots) {
+void apply_smoother_operator(Ctx& c, int l, C* y, const C* x, int N) {
     MG_REQUIRE(l >= 1 && l < c.L - 1 && hat_blocks<C>(c.lev[l]), MGMLMC_EINVAL,
                "smoother operator: only coarse levels above the coarsest");
-    if (!dots) dots = c.scratch<double2>("smop_dots", 2 * (size_t)N);
-    if (!apply_smoother_tc<C>(c, l, y, x, N, dots)) apply_Dhat<C>(c, l, y, x, N, dots);
+    if (!apply_smoother_tc<C>(c, l, y, x, N)) apply_Dhat<C>(c, l, y, x, N, 0, nullptr);
 }
 
 template <typename C>
@@ -183,13 +188,13 @@ void apply_restrict(Ctx& c, int l, C* xc, const C* x, int N) {
 }
 
 template <typename C>
-void apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate) {
+bool apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate, void* xt) {
     const Level& L = c.lev[l];
     const double s = sizeof(C);
     ProfScope ps(c, "P" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
                  (double)L.n * N * s * (accumulate ? 2 : 1) + (double)c.lev[l + 1].n * N * s + (double)L.n * L.nvec * s,
                  8.0 * L.nvec * (double)L.n * N);
-    launch_prolong<C>(x, xc, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, accumulate, c.stream);
+    return launch_prolong<C>(x, xc, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, accumulate, c.stream, xt);
 }
 
 template <typename C> static void coarsest_apply(Ctx& c, C* e, const C* r, int N);
@@ -213,152 +218,184 @@ template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int 
     launch_gemm_nn<float2>(e, L.Dinv32, r, (int)L.n, (int)L.n, N, false, c.stream);
 }
 
-// nu block-Jacobi MR steps from the residual's BF16 tiles rt (overwritten), r and p
-// only as BF16 tiles; yh receives the preconditioned correction.
-static void smooth_tc_tiles(Ctx& c, int l, float2* yh, __nv_bfloat16* rt, int N, int nu, double2* dots) {
-    const Level& L = c.lev[l];
-    __nv_bfloat16* pt =
-        reinterpret_cast<__nv_bfloat16*>(c.scratch_bytes(nm("mr_pt", l, 2), tc_tiles_bytes(L.nsites, N)));
+// Minimal-residual steps are taken in groups of at most kMrGroup: the residuals of a
+// group stay in consecutive slots, and the correction takes sum_s alpha_s r_s once per
+// group.  Slots needed for nu steps:
+constexpr int kMrGroup = 8;
+static int mr_slots(int nu) { return std::min(std::max(nu, 1), kMrGroup); }
+
+// The group loop, for any form of the vectors: image(s, last) forms the image of slot s and
+// its coefficient (the last step of all needs no image), flush(K, first) adds the K slots to
+// the correction, update(s, t) forms the next residual from slot s in slot t.  Returns the
+// slot of the final residual (with need_r), else -1.
+template <typename Image, typename Flush, typename Update>
+static int mr_steps(int nu, bool need_r, Image image, Flush flush, Update update) {
+    const int K = mr_slots(nu);
+    int slot = 0;
     for (int s = 0; s < nu; ++s) {
-        apply_Dhat_tc(c, l, nullptr, pt, rt, N, dots);
-        // traffic: r and p tiles read, r tiles written (4 B per complex), yh read and written
-        ProfScope ps(c, "mr" + std::to_string(l + 1) + ".bf16", (double)L.n * N * (3 * 4 + (s ? 16 : 8)),
-                     16.0 * L.n * N);
-        launch_mr_update_bf16(yh, rt, pt, dots, L.nsites, N, s == 0, c.stream);
+        const bool last = s + 1 == nu && !need_r;
+        image(slot, last);
+        if (slot + 1 == K || s + 1 == nu) flush(slot + 1, s < K);
+        if (last) return -1;
+        const int next = (slot + 1) % K;
+        update(slot, next);
+        slot = next;
     }
+    return slot;
 }
 
 // Post-smoothing of the V-cycle on the tensor cores: the residual r - D_l e is formed
-// from BF16 tiles of e straight into the smoother's BF16 residual tiles (it only
-// feeds the smoother, which needs a few digits), then the BF16 smoother; e += M^{-1} yh.
-template <typename C> static bool residual_smooth_tc(Ctx&, int, C*, const C*, int) { return false; }
-
-// Block-Jacobi MR on the tensor cores.  The residual's BF16 tiles are packed once;
-// when the caller does not need the final residual (post-smoothing), r and p live
-// only as BF16 tiles from there on (the smoother needs a few digits, and FGMRES
-// is flexible), else r stays FP32 and each update writes the next tiles.
-template <typename C> static bool mr_smooth_tc(Ctx&, int, C*, C*, int, int, bool, bool) { return false; }
-template <>
-bool mr_smooth_tc<float2>(Ctx& c, int l, float2* e, float2* r, int N, int nu, bool e_zero, bool need_r) {
+// from BF16 tiles of e (et) straight into the smoother's BF16 residual tiles (it only
+// feeds the smoother, which needs a few digits), then nu block-Jacobi MR steps with r and p
+// only as BF16 tiles; e += M^{-1} sum_s alpha_s r_s.
+template <typename C> static bool post_smooth_tc(Ctx&, int, C*, const C*, int, bool) { return false; }
+template <typename C> static bool post_smooths_tc(const Ctx&, int, int) { return false; }
+template <> bool post_smooths_tc<float2>(const Ctx& c, int l, int N) {
     const Level& L = c.lev[l];
-    if (nu <= 0 || !tc_smoother<float2>(L, N)) return false;
-    float2* yh = c.scratch<float2>(nm("mr_y", l, sizeof(float2)), (size_t)L.n * N);
-    double2* dots = c.scratch<double2>(nm("mr_dots", l, sizeof(float2)), 2 * (size_t)N);
-    __nv_bfloat16* rt = tc_tiles(c, l, N);
-    pack_tiles(c, l, rt, r, N);
-    if (need_r) {
-        float2* p = c.scratch<float2>(nm("mr_p", l, sizeof(float2)), (size_t)L.n * N);
-        for (int s = 0; s < nu; ++s) {
-            apply_Dhat_tc(c, l, p, nullptr, rt, N, dots);
-            const bool more = s + 1 < nu;
-            ProfScope ps(c, "mr" + std::to_string(l + 1) + ".f32", (double)L.n * N * (5 * 8 + (more ? 4 : 0)),
-                         16.0 * L.n * N);
-            launch_mr_update_tc(yh, r, p, dots, L.nsites, N, s == 0, more ? rt : nullptr, c.stream);
-        }
-    } else {
-        smooth_tc_tiles(c, l, yh, rt, N, nu, dots);
-    }
-    ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".f32", 3.0 * L.n * N * sizeof(float2),
-                 8.0 * L.d * (double)L.n * N);
-    launch_block_diag_apply<float2>(e, yh, L.Minv32, L.nsites, L.d, N, !e_zero, c.stream);
-    return true;
+    return c.opt.nu_post > 0 && L.A16 && tc_smoother<float2>(L, N);
 }
 
-// Plain MR on the fine level with r and p in BF16 (mg_precision 16, post-smoothing):
-// the same few digits as the coarse smoother, half the traffic of the FP32 vectors;
-// the correction e stays FP32.
-template <typename C> static bool mr_smooth_fine_bf16(Ctx&, int, C*, C*, int, int, bool, bool) { return false; }
 template <>
-bool mr_smooth_fine_bf16<float2>(Ctx& c, int l, float2* e, float2* r, int N, int nu, bool e_zero, bool need_r) {
-    if (l != 0 || need_r || nu <= 0 || c.opt.mg_precision != 16 || N % 4) return false;
-    const Level& L = c.lev[0];
-    const size_t nN = (size_t)L.n * N;
-    uint32_t* rb = c.scratch<uint32_t>("mrf_rb", nN);
-    uint32_t* pb = c.scratch<uint32_t>("mrf_pb", nN);
-    double2* dots = c.scratch<double2>(nm("mr_dots", 0, sizeof(float2)), 2 * (size_t)N);
-    const int groups = stencil_groups_bf16(L.nsites, N);
-    double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
-    {
-        ProfScope ps(c, "pack1.bf16", (double)nN * (8 + 4), 0.0);
-        launch_pack_bf16(rb, r, (long long)nN, c.stream);
-    }
-    for (int s = 0; s < nu; ++s) {
-        {
-            // algorithmic traffic: BF16 x read and y written once (4 B per complex), links once
-            ProfScope ps(c, "D1.bf16", (double)nN * 8 + 2.0 * L.nsites * 8, 60.0 * L.nsites * N);
-            launch_wilson_bf16(pb, rb, c.U32, c.m0, L.lx, L.lt, N, part, groups, c.stream);
-        }
-        {
-            ProfScope ps(c, "reduce", (double)groups * 2 * N * 16, (double)groups * 2 * N * 2);
-            launch_finalize_rows(dots, part, groups, 2 * N, c.stream);
-        }
-        // traffic: r and p read, r written (4 B each), e read (after the first step) and written
-        ProfScope ps(c, "mr1.bf16", (double)nN * (12 + (e_zero && s == 0 ? 8 : 16)), 16.0 * nN);
-        launch_mr_update_fine_bf16(e, rb, pb, dots, L.n, N, e_zero && s == 0, c.stream);
-    }
-    return true;
-}
-
-// nu MR steps on D_l e = r0 starting from e (or 0); r holds the current residual on
-// entry and is overwritten (with the final residual when need_r).
-template <>
-bool residual_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N) {
+bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bool have_et) {
+    if (!post_smooths_tc<float2>(c, l, N)) return false;
     const Level& L = c.lev[l];
-    const int nu = c.opt.nu_post;
-    if (nu <= 0 || !L.A16 || !tc_smoother<float2>(L, N)) return false;
-    float2* yh = c.scratch<float2>(nm("mr_y", l, sizeof(float2)), (size_t)L.n * N);
-    double2* dots = c.scratch<double2>(nm("mr_dots", l, sizeof(float2)), 2 * (size_t)N);
-    __nv_bfloat16* et =
-        reinterpret_cast<__nv_bfloat16*>(c.scratch_bytes(nm("cyc_et", l, 2), tc_tiles_bytes(L.nsites, N)));
-    __nv_bfloat16* rt = tc_tiles(c, l, N);
-    pack_tiles(c, l, et, e, N);
+    const int nu = c.opt.nu_post, K = mr_slots(nu);
+    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kMrGroup * N);
+    __nv_bfloat16* et = tc_tiles(c, "cyc_et", l, N);
+    __nv_bfloat16* rt = tc_tiles(c, "mr_rt", l, N, K);
+    __nv_bfloat16* pt = tc_tiles(c, "mr_pt", l, N);
+    const size_t slot = tc_tiles_bytes(L.nsites, N) / sizeof(__nv_bfloat16);
+    if (!have_et) pack_tiles(c, l, et, e, N);
     {
         const int groups = block_stencil_tc_groups(L.nsites, N);
-        double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
         // algorithmic traffic: e tiles (4 B per complex) and r (8 B) read, residual tiles written (4 B)
         ProfScope ps(c, "D" + std::to_string(l + 1) + "res.bf16",
                      (double)L.n * N * (4 + 8 + 4) + 5.0 * L.nsites * 8.0 * L.d * L.d,
                      40.0 * L.d * L.d * (double)L.nsites * N);
-        launch_block_stencil_tc(nullptr, rt, r, et, L.A16, L.lx, L.lt, N, part, groups, device_error_flag(c),
+        launch_block_stencil_tc(nullptr, rt, r, et, L.A16, L.lx, L.lt, N, nullptr, groups, device_error_flag(c),
                                 c.stream);
     }
-    smooth_tc_tiles(c, l, yh, rt, N, nu, dots);
-    ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".f32", 3.0 * L.n * N * sizeof(float2),
-                 8.0 * L.d * (double)L.n * N);
-    launch_block_diag_apply<float2>(e, yh, L.Minv32, L.nsites, L.d, N, true, c.stream);
+    mr_steps(
+        nu, false,
+        [&](int s, bool last) { apply_Dhat_tc(c, l, nullptr, last ? nullptr : pt, rt + s * slot, N, alpha + (size_t)s * N); },
+        [&](int k, bool) {
+            // traffic: the K residuals (4 B per complex) read, e read and written
+            ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".bf16", (double)L.n * N * (4 * k + 16),
+                         8.0 * (L.d + k) * (double)L.n * N);
+            launch_block_diag_tiles(e, rt, k, alpha, L.Minv32, L.nsites, N, true, c.stream);
+        },
+        [&](int s, int t) {
+            // traffic: r and p tiles read, the next r tiles written (4 B per complex)
+            ProfScope ps(c, "mr" + std::to_string(l + 1) + ".bf16", (double)L.n * N * 12, 8.0 * L.n * N);
+            launch_mr_update_tiles(rt + t * slot, rt + s * slot, pt, alpha + (size_t)s * N, L.nsites, N, c.stream);
+        });
     return true;
 }
 
-template <typename C>
-static void mr_smooth(Ctx& c, int l, C* e, C* r, int N, int nu, bool e_zero, bool need_r) {
-    if (mr_smooth_tc<C>(c, l, e, r, N, nu, e_zero, need_r)) return;
+// Pre-smoothing with the image on the tensor cores: the residual stays FP32 (the caller
+// restricts it) and each update writes the next step's tiles.
+template <typename C> static bool pre_smooth_tc(Ctx&, int, C*, C*, int, int) { return false; }
+template <>
+bool pre_smooth_tc<float2>(Ctx& c, int l, float2* e, float2* r, int N, int nu) {
     const Level& L = c.lev[l];
-    C* p = c.scratch<C>(nm("mr_p", l, sizeof(C)), (size_t)L.n * N);
-    double2* dots = c.scratch<double2>(nm("mr_dots", l, sizeof(C)), 2 * (size_t)N);
-    if (hat_blocks<C>(L)) {
-        // block-Jacobi MR: minimal residual steps on D M^{-1} (y accumulates the
-        // preconditioned correction), then e += M^{-1} y
-        C* yh = c.scratch<C>(nm("mr_y", l, sizeof(C)), (size_t)L.n * N);
-        for (int s = 0; s < nu; ++s) {
-            apply_Dhat<C>(c, l, p, r, N, dots);
-            ProfScope ps(c, "mr" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)), 5.0 * L.n * N * sizeof(C),
-                         16.0 * L.n * N);
-            launch_mr_update<C>(yh, r, p, dots, L.n, N, s == 0, c.stream);
-        }
-        if (nu > 0) {
-            ProfScope ps(c, "bjac" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
-                         3.0 * L.n * N * sizeof(C), 8.0 * L.d * (double)L.n * N);
-            launch_block_diag_apply<C>(e, yh, minv<C>(L), L.nsites, L.d, N, !e_zero, c.stream);
-        }
-        return;
-    }
-    if (mr_smooth_fine_bf16<C>(c, l, e, r, N, nu, e_zero, need_r)) return;
+    if (!tc_smoother<float2>(L, N)) return false;
+    float2* yh = c.scratch<float2>(nm("mr_y", l, sizeof(float2)), (size_t)L.n * N);
+    float2* p = c.scratch<float2>(nm("mr_p", l, sizeof(float2)), (size_t)L.n * N);
+    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kMrGroup * N);
+    __nv_bfloat16* rt = tc_tiles(c, "mr_rt", l, N);
+    pack_tiles(c, l, rt, r, N);
     for (int s = 0; s < nu; ++s) {
-        apply_D<C>(c, l, p, r, nullptr, N, 2, dots);
-        ProfScope ps(c, "mr" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)), 5.0 * L.n * N * sizeof(C),
+        apply_Dhat_tc(c, l, p, nullptr, rt, N, alpha);
+        const bool more = s + 1 < nu;
+        ProfScope ps(c, "mr" + std::to_string(l + 1) + ".f32", (double)L.n * N * (5 * 8 + (more ? 4 : 0)),
                      16.0 * L.n * N);
-        launch_mr_update<C>(e, r, p, dots, L.n, N, e_zero && s == 0, c.stream);
+        launch_mr_update_tc(yh, r, p, alpha, L.nsites, N, s == 0, more ? rt : nullptr, c.stream);
     }
+    ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".f32", 3.0 * L.n * N * sizeof(float2),
+                 8.0 * L.d * (double)L.n * N);
+    launch_block_diag_apply<float2>(e, yh, L.Minv32, L.nsites, L.d, N, false, c.stream);
+    return true;
+}
+
+// Post-smoothing of the fine level with r and p in BF16 (mg_precision 16): the same few
+// digits as the coarse smoother, half the traffic of the FP32 vectors; the residual r - D e
+// is formed in FP32 and rounded as it is written, the correction e stays FP32.
+template <typename C> static bool post_smooth_fine_bf16(Ctx&, int, C*, const C*, int) { return false; }
+template <>
+bool post_smooth_fine_bf16<float2>(Ctx& c, int l, float2* e, const float2* r, int N) {
+    const int nu = c.opt.nu_post;
+    if (l != 0 || nu <= 0 || c.opt.mg_precision != 16 || N % 4) return false;
+    const Level& L = c.lev[0];
+    const size_t nN = (size_t)L.n * N;
+    uint32_t* rb = c.scratch<uint32_t>("mrf_rb", mr_slots(nu) * nN);
+    uint32_t* pb = c.scratch<uint32_t>("mrf_pb", nN);
+    float2* alpha = c.scratch<float2>(nm("mr_al", 0, sizeof(float2)), (size_t)kMrGroup * N);
+    const int groups = stencil_groups_bf16(L.nsites, N);
+    double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
+    {
+        // algorithmic traffic: e and r read (8 B each), the BF16 residual written
+        ProfScope ps(c, "D1res.bf16", (double)nN * 20 + 2.0 * L.nsites * 8, 60.0 * L.nsites * N);
+        launch_wilson_residual_bf16(rb, e, r, c.U32, c.m0, L.lx, L.lt, N, stencil_groups(L.nsites, N), c.stream);
+    }
+    mr_steps(
+        nu, false,
+        [&](int s, bool last) {
+            {
+                // algorithmic traffic: BF16 x read, y written once (4 B per complex), links once
+                ProfScope ps(c, "D1.bf16", (double)nN * (last ? 4 : 8) + 2.0 * L.nsites * 8, 60.0 * L.nsites * N);
+                launch_wilson_bf16(last ? nullptr : pb, rb + s * nN, c.U32, c.m0, L.lx, L.lt, N, part, groups,
+                                   c.stream);
+            }
+            mr_alpha<float2>(c, alpha + (size_t)s * N, part, groups, N);
+        },
+        [&](int k, bool) {
+            ProfScope ps(c, "mr1sum.bf16", (double)nN * (4 * k + 16), 8.0 * k * nN);
+            launch_mr_combine_bf16(e, rb, nN, k, alpha, L.n, N, false, c.stream);
+        },
+        [&](int s, int t) {
+            // traffic: r and p read, the next r written (4 B each)
+            ProfScope ps(c, "mr1.bf16", (double)nN * 12, 8.0 * nN);
+            launch_mr_update_fine_bf16(rb + t * nN, rb + s * nN, pb, alpha + (size_t)s * N, L.n, N, c.stream);
+        });
+    return true;
+}
+
+// nu MR steps on D_l e = r0 starting from e (or 0); rs has mr_slots(nu) slots, the first
+// holding the current residual.  Returns the slot with the final residual (need_r).  On
+// coarse levels above the coarsest: block-Jacobi MR, minimal-residual steps on D M^{-1}
+// whose preconditioned correction M^{-1} sum_s alpha_s r_s goes to e.
+template <typename C>
+static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool need_r) {
+    const Level& L = c.lev[l];
+    const size_t nN = (size_t)L.n * N;
+    C* p = c.scratch<C>(nm("mr_p", l, sizeof(C)), nN);
+    C* alpha = c.scratch<C>(nm("mr_al", l, sizeof(C)), (size_t)kMrGroup * N);
+    const bool jacobi = hat_blocks<C>(L) != nullptr;
+    const std::string tag = std::to_string(l + 1) + "." + prec_tag(sizeof(C));
+    const int fin = mr_steps(
+        nu, need_r,
+        [&](int s, bool last) {
+            const int mode = last ? 3 : 2;
+            if (jacobi) apply_Dhat<C>(c, l, last ? nullptr : p, rs + s * nN, N, mode, alpha + (size_t)s * N);
+            else apply_D<C>(c, l, last ? nullptr : p, rs + s * nN, nullptr, N, mode, alpha + (size_t)s * N);
+        },
+        [&](int k, bool first) {
+            const bool zero = e_zero && first;
+            if (jacobi) {
+                ProfScope ps(c, "bjac" + tag, (k + (zero ? 1.0 : 2.0)) * nN * sizeof(C), 8.0 * (L.d + k) * (double)nN);
+                launch_block_diag_combine<C>(e, rs, nN, k, alpha, minv<C>(L), L.nsites, L.d, N, !zero, c.stream);
+            } else {
+                ProfScope ps(c, "mr" + std::to_string(l + 1) + "sum." + prec_tag(sizeof(C)),
+                             (k + (zero ? 1.0 : 2.0)) * nN * sizeof(C), 8.0 * k * (double)nN);
+                launch_mr_combine<C>(e, rs, nN, k, alpha, L.n, N, zero, c.stream);
+            }
+        },
+        [&](int s, int t) {
+            ProfScope ps(c, "mr" + tag, 3.0 * nN * sizeof(C), 8.0 * (double)nN);
+            // with a single slot the update is in place
+            launch_mr_update<C>(rs + t * nN, rs + s * nN, p, alpha + (size_t)s * N, L.n, N, c.stream);
+        });
+    return fin >= 0 ? rs + fin * nN : nullptr;
 }
 
 __global__ void k_sqrt_inplace(double* v, int n) {
@@ -492,13 +529,17 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
     }
     const Level& L = c.lev[l];
     const Level& Lc = c.lev[l + 1];
-    C* res = c.scratch<C>(nm("cyc_res", l, sizeof(C)), (size_t)L.n * N);
     C* rc = c.scratch<C>(nm("cyc_rc", l + 1, sizeof(C)), (size_t)Lc.n * N);
     C* ec = c.scratch<C>(nm("cyc_ec", l + 1, sizeof(C)), (size_t)Lc.n * N);
+    const size_t nN = (size_t)L.n * N;
+    auto residual_slots = [&](int nu) { return c.scratch<C>(nm("cyc_res", l, sizeof(C)), mr_slots(nu) * nN); };
     bool e_zero = true;
     if (c.opt.nu_pre > 0) {
-        MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C) * L.n * N, cudaMemcpyDeviceToDevice, c.stream));
-        mr_smooth<C>(c, l, e, res, N, c.opt.nu_pre, true, true);   // leaves res = r - D e
+        C* res = residual_slots(c.opt.nu_pre);
+        MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C) * nN, cudaMemcpyDeviceToDevice, c.stream));
+        // leaves res = r - D e
+        if (!pre_smooth_tc<C>(c, l, e, res, N, c.opt.nu_pre))
+            res = mr_smooth<C>(c, l, e, res, N, c.opt.nu_pre, true, true);
         e_zero = false;
         apply_restrict<C>(c, l, rc, res, N);
     } else {
@@ -508,11 +549,14 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
         kcycle<C>(c, l + 1, ec, rc, N, c.opt.kcycle_iters);
     else
         mg_cycle<C>(c, l + 1, ec, rc, N);
-    apply_prolong<C>(c, l, e, ec, N, !e_zero);
-    if (c.opt.nu_post > 0 && !residual_smooth_tc<C>(c, l, e, r, N)) {
-        apply_D<C>(c, l, res, e, r, N, 1, nullptr);
-        mr_smooth<C>(c, l, e, res, N, c.opt.nu_post, false, false);
-    }
+    // the prolongation also writes the tensor-core smoother's tiles of e where it can
+    void* et = post_smooths_tc<C>(c, l, N) ? tc_tiles(c, "cyc_et", l, N) : nullptr;
+    const bool have_et = apply_prolong<C>(c, l, e, ec, N, !e_zero, et);
+    if (c.opt.nu_post <= 0 || post_smooth_tc<C>(c, l, e, r, N, have_et) || post_smooth_fine_bf16<C>(c, l, e, r, N))
+        return;
+    C* res = residual_slots(c.opt.nu_post);
+    apply_D<C>(c, l, res, e, r, N, 1, nullptr);
+    mr_smooth<C>(c, l, e, res, N, c.opt.nu_post, false, false);
 }
 
 static double read_scalar(Ctx& c, const double* dev) {
@@ -806,11 +850,11 @@ void check_device_error(Ctx& c) {
 }
 
 #define INST(C)                                                                                           \
-    template void apply_D<C>(Ctx&, int, C*, const C*, const C*, int, int, double2*);                        \
+    template void apply_D<C>(Ctx&, int, C*, const C*, const C*, int, int, C*);                              \
     template void apply_restrict<C>(Ctx&, int, C*, const C*, int);                                          \
-    template void apply_prolong<C>(Ctx&, int, C*, const C*, int, bool);                                     \
+    template bool apply_prolong<C>(Ctx&, int, C*, const C*, int, bool, void*);                              \
     template void mg_cycle<C>(Ctx&, int, C*, const C*, int);                                                \
-    template void apply_smoother_operator<C>(Ctx&, int, C*, const C*, int, double2*);                       \
+    template void apply_smoother_operator<C>(Ctx&, int, C*, const C*, int);                                 \
     template long long fgmres<C>(Ctx&, int, const C*, C*, int, double, long long, bool, int*, int);
 INST(double2)
 INST(float2)
