@@ -31,6 +31,11 @@ struct Level {
     // mg_precision 16, d = 16: Ahat as BF16 real 32 x 32 operands of the tensor-core stencil
     __nv_bfloat16* Ahat16 = nullptr;
     __nv_bfloat16* A16 = nullptr;    // the same for D_l itself (the V-cycle residual)
+    // d = 16: the digits of D_l (and, with mg_precision 64, of D M^{-1} and of the coarsest
+    // inverse) for the FP64 products on the tensor cores
+    void* A64t = nullptr;
+    void* Ahat64t = nullptr;
+    void* Dinv64t = nullptr;
     // prolongation to the next level: [site][d][nvec]
     int ax = 0, at = 0, nvec = 0;
     double2* P64 = nullptr;

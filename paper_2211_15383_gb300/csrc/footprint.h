@@ -27,6 +27,10 @@ struct Shape {
     int nu = 4;                      // smoothing steps per level (the larger of pre and post)
 };
 
+// The FP64 coarsest inverse (mg_precision 64) is applied on the tensor cores up to this
+// size: its digits take 64 bytes an entry (1.1 GB at 4096 unknowns, 17 GB at 16384).
+inline bool f64_dense_inverse(long long n) { return n % 16 == 0 && n <= 4096; }
+
 // Residuals that the smoother keeps at once: those of a group of at most 8 steps.
 inline int smoother_slots(int nu) { return std::min(std::max(nu, 1), 8); }
 
@@ -55,7 +59,9 @@ inline size_t footprint_bytes(const Shape& s) {
             b += st * d * d * (24 + 16) + st * 5 * d * d * 24;               // M^{-1}, D M^{-1}, work
             if (bf16) b += st * d * d * 80;                                  // BF16 operand tiles
         }
-        if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * N * 16;            // FP64 Galerkin apply
+        const bool digits = l > 0 && s.d[l] == 16;                           // FP64 products on the tensor cores
+        if (digits) b += st * 5 * 16384 * (f64 && l + 1 < L ? 2 : 1) + st * std::ceil(N / 128) * 57344;
+        if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * (digits ? std::min(N, 16.0) : N) * 16;   // FP64 Galerkin apply
         if (l + 1 < L) {
             const double K = smoother_slots(s.nu);
             const bool tiles = bf16 && l > 0 && s.d[l] == 16;                // smoothed on the tensor cores
@@ -69,6 +75,8 @@ inline size_t footprint_bytes(const Shape& s) {
     }
     b += 2.0 * n0 * nvmax * 16;                                              // setup blocks
     b += nL * nL * 44 + nL * N * 136;                                        // dense coarsest inverse, BF16 solve
+    if (f64 && f64_dense_inverse(s.n[L - 1]))                                // its digits; x digits, partial sums
+        b += nL * nL * 64 + nL / 16 * std::ceil(N / 128) * 57344 + std::ceil(nL / 96) * nL * N * 16;
     b += (2 * m + 1) * n0 * (N * sz + nvmax * 16);                           // FGMRES bases
     b += G * (m + 1) * N * 16 + N * (m + 1) * (m + 4) * 16;                  // Gram-Schmidt partials, Hessenberg
     b += n0 * N * 56;                                                        // refinement blocks

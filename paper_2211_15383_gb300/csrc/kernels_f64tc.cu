@@ -1,0 +1,507 @@
+// FP64 block products on the tensor cores.  GB300 issues 2 FP64 FMA per SM and clock (1/64
+// of its FP32 rate), so the FP64 block stencils (d = 16) and the dense coarsest inverse were
+// bound by that pipe: 4.3 ms for one D_3 x at 32^2 sites x 512 rhs, 2.2 ms for a 1024 x 1024
+// inverse times 64 rhs.  Both are contractions, and an exact integer product of slices of the
+// operands gives the same result on the BF16 tensor cores (the Ozaki scheme: K. Ozaki,
+// T. Ogita, S. Oishi, S. M. Rump, "Error-free transformations of matrix multiplication by
+// using fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
+//
+//  * every rhs of x is scaled by a power of two 2^-ex with |x| < 2^ex (its largest entry) and
+//    rounded to 55 bits, x = 2^ex sum_{j<7} d_j 2^{-6-8j}; the matrix by one power of two,
+//    63 bits, a = 2^ea sum_{i<8} c_i 2^{-6-8i}; all digits are integers in [-128, 127], exact
+//    in BF16.  So x moves by at most 2^-55 of its column's largest entry (FP64 itself keeps
+//    2^-53 of an entry) and a by 2^-63;
+//  * G_g = sum_{i+j=g} sum_k c_i d_j for g = 0..7: products of digits are below 2^14, sums of
+//    at most 192 k and 5 pairs below 2^24, so the FP32 accumulation in TMEM is exact for the
+//    groups g <= 4 (the others weigh at most 2^-40, and their sums can only leave the
+//    exact range by rounding their last place); the dropped pairs i + j > 7 weigh 2^-64;
+//  * sum_g G_g 2^-8g is formed in 128-bit integers and rounded to FP64 once.
+// A product of 160 terms is then closer to the exact one than 160 FP64 FMAs are.
+//
+// Layout: the rhs are the MMA's M (128 rows of x digits, K = 32 reals of a site), the digits
+// of the block are its N: the 8 x 32 rows (i, output real) of a block's tile lie one after
+// another, so digit slice j of x times rows 0 .. 255 - 32j lands on the columns 32j .. 255,
+// which is exactly where G_{i+j} belongs: 7 MMAs (N = 256, 224, ..., 64) per K step, 1120
+// columns for the 35 pairs.  A job is one block of 16 output rows for 128 rhs (5 blocks of
+// the stencil, or up to 6 of a row of the dense matrix); x digits (56 KB) and block digits
+// (16 KB) of each K block move by bulk copies through a 3-stage ring, two 256-column
+// accumulators alternate, eight epilogue warps turn them into FP64.  One CTA per SM (216 KB).
+// Bound: L2 and HBM reads of the digit tiles (72 KB per K block; the MMAs of a stencil job
+// are 5600 cycles, a job takes about 16000).  Measured: D_3 x at 32^2 sites x 512 rhs
+// 4329 -> 217 us, D_2 x at 128^2 sites x 128 rhs (then by P^H D_1 P) 9.4 -> 0.9 ms, the
+// inverse of 1024 unknowns times 64 rhs 2205 -> 33 us; the two passes that scale and slice
+// x move 30 B per real more.
+#include <algorithm>
+
+#include "kernels.cuh"
+#include "tcgen05.cuh"
+
+namespace mg {
+namespace tc {
+namespace f64 {
+constexpr int D = 16, KD = 32;             // block size, reals of a block
+constexpr int NX = 7, NA = 8;              // digit slices of x and of the matrix
+constexpr int XS = 128 * KD * 2;           // 8 KB: one digit slice of a 128-rhs tile
+constexpr int XT = NX * XS;                // 56 KB
+constexpr int AT = NA * KD * KD * 2;       // 16 KB: the digits of one block
+constexpr int NSTG = 3;
+constexpr int STAGE = XT + AT;
+constexpr int SMEM = NSTG * STAGE;         // 216 KB
+constexpr int ACC = NA * KD;               // 256 columns per accumulator
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int KSPLIT = 6;                  // K blocks of a dense job (exact sums, see above)
+
+using u64 = unsigned long long;
+using i64 = long long;
+
+// round(v 2^(BITS - e)) for the biased exponent E of the largest entry (|v| < 2^(E - 1022)).
+template <int BITS>
+__device__ __forceinline__ i64 fixed_point(double v, int E) {
+    const u64 b = (u64)__double_as_longlong(v);
+    const int eb = (int)((b >> 52) & 0x7ff);
+    const u64 m = (b & 0xFFFFFFFFFFFFFull) | (eb ? 1ull << 52 : 0ull);
+    // v = m 2^(max(eb, 1) - 1075); q = m 2^sh
+    const int sh = (eb > 0 ? eb : 1) - 1075 + BITS - (E - 1022);
+    u64 q;
+    if (sh >= 0) q = m << sh;
+    else if (sh < -54) q = 0;
+    else q = (m + (1ull << (-sh - 1))) >> (-sh);
+    return (b >> 63) ? -(i64)q : (i64)q;
+}
+
+// Digit (a byte of the offset fixed-point number) as the float it stands for.
+__device__ __forceinline__ float digit(u64 u, int byte) {
+    return __uint_as_float(0x4B000000u | ((uint32_t)(u >> (8 * byte)) & 0xFFu)) - 8388736.0f;   // 2^23 + 128
+}
+__device__ __forceinline__ uint32_t pack_exact(float lo, float hi) {
+    return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+}
+
+// Largest |re|, |im| per rhs (cols > 1) or of everything (cols == 1: count values of a flat
+// array), as the bit pattern of the double: non-negative doubles order like integers, NaN
+// above all, so the atomic maximum does not depend on the order.
+__global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, const double2* __restrict__ x,
+                                                     long long n, int N) {
+    __shared__ u64 sh[256];
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    u64 m = 0;
+    if (j < N) {
+        const long long S = (long long)gridDim.y * blockDim.y;
+#pragma unroll 4
+        for (long long i = (long long)blockIdx.y * blockDim.y + threadIdx.y; i < n; i += S) {
+            const double2 v = x[i * N + j];
+            const u64 a = (u64)__double_as_longlong(v.x) & 0x7FFFFFFFFFFFFFFFull;
+            const u64 b = (u64)__double_as_longlong(v.y) & 0x7FFFFFFFFFFFFFFFull;
+            m = max(m, max(a, b));
+        }
+    }
+    sh[tid] = m;
+    __syncthreads();
+    for (int st = blockDim.y / 2; st > 0; st >>= 1) {
+        if ((int)threadIdx.y < st) sh[tid] = max(sh[tid], sh[tid + st * blockDim.x]);
+        __syncthreads();
+    }
+    if (threadIdx.y == 0 && j < N && sh[threadIdx.x] != 0) atomicMax(out + j, sh[threadIdx.x]);
+}
+
+// Digit tiles of x: per (site, 128-rhs tile) 7 K-major slices of 8 KB.  Thread = (site,
+// group of 4 components, rhs): four 16-byte loads, seven 16-byte stores.  The rows of a
+// tile beyond the rhs are not written (they only reach the same rows of the product).
+__global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const double2* __restrict__ x,
+                                                 const u64* __restrict__ mx, int nblk, int N, int T) {
+    const int row = threadIdx.x, t = blockIdx.y, j = 128 * t + row;
+    const long long g = (long long)blockIdx.x * blockDim.y + threadIdx.y;    // (block, component group)
+    const int site = (int)(g >> 2), cg = (int)(g & 3);
+    if (site >= nblk || j >= N) return;
+    const int E = (int)(mx[j] >> 52);
+    double2 v[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) v[p] = x[((size_t)site * D + 4 * cg + p) * N + j];
+    u64 qr[4], qi[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        qr[p] = (u64)fixed_point<54>(v[p].x, E) + 0x0080808080808080ull;
+        qi[p] = (u64)fixed_point<54>(v[p].y, E) + 0x0080808080808080ull;
+    }
+    uint8_t* tile = xs + ((size_t)site * T + t) * XT + kmaj32_off(row, 8 * cg);
+#pragma unroll
+    for (int s = 0; s < NX; ++s) {
+        uint32_t w[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) w[p] = pack_exact(digit(qr[p], NX - 1 - s), digit(qi[p], NX - 1 - s));
+        *reinterpret_cast<uint4*>(tile + s * XS) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Digit tiles of 16 x 16 complex blocks in their real 32 x 32 form (row = output real, K =
+// input real; the form of the BF16 stencil operands).  Block q starts at A + base(q) with
+// rows ld apart: the stencil's blocks lie one after another (ld = 16, nb = 0), block (R, C)
+// of a dense n x n matrix starts at (16 R) n + 16 C (nb = n / 16 blocks per row, ld = n).
+// Thread = (block, output real, 8 input reals).
+__global__ void __launch_bounds__(128) k_slice_a(uint8_t* __restrict__ as, const double2* __restrict__ A,
+                                                 const u64* __restrict__ mx, long long nblk, int nb, int ld) {
+    const long long q = blockIdx.x;
+    if (q >= nblk) return;
+    const int n = threadIdx.x >> 2, kg = threadIdx.x & 3;
+    const int co = n >> 1, to = n & 1;
+    const int E = (int)(*mx >> 52);
+    const double2* blk = nb ? A + (q / nb) * D * (long long)ld + (q % nb) * D : A + q * (D * D);
+    u64 u[8];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const double2 a = blk[(long long)co * ld + 4 * kg + p];
+        u[2 * p] = (u64)fixed_point<62>(to ? a.y : a.x, E) + 0x8080808080808080ull;        // times Re x
+        u[2 * p + 1] = (u64)fixed_point<62>(to ? a.x : -a.y, E) + 0x8080808080808080ull;   // times Im x
+    }
+    uint8_t* tile = as + (size_t)q * AT;
+#pragma unroll
+    for (int s = 0; s < NA; ++s) {
+        uint32_t w[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) w[p] = pack_exact(digit(u[2 * p], NA - 1 - s), digit(u[2 * p + 1], NA - 1 - s));
+        *reinterpret_cast<uint4*>(tile + kmaj32_off(s * KD + n, 8 * kg)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// 2^s sum_{g<8} G_g 2^(8 (7 - g)) rounded to FP64 once.  |G_g| < 2^25.
+__device__ __forceinline__ double combine(const int* G, int s) {
+    i64 hi = (((i64)G[0] * 256 + G[1]) * 256 + G[2]) * 256 + G[3];
+    const i64 lo = (((i64)G[4] * 256 + G[5]) * 256 + G[6]) * 256 + G[7];
+    hi += lo >> 32;                               // T = hi 2^32 + l, 0 <= l < 2^32
+    u64 l = (u64)lo & 0xFFFFFFFFull;
+    const bool neg = hi < 0;
+    if (neg) {
+        l = (0x100000000ull - l) & 0xFFFFFFFFull;
+        hi = ~hi + (l == 0 ? 1 : 0);
+    }
+    u64 h = (u64)hi;
+    int e = s + 95;                               // exponent of bit 63 of h
+    if (h == 0) {
+        if (l == 0) return 0.0;
+        h = l;
+        l = 0;
+        e -= 32;
+    }
+    const int z = __clzll((i64)h);                // h < 2^50: z >= 14
+    u64 m = h << z;
+    m |= z >= 32 ? l << (z - 32) : l >> (32 - z);
+    const u64 r = (m >> 11) + ((m >> 10) & 1);    // 2^52 <= r <= 2^53
+    const int E = e - z + 1023;                   // biased exponent of 1.xxx
+    double v;
+    if (E > 0 && E < 2046) v = __longlong_as_double((i64)(((u64)(E - 1) << 52) + r));
+    else v = ldexp((double)(i64)r, E - 1075);     // subnormal or above the range
+    return neg ? -v : v;
+}
+
+// MODE 0: y = A x; 1: y = b - A x; 2: y = A x with the per-rhs dots <y, x>, <y, y>; 3: the
+// dots only; 4: job (R, z) of a dense product, y[z] = its partial sum over K blocks
+// 6z .. 6z + 5.  nblk: sites of the stencil (lx x lt) or block rows of the dense matrix.
+template <int MODE>
+__global__ void __launch_bounds__(THREADS, 1)
+    k_block_f64(double2* __restrict__ y, const double2* __restrict__ b, const double2* __restrict__ x,
+                const uint8_t* __restrict__ xs, const uint8_t* __restrict__ as, const u64* __restrict__ mxx,
+                const u64* __restrict__ mxa, int lx, int lt, int nblk, int splits, int N, double2* __restrict__ part,
+                int* __restrict__ err) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t full[NSTG], empty[NSTG], afull[2], aempty[2];
+    __shared__ uint32_t tmem_holder;
+    __shared__ int abort_flag;
+    volatile int* abrt = &abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int G = gridDim.x, T = gridDim.y, t = blockIdx.y;
+    const int njobs_all = nblk * splits;
+    const int njob = (njobs_all - (int)blockIdx.x + G - 1) / G;
+    const int rows = min(128, N - 128 * t);
+    auto kblocks = [&](int job) { return MODE == 4 ? min(KSPLIT, nblk - (job % splits) * KSPLIT) : 5; };
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
+                     "r"(2 * ACC));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        for (int q = 0; q < NSTG; ++q) {
+            mbar_init(&full[q], 1);
+            mbar_init(&empty[q], 1);
+        }
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(&afull[q], 1);
+            mbar_init(&aempty[q], EPI_WARPS);
+        }
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_holder;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // producer: a tile narrower than 128 rhs moves only its own 8-row groups
+            const uint32_t slice = (uint32_t)((rows + 7) / 8) * 512u;
+            int q = 0;
+            bool ok = true;
+            for (int i = 0; i < njob && ok; ++i) {
+                const int job = blockIdx.x + i * G;
+                const int kb = kblocks(job);
+                for (int o = 0; o < kb; ++o, ++q) {
+                    const int slot = q % NSTG;
+                    if (q >= NSTG && !mbar_wait_ab(&empty[slot], (unsigned)((q / NSTG - 1) & 1), abrt)) {
+                        ok = false;
+                        break;
+                    }
+                    long long xb, ab;
+                    if (MODE == 4) {
+                        xb = (job % splits) * KSPLIT + o;
+                        ab = (long long)(job / splits) * nblk + xb;
+                    } else {
+                        xb = nbr_site(job, o, lx, lt);
+                        ab = (long long)job * 5 + o;
+                    }
+                    uint8_t* st = smem + slot * STAGE;
+                    const uint8_t* xsrc = xs + ((size_t)xb * T + t) * XT;
+                    mbar_expect_tx(&full[slot], slice * NX + AT);
+                    if (slice == (uint32_t)XS) {
+                        bulk_g2s(st, xsrc, XT, &full[slot]);
+                    } else {
+                        for (int s = 0; s < NX; ++s) bulk_g2s(st + s * XS, xsrc + s * XS, slice, &full[slot]);
+                    }
+                    bulk_g2s(st + XT, as + (size_t)ab * AT, AT, &full[slot]);
+                }
+            }
+            if (*abrt)
+                // copies still in flight land before the shared memory goes back
+                for (int q2 = max(0, q - NSTG); q2 < q; ++q2) mbar_wait(&full[q2 % NSTG], (unsigned)((q2 / NSTG) & 1));
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int q = 0, last = -1;
+            bool ok = true;
+            for (int i = 0; i < njob && ok; ++i) {
+                const int as2 = i & 1, kb = kblocks(blockIdx.x + i * G);
+                if (i >= 2 && !mbar_wait_ab(&aempty[as2], (unsigned)(((i >> 1) - 1) & 1), abrt)) break;
+                for (int o = 0; o < kb; ++o, ++q) {
+                    const int slot = q % NSTG;
+                    if (!mbar_wait_ab(&full[slot], (unsigned)((q / NSTG) & 1), abrt)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t sx = smem_u32(smem + slot * STAGE), sa = sx + XT;
+#pragma unroll
+                    for (int j = 0; j < NX; ++j)
+#pragma unroll
+                        for (int ks = 0; ks < 2; ++ks)
+                            mma_bf16(tmem + as2 * ACC + KD * j, smem_desc(sx + j * XS + ks * 256, 128, 512),
+                                     smem_desc(sa + ks * 256, 128, 512), instr_desc(128, ACC - KD * j),
+                                     (o > 0 || j > 0 || ks > 0) ? 1u : 0u);
+                    mma_commit(&empty[slot]);
+                    if (o + 1 == kb) mma_commit(&afull[as2]);
+                    last = q;
+                }
+            }
+            // MMAs in flight complete before the TMEM and shared memory go back
+            if (*abrt && last >= 0) mbar_wait(&empty[last % NSTG], (unsigned)((last / NSTG) & 1));
+        }
+    } else {
+        // epilogue: two warps per TMEM lane quarter, 16 of the 32 output reals each
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        const int jl = quarter * 32 + lane, j = 128 * t + jl;
+        const int ex = j < N ? (int)(mxx[j] >> 52) : 0, ea = (int)(*mxa >> 52);
+        const bool finite = ex != 0x7ff && ea != 0x7ff;
+        const int sc = (ex - 1022) + (ea - 1022) - 68;
+        double2 dyx = make_double2(0.0, 0.0);
+        double dyy = 0.0;
+        bool ok = true;
+        for (int i = 0; i < njob; ++i) {
+            const int as2 = i & 1;
+            if (!mbar_wait_ab(&afull[as2], (unsigned)((i >> 1) & 1), abrt)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int job = blockIdx.x + i * G;
+            const long long row0 = (long long)(MODE == 4 ? job / splits : job) * D;
+            double2* yo = MODE == 4 ? y + (long long)(job % splits) * nblk * D * N : y;
+            const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(as2 * ACC + half * 16);
+#pragma unroll 1
+            for (int c = 0; c < 16; c += 4) {
+                uint32_t r[NA][4];
+#pragma unroll
+                for (int g = 0; g < NA; ++g)
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3])
+                                 : "r"(base + (uint32_t)(g * KD + c)));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (c == 12) {
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&aempty[as2]);      // accumulator may be overwritten
+                }
+                if (j < N) {
+                    double v[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        int Gi[NA];
+#pragma unroll
+                        for (int g = 0; g < NA; ++g) Gi[g] = __float2int_rn(__uint_as_float(r[g][p]));
+                        v[p] = finite ? combine(Gi, sc) : __longlong_as_double(0x7ff8000000000000ll);
+                    }
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        const long long idx = (row0 + half * 8 + (c >> 1) + p) * N + j;
+                        double2 o = make_double2(v[2 * p], v[2 * p + 1]);
+                        if (MODE == 1) o = csub(b[idx], o);
+                        if (MODE != 3) yo[idx] = o;
+                        if (MODE == 2 || MODE == 3) {
+                            cfmac(dyx, o, x[idx]);
+                            dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
+                        }
+                    }
+                }
+            }
+        }
+        if (MODE == 2 || MODE == 3) {
+            // the two halves of a rhs meet in shared memory (the stages are free: every copy
+            // has landed and every MMA has completed once the last accumulator was read)
+            double* red = reinterpret_cast<double*>(smem);
+            asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS));
+            if (half == 1) {
+                red[3 * jl] = dyx.x;
+                red[3 * jl + 1] = dyx.y;
+                red[3 * jl + 2] = dyy;
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS));
+            if (half == 0 && ok && j < N) {
+                part[(long long)j * G + blockIdx.x] = make_double2(dyx.x + red[3 * jl], dyx.y + red[3 * jl + 1]);
+                part[(long long)(N + j) * G + blockIdx.x] = make_double2(dyy + red[3 * jl + 2], 0.0);
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (tid == 0 && abort_flag) atomicExch(err, 1);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * ACC));
+}
+
+// y = sum over the splits of a dense product, in order.
+__global__ void __launch_bounds__(256) k_sum_splits(double2* __restrict__ y, const double2* __restrict__ p,
+                                                    long long count, int splits) {
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
+         e += (long long)gridDim.x * blockDim.x) {
+        double2 s = p[e];
+        for (int z = 1; z < splits; ++z) s = cadd(s, p[z * count + e]);
+        y[e] = s;
+    }
+}
+}  // namespace f64
+}  // namespace tc
+
+using namespace tc::f64;
+
+static int f64_tiles(int N) { return (N + 127) / 128; }
+
+bool f64_tc_supported(int d, int N) { return d == D && f64_tiles(N) <= 65535; }
+size_t f64_tc_operand_bytes(long long nblk) { return (size_t)nblk * AT + 256; }
+size_t f64_tc_scratch_bytes(long long nblk, int N) {
+    return (size_t)nblk * f64_tiles(N) * XT + ((size_t)N * sizeof(u64) + 255) / 256 * 256;
+}
+int f64_dense_splits(int n) { return (n / D + KSPLIT - 1) / KSPLIT; }
+
+static void absmax(u64* out, const double2* x, long long n, int N, cudaStream_t s) {
+    MG_CUDA(cudaMemsetAsync(out, 0, sizeof(u64) * N, s));
+    int bx = 1;
+    while (bx < N && bx < 32) bx *= 2;
+    const int by = 256 / bx, gx = (N + bx - 1) / bx;
+    const long long need = (n + 4 * by - 1) / (4 * by);
+    const int gy = (int)std::max(1LL, std::min(need, 8LL * kNumSM / gx));
+    k_absmax_cols<<<dim3(gx, gy), dim3(bx, by), 0, s>>>(out, x, n, N);
+    MG_LAUNCHED();
+}
+
+// Operand: the digit tiles, then (256-byte aligned) the bits of the largest entry.
+static const u64* operand_max(const void* op, long long nblk) {
+    return reinterpret_cast<const u64*>(reinterpret_cast<const uint8_t*>(op) + (size_t)nblk * AT);
+}
+
+void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int ld, cudaStream_t s) {
+    MG_REQUIRE(nblk >= 1 && nblk <= (1LL << 31) - 1, MGMLMC_EINVAL, "FP64 operand: size");
+    u64* mx = const_cast<u64*>(operand_max(op, nblk));
+    // a flat array as 32 columns: the maximum of its 32 column maxima is taken below
+    absmax(mx, A, nblk * (D * D) / 32, 32, s);
+    tc::f64::k_absmax_cols<<<1, dim3(1, 32), 0, s>>>(mx, reinterpret_cast<const double2*>(mx), 16, 1);
+    MG_LAUNCHED();
+    k_slice_a<<<(unsigned)nblk, 128, 0, s>>>(reinterpret_cast<uint8_t*>(op), A, mx, nblk, nb, nb ? ld : D);
+    MG_LAUNCHED();
+}
+
+// Slices x into the scratch: digit tiles, then the largest entry per rhs.
+static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N, cudaStream_t s) {
+    const int T = f64_tiles(N);
+    u64* mx = reinterpret_cast<u64*>(reinterpret_cast<uint8_t*>(scratch) + (size_t)nblk * T * XT);
+    absmax(mx, x, nblk * D, N, s);
+    int bx = 8;
+    while (bx < N && bx < 128) bx *= 2;
+    const int by = 128 / bx;
+    k_slice_x<<<dim3((unsigned)((4 * nblk + by - 1) / by), T), dim3(bx, by), 0, s>>>(
+        reinterpret_cast<uint8_t*>(scratch), x, mx, (int)nblk, N, T);
+    MG_LAUNCHED();
+    return mx;
+}
+
+template <int MODE>
+static void f64_launch(double2* y, const double2* b, const double2* x, const void* scratch, const void* op,
+                       const u64* mxx, const u64* mxa, int lx, int lt, int nblk, int splits, int N, double2* part,
+                       int groups, int* err, cudaStream_t s) {
+    MG_CUDA(cudaFuncSetAttribute(k_block_f64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
+    k_block_f64<MODE><<<dim3(groups, f64_tiles(N)), THREADS, SMEM, s>>>(
+        y, b, x, reinterpret_cast<const uint8_t*>(scratch), reinterpret_cast<const uint8_t*>(op), mxx, mxa, lx, lt,
+        nblk, splits, N, part, err);
+    MG_LAUNCHED();
+}
+
+int block_stencil_f64_groups(int nsites, int N) {
+    return std::max(1, std::min(nsites, kNumSM / f64_tiles(N)));
+}
+
+void launch_block_stencil_f64(double2* y, const double2* x, const double2* b, const void* op, int lx, int lt, int N,
+                              int mode, void* scratch, double2* part, int groups, int* err, cudaStream_t s) {
+    const int V = lx * lt;
+    MG_REQUIRE(f64_tc_supported(D, N) && groups >= 1 && groups <= V, MGMLMC_EINVAL, "FP64 stencil: size");
+    const u64* mxx = slice_x(scratch, x, V, N, s);
+    const u64* mxa = operand_max(op, 5LL * V);
+    switch (mode) {
+        case 0: f64_launch<0>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
+        case 1: f64_launch<1>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
+        case 2: f64_launch<2>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
+        default: f64_launch<3>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
+    }
+}
+
+size_t f64_dense_scratch_bytes(int n, int N) {
+    const size_t a = (f64_tc_scratch_bytes(n / D, N) + 255) / 256 * 256;
+    return a + (size_t)f64_dense_splits(n) * n * N * sizeof(double2);
+}
+
+void launch_dense_f64(double2* y, const double2* x, const void* op, int n, int N, void* scratch, int* err,
+                      cudaStream_t s) {
+    const int nb = n / D, S = f64_dense_splits(n);
+    MG_REQUIRE(n % D == 0 && f64_tc_supported(D, N), MGMLMC_EINVAL, "FP64 dense product: n % 16 == 0");
+    const u64* mxx = slice_x(scratch, x, nb, N, s);
+    double2* p = reinterpret_cast<double2*>(reinterpret_cast<uint8_t*>(scratch) +
+                                            (f64_tc_scratch_bytes(nb, N) + 255) / 256 * 256);
+    const long long jobs = (long long)nb * S;
+    const int G = (int)std::max(1LL, std::min(jobs, (long long)kNumSM / f64_tiles(N)));
+    f64_launch<4>(S == 1 ? y : p, nullptr, nullptr, scratch, op, mxx, operand_max(op, (long long)nb * nb), 0, 0, nb, S,
+                  N, nullptr, G, err, s);
+    if (S > 1) {
+        const long long cnt = (long long)n * N;
+        k_sum_splits<<<(int)std::min((cnt + 255) / 256, 16LL * kNumSM), 256, 0, s>>>(y, p, cnt, S);
+        MG_LAUNCHED();
+    }
+}
+
+}  // namespace mg

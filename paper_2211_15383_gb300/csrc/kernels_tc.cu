@@ -18,6 +18,7 @@
 // mbarrier wait is bounded: on timeout the CTA records an error flag, frees TMEM
 // and returns.
 #include "kernels.cuh"
+#include "tcgen05.cuh"
 
 namespace mg {
 
@@ -25,48 +26,6 @@ namespace tc {
 
 constexpr int BM = 128;         // rows per tile (TMEM lanes)
 constexpr int BK = 64;          // K per stage (4 MMAs of K = 16)
-constexpr unsigned kWaitLimit = 1u << 26;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// Shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows x
-// 16 bytes; lbo = byte distance between core matrices adjacent along K, sbo =
-// byte distance between 8-row groups; bits 46-48 hold the fixed version 0b001.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
-// Instruction descriptor of kind::f16: D = F32, A = B = BF16, both K-major.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-// Bounded wait for the completion of the phase with the given parity.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
-    const uint32_t a = smem_u32(bar);
-    for (unsigned it = 0; it < kWaitLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
 // Canonical K-major layout of a rows x 64 BF16 tile: 8-row groups of 1024 B
 // (eight 128-byte core matrices along K), rows 16 B apart inside a core matrix.
 // Operands are stored pre-tiled in global memory: a 128 x 64 tile of A' (16 KB) or
@@ -78,20 +37,6 @@ __host__ __device__ __forceinline__ size_t tiled_off(int row, int k, int rows_pe
     const int tile_k = k / 64, kk = k % 64;
     return ((size_t)tile_r * ktiles + tile_k) * (size_t)rows_per_tile * 128 +
            (size_t)((r >> 3) * 1024 + (kk >> 3) * 128 + (r & 7) * 16 + (kk & 7) * 2);
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(
-                     smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(smem_dst)),
-        "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
 }
 
 // Warp-specialised main loop: thread 0 (warp 0) streams stages with bulk copies,
@@ -568,20 +513,8 @@ constexpr int THREADS = 192;               // 6 warps
 constexpr int kCtasPerSm = 3;              // three pipelines per SM
 constexpr int SMEM = NSTG * TILE_A + 2 * B_SITE;   // 68 KB: three CTAs per SM
 constexpr int TCOLS = 64;                  // two accumulators of 32 columns
-constexpr int kMaxDevWait = 1 << 26;
 // direction of the o-th job of a site: the neighbours first, the self block last
 __device__ __forceinline__ int dir_of(int o) { return o == 4 ? 0 : o + 1; }
-
-// Byte offset of (row, k) in a K-major, no-swizzle tile with K = 32: 8-row groups
-// of 512 B, four 128-byte core matrices along K, rows 16 B apart.
-__host__ __device__ __forceinline__ int kmaj32_off(int row, int k) {
-    return (row >> 3) * 512 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
 
 // B(s, dir) for every site: E[(s * 5 + dir) * 1024 + off / 2], element (n = output
 // real, k = input real) of the real form of A(s, dir)^T.
@@ -755,26 +688,6 @@ __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e,
             e[base + (size_t)c * N] = acc[c];
         }
     }
-}
-
-// Bounded wait that also gives up as soon as another role has aborted.
-__device__ __forceinline__ bool mbar_wait_ab(uint64_t* bar, unsigned parity, volatile int* abort_flag) {
-    const uint32_t a = smem_u32(bar);
-    for (int it = 0; it < kMaxDevWait; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (*abort_flag) return false;
-    }
-    *abort_flag = 1;
-    return false;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // FORM 0: y = A x as FP32 rows, with the dots; 1: y as BF16 tiles (yt), with the dots;

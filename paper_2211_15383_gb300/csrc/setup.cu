@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "context.h"
+#include "footprint.h"
 
 namespace mg {
 
@@ -109,6 +110,7 @@ void Ctx::free_hierarchy() {
         dev_free(L.A64); dev_free(L.A32); dev_free(L.P64); dev_free(L.P32); dev_free(L.tv);
         dev_free(L.Minv64); dev_free(L.Minv32); dev_free(L.Ahat64); dev_free(L.Ahat32); dev_free(L.Ahat16); dev_free(L.A16);
         dev_free(L.Dinv64); dev_free(L.Dinv32); dev_free(L.Dinv16);
+        dev_free(L.A64t); dev_free(L.Ahat64t); dev_free(L.Dinv64t);
         L = Level();
     }
     free_deflation();
@@ -234,6 +236,12 @@ void copy_state(Ctx& d, Ctx& s) {
         const size_t nb = (size_t)b.nsites * b.d * b.d;
         a.A64 = dup(d, b.A64, 5 * nb);
         a.A32 = dup(d, b.A32, 5 * nb);
+        auto dup_digits = [&](const void* p, long long nblk) -> void* {
+            return dup(d, reinterpret_cast<const char*>(p), f64_tc_operand_bytes(nblk));
+        };
+        a.A64t = dup_digits(b.A64t, 5LL * b.nsites);
+        a.Ahat64t = dup_digits(b.Ahat64t, 5LL * b.nsites);
+        a.Dinv64t = dup_digits(b.Dinv64t, (b.n / 16) * (b.n / 16));
         a.Minv64 = dup(d, b.Minv64, nb);
         a.Minv32 = dup(d, b.Minv32, nb);
         a.Ahat64 = dup(d, b.Ahat64, 5 * nb);
@@ -366,8 +374,15 @@ static void coarsest_inverse(Ctx& c) {
     if (c.opt.mg_precision == 64) {
         if (!L.Dinv64) L.Dinv64 = c.alloc_n<double2>((size_t)n * n);
         MG_CUDA(cudaMemcpyAsync(L.Dinv64, Dd, sizeof(double2) * n * n, cudaMemcpyDeviceToDevice, c.stream));
-        ProfScope ps(c, "setup.gauss_jordan.f64", 2.0 * n * n * 16 * std::ceil(n / 16.0), 8.0 * n * n * n);
-        launch_gauss_jordan<double2>(L.Dinv64, (int)n, work, c.stream);
+        {
+            ProfScope ps(c, "setup.gauss_jordan.f64", 2.0 * n * n * 16 * std::ceil(n / 16.0), 8.0 * n * n * n);
+            launch_gauss_jordan<double2>(L.Dinv64, (int)n, work, c.stream);
+        }
+        if (f64_dense_inverse(n)) {
+            const long long nb = n / 16;
+            if (!L.Dinv64t) L.Dinv64t = c.dev_alloc(f64_tc_operand_bytes(nb * nb));
+            launch_f64_operand(L.Dinv64t, L.Dinv64, nb * nb, (int)nb, (int)n, c.stream);
+        }
     } else {
         if (!L.Dinv32) L.Dinv32 = c.alloc_n<float2>((size_t)n * n);
         launch_convert<float2, double2>(L.Dinv32, Dd, n * n, c.stream);
@@ -382,6 +397,13 @@ static void coarsest_inverse(Ctx& c) {
     MG_CUDA(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     c.sync();
     MG_REQUIRE(hs == 0, MGMLMC_EINVAL, "coarsest operator is singular (zero pivot)");
+}
+
+// Digits of a level's stencil blocks for the FP64 products on the tensor cores.
+static void f64_stencil_operand(Ctx& c, void*& op, const double2* A, const Level& L) {
+    if (!f64_tc_supported(L.d, 1)) return;
+    if (!op) op = c.dev_alloc(f64_tc_operand_bytes(5LL * L.nsites));
+    launch_f64_operand(op, A, 5LL * L.nsites, 0, 0, c.stream);
 }
 
 // Block-Jacobi smoother of coarse level l: M = block diagonal of D_l (the self
@@ -402,6 +424,7 @@ static void block_jacobi_setup(Ctx& c, int l) {
     launch_precondition_blocks(L.Ahat64, L.A64, L.Minv64, L.lx, L.lt, L.d, c.stream);
     launch_convert<float2, double2>(L.Minv32, L.Minv64, (long long)nb, c.stream);
     launch_convert<float2, double2>(L.Ahat32, L.Ahat64, (long long)nb * 5, c.stream);
+    if (c.opt.mg_precision == 64) f64_stencil_operand(c, L.Ahat64t, L.Ahat64, L);
     if (c.opt.mg_precision == 16 && tc_stencil_supported(L.d, 2)) {
         if (!L.Ahat16) L.Ahat16 = c.alloc_n<__nv_bfloat16>((size_t)L.nsites * 5 * 4 * L.d * L.d);
         if (!L.A16) L.A16 = c.alloc_n<__nv_bfloat16>((size_t)L.nsites * 5 * 4 * L.d * L.d);
@@ -431,6 +454,7 @@ static void rebuild_from(Ctx& c, int l0) {
         ProfScope ps(c, "setup.galerkin", 0, 0);
         launch_galerkin(Lc.A64, L.A64, L.P64, L.lx, L.lt, L.d, L.ax, L.at, L.nvec, T, c.stream);
         launch_convert<float2, double2>(Lc.A32, Lc.A64, (long long)Lc.nsites * 5 * Lc.d * Lc.d, c.stream);
+        f64_stencil_operand(c, Lc.A64t, Lc.A64, Lc);
         if (l + 1 < c.L - 1) block_jacobi_setup(c, l + 1);
     }
     coarsest_inverse(c);

@@ -48,9 +48,34 @@ static bool galerkin_form_cheaper(const Ctx& c, int l) {
     return galerkin < direct;
 }
 
+// FP64 block stencils with d = 16 run on the tensor cores (exact integer digit products, at
+// least as accurate as FP64 sums) from this many right-hand sides on; below it the digits'
+// three extra launches cost more than the FP64 pipe saves.
+constexpr int kF64TcMinRhs = 16;
+template <typename C>
+static bool f64_stencil(Ctx&, const Level&, C*, const C*, const C*, const void*, int, int, double2*, int) {
+    return false;
+}
+static bool f64_stencil_used(const Level& L, const void* op, int N) {
+    return op && N >= kF64TcMinRhs && f64_tc_supported(L.d, N);
+}
+template <>
+bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, const double2* b, const void* op, int N,
+                          int mode, double2* part, int groups) {
+    if (!f64_stencil_used(L, op, N)) return false;
+    launch_block_stencil_f64(y, x, b, op, L.lx, L.lt, N, mode,
+                             c.scratch_bytes("f64_tc", f64_tc_scratch_bytes(L.nsites, N)), part, groups,
+                             device_error_flag(c), c.stream);
+    return true;
+}
+template <typename C> static int bst_groups(const Level& L, const void* op, int N) {
+    return sizeof(C) == 16 && f64_stencil_used(L, op, N) ? block_stencil_f64_groups(L.nsites, N)
+                                                         : block_stencil_groups(L.nsites, L.d, N);
+}
+
 template <typename C> static bool galerkin_apply(Ctx&, C*, const C*, const C*, int, int) { return false; }
 template <> bool galerkin_apply<double2>(Ctx& c, double2* y, const double2* x, const double2* b, int N, int mode) {
-    if (mode >= 2 || !galerkin_form_cheaper(c, 1)) return false;
+    if (mode >= 2 || f64_stencil_used(c.lev[1], c.lev[1].A64t, N) || !galerkin_form_cheaper(c, 1)) return false;
     const Level& F = c.lev[0];
     const Level& Cl = c.lev[1];
     double2* t = c.scratch<double2>("gal64_t", (size_t)F.n * N);
@@ -79,7 +104,7 @@ template <typename C>
 void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* alpha) {
     if (l == 1 && galerkin_apply<C>(c, y, x, b, N, mode)) return;
     const Level& L = c.lev[l];
-    const int groups = (l == 0) ? stencil_groups(L.nsites, N) : block_stencil_groups(L.nsites, L.d, N);
+    const int groups = (l == 0) ? stencil_groups(L.nsites, N) : bst_groups<C>(L, L.A64t, N);
     // algorithmic traffic: read x once, write y once (+ b for the residual form),
     // operator data once; flops: 60 per fine site and rhs, 8 d^2 * 5 per coarse site and rhs
     const double s = sizeof(C);
@@ -93,7 +118,7 @@ void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* al
         ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)), bytes, flops);
         if (l == 0)
             launch_wilson<C>(y, x, b, links<C>(c), c.m0, L.lx, L.lt, N, mode, part, groups, c.stream);
-        else
+        else if (!f64_stencil<C>(c, L, y, x, b, L.A64t, N, mode, part, groups))
             launch_block_stencil<C>(y, x, b, blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
     if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
@@ -149,14 +174,15 @@ static void pack_tiles(Ctx& c, int l, __nv_bfloat16* xt, const float2* x, int N)
 template <typename C>
 static void apply_Dhat(Ctx& c, int l, C* y, const C* x, int N, int mode, C* alpha) {
     const Level& L = c.lev[l];
-    const int groups = block_stencil_groups(L.nsites, L.d, N);
+    const int groups = bst_groups<C>(L, L.Ahat64t, N);
     const double s = sizeof(C);
     double2* part = mode >= 2 ? c.scratch<double2>("part_st", (size_t)groups * 2 * N) : nullptr;
     {
         ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
                      (double)L.n * N * s * (mode == 3 ? 1 : 2) + 5.0 * L.nsites * L.d * L.d * s,
                      40.0 * L.d * L.d * (double)L.nsites * N);
-        launch_block_stencil<C>(y, x, nullptr, hat_blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
+        if (!f64_stencil<C>(c, L, y, x, (const C*)nullptr, L.Ahat64t, N, mode, part, groups))
+            launch_block_stencil<C>(y, x, nullptr, hat_blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
     if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
 }
@@ -203,6 +229,11 @@ static double dinv_flops(const Level& L, int N) { return 8.0 * (double)L.n * L.n
 template <> void coarsest_apply<double2>(Ctx& c, double2* e, const double2* r, int N) {
     const Level& L = c.lev[c.L - 1];
     ProfScope ps(c, "Dinv.f64", dinv_bytes(L, N, 16), dinv_flops(L, N));
+    if (L.Dinv64t && N >= kF64TcMinRhs && f64_tc_supported(16, N)) {
+        void* scr = c.scratch_bytes("f64_dense", f64_dense_scratch_bytes((int)L.n, N));
+        launch_dense_f64(e, r, L.Dinv64t, (int)L.n, N, scr, device_error_flag(c), c.stream);
+        return;
+    }
     launch_gemm_nn<double2>(e, L.Dinv64, r, (int)L.n, (int)L.n, N, false, c.stream);
 }
 template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int N) {
@@ -736,6 +767,7 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
     if (c.opt.mg_precision == 64) {
         const long long it = fgmres<double2>(c, l, b, x, N, tol, maxit, true, ok, 1 << 30);
         c.last_iters = it;
+        check_device_error(c);
         return it;
     }
     // Mixed: FP64 iterative refinement, FP32 FGMRES + FP32 multigrid inside.
