@@ -865,6 +865,7 @@ void release_scratch(Ctx& c) {
     for (auto& kv : c.ws) c.dev_free(kv.second.p);
     c.ws.clear();
     c.dev_err = nullptr;
+    c.dev_max = nullptr;
 }
 
 }  // namespace

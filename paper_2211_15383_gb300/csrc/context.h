@@ -121,6 +121,10 @@ struct Ctx {
     std::string err;
     double* hbuf = nullptr;          // pinned host scratch for scalar read-backs
     int* dev_err = nullptr;          // device error flag of kernels with bounded waits
+    // maxima over the right-hand sides that the host reads back, as bits of doubles: used in
+    // turn, each zero again when its turn comes (the kernel two turns earlier clears it)
+    unsigned long long* dev_max = nullptr;
+    int max_turn = 0;
     size_t hbuf_bytes = 0;
 
     int Lx = 0, Lt = 0;

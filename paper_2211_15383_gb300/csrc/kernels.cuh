@@ -35,9 +35,6 @@ void launch_convert(Cout* y, const Cin* x, long long count, cudaStream_t s);
 // y[i][j] = scale[j] * x[i][j] (scale real, per rhs); scale may be inverted (1/scale, 0 if scale == 0)
 template <typename Cy, typename Cx_>
 void launch_scale_rhs(Cy* y, const Cx_* x, const double* scale, bool invert, long long n, int N, cudaStream_t s);
-// w[:, j] *= s[j] where s[j] != 0 (other columns untouched).
-template <typename C>
-void launch_scale_cols_if(C* w, const double* s, long long n, int N, cudaStream_t st);
 // y[i][j] += sign * alpha[j] * x[i][j]  (alpha complex per rhs, optionally times real beta[j])
 template <typename Cy, typename Cx_>
 void launch_axpy_rhs(Cy* y, const double2* alpha, const double* beta, double sign, const Cx_* x,
@@ -50,35 +47,65 @@ void launch_transpose(double2* out, const double2* in, long long rows, int cols,
 // ------------------------------------------------------------- reductions
 // Number of row groups (partials) used by the reduction kernels for (n, N).
 int reduce_groups(long long n, int N);
-// Row groups of launch_multiaxpy(_norm2): size of the norm partials is axpy_groups * N.
-int axpy_groups(long long n, int N);
 // out[j] = sum_i conj(x[i][j]) * y[i][j]  (double2), via scratch part[groups][N]
 template <typename Cx_, typename Cy>
 void launch_dot(double2* out, const Cx_* x, const Cy* y, long long n, int N, double2* part, cudaStream_t s);
-// out[j] = sum_i |x[i][j]|^2
+// ---- FGMRES and refinement (kernels_krylov.cu)
+// What a norm's reduction writes besides, per rhs (any pointer may be null).
+struct NormOut {
+    double* norm = nullptr;                  // the norm
+    // *max = max(*max, norm mul / den) over the rhs with den > 0 (den null: norm / norm), as the
+    // bits of a double (NaN is the largest); *clear = 0 for a later use
+    unsigned long long* max = nullptr;
+    unsigned long long* clear = nullptr;
+    const double* den = nullptr;
+    const double* mul = nullptr;
+    // a basis vector w = eta v: eta, 1 / eta (0 for a zero vector); where |w| leaves
+    // [2^-32, 2^32], rsc = 1 / |w| for launch_scale_cols_if and eta = 1, else rsc = 0; g0 =
+    // |w| as complex.  With hsub: the norm is |w / eta_prev|, hsub = it (0 if eta_prev is 0).
+    double* eta = nullptr;
+    double* ieta = nullptr;
+    double* rsc = nullptr;
+    double2* g0 = nullptr;
+    double* hsub = nullptr;
+    const double* eta_prev = nullptr;
+};
+// Bytes of the partials of launch_multidot with at most m vectors, and of every norm.
+size_t dot_part_bytes(long long n, int N, int m);
+size_t norm_part_bytes(long long n, int N);
+// For the vectors w_k = V + k n N (k < m) of an unnormalised basis (ieta[k][N] = 1 / eta_k):
+// cf[k][N] = -<w_k, w> / eta_k^2 and H[k][N] (+)= <w_k, w> / (eta_k eta_{m-1}).
 template <typename C>
-void launch_norm2(double* out, const C* x, long long n, int N, double* part, cudaStream_t s);
-// out[k][j] = <V_k, w>_j for k < m; V_k = V + k * n * N.  part: [groups][m][N].
+void launch_multidot(C* cf, double2* H, const C* V, int m, const C* w, long long n, int N, const double* ieta, bool add,
+                     void* part, cudaStream_t s);
+// w (=|+=) sum_{k < m} cf_k V_k; norm (may be null): of the result times nscale[j] (null or 0: 1).
 template <typename C>
-void launch_multidot(double2* out, const C* V, int m, const C* w, long long n, int N, double2* part,
-                     cudaStream_t s);
-// w[i][j] = (accumulate ? w[i][j] : 0) + sign * sum_k c[k][j] V_k[i][j], with
-// c[k][j] = coef[k][j], or coef[k][j] / eta[k][j]^eta_pow (eta_pow 1 or 2; 0 where eta is 0)
-// when eta is given: the coefficients of unnormalised basis vectors V_k = eta_k v_k.
+void launch_multiaxpy(C* w, const C* cf, int m, const C* V, long long n, int N, bool accumulate, const NormOut* norm,
+                      void* npart, const double* nscale, cudaStream_t s);
 template <typename C>
-void launch_multiaxpy(C* w, const double2* coef, int m, const C* V, double sign, long long n, int N,
-                      cudaStream_t s, const double* eta = nullptr, int eta_pow = 0, bool accumulate = true);
-// As launch_multiaxpy (accumulating), and norm2[j] = |w_j / norm_div[j]|^2 of the updated
-// w (norm_div NULL or 0: 1; part: axpy_groups(n, N) * N scratch).
+void launch_norm(const NormOut& o, const C* x, long long n, int N, void* npart, cudaStream_t s);
+// y = scale x (scale null: 1; inverse: x / scale, 0 where scale is 0) and the norms of y.
+template <typename Cy, typename Cx_>
+void launch_scale_norm(const NormOut& o, Cy* y, const Cx_* x, const double* scale, bool inverse, long long n, int N,
+                       void* npart, cudaStream_t s);
+// y (=|+=) sign scale x, and the norms of x (of_x) or of the new y (of_y; at most one of them).
+void launch_refine_axpy(double2* y, const double* scale, double sign, const float2* x, long long n, int N,
+                        bool accumulate, const NormOut* of_x, const NormOut* of_y, void* npart, cudaStream_t s);
+// w[:, j] *= f[j] where f[j] != 0 (other columns untouched).
 template <typename C>
-void launch_multiaxpy_norm2(C* w, const double2* coef, int m, const C* V, double sign, long long n, int N,
-                            double* norm2, double* part, cudaStream_t s, const double* eta = nullptr,
-                            int eta_pow = 0, const double* norm_div = nullptr);
+void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_t s);
+// Givens rotations of the Hessenberg columns j0..j1 (H[j][m + 1][N], subdiagonals hsub[j][N]):
+// rotations cs, sn [j][N], rotated right-hand side g[m + 1][N], irr[j][N] = 1 / R_jj; *max =
+// max(*max, residual / bnorm) after column j1 (max may be null), *clear = 0.
+void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,
+                   const double* bnorm, unsigned long long* max, unsigned long long* clear, int j0, int j1, int m, int N,
+                   cudaStream_t s);
+// cf[i][N] = y_i / eta_i, i <= j, with R y = g.
+template <typename C>
+void launch_back_substitute(C* cf, const double2* H, const double2* g, const double2* irr, const double* ieta, int j,
+                            int m, int N, cudaStream_t s);
 // Sum of partials: out[j] = sum_g part[g][j] (count = values per group).
 void launch_finalize(double2* out, const double2* part, int groups, int count, cudaStream_t s);
-void launch_finalize(double* out, const double* part, int groups, int count, cudaStream_t s);
-// Row-major partials (the stencils' minimal-residual dots): out[i] = sum_g part[i * groups + g].
-void launch_finalize_rows(double2* out, const double2* part, int groups, int count, cudaStream_t s);
 // alpha[j] = <y, x>_j / <y, y>_j (0 where <y, y> is 0) from a stencil's partials of its two dots.
 template <typename C>
 void launch_finalize_alpha(C* alpha, const double2* part, int groups, int N, cudaStream_t s);
@@ -87,7 +114,7 @@ void launch_finalize_alpha(C* alpha, const double2* part, int groups, int N, cud
 // Fine Wilson-Schwinger operator (2 spins, U(1) links U[site][mu]).
 //  mode 0: y = D x;  mode 1: y = b - D x;
 //  mode 2: y = D x and part[0][j][g] = <y, x>_j, part[1][j][g] = <y, y>_j (MR smoother;
-//          row-major in the group index g = blockIdx.y, see launch_finalize_rows)
+//          row-major in the group index g = blockIdx.y, see launch_finalize_alpha)
 //  mode 3: the dots of mode 2 without y (which may be null)
 template <typename C>
 void launch_wilson(C* y, const C* x, const C* b, const C* U, double m0, int lx, int lt, int N,
@@ -252,14 +279,6 @@ size_t galerkin_scratch_count(int lx, int lt, int d, int nvec);
 // status[0] set to 1 if a block is rank deficient.
 void launch_build_prolongator(double2* P, const double2* tv, int lx, int lt, int d, int ax, int at,
                               int nvec, int* status, cudaStream_t s);
-// Small per-rhs FGMRES bookkeeping (one thread per rhs).
-void launch_arnoldi_column(double2* H, double* cs, double2* sn, double2* g, double* resid,
-                           const double2* h, const double* hnorm, int j, int m, int N, cudaStream_t s);
-void launch_back_substitute(double2* y, const double2* H, const double2* g, int j, int m, int N,
-                            cudaStream_t s);
-void launch_init_g(double2* g, const double* beta, int m, int N, cudaStream_t s);
-// max over rhs of resid[j] / bnorm[j] -> out (device scalar)
-void launch_max_ratio(double* out, const double* resid, const double* bnorm, int N, cudaStream_t s);
 // samples: s[j] = sign * <x, z>_j + s[j] (accumulate) helpers live in the estimator.
 void launch_deflation_correction(double2* s, const double2* A, const double2* B, const double* a, int k,
                                  int N, cudaStream_t s_);

@@ -173,117 +173,6 @@ void launch_build_prolongator(double2* P, const double2* tv, int lx, int lt, int
     MG_LAUNCHED();
 }
 
-// ------------------------------------------------------------- FGMRES bookkeeping
-// Per rhs r: H[r][i][j] (i <= j) the rotated upper-triangular Hessenberg,
-// cs[r][j] real cosines, sn[r][j] complex sines, g[r][0..m] the rotated rhs.
-__global__ void k_init_g(double2* g, const double* beta, int m, int N) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    for (int i = 0; i <= m; ++i) g[(long long)r * (m + 1) + i] = make_double2(i == 0 ? beta[r] : 0.0, 0.0);
-}
-
-__global__ void k_arnoldi_column(double2* H, double* cs, double2* sn, double2* g, double* resid, const double2* h,
-                                 const double* hnorm, int j, int m, int N) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    double2* Hr = H + (long long)r * (m + 1) * m;
-    double* c_r = cs + (long long)r * m;
-    double2* s_r = sn + (long long)r * m;
-    double2* g_r = g + (long long)r * (m + 1);
-    double2 col[65];
-    for (int i = 0; i <= j; ++i) col[i] = h[(long long)i * N + r];
-    col[j + 1] = make_double2(hnorm[r], 0.0);
-    // previous rotations: (a, b) <- (c a + s b, -conj(s) a + c b)
-    for (int i = 0; i < j; ++i) {
-        const double c = c_r[i];
-        const double2 s = s_r[i];
-        const double2 a = col[i], b = col[i + 1];
-        const double2 sb = cmul(s, b);
-        const double2 sca = cmulc(s, a);
-        col[i] = make_double2(c * a.x + sb.x, c * a.y + sb.y);
-        col[i + 1] = make_double2(c * b.x - sca.x, c * b.y - sca.y);
-    }
-    // new rotation zeroing col[j+1]
-    const double2 a = col[j], b = col[j + 1];
-    const double na = sqrt(a.x * a.x + a.y * a.y), nb = sqrt(b.x * b.x + b.y * b.y);
-    const double rho = sqrt(na * na + nb * nb);
-    double c;
-    double2 s, rr;
-    if (rho == 0.0) {
-        c = 1.0; s = make_double2(0, 0); rr = make_double2(0, 0);
-    } else if (na == 0.0) {
-        c = 0.0; s = make_double2(b.x / nb, -b.y / nb); rr = make_double2(nb, 0);   // s = conj(b)/|b|
-    } else {
-        const double2 ph = make_double2(a.x / na, a.y / na);
-        c = na / rho;
-        s = cmul(ph, make_double2(b.x / rho, -b.y / rho));      // (a/|a|) conj(b) / rho
-        rr = make_double2(ph.x * rho, ph.y * rho);
-    }
-    c_r[j] = c;
-    s_r[j] = s;
-    col[j] = rr;
-    for (int i = 0; i <= j; ++i) Hr[(long long)i * m + j] = col[i];
-    const double2 gj = g_r[j];
-    const double2 sg = cmulc(s, gj);
-    g_r[j] = make_double2(c * gj.x, c * gj.y);
-    g_r[j + 1] = make_double2(-sg.x, -sg.y);
-    resid[r] = sqrt(sg.x * sg.x + sg.y * sg.y);
-}
-
-__global__ void k_back_substitute(double2* y, const double2* H, const double2* g, int j, int m, int N) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    const double2* Hr = H + (long long)r * (m + 1) * m;
-    const double2* g_r = g + (long long)r * (m + 1);
-    double2 yv[64];
-    for (int i = j; i >= 0; --i) {
-        double2 acc = g_r[i];
-        for (int l = i + 1; l <= j; ++l) acc = csub(acc, cmul(Hr[(long long)i * m + l], yv[l]));
-        const double2 hd = Hr[(long long)i * m + i];
-        const double den = hd.x * hd.x + hd.y * hd.y;
-        yv[i] = (den > 0.0) ? make_double2((acc.x * hd.x + acc.y * hd.y) / den, (acc.y * hd.x - acc.x * hd.y) / den)
-                            : make_double2(0, 0);
-    }
-    for (int i = 0; i <= j; ++i) y[(long long)i * N + r] = yv[i];
-}
-
-__global__ void k_max_ratio(double* out, const double* resid, const double* bnorm, int N) {
-    __shared__ double sh[256];
-    double m = 0;
-    for (int r = threadIdx.x; r < N; r += blockDim.x) {
-        const double b = bnorm[r];
-        double v = (b > 0.0) ? resid[r] / b : 0.0;
-        if (v != v) v = __longlong_as_double(0x7ff8000000000000ll);   // keep NaN visible
-        if (!(v <= m)) m = v;
-    }
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st && !(sh[threadIdx.x + st] <= sh[threadIdx.x])) sh[threadIdx.x] = sh[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = sh[0];
-}
-
-void launch_init_g(double2* g, const double* beta, int m, int N, cudaStream_t s) {
-    k_init_g<<<(N + 127) / 128, 128, 0, s>>>(g, beta, m, N);
-    MG_LAUNCHED();
-}
-void launch_arnoldi_column(double2* H, double* cs, double2* sn, double2* g, double* resid, const double2* h,
-                           const double* hnorm, int j, int m, int N, cudaStream_t s) {
-    MG_REQUIRE(m <= 64, MGMLMC_EINVAL, "FGMRES restart length above 64");
-    k_arnoldi_column<<<(N + 63) / 64, 64, 0, s>>>(H, cs, sn, g, resid, h, hnorm, j, m, N);
-    MG_LAUNCHED();
-}
-void launch_back_substitute(double2* y, const double2* H, const double2* g, int j, int m, int N, cudaStream_t s) {
-    k_back_substitute<<<(N + 63) / 64, 64, 0, s>>>(y, H, g, j, m, N);
-    MG_LAUNCHED();
-}
-void launch_max_ratio(double* out, const double* resid, const double* bnorm, int N, cudaStream_t s) {
-    k_max_ratio<<<1, 256, 0, s>>>(out, resid, bnorm, N);
-    MG_LAUNCHED();
-}
-
 // ------------------------------------------------------------- sample assembly
 // s[j] -= sum_i a_i conj(B[i][j]) A[i][j]   (deflated part of the coarsest term)
 __global__ void k_deflation_correction(double2* s, const double2* A, const double2* B, const double* a, int k, int N) {

@@ -78,6 +78,7 @@ void Ctx::release_all() {
     live_bytes = 0;
     ws.clear();
     dev_err = nullptr;
+    dev_max = nullptr;
     for (auto& L : lev) L = Level();
     U64 = nullptr;
     U32 = nullptr;

@@ -429,80 +429,130 @@ static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool
     return fin >= 0 ? rs + fin * nN : nullptr;
 }
 
-__global__ void k_sqrt_inplace(double* v, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) v[i] = sqrt(v[i]);
-}
-__global__ void k_add2(double2* a, const double2* b, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = make_double2(a[i].x + b[i].x, a[i].y + b[i].y);
-}
-
-// Unnormalised basis vectors are kept while eta = |w| lies in [2^-32, 2^32]: their FP32
-// entries, dot products and squared sums then stay far inside the normal range.
-constexpr double kEtaLow = 0x1p-32, kEtaHigh = 0x1p32;
-__device__ __forceinline__ void keep_eta(double* eta, double* rsc, double en) {
-    const bool out = en > 0.0 && (en < kEtaLow || en > kEtaHigh);
-    *rsc = out ? 1.0 / en : 0.0;   // the vector is rescaled to unit norm where rsc != 0
-    *eta = out ? 1.0 : en;
-}
-
-// Arnoldi column j of FGMRES with an unnormalised basis w_i = eta_i v_i (per rhs r):
-// on entry h[i] = <w_i, u> summed over the Gram-Schmidt passes and hn2 = |u' / eta_j|^2
-// for the orthogonalised u' (u = D M(w_j)); on exit h[i] = H_ij = h[i] / (eta_i eta_j),
-// hn2 = H_{j+1,j} = |u'| / eta_j, and w_{j+1} = u' has eta_{j+1} = |u'| (or is marked in
-// rsc for rescaling, eta_{j+1} = 1).  A zero eta_j (a zero vector, as a zero rhs or an
-// exhausted Krylov space gives) leaves a zero column.
-__global__ void k_lazy_column(double2* __restrict__ h, double* __restrict__ hn2, double* __restrict__ eta,
-                              double* __restrict__ rsc, int j, int N) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    const double ej = eta[(long long)j * N + r];
-    const double hs = sqrt(hn2[r]);
-    for (int i = 0; i <= j; ++i) {
-        const double d = eta[(long long)i * N + r] * ej;
-        const double f = (d != 0.0) ? 1.0 / d : 0.0;
-        const double2 v = h[(long long)i * N + r];
-        h[(long long)i * N + r] = make_double2(v.x * f, v.y * f);
+// A maximum that the next reduction writes (NormOut::max and ::clear, or launch_rotate's) and
+// read_max returns.  Four in turn: at most two are taken between two reads.
+constexpr int kMaxSlots = 4;
+struct MaxSlot {
+    int i = 0;
+    unsigned long long *at = nullptr, *clear = nullptr;
+};
+static MaxSlot take_max(Ctx& c) {
+    if (!c.dev_max) {
+        c.dev_max = c.scratch<unsigned long long>("dev_max", kMaxSlots);
+        MG_CUDA(cudaMemsetAsync(c.dev_max, 0, kMaxSlots * sizeof(unsigned long long), c.stream));
+        c.max_turn = 0;
     }
-    hn2[r] = (ej != 0.0) ? hs : 0.0;
-    keep_eta(eta + (long long)(j + 1) * N + r, rsc + r, hs * ej);
+    MaxSlot m;
+    m.i = c.max_turn;
+    m.at = c.dev_max + m.i;
+    m.clear = c.dev_max + (m.i + 2) % kMaxSlots;
+    c.max_turn = (m.i + 1) % kMaxSlots;
+    return m;
 }
-
-// The same range check for the first basis vector of a cycle (eta_0 = |r|).
-__global__ void k_eta_range(double* __restrict__ eta, double* __restrict__ rsc, int N) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < N) keep_eta(eta + r, rsc + r, eta[r]);
-}
-
-// out = max_j a_j b_j / c_j (terms with c_j = 0 skipped; NaN kept visible).
-__global__ void k_max_scaled_ratio(double* out, const double* a, const double* b, const double* cden, int N) {
-    __shared__ double sh[256];
-    double m = 0.0;
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        double v = (cden[j] > 0.0) ? a[j] * b[j] / cden[j] : 0.0;
-        if (v != v) v = __longlong_as_double(0x7ff8000000000000ll);
-        if (!(v <= m)) m = v;
-    }
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st && !(sh[threadIdx.x + st] <= sh[threadIdx.x])) sh[threadIdx.x] = sh[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = sh[0];
-}
-
-static void sqrt_inplace(Ctx& c, double* v, int n) {
-    k_sqrt_inplace<<<(n + 127) / 128, 128, 0, c.stream>>>(v, n);
-    MG_LAUNCHED();
+// Value of one slot (and of another read with it); waits for the stream.
+static double read_max(Ctx& c, const MaxSlot& m, const MaxSlot* also = nullptr, double* also_v = nullptr) {
+    MG_CUDA(cudaMemcpyAsync(c.hbuf, c.dev_max, kMaxSlots * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+    c.sync();
+    if (also) *also_v = c.hbuf[also->i];
+    return c.hbuf[m.i];
 }
 
 template <typename C>
-static void norms(Ctx& c, double* out, const C* x, long long n, int N) {
-    double* part = c.scratch<double>("part_nrm", (size_t)reduce_groups(n, N) * N);
-    launch_norm2<C>(out, x, n, N, part, c.stream);
-    sqrt_inplace(c, out, N);
+static void norms(Ctx& c, const NormOut& o, const C* x, long long n, int N) {
+    launch_norm<C>(o, x, n, N, c.scratch_bytes("part_nrm", norm_part_bytes(n, N)), c.stream);
+}
+
+// One Arnoldi basis of the multi-RHS flexible GMRES with its per-rhs bookkeeping.
+//
+// The basis is kept unnormalised, w_i = eta_i v_i with eta_i = |w_i| per rhs: the
+// Gram-Schmidt coefficients are divided by eta_i^2, the Hessenberg column by eta_i eta_j, and
+// the correction takes y_j / eta_j of z_j = M(w_j).  This is FGMRES on the normalised basis
+// exactly (the preconditioner of each step is whatever maps v_j to z_j / eta_j: no property
+// of M is assumed) and saves the pass that would scale each new vector.  A vector whose eta
+// leaves [2^-32, 2^32] (an iteration run on past convergence shrinks it by the FP32
+// rounding level each step) is rescaled to unit norm, only for that rhs.
+template <typename C>
+struct Basis {
+    C *V, *Z, *cf;
+    double2 *H, *g, *sn, *irr;
+    double *hsub, *cs, *eta, *ieta, *rsc;
+    void *part, *npart;
+    long long n;
+    int N, m;
+    C* v(int j) const { return V + (size_t)j * n * N; }
+    C* z(int j) const { return Z + (size_t)j * n * N; }
+};
+
+template <typename C>
+static Basis<C> basis(Ctx& c, const char* name, int l, long long n, int m, int N) {
+    const size_t sz = sizeof(C), nN = (size_t)n * N;
+    const std::string p = name;
+    Basis<C> B;
+    B.n = n;
+    B.N = N;
+    B.m = m;
+    B.V = c.scratch<C>(nm((p + "_V").c_str(), l, sz), (size_t)(m + 1) * nN);
+    B.Z = c.scratch<C>(nm((p + "_Z").c_str(), l, sz), (size_t)m * nN);
+    B.cf = c.scratch<C>(nm((p + "_cf").c_str(), l, sz), (size_t)(m + 1) * N);
+    B.H = c.scratch<double2>(nm((p + "_H").c_str(), l, sz), (size_t)m * (m + 1) * N);
+    B.g = c.scratch<double2>(nm((p + "_g").c_str(), l, sz), (size_t)(m + 1) * N);
+    B.sn = c.scratch<double2>(nm((p + "_sn").c_str(), l, sz), (size_t)m * N);
+    B.irr = c.scratch<double2>(nm((p + "_irr").c_str(), l, sz), (size_t)m * N);
+    B.hsub = c.scratch<double>(nm((p + "_hs").c_str(), l, sz), (size_t)m * N);
+    B.cs = c.scratch<double>(nm((p + "_cs").c_str(), l, sz), (size_t)m * N);
+    B.eta = c.scratch<double>(nm((p + "_eta").c_str(), l, sz), (size_t)(m + 1) * N);
+    B.ieta = c.scratch<double>(nm((p + "_ieta").c_str(), l, sz), (size_t)(m + 1) * N);
+    B.rsc = c.scratch<double>(nm((p + "_rsc").c_str(), l, sz), N);
+    // own partials: a K-cycle runs inside an outer step
+    B.part = c.scratch_bytes(nm((p + "_part").c_str(), l, sz), dot_part_bytes(n, N, m));
+    B.npart = c.scratch_bytes(nm((p + "_npart").c_str(), l, sz), norm_part_bytes(n, N));
+    return B;
+}
+
+// The reduction of the first vector's norm: eta_0 and g_0 with it.
+template <typename C>
+static NormOut basis_start(const Basis<C>& B) {
+    NormOut o;
+    o.eta = B.eta;
+    o.ieta = B.ieta;
+    o.rsc = B.rsc;
+    o.g0 = B.g;
+    return o;
+}
+
+// Step j after u = D M(w_j) was formed in v(j + 1): classical Gram-Schmidt (passes times) and
+// the Hessenberg column j.
+template <typename C>
+static void arnoldi_step(Ctx& c, const Basis<C>& B, int j, int passes) {
+    const double nN = (double)B.n * B.N, sz = sizeof(C);
+    // algorithmic bytes: the j+1 basis vectors read once per Gram-Schmidt pass; the
+    // implementation reads them twice (dot products, then the update) and reads w twice and
+    // writes it once per pass: (2j + 5) vectors
+    ProfScope ps(c, std::string("orth.") + prec_tag(sizeof(C)), passes * (j + 1) * nN * sz,
+                 passes * 2.0 * 8.0 * (j + 1) * nN, passes * (2 * j + 5) * nN * sz);
+    C* u = B.v(j + 1);
+    double2* H = B.H + (size_t)j * (B.m + 1) * B.N;
+    NormOut o;
+    o.eta = B.eta + (size_t)(j + 1) * B.N;
+    o.ieta = B.ieta + (size_t)(j + 1) * B.N;
+    o.rsc = B.rsc;
+    o.hsub = B.hsub + (size_t)j * B.N;
+    o.eta_prev = B.eta + (size_t)j * B.N;
+    for (int p = 0; p < passes; ++p) {
+        launch_multidot<C>(B.cf, H, B.V, j + 1, u, B.n, B.N, B.ieta, p > 0, B.part, c.stream);
+        // the norm is summed over u / eta_j (FP32 squares of a small vector would leave the
+        // normal range)
+        launch_multiaxpy<C>(u, B.cf, j + 1, B.V, B.n, B.N, true, p + 1 == passes ? &o : nullptr, B.npart,
+                            B.ieta + (size_t)j * B.N, c.stream);
+    }
+    if (j + 1 < B.m) launch_scale_cols_if<C>(u, B.rsc, B.n, B.N, c.stream);
+}
+
+// x (=|+=) Z y after column j.
+template <typename C>
+static void basis_update(Ctx& c, const Basis<C>& B, int j, C* x, bool accumulate) {
+    launch_back_substitute<C>(B.cf, B.H, B.g, B.irr, B.ieta, j, B.m, B.N, c.stream);
+    launch_multiaxpy<C>(x, B.cf, j + 1, B.Z, B.n, B.N, accumulate, nullptr, nullptr, nullptr, c.stream);
 }
 
 // K-cycle coarse-grid correction: e ~ D_l^{-1} r by k steps of flexible GMRES from
@@ -511,45 +561,17 @@ static void norms(Ctx& c, double* out, const C* x, long long n, int N) {
 // bookkeeping (Givens rotations, least-squares solve) runs per rhs on the device.
 template <typename C>
 static void kcycle(Ctx& c, int l, C* e, const C* r, int N, int k) {
-    const Level& L = c.lev[l];
-    const long long n = L.n;
-    const size_t nN = (size_t)n * N;
-    const size_t sz = sizeof(C);
-    C* V = c.scratch<C>(nm("kc_V", l, sz), (size_t)(k + 1) * nN);
-    C* Z = c.scratch<C>(nm("kc_Z", l, sz), (size_t)k * nN);
-    double* beta = c.scratch<double>(nm("kc_beta", l, sz), N);
-    double* hnorm = c.scratch<double>(nm("kc_hn", l, sz), N);
-    double* resid = c.scratch<double>(nm("kc_res", l, sz), N);
-    double2* h = c.scratch<double2>(nm("kc_h", l, sz), (size_t)(k + 1) * N);
-    double2* y = c.scratch<double2>(nm("kc_y", l, sz), (size_t)(k + 1) * N);
-    double2* H = c.scratch<double2>(nm("kc_H", l, sz), (size_t)N * (k + 1) * k);
-    double* cs = c.scratch<double>(nm("kc_cs", l, sz), (size_t)N * k);
-    double2* sn = c.scratch<double2>(nm("kc_sn", l, sz), (size_t)N * k);
-    double2* g = c.scratch<double2>(nm("kc_g", l, sz), (size_t)N * (k + 1));
-    // own partials: the caller's FGMRES holds the pointer of its "part_md" across this call
-    double2* part = c.scratch<double2>(nm("kc_part", l, sz), (size_t)reduce_groups(n, N) * (k + 1) * N);
-    double* npart = c.scratch<double>(nm("kc_npart", l, sz), (size_t)axpy_groups(n, N) * N);
-    norms<C>(c, beta, r, n, N);
-    launch_scale_rhs<C, C>(V, r, beta, true, n, N, c.stream);
-    launch_init_g(g, beta, k, N, c.stream);
+    const long long n = c.lev[l].n;
+    const Basis<C> B = basis<C>(c, "kc", l, n, k, N);
+    launch_scale_norm<C, C>(basis_start(B), B.V, r, nullptr, false, n, N, B.npart, c.stream);
+    launch_scale_cols_if<C>(B.V, B.rsc, n, N, c.stream);
     for (int j = 0; j < k; ++j) {
-        C* Vj = V + (size_t)j * nN;
-        C* Vn = V + (size_t)(j + 1) * nN;
-        C* Zj = Z + (size_t)j * nN;
-        mg_cycle<C>(c, l, Zj, Vj, N);
-        apply_D<C>(c, l, Vn, Zj, nullptr, N, 0, nullptr);
-        {
-            ProfScope ps(c, "orth." + std::string(prec_tag(sz)), (j + 1) * (double)nN * sz,
-                         2.0 * 8.0 * (j + 1) * (double)nN, (2 * j + 5) * (double)nN * sz);
-            launch_multidot<C>(h, V, j + 1, Vn, n, N, part, c.stream);
-            launch_multiaxpy_norm2<C>(Vn, h, j + 1, V, -1.0, n, N, hnorm, npart, c.stream);
-        }
-        sqrt_inplace(c, hnorm, N);
-        if (j + 1 < k) launch_scale_rhs<C, C>(Vn, Vn, hnorm, true, n, N, c.stream);
-        launch_arnoldi_column(H, cs, sn, g, resid, h, hnorm, j, k, N, c.stream);
+        mg_cycle<C>(c, l, B.z(j), B.v(j), N);
+        apply_D<C>(c, l, B.v(j + 1), B.z(j), nullptr, N, 0, nullptr);
+        arnoldi_step<C>(c, B, j, 1);
     }
-    launch_back_substitute(y, H, g, k - 1, k, N, c.stream);
-    launch_multiaxpy<C>(e, y, k, Z, 1.0, n, N, c.stream, nullptr, 0, false);   // e = Z y
+    launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, nullptr, nullptr, nullptr, 0, k - 1, k, N, c.stream);
+    basis_update<C>(c, B, k - 1, e, false);
 }
 
 template <typename C>
@@ -590,148 +612,92 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
     mr_smooth<C>(c, l, e, res, N, c.opt.nu_post, false, false);
 }
 
-static double read_scalar(Ctx& c, const double* dev) {
-    MG_CUDA(cudaMemcpyAsync(c.hbuf, dev, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    c.sync();
-    return c.hbuf[0];
+// One Arnoldi cycle from the started basis B (first vector, eta_0, g_0): at most B.m steps,
+// ended once the residual estimate (relative to bnorm) reaches tol or it reaches maxit; then
+// x (=|+=) the correction.
+template <typename C>
+static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate, const double* bnorm, double tol,
+                         long long& it, long long maxit, bool inner) {
+    const int N = B.N, m = B.m;
+    // Inner cycles of the refinement loop converge in a repeatable number of steps per level
+    // and tolerance: the host reads the residual estimate (a round trip that leaves the GPU
+    // idle) only from two steps before the last such count on.
+    int* hint = nullptr;
+    if (inner) {
+        const int dec = std::min(15, std::max(0, (int)std::floor(-std::log10(tol))));
+        hint = &c.cycle_hint[((long long)l * 16 + dec) * (1LL << 32) + N];
+    }
+    const int check_from = hint ? std::max(1, *hint - 2) : 1;
+    // classical Gram-Schmidt: twice in FP64; once in the FP32 inner solve of the refinement
+    // loop, whose FP64 residual absorbs the loss of orthogonality
+    const int passes = sizeof(C) == sizeof(double2) ? 2 : 1;
+    int j = 0, rotated = 0;
+    for (;; ++j) {
+        mg_cycle<C>(c, l, B.z(j), B.v(j), N);
+        apply_D<C>(c, l, B.v(j + 1), B.z(j), nullptr, N, 0, nullptr);
+        arnoldi_step<C>(c, B, j, passes);
+        ++it;
+        if (j + 1 < check_from && j + 1 < m && it < maxit) continue;
+        const MaxSlot ms = take_max(c);
+        launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, ms.at, ms.clear, rotated, j, m, N, c.stream);
+        rotated = j + 1;
+        const double est = read_max(c, ms);
+        if (est != est) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
+        if (est <= tol || it >= maxit || j + 1 >= m) break;
+    }
+    if (hint) *hint = j + 1;
+    basis_update<C>(c, B, j, x, accumulate);
 }
 
 template <typename C>
 long long fgmres(Ctx& c, int l, const C* b, C* x, int N, double tol, long long maxit, bool x_zero, int* ok,
                  int max_cycles) {
-    const Level& L = c.lev[l];
-    const long long n = L.n;
-    const int m = c.opt.fgmres_restart;
-    const size_t nN = (size_t)n * N;
-    const size_t sz = sizeof(C);
-    C* V = c.scratch<C>(nm("fg_V", 0, sz), (size_t)(m + 1) * nN);
-    C* Z = c.scratch<C>(nm("fg_Z", 0, sz), (size_t)m * nN);
-    double* bnorm = c.scratch<double>(nm("fg_bn", 0, sz), N);
-    double* beta = c.scratch<double>(nm("fg_beta", 0, sz), N);
-    double* hnorm = c.scratch<double>(nm("fg_hn", 0, sz), N);
-    double* resid = c.scratch<double>(nm("fg_res", 0, sz), N);
-    double* maxr = c.scratch<double>(nm("fg_maxr", 0, sz), 1);
-    double2* h = c.scratch<double2>(nm("fg_h", 0, sz), (size_t)(m + 1) * N);
-    double2* h2 = c.scratch<double2>(nm("fg_h2", 0, sz), (size_t)(m + 1) * N);
-    double2* y = c.scratch<double2>(nm("fg_y", 0, sz), (size_t)(m + 1) * N);
-    double2* H = c.scratch<double2>(nm("fg_H", 0, sz), (size_t)N * (m + 1) * m);
-    double* cs = c.scratch<double>(nm("fg_cs", 0, sz), (size_t)N * m);
-    double2* sn = c.scratch<double2>(nm("fg_sn", 0, sz), (size_t)N * m);
-    double2* g = c.scratch<double2>(nm("fg_g", 0, sz), (size_t)N * (m + 1));
-    double2* part = c.scratch<double2>("part_md", (size_t)reduce_groups(n, N) * (m + 1) * N);
-
-    // The Arnoldi basis is kept unnormalised, w_i = eta_i v_i with eta_i = |w_i| per rhs
-    // (eta: (m + 1) x N): the Gram-Schmidt coefficients are divided by eta_i^2, the
-    // Hessenberg column by eta_i eta_j, and the correction takes y_j / eta_j of z_j =
-    // M(w_j).  This is FGMRES on the normalised basis exactly (the preconditioner of
-    // each step is whatever maps v_j to z_j / eta_j: no property of M is assumed) and
-    // saves the pass that would scale each new vector.  A vector whose eta leaves
-    // [2^-32, 2^32] (an iteration run on past convergence shrinks it by the FP32
-    // rounding level each step) is rescaled to unit norm, only for that rhs.
-    double* eta = c.scratch<double>(nm("fg_eta", 0, sz), (size_t)(m + 1) * N);
-    double* rsc = c.scratch<double>(nm("fg_rsc", 0, sz), N);
-    MG_REQUIRE(b != V || (x_zero && max_cycles == 1), MGMLMC_EINVAL,
-               "fgmres: a right-hand side in the basis needs x = 0 and one cycle");
-    norms<C>(c, bnorm, b, n, N);
+    const long long n = c.lev[l].n;
+    const Basis<C> B = basis<C>(c, "fg", 0, n, c.opt.fgmres_restart, N);
+    double* bnorm = c.scratch<double>(nm("fg_bn", 0, sizeof(C)), N);
     // x = 0 is not written: the first correction overwrites x (or x is zeroed on exit)
     bool x_unset = x_zero;
     long long it = 0;
     int cycles = 0;
     *ok = 0;
+    if (!x_unset) {
+        NormOut o;
+        o.norm = bnorm;
+        norms<C>(c, o, b, n, N);
+    }
     for (;;) {
+        const MaxSlot ms = take_max(c);
+        NormOut o = basis_start(B);
+        o.max = ms.at;
+        o.clear = ms.clear;
         if (x_unset) {
-            if (b != V) MG_CUDA(cudaMemcpyAsync(V, b, sz * nN, cudaMemcpyDeviceToDevice, c.stream));
-            MG_CUDA(cudaMemcpyAsync(eta, bnorm, sizeof(double) * N, cudaMemcpyDeviceToDevice, c.stream));
+            o.norm = bnorm;
+            launch_scale_norm<C, C>(o, B.V, b, nullptr, false, n, N, B.npart, c.stream);
         } else {
-            apply_D<C>(c, l, V, x, b, N, 1, nullptr);
-            norms<C>(c, eta, V, n, N);
+            o.den = bnorm;
+            apply_D<C>(c, l, B.V, x, b, N, 1, nullptr);
+            launch_norm<C>(o, B.V, n, N, B.npart, c.stream);
         }
-        launch_max_ratio(maxr, eta, bnorm, N, c.stream);
-        const double ratio = read_scalar(c, maxr);
+        const double ratio = read_max(c, ms);
         if (ratio != ratio) throw Error(MGMLMC_ENAN, "FGMRES: NaN residual");
         if (c.opt.verbose)
-            fprintf(stderr, "[mgmlmc] fgmres level %d prec %zu it %lld true rel res %.3e\n", l + 1, sz * 4, it,
+            fprintf(stderr, "[mgmlmc] fgmres level %d prec %zu it %lld true rel res %.3e\n", l + 1, sizeof(C) * 4, it,
                     ratio);
         if (ratio <= tol) {
             *ok = 1;
             break;
         }
         if (it >= maxit) break;
-        launch_init_g(g, eta, m, N, c.stream);
-        k_eta_range<<<(N + 127) / 128, 128, 0, c.stream>>>(eta, rsc, N);
-        MG_LAUNCHED();
-        launch_scale_cols_if<C>(V, rsc, n, N, c.stream);
-        int j_end = -1;
-        // Inner cycles of the refinement loop converge in a repeatable number of steps
-        // per level and tolerance: the host reads the residual estimate (a round trip
-        // that leaves the GPU idle) only from two steps before the last such count on.
-        int* hint = nullptr;
-        if (max_cycles == 1) {
-            const int dec = std::min(15, std::max(0, (int)std::floor(-std::log10(tol))));
-            hint = &c.cycle_hint[((long long)l * 16 + dec) * (1LL << 32) + N];
-        }
-        const int check_from = hint ? std::max(1, *hint - 2) : 1;
-        for (int j = 0; j < m; ++j) {
-            C* Vj = V + (size_t)j * nN;
-            C* Vn = V + (size_t)(j + 1) * nN;
-            C* Zj = Z + (size_t)j * nN;
-            mg_cycle<C>(c, l, Zj, Vj, N);
-            apply_D<C>(c, l, Vn, Zj, nullptr, N, 0, nullptr);
-            // classical Gram-Schmidt: twice in FP64; once in the FP32 inner solve of the
-            // refinement loop, whose FP64 residual absorbs the loss of orthogonality
-            {
-                // algorithmic bytes: the j+1 basis vectors read once per Gram-Schmidt pass;
-                // the implementation reads them twice (dot products, then the update) and
-                // reads w twice and writes it once per pass: (2j + 5) vectors
-                const int passes = (sz == sizeof(double2)) ? 2 : 1;
-                ProfScope ps(c, "orth." + std::string(prec_tag(sz)), passes * (j + 1) * (double)nN * sz,
-                             passes * 2.0 * 8.0 * (j + 1) * (double)nN, passes * (2 * j + 5) * (double)nN * sz);
-                // the last axpy also returns |Vn|^2 (its partials), saving a pass over Vn
-                double* npart = c.scratch<double>("part_nrm_ax", (size_t)axpy_groups(n, N) * N);
-                launch_multidot<C>(h, V, j + 1, Vn, n, N, part, c.stream);
-                if (passes == 2) {
-                    launch_multiaxpy<C>(Vn, h, j + 1, V, -1.0, n, N, c.stream, eta, 2);
-                    launch_multidot<C>(h2, V, j + 1, Vn, n, N, part, c.stream);
-                    launch_multiaxpy_norm2<C>(Vn, h2, j + 1, V, -1.0, n, N, hnorm, npart, c.stream, eta, 2,
-                                              eta + (size_t)j * N);
-                    k_add2<<<((j + 1) * N + 127) / 128, 128, 0, c.stream>>>(h, h2, (j + 1) * N);
-                    MG_LAUNCHED();
-                } else {
-                    launch_multiaxpy_norm2<C>(Vn, h, j + 1, V, -1.0, n, N, hnorm, npart, c.stream, eta, 2,
-                                              eta + (size_t)j * N);
-                }
-            }
-            k_lazy_column<<<(N + 127) / 128, 128, 0, c.stream>>>(h, hnorm, eta, rsc, j, N);
-            MG_LAUNCHED();
-            launch_scale_cols_if<C>(Vn, rsc, n, N, c.stream);
-            launch_arnoldi_column(H, cs, sn, g, resid, h, hnorm, j, m, N, c.stream);
-            ++it;
-            j_end = j;
-            if (j + 1 < check_from && j + 1 < m && it < maxit) continue;
-            launch_max_ratio(maxr, resid, bnorm, N, c.stream);
-            const double est = read_scalar(c, maxr);
-            if (est != est) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
-            if (est <= tol || it >= maxit) break;
-        }
-        if (hint) *hint = j_end + 1;
-        launch_back_substitute(y, H, g, j_end, m, N, c.stream);
-        launch_multiaxpy<C>(x, y, j_end + 1, Z, 1.0, n, N, c.stream, eta, 1, !x_unset);
+        launch_scale_cols_if<C>(B.V, B.rsc, n, N, c.stream);
+        fgmres_cycle<C>(c, l, B, x, !x_unset, bnorm, tol, it, maxit, max_cycles == 1);
         x_unset = false;
         if (++cycles >= max_cycles) {
-            // the caller checks the residual itself (inner solve of the refinement loop)
             *ok = 1;
             break;
         }
     }
-    if (x_unset) launch_zero<C>(x, (long long)nN, c.stream);
+    if (x_unset) launch_zero<C>(x, n * N, c.stream);
     return it;
-}
-
-// The Krylov basis block of fgmres<C> for N right-hand sides on level l: a caller that
-// builds its rhs there (x = 0, one cycle) saves the copy into the basis.
-template <typename C>
-static C* fgmres_basis(Ctx& c, int l, int N) {
-    return c.scratch<C>(nm("fg_V", 0, sizeof(C)), (size_t)(c.opt.fgmres_restart + 1) * c.lev[l].n * N);
 }
 
 static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N, double tol, int* ok);
@@ -771,16 +737,16 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
         return it;
     }
     // Mixed: FP64 iterative refinement, FP32 FGMRES + FP32 multigrid inside.
-    const Level& L = c.lev[l];
-    const long long n = L.n;
+    const long long n = c.lev[l].n;
     const size_t nN = (size_t)n * N;
     double2* r = c.scratch<double2>("ir_r", nN);
     // the FP32 rhs of each inner cycle is built in the inner FGMRES's first basis vector
-    float2* r32 = fgmres_basis<float2>(c, l, N);
+    const Basis<float2> B = basis<float2>(c, "fg", 0, n, c.opt.fgmres_restart, N);
     float2* e32 = c.scratch<float2>("ir_e32", nN);
     double* bnorm = c.scratch<double>("ir_bn", N);
     double* rnorm = c.scratch<double>("ir_rn", N);
-    double* maxr = c.scratch<double>("ir_maxr", 1);
+    double* inorm = c.scratch<double>("ir_in", N);
+    void* npart = c.scratch_bytes("part_nrm", norm_part_bytes(n, N));
     // inner tolerance: the reduction still needed this cycle (with margin), but no
     // tighter than FP32 arithmetic can deliver
     const double inner_floor = 2e-7;
@@ -806,18 +772,39 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
     constexpr double kRecursiveResidual = 500.0;
     const bool fp32_updates = c.fp32_residual_updates;
     const double dnorm = std::fabs(c.m0 + 2.0) + 4.0;
-    double* enorm = c.scratch<double>("ir_en", N);
     double drift = 0.0;
-    norms<double2>(c, bnorm, b, n, N);
-    launch_zero<double2>(x, (long long)nN, c.stream);
-    MG_CUDA(cudaMemcpyAsync(r, b, sizeof(double2) * nN, cudaMemcpyDeviceToDevice, c.stream));
+    // r = b, its norm; a reduction that gives |r| also gives max |r| / |b|
+    const double* rn = bnorm;
+    auto residual_norm = [&](const MaxSlot& ms) {
+        NormOut o;
+        o.norm = rnorm;
+        o.den = bnorm;
+        o.max = ms.at;
+        o.clear = ms.clear;
+        rn = rnorm;
+        return o;
+    };
+    double ratio;
+    {
+        const MaxSlot ms = take_max(c);
+        NormOut o;
+        o.norm = bnorm;
+        o.max = ms.at;
+        o.clear = ms.clear;
+        launch_scale_norm<double2, double2>(o, r, b, nullptr, false, n, N, npart, c.stream);
+        ratio = read_max(c, ms);
+    }
+    auto fp64_residual = [&] {
+        apply_D<double2>(c, l, r, x, b, N, 1, nullptr);
+        const MaxSlot ms = take_max(c);
+        launch_norm<double2>(residual_norm(ms), r, n, N, npart, c.stream);
+        ratio = read_max(c, ms);
+    };
     long long it = 0;
+    bool x_unset = true;                         // x = 0 is written by the first correction
     *ok = 0;
     // cycles until the FP64 residual meets tol or the iteration budget is spent
     for (int cycle = 0;; ++cycle) {
-        norms<double2>(c, rnorm, r, n, N);
-        launch_max_ratio(maxr, rnorm, bnorm, N, c.stream);
-        const double ratio = read_scalar(c, maxr);
         if (ratio != ratio) throw Error(MGMLMC_ENAN, "refinement: NaN residual");
         if (drift > 0.0 && (drift > 1e-2 * ratio || (ratio <= tol && drift > tol / 20))) {
             double2* rrec = nullptr;
@@ -825,14 +812,18 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
                 rrec = c.scratch<double2>("ir_rrec", nN);
                 MG_CUDA(cudaMemcpyAsync(rrec, r, sizeof(double2) * nN, cudaMemcpyDeviceToDevice, c.stream));
             }
-            apply_D<double2>(c, l, r, x, b, N, 1, nullptr);
+            fp64_residual();
             if (rrec) {
                 // the error the FP32 updates actually made, against the bound
                 launch_axpy_rhs<double2, double2>(rrec, nullptr, nullptr, -1.0, r, n, N, c.stream);
-                norms<double2>(c, rnorm, rrec, n, N);
-                launch_max_ratio(maxr, rnorm, bnorm, N, c.stream);
+                const MaxSlot ms = take_max(c);
+                NormOut o;
+                o.den = bnorm;
+                o.max = ms.at;
+                o.clear = ms.clear;
+                launch_norm<double2>(o, rrec, n, N, npart, c.stream);
                 fprintf(stderr, "[mgmlmc] refine level %d FP64 residual: FP32 drift %.3e (bound %.3e)\n", l + 1,
-                        read_scalar(c, maxr), drift);
+                        read_max(c, ms), drift);
             }
             drift = 0.0;
             continue;
@@ -844,27 +835,40 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
             break;
         }
         if (it >= maxit) break;
-        launch_scale_rhs<float2, double2>(r32, r, rnorm, true, n, N, c.stream);
-        const double inner_tol = std::max(inner_floor, 0.3 * tol / ratio);
-        int iok = 0;
-        // one FGMRES cycle in FP32: its own FP32 residual cannot certify more than
+        // one FGMRES cycle in FP32 on r / |r|: its own FP32 residual cannot certify more than
         // ~1e-6 relative, so the FP64 residual of this loop decides on restarts
-        it += fgmres<float2>(c, l, r32, e32, N, inner_tol, maxit - it, true, &iok, 1);
-        launch_axpy_rhs<double2, float2>(x, nullptr, rnorm, 1.0, e32, n, N, c.stream);
+        const double inner_tol = std::max(inner_floor, 0.3 * tol / ratio);
+        NormOut start = basis_start(B);
+        start.norm = inorm;
+        launch_scale_norm<float2, double2>(start, B.V, r, rn, true, n, N, npart, c.stream);
+        fgmres_cycle<float2>(c, l, B, e32, false, inorm, inner_tol, it, maxit, true);
         if (!fp32_updates && ratio > kRecursiveResidual * tol) {
-            apply_D<double2>(c, l, r, x, b, N, 1, nullptr);
+            launch_refine_axpy(x, rn, 1.0, e32, n, N, !x_unset, nullptr, nullptr, npart, c.stream);
+            x_unset = false;
+            fp64_residual();
             continue;
         }
+        // x += |r| e and, for the bound of this update, max_j |e_j| |r_j| / |b_j|; then
+        // r -= |r| D e (without fp32_updates the last cycle: accepted on this residual)
+        const MaxSlot md = take_max(c);
+        NormOut oe;
+        oe.max = md.at;
+        oe.clear = md.clear;
+        oe.den = bnorm;
+        oe.mul = rn;
+        launch_refine_axpy(x, rn, 1.0, e32, n, N, !x_unset, &oe, nullptr, npart, c.stream);
+        x_unset = false;
         float2* de = c.scratch<float2>("ir_de32", nN);
         apply_D<float2>(c, l, de, e32, nullptr, N, 0, nullptr);
-        launch_axpy_rhs<double2, float2>(r, nullptr, rnorm, -1.0, de, n, N, c.stream);
-        if (!fp32_updates) continue;   // the last cycle: accepted on this residual
-        // the bound of this update: max_j |e_j| |r_j| / |b_j|
-        norms<float2>(c, enorm, e32, n, N);
-        k_max_scaled_ratio<<<1, 256, 0, c.stream>>>(maxr, enorm, rnorm, bnorm, N);
-        MG_LAUNCHED();
-        drift += kFp32Product * dnorm * read_scalar(c, maxr);
+        const MaxSlot ms = take_max(c);
+        const double* scale = rn;
+        const NormOut orr = residual_norm(ms);
+        launch_refine_axpy(r, scale, -1.0, de, n, N, true, nullptr, &orr, npart, c.stream);
+        double er = 0.0;
+        ratio = read_max(c, ms, &md, &er);
+        if (fp32_updates) drift += kFp32Product * dnorm * er;
     }
+    if (x_unset) launch_zero<double2>(x, (long long)nN, c.stream);
     c.last_iters = it;
     check_device_error(c);
     return it;
@@ -894,7 +898,11 @@ INST(float2)
 }  // namespace mg
 
 namespace mg {
-void column_norms(Ctx& c, double* out, const double2* x, long long n, int N) { norms<double2>(c, out, x, n, N); }
+void column_norms(Ctx& c, double* out, const double2* x, long long n, int N) {
+    NormOut o;
+    o.norm = out;
+    norms<double2>(c, o, x, n, N);
+}
 
 void approx_inverse(Ctx& c, int l, const double2* b, double2* x, int N) {
     int ok = 0;
