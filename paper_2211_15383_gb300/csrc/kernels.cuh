@@ -283,10 +283,9 @@ void launch_build_prolongator(double2* P, const double2* tv, int lx, int lt, int
 void launch_deflation_correction(double2* s, const double2* A, const double2* B, const double* a, int k,
                                  int N, cudaStream_t s_);
 void launch_sample_stats(double* acc, const double2* samples, int N, cudaStream_t s);
-// Block-Jacobi smoother data: Minv[s] = A[s][0]^{-1} (work: nsites d^2 scratch) and the
+// Block-Jacobi smoother data: Minv[s] = A[s][0]^{-1} and the
 // block stencil Ahat of D M^{-1} (Ahat[s][dir] = A[s][dir] Minv[nbr(s,dir)]).
-void launch_block_diag_inverse(double2* Minv, double2* work, const double2* A, int nsites, int d, int* status,
-                               cudaStream_t s);
+void launch_block_diag_inverse(double2* Minv, const double2* A, int nsites, int d, int* status, cudaStream_t s);
 void launch_precondition_blocks(double2* Ahat, const double2* A, const double2* Minv, int lx, int lt, int d,
                                 cudaStream_t s);
 // y[s] (+)= Minv[s] sum_{q < K} alpha_q x_q[s] over K slots of x.

@@ -332,23 +332,248 @@ __global__ void __launch_bounds__(32 * kGJRowsPerCTA) k_gj_eliminate(C* A, int n
     }
 }
 
-// The panel's row swaps on the other columns (in the order they were taken), then a
-// copy of the pivot rows R[s][c] = A[k0 + s][c]: one thread per column.
+// All steps of a panel in one launch: a cluster of 8 CTAs holds the panel's n x kb entries in
+// its shared memory (at most 6144 rows: 768 rows x 256 B a CTA).  Per column every CTA sends
+// its pivot candidate with that candidate's panel row, and the owner row k, to all CTAs
+// through distributed shared memory; after one cluster barrier each CTA knows the pivot
+// (largest max(|Re|, |Im|), ties to the smallest row), scales its own copy of the pivot row
+// and eliminates its rows, which also gives the candidates of the next column.  What a
+// column costs is that chain (exchange, barrier, scale, eliminate: about 2 us), where the two
+// launches per column of k_gj_pivot and k_gj_eliminate cost 17 us at n = 1024 and 23 us at
+// n = 4096; larger matrices keep those.
+constexpr int kGJCluster = 8, kGJPanelThreads = 512, kGJPanelRows = 768;
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Address of this CTA's shared variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_map(const void* p, unsigned rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, float2 v) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, double2 v) {
+    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+template <typename C> __device__ __forceinline__ re_t<C> gj_size(C v) { return fmax(fabs(v.x), fabs(v.y)); }
+
+// 1 / p.  FP32: scaled by the larger part, then one Newton step, which leaves the rounding of
+// the last operation.
+__device__ __forceinline__ float2 gj_reciprocal(float2 p) {
+    const float m = 1.f / fmaxf(fabsf(p.x), fabsf(p.y));
+    const float x = p.x * m, y = p.y * m;
+    const float q = m / fmaf(x, x, y * y);
+    float2 r = mk(x * q, -y * q);
+    const float ex = fmaf(-p.x, r.x, fmaf(p.y, r.y, 1.f)), ey = fmaf(-p.x, r.y, -p.y * r.x);
+    return mk(fmaf(r.x, ex, fmaf(-r.y, ey, r.x)), fmaf(r.x, ey, fmaf(r.y, ex, r.y)));
+}
+__device__ __forceinline__ double2 gj_reciprocal(double2 p) {
+    const double den = p.x * p.x + p.y * p.y;
+    return mk(p.x / den, -p.y / den);
+}
+
 template <typename C>
-__global__ void __launch_bounds__(256) k_gj_swap_rows(C* A, int n, int k0, int kb, GJWork w) {
+__global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 1, 1)
+    k_gj_panel(C* A, int n, int k0, int kb, int R, GJWork w) {
+    using T = re_t<C>;
+    constexpr int B = GJPanel<C>::B;             // columns of a panel row: 256 bytes
+    constexpr int U = 16 / (int)sizeof(C);       // columns per 16 bytes
+    struct alignas(16) Unit { C v[U]; };
+    extern __shared__ __align__(16) unsigned char smem_gj[];
+    C* P = reinterpret_cast<C*>(smem_gj);        // this CTA's rows
+    __shared__ __align__(16) C xrow[2][kGJCluster][B], krow[2][B];
+    __shared__ T xval[2][kGJCluster];
+    __shared__ int xidx[2][kGJCluster];
+    __shared__ __align__(16) C srow[B];
+    __shared__ T rv[kGJPanelThreads / 32];
+    __shared__ int ri[kGJPanelThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int rank = (int)cluster_rank();
+    const int row0 = rank * R, rows = max(0, min(R, n - row0));
+    for (int e = tid; e < rows * B; e += kGJPanelThreads) {
+        const int r = e / B, c = e % B;
+        P[e] = c < kb ? A[(long long)(row0 + r) * n + k0 + c] : czero<C>();
+    }
+    __syncthreads();
+    // the CTA's candidate (value, local row) from per-thread ones: lane 0 of every warp, then warp 0
+    auto reduce = [&](T bv, int bi) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+        }
+        if (lane == 0) { rv[wid] = bv; ri[wid] = bi; }
+        __syncthreads();
+        bv = rv[lane % (kGJPanelThreads / 32)];
+        bi = ri[lane % (kGJPanelThreads / 32)];
+#pragma unroll
+        for (int o = kGJPanelThreads / 64; o > 0; o >>= 1) {
+            const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+        }
+        return bi;
+    };
+    T cv = (T)-1;
+    int ci = 0x7fffffff;
+    for (int r = tid; r < rows; r += kGJPanelThreads)
+        if (row0 + r >= k0) {
+            const T m = gj_size(P[r * B]);
+            if (m > cv) { cv = m; ci = r; }
+        }
+    for (int c = 0; c < kb; ++c) {
+        const int k = k0 + c, par = c & 1;
+        const int bi = reduce(cv, ci);           // local row, or none
+        const bool mine = bi < rows;
+        // warp q (< 8) sends to CTA q
+        if (wid < kGJCluster) {
+            if (lane < B) {
+                if (mine) cluster_store(cluster_map(&xrow[par][rank][lane], wid), P[bi * B + lane]);
+                if (k >= row0 && k < row0 + rows) cluster_store(cluster_map(&krow[par][lane], wid), P[(k - row0) * B + lane]);
+            }
+            if (lane == 0) {
+                cluster_store(cluster_map(&xval[par][rank], wid), mine ? gj_size(P[bi * B + c]) : (T)-1);
+                cluster_store(cluster_map(&xidx[par][rank], wid), mine ? row0 + bi : 0x7fffffff);
+            }
+        }
+        cluster_barrier();
+        int best = 0;
+#pragma unroll
+        for (int q = 1; q < kGJCluster; ++q)
+            if (xval[par][q] > xval[par][best] || (xval[par][q] == xval[par][best] && xidx[par][q] < xidx[par][best]))
+                best = q;
+        const bool ok = xval[par][best] > (T)0;
+        const int p = xidx[par][best] < n ? xidx[par][best] : k;
+        if (wid == 0) {
+            const C raw = lane < B ? xrow[par][best][lane] : czero<C>();
+            C piv = mk(__shfl_sync(0xffffffffu, raw.x, c), __shfl_sync(0xffffffffu, raw.y, c));
+            if (!ok) piv = mk((T)1, (T)0);
+            const C inv = gj_reciprocal(piv);
+            const C sv = lane == c ? inv : cmul(raw, inv);
+            if (lane < B) {
+                srow[lane] = sv;
+                if (k >= row0 && k < row0 + rows) P[(k - row0) * B + lane] = sv;
+            }
+            if (rank == 0 && lane == 0) {
+                w.perm[k] = p;
+                if (!ok) *w.status = 1;
+            }
+        } else if (wid == 1 && lane < B && p != k && p >= row0 && p < row0 + rows) {
+            P[(p - row0) * B + lane] = krow[par][lane];
+        }
+        __syncthreads();
+        // eliminate column k from the other rows: 8 threads per row
+        const int sub = tid & 7;
+        cv = (T)-1;
+        ci = 0x7fffffff;
+        // thread `sub` of a row's eight holds the 16-byte units sub and sub + 8
+        Unit s[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) s[q] = *reinterpret_cast<const Unit*>(srow + (sub + 8 * q) * U);
+        for (int r0 = 0; r0 < rows; r0 += kGJPanelThreads / 8) {
+            const int r = r0 + (tid >> 3);
+            const bool in = r < rows && row0 + r != k;
+            C f = czero<C>();
+            if (in) f = P[r * B + c];
+            __syncwarp();
+            if (in) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    Unit* pu = reinterpret_cast<Unit*>(P + r * B + (sub + 8 * q) * U);
+                    Unit o = *pu;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int cc = (sub + 8 * q) * U + u;
+                        o.v[u] = csub(cc == c ? czero<C>() : o.v[u], cmul(f, s[q].v[u]));
+                        if (cc == c + 1 && row0 + r > k) {
+                            const T m = gj_size(o.v[u]);
+                            if (m > cv) { cv = m; ci = r; }
+                        }
+                    }
+                    *pu = o;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < rows * B; e += kGJPanelThreads) {
+        const int r = e / B, c = e % B;
+        if (c < kb) A[(long long)(row0 + r) * n + k0 + c] = P[e];
+    }
+}
+
+// The panel's row swaps on the other columns (as they were taken), then a copy of the pivot
+// rows R[s][c] = A[k0 + s][c]: one thread per column.  Warp 0 first composes the swaps (lane
+// s: the row that ends in panel row k0 + s, and of up to kb rows outside the panel), so that
+// a thread's loads are independent: taken one swap after another they were a chain of kb
+// round trips.
+template <typename C>
+__global__ void __launch_bounds__(128) k_gj_swap_rows(C* A, int n, int k0, int kb, GJWork w) {
+    constexpr int B = GJPanel<C>::B;
+    __shared__ int from_in[32], row_out[32], from_out[32];
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int fi = k0 + lane, ro = -1, fo = -1, cnt = 0;
+        const int mine = lane < kb ? w.perm[k0 + lane] : 0;
+        for (int j = 0; j < kb; ++j) {
+            const int p = __shfl_sync(0xffffffffu, mine, j);
+            if (p == k0 + j) continue;           // uniform
+            const int fj = __shfl_sync(0xffffffffu, fi, j);
+            if (p < k0 + kb) {
+                const int fp = __shfl_sync(0xffffffffu, fi, p - k0);
+                if (lane == j) fi = fp;
+                if (lane == p - k0) fi = fj;
+            } else {
+                const unsigned hit = __ballot_sync(0xffffffffu, ro == p);
+                const int slot = hit ? __ffs(hit) - 1 : cnt++;
+                if (lane == slot && !hit) { ro = p; fo = p; }
+                const int fp = __shfl_sync(0xffffffffu, fo, slot);
+                if (lane == j) fi = fp;
+                if (lane == slot) fo = fj;
+            }
+        }
+        from_in[lane] = fi;
+        row_out[lane] = ro;
+        from_out[lane] = fo;
+    }
+    __syncthreads();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     C* R = reinterpret_cast<C*>(w.rows);
     const bool in_panel = c >= k0 && c < k0 + kb;
-    for (int j = k0; j < k0 + kb; ++j) {
-        const int p = w.perm[j];
-        if (!in_panel && p != j) {
-            const C t = A[(long long)j * n + c];
-            A[(long long)j * n + c] = A[(long long)p * n + c];
-            A[(long long)p * n + c] = t;
+    C a[B], o[B];
+#pragma unroll
+    for (int s = 0; s < B; ++s)
+        if (s < kb) {
+            a[s] = A[(long long)(in_panel ? k0 + s : from_in[s]) * n + c];
+            if (!in_panel && row_out[s] >= 0) o[s] = A[(long long)from_out[s] * n + c];
         }
-        R[(long long)(j - k0) * n + c] = A[(long long)j * n + c];
-    }
+#pragma unroll
+    for (int s = 0; s < B; ++s)
+        if (s < kb) {
+            R[(long long)s * n + c] = a[s];
+            if (!in_panel) {
+                if (from_in[s] != k0 + s) A[(long long)(k0 + s) * n + c] = a[s];
+                if (row_out[s] >= 0) A[(long long)row_out[s] * n + c] = o[s];
+            }
+        }
 }
 
 // A[i][c] = [i outside S] A[i][c] + sum_s A[i][k0 + s] R[s][c] for every column c
@@ -432,15 +657,23 @@ void launch_gauss_jordan(C* A, int n, void* work, cudaStream_t s) {
     long long launches = 0;
     const dim3 tiles((n + 63) / 64, (n + 63) / 64);
     const int ncand = (n + kGJRowsPerCTA - 1) / kGJRowsPerCTA;   // <= n slots of 16 B
+    const int R = (n + kGJCluster - 1) / kGJCluster;             // rows per CTA of the panel cluster
+    const bool cluster = R <= kGJPanelRows;
+    if (cluster)
+        MG_CUDA(cudaFuncSetAttribute(k_gj_panel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGJPanelRows * 256));
     for (int k0 = 0; k0 < n; k0 += B) {
         const int kb = n - k0 < B ? n - k0 : B;
-        for (int k = k0; k < k0 + kb; ++k) {
-            k_gj_pivot<C><<<1, 1024, 0, s>>>(A, n, k, k0, kb, w, k > k0 ? ncand : 0);
-            k_gj_eliminate<C><<<ncand, 32 * kGJRowsPerCTA, 0, s>>>(A, n, k, k0, kb, w);
+        if (cluster) {
+            k_gj_panel<C><<<kGJCluster, kGJPanelThreads, (size_t)R * 256, s>>>(A, n, k0, kb, R, w);
+        } else {
+            for (int k = k0; k < k0 + kb; ++k) {
+                k_gj_pivot<C><<<1, 1024, 0, s>>>(A, n, k, k0, kb, w, k > k0 ? ncand : 0);
+                k_gj_eliminate<C><<<ncand, 32 * kGJRowsPerCTA, 0, s>>>(A, n, k, k0, kb, w);
+            }
         }
-        k_gj_swap_rows<C><<<(n + 255) / 256, 256, 0, s>>>(A, n, k0, kb, w);
+        k_gj_swap_rows<C><<<(n + 127) / 128, 128, 0, s>>>(A, n, k0, kb, w);
         k_gj_update<C, B><<<tiles, 256, 0, s>>>(A, n, k0, kb, w);
-        launches += 2LL * kb + 2;
+        launches += (cluster ? 1LL : 2LL * kb) + 2;
     }
     launch_counter().fetch_add(launches - 1);
     MG_LAUNCHED();

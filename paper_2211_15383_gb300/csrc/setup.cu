@@ -419,9 +419,8 @@ static void block_jacobi_setup(Ctx& c, int l) {
         L.Ahat32 = c.alloc_n<float2>(nb * 5);
     }
     int* status = c.scratch<int>("status_bj", 4);
-    double2* work = c.scratch<double2>("bj_work", nb);
     MG_CUDA(cudaMemsetAsync(status, 0, sizeof(int), c.stream));
-    launch_block_diag_inverse(L.Minv64, work, L.A64, L.nsites, L.d, status, c.stream);
+    launch_block_diag_inverse(L.Minv64, L.A64, L.nsites, L.d, status, c.stream);
     launch_precondition_blocks(L.Ahat64, L.A64, L.Minv64, L.lx, L.lt, L.d, c.stream);
     launch_convert<float2, double2>(L.Minv32, L.Minv64, (long long)nb, c.stream);
     launch_convert<float2, double2>(L.Ahat32, L.Ahat64, (long long)nb * 5, c.stream);

@@ -1,5 +1,5 @@
-"""The block FGMRES on its own (no smoothing, rough test vectors: a weak preconditioner, so
-that one cycle runs to the restart length): restart lengths below, at and above 32 vectors,
+"""The block FGMRES with a weak preconditioner (one smoothing step, one rough test vector: one
+cycle runs to the restart length): restart lengths below, at and above 32 vectors,
 narrow and ragged blocks, zero right-hand sides among the others."""
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ from oracle import hierarchy as ohier
 from gpu_common import make_ctx, rand_complex, require_gpu, small_problem
 
 pytestmark = pytest.mark.gpu
-AGG, NVEC, M0 = ((2, 2),), (1,), 0.05
+AGG, NVEC, M0 = ((2, 2),), (1,), 0.4
 
 
 @pytest.fixture(scope="module")
@@ -27,7 +27,7 @@ def test_solve(pkg, prec, nrhs, restart):
     b *= np.exp2(np.arange(nrhs) % 5 * 20.0 - 40.0)[:, None]
     if nrhs > 2:
         b[1] = 0
-    with make_ctx(pkg, theta, M0, AGG, NVEC, sv, 0, mg_precision=prec, fgmres_restart=restart, nu_post=0,
+    with make_ctx(pkg, theta, M0, AGG, NVEC, sv, 0, mg_precision=prec, fgmres_restart=restart, nu_post=1,
                   max_iters=20000) as ctx:
         x, iters = ctx.solve(1, b)
         zero, none = ctx.solve(1, np.zeros_like(b))
