@@ -10,20 +10,23 @@
 namespace mg {
 
 // ------------------------------------------------------------------ GEMM nn
-// Tile 64 x 32 (rows x cols), K step 16; thread (tx, ty) owns column tx and rows
-// ty*8 .. ty*8+7.  All threads of a warp share ty, so A reads are broadcasts.
-constexpr int GM = 64, GN = 32, GK = 16;
+// Tile 8 RT x 32 (rows x cols), K step 16; thread (tx, ty) owns column tx and rows
+// ty*RT .. ty*RT+RT-1.  All threads of a warp share ty, so A reads are broadcasts.  RT = 8 where
+// that gives every SM a tile, else 1: in FP64 an SM does 2 operations per clock, so idle SMs
+// cost more than the extra reads of B (1024 x 64 x 64: 134 us with RT = 8 on 32 SMs).
+constexpr int GN = 32, GK = 16;
 
-template <typename S, typename C>
+template <typename S, typename C, int RT>
 __global__ void __launch_bounds__(256) k_gemm_nn(S* __restrict__ Cm, const S* __restrict__ A,
                                                  const S* __restrict__ B, int M, int K, int Nc, bool accumulate) {
+    constexpr int GM = 8 * RT;
     __shared__ C As[GM][GK + 1];
     __shared__ C Bs[GK][GN];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
     const int row0 = blockIdx.y * GM, col0 = blockIdx.x * GN;
-    C acc[8];
+    C acc[RT];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) acc[r] = czero<C>();
+    for (int r = 0; r < RT; ++r) acc[r] = czero<C>();
     for (int k0 = 0; k0 < K; k0 += GK) {
         for (int e = tid; e < GM * GK; e += 256) {
             const int r = e / GK, k = e % GK;
@@ -40,15 +43,15 @@ __global__ void __launch_bounds__(256) k_gemm_nn(S* __restrict__ Cm, const S* __
         for (int k = 0; k < GK; ++k) {
             const C bv = Bs[k][tx];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) cfma(acc[r], As[ty * 8 + r][k], bv);
+            for (int r = 0; r < RT; ++r) cfma(acc[r], As[ty * RT + r][k], bv);
         }
         __syncthreads();
     }
     const int gc = col0 + tx;
     if (gc >= Nc) return;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int gr = row0 + ty * 8 + r;
+    for (int r = 0; r < RT; ++r) {
+        const int gr = row0 + ty * RT + r;
         if (gr < M) {
             const long long idx = (long long)gr * Nc + gc;
             const S v = cvtc(acc[r], S{});
@@ -92,24 +95,30 @@ __global__ void __launch_bounds__(128) k_gemm_nn8(C* __restrict__ Cm, const C* _
     }
 }
 
+template <typename S, typename C>
+static void gemm_nn(S* Cm, const S* A, const S* B, int M, int K, int Nc, bool accumulate, cudaStream_t s) {
+    const int gx = (Nc + GN - 1) / GN;
+    if ((long long)gx * ((M + 63) / 64) < kNumSM && (M + 7) / 8 <= 65535)
+        k_gemm_nn<S, C, 1><<<dim3(gx, (M + 7) / 8), dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
+    else
+        k_gemm_nn<S, C, 8><<<dim3(gx, (M + 63) / 64), dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
+    MG_LAUNCHED();
+}
+
 template <typename C>
 void launch_gemm_nn(C* Cm, const C* A, const C* B, int M, int K, int Nc, bool accumulate, cudaStream_t s) {
-    MG_REQUIRE((M + 15) / 16 <= 65535 || (Nc > 8 && (M + GM - 1) / GM <= 65535), MGMLMC_EINVAL, "gemm_nn: M too large");
+    MG_REQUIRE((M + 15) / 16 <= 65535 || (Nc > 8 && (M + 63) / 64 <= 65535), MGMLMC_EINVAL, "gemm_nn: M too large");
     if (Nc <= 8) {
         dim3 g(1, (M + 15) / 16);
         k_gemm_nn8<C><<<g, dim3(8, 16), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
         MG_LAUNCHED();
         return;
     }
-    dim3 g((Nc + GN - 1) / GN, (M + GM - 1) / GM);
-    k_gemm_nn<C, C><<<g, dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
-    MG_LAUNCHED();
+    gemm_nn<C, C>(Cm, A, B, M, K, Nc, accumulate, s);
 }
 
 void launch_gemm_nn_fp32(double2* Cm, const double2* A, const double2* B, int M, int K, int Nc, cudaStream_t s) {
-    dim3 g((Nc + GN - 1) / GN, (M + GM - 1) / GM);
-    k_gemm_nn<double2, float2><<<g, dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, false);
-    MG_LAUNCHED();
+    gemm_nn<double2, float2>(Cm, A, B, M, K, Nc, false, s);
 }
 
 // ------------------------------------------------------------------ GEMM hn
@@ -158,7 +167,7 @@ int gemm_hn_groups(long long n, int ka, int kb) {
     const long long tiles = (long long)((ka + 31) / 32) * ((kb + 31) / 32);
     long long g = (4LL * kNumSM) / tiles;
     if (g < 1) g = 1;
-    const long long maxg = (n + 63) / 64;
+    const long long maxg = (n + 15) / 16;         // a slice is at least one stage of 16 rows
     if (g > maxg) g = maxg;
     return (int)g;
 }
@@ -698,6 +707,7 @@ void launch_gauss_jordan(C* A, int n, void* work, cudaStream_t s) {
 // eigenvectors in the matching columns of W.
 namespace jac {
 constexpr int kThreads = 256;
+constexpr int kLocalRot = 64;                 // rotations of a round that every CTA forms itself
 constexpr long long kSpinLimit = 1LL << 24;   // x ~64 ns sleep: a barrier gives up after ~1 s
 
 struct Sync {
@@ -755,11 +765,12 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
     __shared__ double red_off[kThreads], red_tot[kThreads];
     __shared__ int stop;
     const unsigned G = gridDim.x;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nthr = (long long)G * blockDim.x;
-    const long long bb = (long long)bp * bp;
-    for (long long e = tid; e < bb; e += nthr) {
-        const int i = (int)(e / bp), j = (int)(e % bp);
+    // consecutive warps of work go to different CTAs: few items still use every SM's FP64 pipe
+    const int tid = (int)(((threadIdx.x >> 5) * G + blockIdx.x) * 32 + (threadIdx.x & 31));
+    const int nthr = (int)(G * blockDim.x);
+    const int bb = bp * bp;
+    for (int e = tid; e < bb; e += nthr) {
+        const int i = e / bp, j = e % bp;
         A0[e] = (i < b && j < b) ? Hin[(long long)i * b + j] : make_double2(0.0, 0.0);
         Wp[e] = make_double2(i == j ? 1.0 : 0.0, 0.0);
     }
@@ -768,7 +779,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
     double2* nxt = A1;
     for (int sw = 0; sw < sweeps; ++sw) {
         double lo = 0.0, lt = 0.0;
-        for (long long e = tid; e < bb; e += nthr) {
+        for (int e = tid; e < bb; e += nthr) {
             const double2 v = __ldcg(cur + e);
             const double m = v.x * v.x + v.y * v.y;
             lt += m;
@@ -801,48 +812,63 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
         if (stop) break;
         for (int r = 0; r < bp - 1; ++r) {
             // each rotation of the round once, grid-wide (FP64 square roots and divisions
-            // run at 1/64 of the FP32 rate: computing all of them in every CTA cost more
-            // than the block updates), published in rot[4][half] ...
-            for (long long k = tid; k < half; k += nthr) {
-                int p = ord((int)k, r, bp), q = ord(bp - 1 - (int)k, r, bp);
+            // run at 1/64 of the FP32 rate: when every CTA computed all of them, that cost
+            // more than the block updates at b = 1024), published in rot[4][half] and staged
+            // by every CTA after a barrier; up to kLocalRot pairs (two warps' work) every
+            // CTA forms them itself, which saves that barrier
+            const bool local = half <= kLocalRot;
+            for (int k = local ? (int)threadIdx.x : tid; k < half; k += local ? (int)blockDim.x : nthr) {
+                int p = ord(k, r, bp), q = ord(bp - 1 - k, r, bp);
                 if (p > q) { const int t = p; p = q; q = t; }
                 double c = 1.0, sn = 0.0, pr = 1.0, pi = 0.0;
                 if (q < b) {
                     const double2 hpq = __ldcg(cur + (long long)p * bp + q);
-                    const double a = sqrt(hpq.x * hpq.x + hpq.y * hpq.y);
+                    const double hpp = __ldcg(cur + (long long)p * bp + p).x;
+                    const double hqq = __ldcg(cur + (long long)q * bp + q).x;
+                    const double a2 = hpq.x * hpq.x + hpq.y * hpq.y;
+                    const double a = sqrt(a2);
                     if (a > 0.0) {
-                        const double hpp = __ldcg(cur + (long long)p * bp + p).x;
-                        const double hqq = __ldcg(cur + (long long)q * bp + q).x;
-                        const double tau = (hqq - hpp) / (2.0 * a);
+                        const double ia = 1.0 / a;
+                        const double tau = (hqq - hpp) * (0.5 * ia);
                         const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + t * t);
+                        c = rsqrt(1.0 + t * t);
                         sn = t * c;
-                        pr = hpq.x / a;
-                        pi = hpq.y / a;
+                        pr = hpq.x * ia;
+                        pi = hpq.y * ia;
                     }
                 }
-                rot[k] = c;
-                rot[half + k] = sn;
-                rot[2 * half + k] = pr;
-                rot[3 * half + k] = pi;
+                if (local) {
+                    rc[k] = c;
+                    rs[k] = sn;
+                    rpr[k] = pr;
+                    rpi[k] = pi;
+                    rp[k] = p;
+                    rq[k] = q;
+                } else {
+                    rot[k] = c;
+                    rot[half + k] = sn;
+                    rot[2 * half + k] = pr;
+                    rot[3 * half + k] = pi;
+                }
             }
-            if (!grid_barrier(sy, G)) return;
-            // ... and staged by every CTA into shared memory with the pair indices
-            for (int k = threadIdx.x; k < half; k += blockDim.x) {
-                int p = ord(k, r, bp), q = ord(bp - 1 - k, r, bp);
-                if (p > q) { const int t = p; p = q; q = t; }
-                rc[k] = __ldcg(rot + k);
-                rs[k] = __ldcg(rot + half + k);
-                rpr[k] = __ldcg(rot + 2 * half + k);
-                rpi[k] = __ldcg(rot + 3 * half + k);
-                rp[k] = p;
-                rq[k] = q;
+            if (!local) {
+                if (!grid_barrier(sy, G)) return;
+                for (int k = threadIdx.x; k < half; k += blockDim.x) {
+                    int p = ord(k, r, bp), q = ord(bp - 1 - k, r, bp);
+                    if (p > q) { const int t = p; p = q; q = t; }
+                    rc[k] = __ldcg(rot + k);
+                    rs[k] = __ldcg(rot + half + k);
+                    rpr[k] = __ldcg(rot + 2 * half + k);
+                    rpi[k] = __ldcg(rot + 3 * half + k);
+                    rp[k] = p;
+                    rq[k] = q;
+                }
             }
             __syncthreads();
             // 2x2 blocks (P, Q): out = G_P^H B G_Q
-            const long long nblk = (long long)half * half;
-            for (long long e = tid; e < nblk; e += nthr) {
-                const int P = (int)(e / half), Q = (int)(e % half);
+            const int nblk = half * half;
+            for (int e = tid; e < nblk; e += nthr) {
+                const int P = e / half, Q = e % half;
                 const int p1 = rp[P], q1 = rq[P], p2 = rp[Q], q2 = rq[Q];
                 const double c1 = rc[P], s1 = rs[P], c2 = rc[Q], s2 = rs[Q];
                 const double2 f1 = make_double2(rpr[P], rpi[P]);
@@ -864,9 +890,9 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
                 nxt[(long long)q1 * bp + q2] = make_double2(s2 * r10.x + c2 * g11.x, s2 * r10.y + c2 * g11.y);
             }
             // eigenvectors: W(:, P) <- W(:, P) G_P, in place (disjoint columns)
-            const long long nw = (long long)bp * half;
-            for (long long e = tid; e < nw; e += nthr) {
-                const int i = (int)(e / half), P = (int)(e % half);
+            const int nw = bp * half;
+            for (int e = tid; e < nw; e += nthr) {
+                const int i = e / half, P = e % half;
                 const int p = rp[P], q = rq[P];
                 const double c = rc[P], sn = rs[P];
                 const double2 fc = make_double2(rpr[P], -rpi[P]);
@@ -882,7 +908,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
         }
     }
     // the diagonal of the last matrix goes to part[0 .. b) for the sorting kernel
-    for (long long i = tid; i < b; i += nthr) part[2 * G + i] = __ldcg(cur + i * bp + i).x;
+    for (int i = tid; i < b; i += nthr) part[2 * G + i] = __ldcg(cur + (long long)i * bp + i).x;
 }
 
 // rank of every eigenvalue by |lambda| (ties by index), then lam and the columns
@@ -953,16 +979,24 @@ namespace chol {
 __global__ void __launch_bounds__(jac::kThreads) k_cholesky_grid(double2* G, double2* Rinv, double2* R, double2* Tt,
                                                                  int b, int* status, jac::Sync* sy) {
     const unsigned NB = gridDim.x;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nthr = (long long)NB * blockDim.x;
+    // consecutive warps of work go to different CTAs (see the eigensolver), and the square root
+    // and quotient of a column are formed once per CTA: FP64 runs at 1/64 of the FP32 rate
+    const int tid = (int)(((threadIdx.x >> 5) * NB + blockIdx.x) * 32 + (threadIdx.x & 31));
+    const int nthr = (int)(NB * blockDim.x);
+    __shared__ double piv[2];
     for (int j = 0; j < b; ++j) {
-        double d = __ldcg(G + (long long)j * b + j).x;
-        if (!(d > 0.0)) {
-            if (tid == 0) *status = 1;
-            d = 1e-300;
+        if (threadIdx.x == 0) {
+            double d = __ldcg(G + (long long)j * b + j).x;
+            if (!(d > 0.0)) {
+                *status = 1;
+                d = 1e-300;
+            }
+            piv[0] = sqrt(d);
+            piv[1] = 1.0 / piv[0];
         }
-        const double rd = sqrt(d), inv = 1.0 / rd;
-        for (long long i = tid; i < b; i += nthr) {
+        __syncthreads();
+        const double rd = piv[0], inv = piv[1], id = inv * inv;
+        for (int i = tid; i < b; i += nthr) {
             double2 v = make_double2(0.0, 0.0);
             if (i == j) v = make_double2(rd, 0.0);
             else if (i > j) {
@@ -971,23 +1005,23 @@ __global__ void __launch_bounds__(jac::kThreads) k_cholesky_grid(double2* G, dou
             }
             R[(long long)j * b + i] = v;
         }
-        const long long m = b - j - 1;
-        for (long long e = tid; e < m * m; e += nthr) {
-            const int p = j + 1 + (int)(e / m), q = j + 1 + (int)(e % m);
+        const int m = b - j - 1;
+        for (int e = tid; e < m * m; e += nthr) {
+            const int p = j + 1 + e / m, q = j + 1 + e % m;
             if (q < p) continue;
             const double2 gp = __ldcg(G + (long long)j * b + p), gq = __ldcg(G + (long long)j * b + q);
             const double2 g = __ldcg(G + (long long)p * b + q);
             // conj(R[j][p]) R[j][q] = conj(gp) gq / d
-            G[(long long)p * b + q] = make_double2(g.x - (gp.x * gq.x + gp.y * gq.y) / d,
-                                                   g.y - (gp.x * gq.y - gp.y * gq.x) / d);
+            G[(long long)p * b + q] = make_double2(g.x - (gp.x * gq.x + gp.y * gq.y) * id,
+                                                   g.y - (gp.x * gq.y - gp.y * gq.x) * id);
         }
         if (!jac::grid_barrier(sy, NB)) return;
     }
     const int lane = threadIdx.x & 31;
-    const long long warp = tid >> 5, nwarps = nthr >> 5;
-    for (long long c = warp; c < b; c += nwarps) {
-        double2* t = Tt + c * b;
-        for (int i = (int)c; i >= 0; --i) {
+    const int warp = (int)((threadIdx.x >> 5) * NB + blockIdx.x), nwarps = (int)(NB * (blockDim.x >> 5));
+    for (int c = warp; c < b; c += nwarps) {
+        double2* t = Tt + (long long)c * b;
+        for (int i = c; i >= 0; --i) {
             double sr = 0.0, si = 0.0;
             for (int k = i + 1 + lane; k <= c; k += 32) {
                 const double2 r = __ldcg(R + (long long)i * b + k), tk = t[k];
@@ -1000,17 +1034,17 @@ __global__ void __launch_bounds__(jac::kThreads) k_cholesky_grid(double2* G, dou
                 si += __shfl_xor_sync(0xffffffffu, si, o);
             }
             if (lane == 0) {
-                const double rii = __ldcg(R + (long long)i * b + i).x;
-                t[i] = make_double2(((i == c ? 1.0 : 0.0) - sr) / rii, -si / rii);
+                const double ir = 1.0 / __ldcg(R + (long long)i * b + i).x;
+                t[i] = make_double2(((i == c ? 1.0 : 0.0) - sr) * ir, -si * ir);
             }
             __syncwarp();
         }
-        for (int i = (int)c + 1 + lane; i < b; i += 32) t[i] = make_double2(0.0, 0.0);
+        for (int i = c + 1 + lane; i < b; i += 32) t[i] = make_double2(0.0, 0.0);
     }
     if (!jac::grid_barrier(sy, NB)) return;
-    for (long long e = tid; e < (long long)b * b; e += nthr) {
-        const long long i = e / b, c = e % b;
-        Rinv[e] = __ldcg(Tt + c * b + i);
+    for (int e = tid; e < b * b; e += nthr) {
+        const int i = e / b, c = e % b;
+        Rinv[e] = __ldcg(Tt + (long long)c * b + i);
     }
 }
 
@@ -1023,7 +1057,8 @@ size_t cholesky_work_bytes(int b) { return 2 * (size_t)b * b * sizeof(double2) +
 
 void launch_cholesky_inv(double2* G, double2* Rinv, int b, void* work, int* status, int* err, cudaStream_t s) {
     MG_REQUIRE(b >= 1 && b <= 4096, MGMLMC_EINVAL, "cholesky: 1 <= b <= 4096");
-    const int NB = jacobi_grid_size();
+    // one CTA per SM, or one per warp of the trailing update where there are fewer
+    const int NB = (int)std::min((long long)jacobi_grid_size(), std::max(1LL, ((long long)b * b + 63) / 64));
     double2* R = reinterpret_cast<double2*>(work);
     double2* Tt = R + (size_t)b * b;
     jac::Sync* sy = reinterpret_cast<jac::Sync*>(Tt + (size_t)b * b);
@@ -1040,7 +1075,10 @@ void launch_jacobi_eig(double2* H, double2* W, double* lam, int b, int sweeps, v
                        bool descending) {
     MG_REQUIRE(b >= 1 && b <= 2048, MGMLMC_EINVAL, "jacobi: 1 <= b <= 2048");
     const int bp = b + (b & 1);
-    const int G = jacobi_grid_size();
+    // one CTA per SM, or one per warp of 2 x 2 blocks where there are fewer (fewer arrivals
+    // at the barriers)
+    const long long half2 = (long long)(bp / 2) * (bp / 2);
+    const int G = (int)std::min((long long)jacobi_grid_size(), std::max(1LL, (half2 + 31) / 32));
     MG_REQUIRE(G <= 4 * kNumSM, MGMLMC_ECUDA, "jacobi: more SMs than the work space assumes");
     char* w = reinterpret_cast<char*>(work);
     const size_t mat = (size_t)bp * bp * sizeof(double2);
