@@ -46,6 +46,38 @@ std::atomic<long long>& launch_counter();   // all contexts, thread-safe
         if (!(cond)) throw ::mg::Error((code), (msg));                                  \
     } while (0)
 
+// ---- programmatic dependent launch
+// Kernels of the solver's chain are launched so that a kernel may be set up while the one
+// before it in the stream still runs: without it each launch starts about 2 us after the end
+// of its predecessor, as long as many of these kernels run.  Every kernel launched by
+// MG_LAUNCH begins with `if (grid_dependency()) return;`: it waits until the kernels before it
+// have completed and their writes are visible (so a chain orders as plain launches do), then
+// lets the next one be set up.  The result is always false; the branch on it keeps the
+// compiler from moving reads through const __restrict__ pointers, which it takes for
+// invariant, above the wait.
+__device__ __forceinline__ bool grid_dependency() {
+    int z;
+    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n mov.u32 %0, 0;" : "=r"(z)::"memory");
+    return z != 0;
+}
+
+template <typename... P, typename... A>
+inline void launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    MG_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+}
+// MG_LAUNCH(grid, block, smem, stream, (kernel<...>), args...)
+#define MG_LAUNCH(g, b, sm, s, k, ...) ::mg::launch_dependent(k, g, b, sm, s, __VA_ARGS__)
+
 // ---- complex type per real type --------------------------------------------------
 template <typename R> struct Cx;
 template <> struct Cx<double> { using T = double2; };

@@ -19,6 +19,7 @@ constexpr int GN = 32, GK = 16;
 template <typename S, typename C, int RT>
 __global__ void __launch_bounds__(256) k_gemm_nn(S* __restrict__ Cm, const S* __restrict__ A,
                                                  const S* __restrict__ B, int M, int K, int Nc, bool accumulate) {
+    if (grid_dependency()) return;
     constexpr int GM = 8 * RT;
     __shared__ C As[GM][GK + 1];
     __shared__ C Bs[GK][GN];
@@ -66,6 +67,7 @@ __global__ void __launch_bounds__(256) k_gemm_nn(S* __restrict__ Cm, const S* __
 template <typename C>
 __global__ void __launch_bounds__(128) k_gemm_nn8(C* __restrict__ Cm, const C* __restrict__ A,
                                                   const C* __restrict__ B, int M, int K, int Nc, bool accumulate) {
+    if (grid_dependency()) return;
     constexpr int ROWS = 16, KT = 64;
     __shared__ C As[ROWS][KT + 1];
     __shared__ C Bs[KT][8];
@@ -99,9 +101,9 @@ template <typename S, typename C>
 static void gemm_nn(S* Cm, const S* A, const S* B, int M, int K, int Nc, bool accumulate, cudaStream_t s) {
     const int gx = (Nc + GN - 1) / GN;
     if ((long long)gx * ((M + 63) / 64) < kNumSM && (M + 7) / 8 <= 65535)
-        k_gemm_nn<S, C, 1><<<dim3(gx, (M + 7) / 8), dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
+        MG_LAUNCH(dim3(gx, (M + 7) / 8), dim3(32, 8), 0, s, (k_gemm_nn<S, C, 1>), Cm, A, B, M, K, Nc, accumulate);
     else
-        k_gemm_nn<S, C, 8><<<dim3(gx, (M + 63) / 64), dim3(32, 8), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
+        MG_LAUNCH(dim3(gx, (M + 63) / 64), dim3(32, 8), 0, s, (k_gemm_nn<S, C, 8>), Cm, A, B, M, K, Nc, accumulate);
     MG_LAUNCHED();
 }
 
@@ -110,7 +112,7 @@ void launch_gemm_nn(C* Cm, const C* A, const C* B, int M, int K, int Nc, bool ac
     MG_REQUIRE((M + 15) / 16 <= 65535 || (Nc > 8 && (M + 63) / 64 <= 65535), MGMLMC_EINVAL, "gemm_nn: M too large");
     if (Nc <= 8) {
         dim3 g(1, (M + 15) / 16);
-        k_gemm_nn8<C><<<g, dim3(8, 16), 0, s>>>(Cm, A, B, M, K, Nc, accumulate);
+        MG_LAUNCH(g, dim3(8, 16), 0, s, (k_gemm_nn8<C>), Cm, A, B, M, K, Nc, accumulate);
         MG_LAUNCHED();
         return;
     }
@@ -128,6 +130,7 @@ template <typename S, typename C>
 __global__ void __launch_bounds__(256) k_gemm_hn(double2* __restrict__ part, const S* __restrict__ A,
                                                  const S* __restrict__ B, long long n, int ka, int kb,
                                                  long long slice) {
+    if (grid_dependency()) return;
     __shared__ C As[16][33];
     __shared__ C Bs[16][33];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
@@ -178,7 +181,7 @@ void launch_gemm_hn(double2* Cm, const C* A, const C* B, long long n, int ka, in
     long long slice = (n + groups - 1) / groups;
     slice = ((slice + 15) / 16) * 16;
     dim3 g((kb + 31) / 32, (ka + 31) / 32, groups);
-    k_gemm_hn<C, C><<<g, dim3(32, 8), 0, s>>>(part, A, B, n, ka, kb, slice);
+    MG_LAUNCH(g, dim3(32, 8), 0, s, (k_gemm_hn<C, C>), part, A, B, n, ka, kb, slice);
     MG_LAUNCHED();
     launch_finalize(Cm, part, groups, ka * kb, s);
 }
@@ -196,7 +199,7 @@ void launch_gemm_hn_fp32(double2* Cm, const double2* A, const double2* B, long l
     long long slice = (n + groups - 1) / groups;
     slice = ((slice + 15) / 16) * 16;
     dim3 g((kb + 31) / 32, (ka + 31) / 32, groups);
-    k_gemm_hn<double2, float2><<<g, dim3(32, 8), 0, s>>>(part, A, B, n, ka, kb, slice);
+    MG_LAUNCH(g, dim3(32, 8), 0, s, (k_gemm_hn<double2, float2>), part, A, B, n, ka, kb, slice);
     MG_LAUNCHED();
     launch_finalize(Cm, part, groups, ka * kb, s);
 }
@@ -246,6 +249,7 @@ template <> struct GJPanel<double2> { static constexpr int B = 16; };
 // pivot: the largest |A[i][k]|^2, ties to the smallest row index.
 template <typename C>
 __global__ void __launch_bounds__(1024) k_gj_pivot(C* A, int n, int k, int k0, int kb, GJWork w, int ncand) {
+    if (grid_dependency()) return;
     __shared__ double best[1024];
     __shared__ int bidx[1024];
     double bv = -1.0;
@@ -306,6 +310,7 @@ __global__ void __launch_bounds__(1024) k_gj_pivot(C* A, int n, int k, int k0, i
 // the pivot candidate of that column among its rows i > k (w.cand[blockIdx.x]).
 template <typename C>
 __global__ void __launch_bounds__(32 * kGJRowsPerCTA) k_gj_eliminate(C* A, int n, int k, int k0, int kb, GJWork w) {
+    if (grid_dependency()) return;
     __shared__ double cm[kGJRowsPerCTA];
     __shared__ int ci[kGJRowsPerCTA];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -535,6 +540,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
 // round trips.
 template <typename C>
 __global__ void __launch_bounds__(128) k_gj_swap_rows(C* A, int n, int k0, int kb, GJWork w) {
+    if (grid_dependency()) return;
     constexpr int B = GJPanel<C>::B;
     __shared__ int from_in[32], row_out[32], from_out[32];
     if (threadIdx.x < 32) {
@@ -590,6 +596,7 @@ __global__ void __launch_bounds__(128) k_gj_swap_rows(C* A, int n, int k0, int k
 // tx + 16b (a, b < 4); the panel columns are read, never written.
 template <typename C, int B>
 __global__ void __launch_bounds__(256) k_gj_update(C* A, int n, int k0, int kb, GJWork w) {
+    if (grid_dependency()) return;
     __shared__ C Ts[64][B + 1];
     __shared__ C Rs[B][64];
     const C* R = reinterpret_cast<const C*>(w.rows);
@@ -635,6 +642,7 @@ __global__ void __launch_bounds__(256) k_gj_update(C* A, int n, int k0, int kb, 
 
 template <typename C>
 __global__ void k_gj_unpermute(C* A, int n, GJWork w) {
+    if (grid_dependency()) return;
     // column swaps in reverse order of the row swaps; one thread per row
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -676,17 +684,17 @@ void launch_gauss_jordan(C* A, int n, void* work, cudaStream_t s) {
             k_gj_panel<C><<<kGJCluster, kGJPanelThreads, (size_t)R * 256, s>>>(A, n, k0, kb, R, w);
         } else {
             for (int k = k0; k < k0 + kb; ++k) {
-                k_gj_pivot<C><<<1, 1024, 0, s>>>(A, n, k, k0, kb, w, k > k0 ? ncand : 0);
-                k_gj_eliminate<C><<<ncand, 32 * kGJRowsPerCTA, 0, s>>>(A, n, k, k0, kb, w);
+                MG_LAUNCH(1, 1024, 0, s, (k_gj_pivot<C>), A, n, k, k0, kb, w, k > k0 ? ncand : 0);
+                MG_LAUNCH(ncand, 32 * kGJRowsPerCTA, 0, s, (k_gj_eliminate<C>), A, n, k, k0, kb, w);
             }
         }
-        k_gj_swap_rows<C><<<(n + 127) / 128, 128, 0, s>>>(A, n, k0, kb, w);
-        k_gj_update<C, B><<<tiles, 256, 0, s>>>(A, n, k0, kb, w);
+        MG_LAUNCH((n + 127) / 128, 128, 0, s, (k_gj_swap_rows<C>), A, n, k0, kb, w);
+        MG_LAUNCH(tiles, 256, 0, s, (k_gj_update<C, B>), A, n, k0, kb, w);
         launches += (cluster ? 1LL : 2LL * kb) + 2;
     }
     launch_counter().fetch_add(launches - 1);
     MG_LAUNCHED();
-    k_gj_unpermute<C><<<(n + 127) / 128, 128, 0, s>>>(A, n, w);
+    MG_LAUNCH((n + 127) / 128, 128, 0, s, (k_gj_unpermute<C>), A, n, w);
     MG_LAUNCHED();
 }
 
@@ -914,6 +922,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(const double2* __restr
 // rank of every eigenvalue by |lambda| (ties by index), then lam and the columns
 // of W permuted to that order; a barrier failure is passed to the caller's flag.
 __global__ void k_jacobi_rank(const double* diag, int* rank, int b, int descending) {
+    if (grid_dependency()) return;
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     if (col >= b) return;
     const double lc = descending ? -fabs(diag[col]) : fabs(diag[col]);
@@ -927,6 +936,7 @@ __global__ void k_jacobi_rank(const double* diag, int* rank, int b, int descendi
 
 __global__ void k_jacobi_permute(const double* diag, const int* rank, const double2* Wp, double2* W, double* lam,
                                  int b, int bp, const Sync* sy, int* err) {
+    if (grid_dependency()) return;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nthr = (long long)gridDim.x * blockDim.x;
     for (long long e = tid; e < (long long)b * b; e += nthr) {
@@ -1049,6 +1059,7 @@ __global__ void __launch_bounds__(jac::kThreads) k_cholesky_grid(double2* G, dou
 }
 
 __global__ void k_flag(const jac::Sync* sy, int* err) {
+    if (grid_dependency()) return;
     if (err && sy->err) *err = 1;
 }
 }  // namespace chol
@@ -1067,7 +1078,7 @@ void launch_cholesky_inv(double2* G, double2* Rinv, int b, void* work, int* stat
     MG_CUDA(cudaLaunchCooperativeKernel((const void*)chol::k_cholesky_grid, dim3(NB), dim3(jac::kThreads), args, 0,
                                         s));
     MG_LAUNCHED();
-    chol::k_flag<<<1, 1, 0, s>>>(sy, err);
+    MG_LAUNCH(1, 1, 0, s, chol::k_flag, sy, err);
     MG_LAUNCHED();
 }
 
@@ -1097,9 +1108,9 @@ void launch_jacobi_eig(double2* H, double2* W, double* lam, int b, int sweeps, v
     MG_CUDA(cudaLaunchCooperativeKernel((const void*)jac::k_jacobi_grid, dim3(G), dim3(jac::kThreads), args, sm, s));
     MG_LAUNCHED();
     int* rank = reinterpret_cast<int*>(sy + 1);
-    jac::k_jacobi_rank<<<(b + 255) / 256, 256, 0, s>>>(part + 2 * G, rank, b, descending ? 1 : 0);
+    MG_LAUNCH((b + 255) / 256, 256, 0, s, jac::k_jacobi_rank, part + 2 * G, rank, b, descending ? 1 : 0);
     MG_LAUNCHED();
-    jac::k_jacobi_permute<<<2 * kNumSM, 256, 0, s>>>(part + 2 * G, rank, Wp, W, lam, b, bp, sy, err);
+    MG_LAUNCH(2 * kNumSM, 256, 0, s, jac::k_jacobi_permute, part + 2 * G, rank, Wp, W, lam, b, bp, sy, err);
     MG_LAUNCHED();
 }
 

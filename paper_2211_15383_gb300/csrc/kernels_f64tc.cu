@@ -83,6 +83,7 @@ __device__ __forceinline__ uint32_t pack_exact(float lo, float hi) {
 // above all, so the atomic maximum does not depend on the order.
 __global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, const double2* __restrict__ x,
                                                      long long n, int N) {
+    if (grid_dependency()) return;
     __shared__ u64 sh[256];
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, cons
 // tile beyond the rhs are not written (they only reach the same rows of the product).
 __global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const double2* __restrict__ x,
                                                  const u64* __restrict__ mx, int nblk, int N, int T) {
+    if (grid_dependency()) return;
     const int row = threadIdx.x, t = blockIdx.y, j = 128 * t + row;
     const long long g = (long long)blockIdx.x * blockDim.y + threadIdx.y;    // (block, component group)
     const int site = (int)(g >> 2), cg = (int)(g & 3);
@@ -142,6 +144,7 @@ __global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const
 // Thread = (block, output real, 8 input reals).
 __global__ void __launch_bounds__(128) k_slice_a(uint8_t* __restrict__ as, const double2* __restrict__ A,
                                                  const u64* __restrict__ mx, long long nblk, int nb, int ld) {
+    if (grid_dependency()) return;
     const long long q = blockIdx.x;
     if (q >= nblk) return;
     const int n = threadIdx.x >> 2, kg = threadIdx.x & 3;
@@ -204,6 +207,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const uint8_t* __restrict__ xs, const uint8_t* __restrict__ as, const u64* __restrict__ mxx,
                 const u64* __restrict__ mxa, int lx, int lt, int nblk, int splits, int N, double2* __restrict__ part,
                 int* __restrict__ err) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[NSTG], empty[NSTG], afull[2], aempty[2];
     __shared__ uint32_t tmem_holder;
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // y = sum over the splits of a dense product, in order.
 __global__ void __launch_bounds__(256) k_sum_splits(double2* __restrict__ y, const double2* __restrict__ p,
                                                     long long count, int splits) {
+    if (grid_dependency()) return;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
          e += (long long)gridDim.x * blockDim.x) {
         double2 s = p[e];
@@ -418,7 +423,7 @@ static void absmax(u64* out, const double2* x, long long n, int N, cudaStream_t 
     const int by = 256 / bx, gx = (N + bx - 1) / bx;
     const long long need = (n + 4 * by - 1) / (4 * by);
     const int gy = (int)std::max(1LL, std::min(need, 8LL * kNumSM / gx));
-    k_absmax_cols<<<dim3(gx, gy), dim3(bx, by), 0, s>>>(out, x, n, N);
+    MG_LAUNCH(dim3(gx, gy), dim3(bx, by), 0, s, k_absmax_cols, out, x, n, N);
     MG_LAUNCHED();
 }
 
@@ -432,9 +437,9 @@ void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int 
     u64* mx = const_cast<u64*>(operand_max(op, nblk));
     // a flat array as 32 columns: the maximum of its 32 column maxima is taken below
     absmax(mx, A, nblk * (D * D) / 32, 32, s);
-    tc::f64::k_absmax_cols<<<1, dim3(1, 32), 0, s>>>(mx, reinterpret_cast<const double2*>(mx), 16, 1);
+    MG_LAUNCH(1, dim3(1, 32), 0, s, tc::f64::k_absmax_cols, mx, reinterpret_cast<const double2*>(mx), 16, 1);
     MG_LAUNCHED();
-    k_slice_a<<<(unsigned)nblk, 128, 0, s>>>(reinterpret_cast<uint8_t*>(op), A, mx, nblk, nb, nb ? ld : D);
+    MG_LAUNCH((unsigned)nblk, 128, 0, s, k_slice_a, reinterpret_cast<uint8_t*>(op), A, mx, nblk, nb, nb ? ld : D);
     MG_LAUNCHED();
 }
 
@@ -446,8 +451,7 @@ static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N
     int bx = 8;
     while (bx < N && bx < 128) bx *= 2;
     const int by = 128 / bx;
-    k_slice_x<<<dim3((unsigned)((4 * nblk + by - 1) / by), T), dim3(bx, by), 0, s>>>(
-        reinterpret_cast<uint8_t*>(scratch), x, mx, (int)nblk, N, T);
+    MG_LAUNCH(dim3((unsigned)((4 * nblk + by - 1) / by), T), dim3(bx, by), 0, s, k_slice_x, reinterpret_cast<uint8_t*>(scratch), x, mx, (int)nblk, N, T);
     MG_LAUNCHED();
     return mx;
 }
@@ -457,8 +461,7 @@ static void f64_launch(double2* y, const double2* b, const double2* x, const voi
                        const u64* mxx, const u64* mxa, int lx, int lt, int nblk, int splits, int N, double2* part,
                        int groups, int* err, cudaStream_t s) {
     MG_CUDA(cudaFuncSetAttribute(k_block_f64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-    k_block_f64<MODE><<<dim3(groups, f64_tiles(N)), THREADS, SMEM, s>>>(
-        y, b, x, reinterpret_cast<const uint8_t*>(scratch), reinterpret_cast<const uint8_t*>(op), mxx, mxa, lx, lt,
+    MG_LAUNCH(dim3(groups, f64_tiles(N)), THREADS, SMEM, s, (k_block_f64<MODE>), y, b, x, reinterpret_cast<const uint8_t*>(scratch), reinterpret_cast<const uint8_t*>(op), mxx, mxa, lx, lt,
         nblk, splits, N, part, err);
     MG_LAUNCHED();
 }
@@ -499,7 +502,7 @@ void launch_dense_f64(double2* y, const double2* x, const void* op, int n, int N
                   N, nullptr, G, err, s);
     if (S > 1) {
         const long long cnt = (long long)n * N;
-        k_sum_splits<<<(int)std::min((cnt + 255) / 256, 16LL * kNumSM), 256, 0, s>>>(y, p, cnt, S);
+        MG_LAUNCH((int)std::min((cnt + 255) / 256, 16LL * kNumSM), 256, 0, s, k_sum_splits, y, p, cnt, S);
         MG_LAUNCHED();
     }
 }

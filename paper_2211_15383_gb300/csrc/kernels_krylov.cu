@@ -99,6 +99,7 @@ template <typename C, int M, int V, int R>
 __global__ void __launch_bounds__(256, (DotRegs<C, M, V, R>::blocks))
     k_multidot(CSum<C>* __restrict__ part, const C* __restrict__ Vb, int m, int mt, const C* __restrict__ w,
                long long n, int N) {
+    if (grid_dependency()) return;
     constexpr int KC = 4;                        // vectors reduced at once
     constexpr int KL = M < 8 ? M : 8;            // vectors loaded at once
     __shared__ C sh[KC][256 * V];
@@ -172,6 +173,7 @@ template <typename C>
 __global__ void __launch_bounds__(256) k_finalize_dots(C* __restrict__ cf, double2* __restrict__ H,
                                                        const CSum<C>* __restrict__ part, int groups, int m, int N,
                                                        const double* __restrict__ ieta, bool add) {
+    if (grid_dependency()) return;
     __shared__ CSum<C> sh[256];
     const int r = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
     CSum<C> s;
@@ -208,6 +210,7 @@ __global__ void __launch_bounds__(256, 4) k_multiaxpy(C* __restrict__ w, const C
                                                       const C* __restrict__ Vb, long long n, int N, bool accumulate,
                                                       sum_t<C>* __restrict__ npart,
                                                       const double* __restrict__ nscale) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     constexpr int KC = V * sizeof(C) == 8 ? 8 : 4;
     __shared__ Vec<C, V> cs[64 * 32];
@@ -268,6 +271,7 @@ __global__ void __launch_bounds__(256, 4) k_multiaxpy(C* __restrict__ w, const C
 template <typename C, int V>
 __global__ void __launch_bounds__(256) k_norm2(sum_t<C>* __restrict__ npart, const C* __restrict__ x, long long n,
                                                int N) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     __shared__ sum_t<C> sh[256];
     const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -297,6 +301,7 @@ template <typename Cy, typename Cx_, int V>
 __global__ void __launch_bounds__(256) k_scale_norm(Cy* __restrict__ y, const Cx_* __restrict__ x,
                                                     const double* __restrict__ scale, bool inverse, long long n, int N,
                                                     sum_t<Cy>* __restrict__ npart) {
+    if (grid_dependency()) return;
     using R = re_t<Cy>;
     __shared__ sum_t<Cy> sh[256];
     __shared__ R sc[32 * V];
@@ -342,6 +347,7 @@ template <bool OF_X>
 __global__ void __launch_bounds__(256) k_refine_axpy(double2* __restrict__ y, const double* __restrict__ s, double sign,
                                                      const float2* __restrict__ x, long long n, int N, bool accumulate,
                                                      void* __restrict__ npart) {
+    if (grid_dependency()) return;
     __shared__ PairF shf[256];
     __shared__ SumD shd[256];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -387,6 +393,7 @@ __device__ __forceinline__ void atomic_max_double(u64* m, double v) {
 // norm_j = sqrt(sum of the partials), and with it what the caller's next kernels need (NormOut).
 template <typename S>
 __global__ void __launch_bounds__(256) k_finalize_norm(NormOut o, const S* __restrict__ part, int groups, int N) {
+    if (grid_dependency()) return;
     __shared__ S sh[256];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     S s;
@@ -424,6 +431,7 @@ __global__ void __launch_bounds__(256) k_finalize_norm(NormOut o, const S* __res
 template <typename C>
 __global__ void __launch_bounds__(256) k_scale_cols_if(C* __restrict__ w, const double* __restrict__ s, long long n,
                                                        int N) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
@@ -446,6 +454,7 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
                                                double2* __restrict__ g, double2* __restrict__ irr,
                                                const double* __restrict__ bnorm, u64* max, u64* clear, int j0, int j1,
                                                int m, int N) {
+    if (grid_dependency()) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (clear && r == 0) *clear = 0;
     if (r >= N) return;
@@ -504,6 +513,7 @@ template <typename C>
 __global__ void __launch_bounds__(32) k_back_substitute(C* __restrict__ cf, const double2* __restrict__ H,
                                                         const double2* __restrict__ g, const double2* __restrict__ irr,
                                                         const double* __restrict__ ieta, int j, int m, int N) {
+    if (grid_dependency()) return;
     const int r = blockIdx.x, l = threadIdx.x;
     double2 v[2], d[2], col[2], nxt[2];
     auto load = [&](int i, double2* c) {
@@ -567,20 +577,20 @@ void launch_multidot(C* cf, double2* H, const C* V, int m, const C* w, long long
         const C* Vk = V + (size_t)k0 * n * N;
         CSum<C>* pk = p + (size_t)k0 * N;
         if (W == 2 && mk_ <= 16) {
-            if (mk_ <= 4) k_multidot<C, 4, W2, 2><<<s2.g, s2.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
-            else if (mk_ <= 8) k_multidot<C, 8, W2, 1><<<s2.g, s2.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
-            else k_multidot<C, 16, W2, 1><<<s2.g, s2.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
+            if (mk_ <= 4) MG_LAUNCH(s2.g, s2.b, 0, s, (k_multidot<C, 4, W2, 2>), pk, Vk, mk_, m, w, n, N);
+            else if (mk_ <= 8) MG_LAUNCH(s2.g, s2.b, 0, s, (k_multidot<C, 8, W2, 1>), pk, Vk, mk_, m, w, n, N);
+            else MG_LAUNCH(s2.g, s2.b, 0, s, (k_multidot<C, 16, W2, 1>), pk, Vk, mk_, m, w, n, N);
         } else {
-            if (mk_ <= 4) k_multidot<C, 4, 1, 2><<<s1.g, s1.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
-            else if (mk_ <= 8) k_multidot<C, 8, 1, 1><<<s1.g, s1.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
-            else if (mk_ <= 16) k_multidot<C, 16, 1, 1><<<s1.g, s1.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
-            else k_multidot<C, 32, 1, 1><<<s1.g, s1.b, 0, s>>>(pk, Vk, mk_, m, w, n, N);
+            if (mk_ <= 4) MG_LAUNCH(s1.g, s1.b, 0, s, (k_multidot<C, 4, 1, 2>), pk, Vk, mk_, m, w, n, N);
+            else if (mk_ <= 8) MG_LAUNCH(s1.g, s1.b, 0, s, (k_multidot<C, 8, 1, 1>), pk, Vk, mk_, m, w, n, N);
+            else if (mk_ <= 16) MG_LAUNCH(s1.g, s1.b, 0, s, (k_multidot<C, 16, 1, 1>), pk, Vk, mk_, m, w, n, N);
+            else MG_LAUNCH(s1.g, s1.b, 0, s, (k_multidot<C, 32, 1, 1>), pk, Vk, mk_, m, w, n, N);
         }
         MG_LAUNCHED();
     }
     int bx = 1;
     while (bx < N && bx < 16) bx *= 2;
-    k_finalize_dots<C><<<dim3((N + bx - 1) / bx, m), dim3(bx, 128 / bx), 0, s>>>(cf, H, p, G, m, N, ieta, add);
+    MG_LAUNCH(dim3((N + bx - 1) / bx, m), dim3(bx, 128 / bx), 0, s, (k_finalize_dots<C>), cf, H, p, G, m, N, ieta, add);
     MG_LAUNCHED();
 }
 
@@ -588,8 +598,7 @@ template <typename C>
 static void launch_finalize_norm(const NormOut& o, const void* part, int groups, int N, cudaStream_t s) {
     int bx = 1;
     while (bx < N && bx < 8) bx *= 2;
-    k_finalize_norm<sum_t<C>><<<(N + bx - 1) / bx, dim3(bx, 256 / bx), 0, s>>>(
-        o, reinterpret_cast<const sum_t<C>*>(part), groups, N);
+    MG_LAUNCH((N + bx - 1) / bx, dim3(bx, 256 / bx), 0, s, (k_finalize_norm<sum_t<C>>), o, reinterpret_cast<const sum_t<C>*>(part), groups, N);
     MG_LAUNCHED();
 }
 
@@ -602,10 +611,10 @@ void launch_multiaxpy(C* w, const C* cf, int m, const C* V, long long n, int N, 
     const int G = axpy_groups(n, N);
     if (width<C>(N) == 2) {
         const Shape2 sh = shape(n, N, W2, G);
-        k_multiaxpy<C, W2><<<sh.g, sh.b, 0, s>>>(w, cf, m, V, n, N, accumulate, np, nscale);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_multiaxpy<C, W2>), w, cf, m, V, n, N, accumulate, np, nscale);
     } else {
         const Shape2 sh = shape(n, N, 1, G);
-        k_multiaxpy<C, 1><<<sh.g, sh.b, 0, s>>>(w, cf, m, V, n, N, accumulate, np, nscale);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_multiaxpy<C, 1>), w, cf, m, V, n, N, accumulate, np, nscale);
     }
     MG_LAUNCHED();
     if (norm) launch_finalize_norm<C>(*norm, np, G, N, s);
@@ -618,10 +627,10 @@ void launch_norm(const NormOut& o, const C* x, long long n, int N, void* part, c
     const int G = dot_groups(n, N);
     if (width<C>(N) == 2) {
         const Shape2 sh = shape(n, N, W2, G);
-        k_norm2<C, W2><<<sh.g, sh.b, 0, s>>>(np, x, n, N);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_norm2<C, W2>), np, x, n, N);
     } else {
         const Shape2 sh = shape(n, N, 1, G);
-        k_norm2<C, 1><<<sh.g, sh.b, 0, s>>>(np, x, n, N);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_norm2<C, 1>), np, x, n, N);
     }
     MG_LAUNCHED();
     launch_finalize_norm<C>(o, np, G, N, s);
@@ -635,10 +644,10 @@ void launch_scale_norm(const NormOut& o, Cy* y, const Cx_* x, const double* scal
     const int G = dot_groups(n, N);
     if (width<Cy>(N) == 2) {
         const Shape2 sh = shape(n, N, W2, G);
-        k_scale_norm<Cy, Cx_, W2><<<sh.g, sh.b, 0, s>>>(y, x, scale, inverse, n, N, np);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_norm<Cy, Cx_, W2>), y, x, scale, inverse, n, N, np);
     } else {
         const Shape2 sh = shape(n, N, 1, G);
-        k_scale_norm<Cy, Cx_, 1><<<sh.g, sh.b, 0, s>>>(y, x, scale, inverse, n, N, np);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_norm<Cy, Cx_, 1>), y, x, scale, inverse, n, N, np);
     }
     MG_LAUNCHED();
     launch_finalize_norm<Cy>(o, np, G, N, s);
@@ -649,11 +658,11 @@ void launch_refine_axpy(double2* y, const double* scale, double sign, const floa
     const int G = dot_groups(n, N);
     const Shape2 sh = shape(n, N, 1, G);
     if (of_y) {
-        k_refine_axpy<false><<<sh.g, sh.b, 0, s>>>(y, scale, sign, x, n, N, accumulate, part);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_refine_axpy<false>), y, scale, sign, x, n, N, accumulate, part);
         MG_LAUNCHED();
         launch_finalize_norm<double2>(*of_y, part, G, N, s);
     } else {
-        k_refine_axpy<true><<<sh.g, sh.b, 0, s>>>(y, scale, sign, x, n, N, accumulate, of_x ? part : nullptr);
+        MG_LAUNCH(sh.g, sh.b, 0, s, (k_refine_axpy<true>), y, scale, sign, x, n, N, accumulate, of_x ? part : nullptr);
         MG_LAUNCHED();
         if (of_x) launch_finalize_norm<float2>(*of_x, part, G, N, s);
     }
@@ -662,14 +671,14 @@ void launch_refine_axpy(double2* y, const double* scale, double sign, const floa
 template <typename C>
 void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_t s) {
     const Shape2 sh = shape(n, N, 1, groups_of(n, N, 1, 4));
-    k_scale_cols_if<C><<<sh.g, sh.b, 0, s>>>(w, f, n, N);
+    MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_cols_if<C>), w, f, n, N);
     MG_LAUNCHED();
 }
 
 void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,
                    const double* bnorm, unsigned long long* max, unsigned long long* clear, int j0, int j1, int m, int N,
                    cudaStream_t s) {
-    k_rotate<<<(N + 31) / 32, 32, 0, s>>>(H, hsub, cs, sn, g, irr, bnorm, max, clear, j0, j1, m, N);
+    MG_LAUNCH((N + 31) / 32, 32, 0, s, k_rotate, H, hsub, cs, sn, g, irr, bnorm, max, clear, j0, j1, m, N);
     MG_LAUNCHED();
 }
 
@@ -677,7 +686,7 @@ template <typename C>
 void launch_back_substitute(C* cf, const double2* H, const double2* g, const double2* irr, const double* ieta, int j,
                             int m, int N, cudaStream_t s) {
     MG_REQUIRE(j < 64, MGMLMC_EINVAL, "FGMRES restart length above 64");
-    k_back_substitute<C><<<N, 32, 0, s>>>(cf, H, g, irr, ieta, j, m, N);
+    MG_LAUNCH(N, 32, 0, s, (k_back_substitute<C>), cf, H, g, irr, ieta, j, m, N);
     MG_LAUNCHED();
 }
 

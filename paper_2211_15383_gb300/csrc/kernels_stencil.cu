@@ -30,6 +30,7 @@ template <typename C, int MODE>
 __global__ void __launch_bounds__(256) k_wilson(C* __restrict__ y, const C* __restrict__ x, const C* __restrict__ b,
                                                 const C* __restrict__ U, re_t<C> mass, int lx, int lt, int N,
                                                 double2* __restrict__ part) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     const int V = lx * lt;
@@ -109,6 +110,7 @@ template <typename C, int RPT, int MODE>
 __global__ void __launch_bounds__(256) k_block_stencil(C* __restrict__ y, const C* __restrict__ x,
                                                        const C* __restrict__ b, const C* __restrict__ A, int lx,
                                                        int lt, int d, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* As = reinterpret_cast<C*>(smem_raw);
@@ -179,6 +181,7 @@ template <typename C, int D, int MODE>
 __global__ void __launch_bounds__(128) k_block_stencil_d(C* __restrict__ y, const C* __restrict__ x,
                                                          const C* __restrict__ b, const C* __restrict__ A, int lx,
                                                          int lt, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     __shared__ C At[5 * D * D];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -237,6 +240,7 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(128) k_block_stencil_f2(float2* __restrict__ y, const float2* __restrict__ x,
                                                           const float2* __restrict__ b, const float2* __restrict__ A,
                                                           int lx, int lt, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     __shared__ float2 At[5 * D * D];
     // blockDim.x threads (32..128) x 2 rhs each: blocks of 64 rhs use one-warp CTAs
     const int j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -317,6 +321,7 @@ template <int MODE>
 __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y, const float2* __restrict__ x,
                                                           const float2* __restrict__ b, const float2* __restrict__ A,
                                                           int lx, int lt, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     constexpr int D = 16, H = 8;
     __shared__ float2 At[5 * D * D];
     __shared__ float red[MODE >= 2 ? 64 * 12 : 1];     // half 1's dots, T <= 64
@@ -428,6 +433,7 @@ template <typename C, int D, int MODE>
 __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ y, const C* __restrict__ x,
                                                                 const C* __restrict__ b, const C* __restrict__ A,
                                                                 int lx, int lt, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     using R = re_t<C>;
     __shared__ C As[5 * D * D];
     __shared__ double2 red[2][D][8];
@@ -487,6 +493,7 @@ __global__ void __launch_bounds__(128) k_block_diag_apply(C* __restrict__ y, con
                                                           int K, const C* __restrict__ alpha,
                                                           const C* __restrict__ Minv, int nsites, int d, int N,
                                                           bool accumulate) {
+    if (grid_dependency()) return;
     __shared__ C Ms[32 * 32];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     for (int site = blockIdx.y; site < nsites; site += gridDim.y) {
@@ -511,6 +518,7 @@ __global__ void __launch_bounds__(128) k_block_diag_apply_d(C* __restrict__ y, c
                                                             int K, const C* __restrict__ alpha,
                                                             const C* __restrict__ Minv, int nsites, int N,
                                                             bool accumulate) {
+    if (grid_dependency()) return;
     __shared__ C Ms[D * D];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     for (int site = blockIdx.y; site < nsites; site += gridDim.y) {
@@ -553,9 +561,9 @@ void launch_block_diag_combine(C* y, const C* x, size_t slot, int K, const C* al
     if (G > nsites) G = nsites;
     if (G < 1) G = 1;
     const dim3 g(tiles, G);
-    if (d == 16) k_block_diag_apply_d<C, 16><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, N, accumulate);
-    else if (d == 8) k_block_diag_apply_d<C, 8><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, N, accumulate);
-    else k_block_diag_apply<C><<<g, th, 0, s>>>(y, x, slot, K, alpha, Minv, nsites, d, N, accumulate);
+    if (d == 16) MG_LAUNCH(g, th, 0, s, (k_block_diag_apply_d<C, 16>), y, x, slot, K, alpha, Minv, nsites, N, accumulate);
+    else if (d == 8) MG_LAUNCH(g, th, 0, s, (k_block_diag_apply_d<C, 8>), y, x, slot, K, alpha, Minv, nsites, N, accumulate);
+    else MG_LAUNCH(g, th, 0, s, (k_block_diag_apply<C>), y, x, slot, K, alpha, Minv, nsites, d, N, accumulate);
     MG_LAUNCHED();
 }
 
@@ -569,6 +577,7 @@ void launch_block_diag_apply(C* y, const C* x, const C* Minv, int nsites, int d,
 template <typename C>
 __global__ void k_restrict(C* __restrict__ xc, const C* __restrict__ x, const C* __restrict__ P, int lx, int lt,
                            int d, int ax, int at, int nvec, int N) {
+    if (grid_dependency()) return;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
     const int cx = lx / ax, ct = lt / at, dc = 2 * nvec, hd = d / 2;
@@ -592,6 +601,7 @@ __global__ void k_restrict(C* __restrict__ xc, const C* __restrict__ x, const C*
 template <typename C>
 __global__ void k_prolong(C* __restrict__ x, const C* __restrict__ xc, const C* __restrict__ P, int lx, int lt,
                           int d, int ax, int at, int nvec, int N, bool accumulate) {
+    if (grid_dependency()) return;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
     const int cx = lx / ax, dc = 2 * nvec, hd = d / 2;
@@ -618,6 +628,7 @@ template <typename C, int NV>
 __global__ void __launch_bounds__(128) k_restrict_nv(C* __restrict__ xc, const C* __restrict__ x,
                                                      const C* __restrict__ P, int lx, int lt, int d, int ax, int at,
                                                      int N) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -661,6 +672,7 @@ template <typename C, int NV>
 __global__ void __launch_bounds__(128) k_prolong_nv(C* __restrict__ x, const C* __restrict__ xc,
                                                     const C* __restrict__ P, int lx, int lt, int d, int ax, int at,
                                                     int N, bool accumulate) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -716,6 +728,7 @@ __device__ __forceinline__ void store_bf16_row(uint8_t* xt, int site, int j, int
 template <typename C, int NV, int D, int QB>
 __global__ void __launch_bounds__(128) k_restrict_nvd(C* __restrict__ xc, const C* __restrict__ x,
                                                       const C* __restrict__ P, int lx, int lt, int ax, int at, int N) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     constexpr int HD = D / 2;
@@ -766,6 +779,7 @@ template <typename C, int NV, int D, int QB>
 __global__ void __launch_bounds__(128) k_prolong_nvd(C* __restrict__ x, const C* __restrict__ xc,
                                                      const C* __restrict__ P, int lx, int lt, int ax, int at, int N,
                                                      bool accumulate, uint8_t* __restrict__ xt) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     constexpr int HD = D / 2;
@@ -829,6 +843,7 @@ template <typename T, int V> struct alignas(sizeof(T) * V) VecOf { T v[V]; };
 template <typename C, int V>
 __global__ void __launch_bounds__(256) k_mr_update(C* rn, const C* r, const C* __restrict__ p,
                                                    const C* __restrict__ alpha, long long n, int N) {
+    if (grid_dependency()) return;
     const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
     C a[V];
@@ -862,6 +877,7 @@ constexpr int kMrGroup = 8;   // as in the solver's group loop
 template <typename C, int V>
 __global__ void __launch_bounds__(256) k_mr_combine(C* __restrict__ e, const C* __restrict__ rs, size_t slot, int K,
                                                     const C* __restrict__ alpha, long long n, int N, bool e_is_zero) {
+    if (grid_dependency()) return;
     const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
     for (long long i = (long long)blockIdx.y * blockDim.y + threadIdx.y; i < n;
@@ -889,6 +905,7 @@ __global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* __restric
                                                              const uint32_t* __restrict__ r,
                                                              const uint32_t* __restrict__ p,
                                                              const float2* __restrict__ alpha, long long n, int N) {
+    if (grid_dependency()) return;
     const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
     float2 a[4];
@@ -921,6 +938,7 @@ __global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* __restric
 __global__ void __launch_bounds__(256) k_mr_combine_bf16(float2* __restrict__ e, const uint32_t* __restrict__ rs,
                                                          size_t slot, int K, const float2* __restrict__ alpha,
                                                          long long n, int N, bool e_is_zero) {
+    if (grid_dependency()) return;
     const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
     for (long long i = (long long)blockIdx.y * blockDim.y + threadIdx.y; i < n;
@@ -950,6 +968,7 @@ __global__ void __launch_bounds__(256) k_mr_combine_bf16(float2* __restrict__ e,
 
 template <typename C>
 __global__ void k_gamma5(C* __restrict__ y, const C* __restrict__ x, long long rows, int d, int N) {
+    if (grid_dependency()) return;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
     for (long long i = (long long)blockIdx.y * kRowLanes + threadIdx.y; i < rows;
@@ -979,6 +998,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const float2* __restrict__ x,
                                                    const float2* __restrict__ b, const float2* __restrict__ U,
                                                    float mass, int lx, int lt, int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     const int j = 2 * (blockIdx.x * kRhsTile + threadIdx.x);
     const int V = lx * lt;
     float2 dyx[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -1095,10 +1115,10 @@ bool wilson_f2<float2>(float2* y, const float2* x, const float2* b, const float2
     if (N % 2) return false;
     dim3 g((N / 2 + kRhsTile - 1) / kRhsTile, groups);
     switch (mode) {
-        case 0: k_wilson_f2<0><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        case 1: k_wilson_f2<1><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        case 2: k_wilson_f2<2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        default: k_wilson_f2<3><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        case 0: MG_LAUNCH(g, blk(), 0, s, (k_wilson_f2<0>), y, x, b, U, mass, lx, lt, N, part); break;
+        case 1: MG_LAUNCH(g, blk(), 0, s, (k_wilson_f2<1>), y, x, b, U, mass, lx, lt, N, part); break;
+        case 2: MG_LAUNCH(g, blk(), 0, s, (k_wilson_f2<2>), y, x, b, U, mass, lx, lt, N, part); break;
+        default: MG_LAUNCH(g, blk(), 0, s, (k_wilson_f2<3>), y, x, b, U, mass, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
     return true;
@@ -1119,6 +1139,7 @@ template <int RPT, bool STORE>
 __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y, const uint32_t* __restrict__ x,
                                                         const float2* __restrict__ U, float mass, int lx, int lt,
                                                         int N, double2* __restrict__ part) {
+    if (grid_dependency()) return;
     const int j = RPT * (blockIdx.x * kRhsTile + threadIdx.x);
     const int V = lx * lt;
     float2 dyx[RPT];
@@ -1230,12 +1251,12 @@ void launch_wilson_bf16(uint32_t* y, const uint32_t* x, const float2* U, double 
     MG_REQUIRE(N % 4 == 0, MGMLMC_EINVAL, "BF16 Wilson operator: N a multiple of 4");
     if (N % 128 == 0) {
         dim3 g(N / 128, groups);
-        if (y) k_wilson_bf16<4, true><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
-        else k_wilson_bf16<4, false><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        if (y) MG_LAUNCH(g, blk(), 0, s, (k_wilson_bf16<4, true>), y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        else MG_LAUNCH(g, blk(), 0, s, (k_wilson_bf16<4, false>), y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
     } else {
         dim3 g((N / 2 + kRhsTile - 1) / kRhsTile, groups);
-        if (y) k_wilson_bf16<2, true><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
-        else k_wilson_bf16<2, false><<<g, blk(), 0, s>>>(y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        if (y) MG_LAUNCH(g, blk(), 0, s, (k_wilson_bf16<2, true>), y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
+        else MG_LAUNCH(g, blk(), 0, s, (k_wilson_bf16<2, false>), y, x, U, (float)(m0 + 2.0), lx, lt, N, part);
     }
     MG_LAUNCHED();
 }
@@ -1244,7 +1265,7 @@ void launch_wilson_residual_bf16(uint32_t* y, const float2* x, const float2* b, 
                                  int lt, int N, int groups, cudaStream_t s) {
     MG_REQUIRE(N % 2 == 0, MGMLMC_EINVAL, "BF16 Wilson residual: N even");
     dim3 g((N / 2 + kRhsTile - 1) / kRhsTile, groups);
-    k_wilson_f2<4><<<g, blk(), 0, s>>>(reinterpret_cast<float2*>(y), x, b, U, (float)(m0 + 2.0), lx, lt, N, nullptr);
+    MG_LAUNCH(g, blk(), 0, s, (k_wilson_f2<4>), reinterpret_cast<float2*>(y), x, b, U, (float)(m0 + 2.0), lx, lt, N, nullptr);
     MG_LAUNCHED();
 }
 
@@ -1256,10 +1277,10 @@ void launch_wilson(C* y, const C* x, const C* b, const C* U, double m0, int lx, 
     const R mass = (R)(m0 + 2.0);
     if (wilson_f2<C>(y, x, b, U, mass, lx, lt, N, mode, part, groups, s)) return;
     switch (mode) {
-        case 0: k_wilson<C, 0><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        case 1: k_wilson<C, 1><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        case 2: k_wilson<C, 2><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
-        default: k_wilson<C, 3><<<g, blk(), 0, s>>>(y, x, b, U, mass, lx, lt, N, part); break;
+        case 0: MG_LAUNCH(g, blk(), 0, s, (k_wilson<C, 0>), y, x, b, U, mass, lx, lt, N, part); break;
+        case 1: MG_LAUNCH(g, blk(), 0, s, (k_wilson<C, 1>), y, x, b, U, mass, lx, lt, N, part); break;
+        case 2: MG_LAUNCH(g, blk(), 0, s, (k_wilson<C, 2>), y, x, b, U, mass, lx, lt, N, part); break;
+        default: MG_LAUNCH(g, blk(), 0, s, (k_wilson<C, 3>), y, x, b, U, mass, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
 }
@@ -1278,10 +1299,10 @@ static void bs_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int lt
         MG_CUDA(cudaFuncSetAttribute(k_block_stencil<C, RPT, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     }
     switch (mode) {
-        case 0: k_block_stencil<C, RPT, 0><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
-        case 1: k_block_stencil<C, RPT, 1><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
-        case 2: k_block_stencil<C, RPT, 2><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
-        default: k_block_stencil<C, RPT, 3><<<g, blk(), sm, s>>>(y, x, b, A, lx, lt, d, N, part); break;
+        case 0: MG_LAUNCH(g, blk(), sm, s, (k_block_stencil<C, RPT, 0>), y, x, b, A, lx, lt, d, N, part); break;
+        case 1: MG_LAUNCH(g, blk(), sm, s, (k_block_stencil<C, RPT, 1>), y, x, b, A, lx, lt, d, N, part); break;
+        case 2: MG_LAUNCH(g, blk(), sm, s, (k_block_stencil<C, RPT, 2>), y, x, b, A, lx, lt, d, N, part); break;
+        default: MG_LAUNCH(g, blk(), sm, s, (k_block_stencil<C, RPT, 3>), y, x, b, A, lx, lt, d, N, part); break;
     }
     MG_LAUNCHED();
 }
@@ -1295,10 +1316,10 @@ static bool bsd_f2(float2* y, const float2* x, const float2* b, const float2* A,
         const int T = std::min(64, (N / 4 + 31) / 32 * 32);
         dim3 g((N / 4 + T - 1) / T, groups);
         switch (mode) {
-            case 0: k_block_stencil_f4<0><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-            case 1: k_block_stencil_f4<1><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-            case 2: k_block_stencil_f4<2><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-            default: k_block_stencil_f4<3><<<g, 2 * T, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+            case 0: MG_LAUNCH(g, 2 * T, 0, s, (k_block_stencil_f4<0>), y, x, b, A, lx, lt, N, part); break;
+            case 1: MG_LAUNCH(g, 2 * T, 0, s, (k_block_stencil_f4<1>), y, x, b, A, lx, lt, N, part); break;
+            case 2: MG_LAUNCH(g, 2 * T, 0, s, (k_block_stencil_f4<2>), y, x, b, A, lx, lt, N, part); break;
+            default: MG_LAUNCH(g, 2 * T, 0, s, (k_block_stencil_f4<3>), y, x, b, A, lx, lt, N, part); break;
         }
         MG_LAUNCHED();
         return true;
@@ -1306,10 +1327,10 @@ static bool bsd_f2(float2* y, const float2* x, const float2* b, const float2* A,
     const int threads = std::min(128, (N / 2 + 31) / 32 * 32);
     dim3 g((N / 2 + threads - 1) / threads, groups);
     switch (mode) {
-        case 0: k_block_stencil_f2<D, 0><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 1: k_block_stencil_f2<D, 1><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 2: k_block_stencil_f2<D, 2><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        default: k_block_stencil_f2<D, 3><<<g, threads, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 0: MG_LAUNCH(g, threads, 0, s, (k_block_stencil_f2<D, 0>), y, x, b, A, lx, lt, N, part); break;
+        case 1: MG_LAUNCH(g, threads, 0, s, (k_block_stencil_f2<D, 1>), y, x, b, A, lx, lt, N, part); break;
+        case 2: MG_LAUNCH(g, threads, 0, s, (k_block_stencil_f2<D, 2>), y, x, b, A, lx, lt, N, part); break;
+        default: MG_LAUNCH(g, threads, 0, s, (k_block_stencil_f2<D, 3>), y, x, b, A, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
     return true;
@@ -1327,10 +1348,10 @@ static void bsd_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int l
     const int th = cta_threads(N);
     dim3 g((N + th - 1) / th, groups);
     switch (mode) {
-        case 0: k_block_stencil_d<C, D, 0><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 1: k_block_stencil_d<C, D, 1><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 2: k_block_stencil_d<C, D, 2><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        default: k_block_stencil_d<C, D, 3><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 0: MG_LAUNCH(g, th, 0, s, (k_block_stencil_d<C, D, 0>), y, x, b, A, lx, lt, N, part); break;
+        case 1: MG_LAUNCH(g, th, 0, s, (k_block_stencil_d<C, D, 1>), y, x, b, A, lx, lt, N, part); break;
+        case 2: MG_LAUNCH(g, th, 0, s, (k_block_stencil_d<C, D, 2>), y, x, b, A, lx, lt, N, part); break;
+        default: MG_LAUNCH(g, th, 0, s, (k_block_stencil_d<C, D, 3>), y, x, b, A, lx, lt, N, part); break;
     }
     MG_LAUNCHED();
 }
@@ -1340,10 +1361,10 @@ static void bsn_dispatch(C* y, const C* x, const C* b, const C* A, int lx, int l
                          int groups, cudaStream_t s) {
     const dim3 g((N + 7) / 8, groups), th(8, D);
     switch (mode) {
-        case 0: k_block_stencil_narrow<C, D, 0><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 1: k_block_stencil_narrow<C, D, 1><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        case 2: k_block_stencil_narrow<C, D, 2><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
-        default: k_block_stencil_narrow<C, D, 3><<<g, th, 0, s>>>(y, x, b, A, lx, lt, N, part); break;
+        case 0: MG_LAUNCH(g, th, 0, s, (k_block_stencil_narrow<C, D, 0>), y, x, b, A, lx, lt, N, part); break;
+        case 1: MG_LAUNCH(g, th, 0, s, (k_block_stencil_narrow<C, D, 1>), y, x, b, A, lx, lt, N, part); break;
+        case 2: MG_LAUNCH(g, th, 0, s, (k_block_stencil_narrow<C, D, 2>), y, x, b, A, lx, lt, N, part); break;
+        default: MG_LAUNCH(g, th, 0, s, (k_block_stencil_narrow<C, D, 3>), y, x, b, A, lx, lt, N, part); break;
     }
 }
 
@@ -1396,21 +1417,21 @@ static void rp_launch(bool restrict_op, C* xc_or_x, const C* in, const C* P, int
     if (G < 1) G = 1;
     const size_t sm = (size_t)ax * at * d * NV * sizeof(C);
     if (d == 2) {
-        if (restrict_op) k_restrict_nvd<C, NV, 2, 4><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N);
-        else k_prolong_nvd<C, NV, 2, 4><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr);
+        if (restrict_op) MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nvd<C, NV, 2, 4>), xc_or_x, in, P, lx, lt, ax, at, N);
+        else MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nvd<C, NV, 2, 4>), xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr);
         MG_LAUNCHED();
         return;
     }
     if (d == 16) {
-        if (restrict_op) k_restrict_nvd<C, NV, 16, 1><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N);
-        else k_prolong_nvd<C, NV, 16, 1><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt);
+        if (restrict_op) MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nvd<C, NV, 16, 1>), xc_or_x, in, P, lx, lt, ax, at, N);
+        else MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nvd<C, NV, 16, 1>), xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt);
         MG_LAUNCHED();
         return;
     }
     if (restrict_op)
-        k_restrict_nv<C, NV><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, d, ax, at, N);
+        MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nv<C, NV>), xc_or_x, in, P, lx, lt, d, ax, at, N);
     else
-        k_prolong_nv<C, NV><<<dim3(tiles, G), th, sm, s>>>(xc_or_x, in, P, lx, lt, d, ax, at, N, accumulate);
+        MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nv<C, NV>), xc_or_x, in, P, lx, lt, d, ax, at, N, accumulate);
     MG_LAUNCHED();
 }
 
@@ -1432,7 +1453,7 @@ void launch_restrict(C* xc, const C* x, const C* P, int lx, int lt, int d, int a
     if (rp_fast<C>(true, xc, x, P, lx, lt, d, ax, at, nvec, N, false, nullptr, s)) return;
     const int ncs = (lx / ax) * (lt / at);
     int G = row_groups((long long)ncs * kRowLanes, N, 4);
-    k_restrict<C><<<dim3(rhs_tiles(N), G), blk(), 0, s>>>(xc, x, P, lx, lt, d, ax, at, nvec, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), G), blk(), 0, s, (k_restrict<C>), xc, x, P, lx, lt, d, ax, at, nvec, N);
     MG_LAUNCHED();
 }
 
@@ -1442,7 +1463,7 @@ bool launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax
     uint8_t* tiles = (sizeof(C) == 8 && d == 16) ? reinterpret_cast<uint8_t*>(xt) : nullptr;
     if (rp_fast<C>(false, x, xc, P, lx, lt, d, ax, at, nvec, N, accumulate, tiles, s)) return tiles != nullptr;
     const long long rows = (long long)lx * lt * d;
-    k_prolong<C><<<dim3(rhs_tiles(N), row_groups(rows, N)), blk(), 0, s>>>(x, xc, P, lx, lt, d, ax, at, nvec, N,
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(rows, N)), blk(), 0, s, (k_prolong<C>), x, xc, P, lx, lt, d, ax, at, nvec, N,
                                                                              accumulate);
     MG_LAUNCHED();
     return false;
@@ -1465,10 +1486,10 @@ void launch_mr_update(C* rn, const C* r, const C* p, const C* alpha, long long n
     dim3 g, b;
     if (sizeof(C) == 8 && N % 2 == 0) {
         row_shape(n, N, 2, 8, g, b);
-        k_mr_update<C, sizeof(C) == 8 ? 2 : 1><<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+        MG_LAUNCH(g, b, 0, s, (k_mr_update<C, sizeof(C) == 8 ? 2 : 1>), rn, r, p, alpha, n, N);
     } else {
         row_shape(n, N, 1, 8, g, b);
-        k_mr_update<C, 1><<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+        MG_LAUNCH(g, b, 0, s, (k_mr_update<C, 1>), rn, r, p, alpha, n, N);
     }
     MG_LAUNCHED();
 }
@@ -1480,10 +1501,10 @@ void launch_mr_combine(C* e, const C* rs, size_t slot, int K, const C* alpha, lo
     dim3 g, b;
     if (sizeof(C) == 8 && N % 2 == 0) {
         row_shape(n, N, 2, 8, g, b);
-        k_mr_combine<C, sizeof(C) == 8 ? 2 : 1><<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
+        MG_LAUNCH(g, b, 0, s, (k_mr_combine<C, sizeof(C) == 8 ? 2 : 1>), e, rs, slot, K, alpha, n, N, e_is_zero);
     } else {
         row_shape(n, N, 1, 8, g, b);
-        k_mr_combine<C, 1><<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
+        MG_LAUNCH(g, b, 0, s, (k_mr_combine<C, 1>), e, rs, slot, K, alpha, n, N, e_is_zero);
     }
     MG_LAUNCHED();
 }
@@ -1493,7 +1514,7 @@ void launch_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r, const uint32_t*
     MG_REQUIRE(N % 4 == 0, MGMLMC_EINVAL, "BF16 MR update: N a multiple of 4");
     dim3 g, b;
     row_shape(n, N, 4, 8, g, b);
-    k_mr_update_fine_bf16<<<g, b, 0, s>>>(rn, r, p, alpha, n, N);
+    MG_LAUNCH(g, b, 0, s, k_mr_update_fine_bf16, rn, r, p, alpha, n, N);
     MG_LAUNCHED();
 }
 
@@ -1502,14 +1523,14 @@ void launch_mr_combine_bf16(float2* e, const uint32_t* rs, size_t slot, int K, c
     MG_REQUIRE(N % 4 == 0 && K >= 1 && K <= kMrGroup, MGMLMC_EINVAL, "BF16 MR sum: N a multiple of 4, group size");
     dim3 g, b;
     row_shape(n, N, 4, 8, g, b);
-    k_mr_combine_bf16<<<g, b, 0, s>>>(e, rs, slot, K, alpha, n, N, e_is_zero);
+    MG_LAUNCH(g, b, 0, s, k_mr_combine_bf16, e, rs, slot, K, alpha, n, N, e_is_zero);
     MG_LAUNCHED();
 }
 
 template <typename C>
 void launch_gamma5(C* y, const C* x, long long nsites, int d, int N, cudaStream_t s) {
     const long long rows = nsites * d;
-    k_gamma5<C><<<dim3(rhs_tiles(N), row_groups(rows, N)), blk(), 0, s>>>(y, x, rows, d, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(rows, N)), blk(), 0, s, (k_gamma5<C>), y, x, rows, d, N);
     MG_LAUNCHED();
 }
 

@@ -47,6 +47,7 @@ template <int NT, int ST>
 __global__ void __launch_bounds__(128, 1)
     k_tc_gemm_bf16(float* __restrict__ Y, const __nv_bfloat16* __restrict__ At, const __nv_bfloat16* __restrict__ Bt,
                    int M, int K, int Ncols, int* __restrict__ err) {
+    if (grid_dependency()) return;
     constexpr int A_BYTES = BM * BK * 2;
     constexpr int B_BYTES = NT * BK * 2;
     constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(128, 1)
 
 // A' = [Re A | Im A] (n x 2n) written pre-tiled (128-row tiles).
 __global__ void k_embed_a(__nv_bfloat16* __restrict__ E, const float2* __restrict__ A, int n) {
+    if (grid_dependency()) return;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= (long long)n * n) return;
     const int i = (int)(e / n), k = (int)(e % n);
@@ -188,6 +190,7 @@ __global__ void k_embed_a(__nv_bfloat16* __restrict__ E, const float2* __restric
 //   k >= n: p = 0 -> -Im X[k-n][j],    p = 1 -> Re X[k-n][j]
 __global__ void k_pack_bt(__nv_bfloat16* __restrict__ Bt, const float2* __restrict__ X, int n, int N, int Ncols,
                           int NT) {
+    if (grid_dependency()) return;
     __shared__ float2 t[32][33];
     const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;   // rows of X, rhs
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -210,6 +213,7 @@ __global__ void k_pack_bt(__nv_bfloat16* __restrict__ Bt, const float2* __restri
 
 // Y[i][j] = sum over splits of Yp[z][i][c] (fixed order), complex output unpadded.
 __global__ void k_reduce_y(float2* __restrict__ Y, const float* __restrict__ Yp, int n, int N, int Ncols, int splits) {
+    if (grid_dependency()) return;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= (long long)n * N) return;
     const long long i = e / N, j = e % N;
@@ -226,7 +230,7 @@ __global__ void k_reduce_y(float2* __restrict__ Y, const float* __restrict__ Yp,
 
 void launch_embed_bf16(__nv_bfloat16* E, const float2* A, int n, cudaStream_t s) {
     const long long tot = (long long)n * n;
-    tc::k_embed_a<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(E, A, n);
+    MG_LAUNCH((unsigned)((tot + 255) / 256), 256, 0, s, tc::k_embed_a, E, A, n);
     MG_LAUNCHED();
 }
 
@@ -260,7 +264,7 @@ static void launch_tc_st(float* Y, const __nv_bfloat16* A, const __nv_bfloat16* 
     constexpr int smem = ST * (tc::BM * tc::BK * 2 + NT * tc::BK * 2);
     MG_CUDA(cudaFuncSetAttribute(tc::k_tc_gemm_bf16<NT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     dim3 g(Ncols / NT, M / tc::BM, splits);
-    tc::k_tc_gemm_bf16<NT, ST><<<g, 128, smem, s>>>(Y, A, Bt, M, K, Ncols, err);
+    MG_LAUNCH(g, 128, smem, s, (tc::k_tc_gemm_bf16<NT, ST>), Y, A, Bt, M, K, Ncols, err);
     MG_LAUNCHED();
 }
 
@@ -274,7 +278,7 @@ static void launch_tc(int NT, float* Y, const __nv_bfloat16* A, const __nv_bfloa
 
 static void launch_pack(__nv_bfloat16* Bt, const float2* X, int n, int N, int Ncols, int NT, cudaStream_t s) {
     dim3 g((Ncols / 2 + 31) / 32, (n + 31) / 32);
-    tc::k_pack_bt<<<g, dim3(32, 8), 0, s>>>(Bt, X, n, N, Ncols, NT);
+    MG_LAUNCH(g, dim3(32, 8), 0, s, tc::k_pack_bt, Bt, X, n, N, Ncols, NT);
     MG_LAUNCHED();
 }
 
@@ -291,7 +295,7 @@ void launch_coarse_inverse_bf16(float2* Y, const float2* X, const __nv_bfloat16*
     launch_tc(NT, direct ? reinterpret_cast<float*>(Y) : Yp, E, Bt, n, 2 * n, Ncols, S, err, s);
     if (!direct) {
         const long long tot = (long long)n * N;
-        tc::k_reduce_y<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(Y, Yp, n, N, Ncols, S);
+        MG_LAUNCH((unsigned)((tot + 255) / 256), 256, 0, s, tc::k_reduce_y, Y, Yp, n, N, Ncols, S);
         MG_LAUNCHED();
     }
 }
@@ -315,6 +319,7 @@ namespace tc {
 // 3k + m: -Im L; rows >= 4k zero.  Rounding: FP64 -> FP32 -> BF16, both to nearest.
 __global__ void k_embed_defl(__nv_bfloat16* __restrict__ W, const double2* __restrict__ R,
                              const double2* __restrict__ L, int n, int k, int Mpad) {
+    if (grid_dependency()) return;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= (long long)n * Mpad) return;
     const int i = (int)(e / Mpad), m = (int)(e % Mpad);
@@ -330,6 +335,7 @@ __global__ void k_embed_defl(__nv_bfloat16* __restrict__ W, const double2* __res
 // X^T pre-tiled in NT-row tiles (row j = rhs, K = n): the real part of X, zero for j >= N.
 __global__ void k_pack_x_real(__nv_bfloat16* __restrict__ Bt, const double2* __restrict__ X, int n, int N, int Ncols,
                               int NT) {
+    if (grid_dependency()) return;
     __shared__ float t[32][33];
     const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -351,6 +357,7 @@ __device__ __forceinline__ double2 bf16_round(double2 z) {
 // t[m] = R~_m^H L~_m in FP64 over the BF16-rounded factors (one CTA per m, fixed tree).
 __global__ void k_defl_tau(double2* __restrict__ t, const double2* __restrict__ R, const double2* __restrict__ L,
                            int n, int k) {
+    if (grid_dependency()) return;
     __shared__ double sr[256], si[256];
     const int m = blockIdx.x;
     double re = 0, im = 0;
@@ -376,6 +383,7 @@ __global__ void k_defl_tau(double2* __restrict__ t, const double2* __restrict__ 
 // CTA per rhs, fixed order over splits and a fixed reduction tree over m).
 __global__ void k_defl_correction_tc(double2* __restrict__ smp, const float* __restrict__ Yp,
                                      const double* __restrict__ a, int k, int Mpad, int Ncols, int splits) {
+    if (grid_dependency()) return;
     __shared__ double sr[256], si[256];
     const int j = blockIdx.x;
     const size_t slab = (size_t)Mpad * Ncols;
@@ -415,12 +423,12 @@ void launch_embed_deflation_bf16(__nv_bfloat16* W, const double2* R, const doubl
     MG_REQUIRE(tc_deflation_supported(n, k), MGMLMC_EINVAL, "tensor-core deflation needs n % 64 == 0");
     const int Mpad = tc_deflation_rows(k);
     const long long tot = n * Mpad;
-    tc::k_embed_defl<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(W, R, L, (int)n, k, Mpad);
+    MG_LAUNCH((unsigned)((tot + 255) / 256), 256, 0, s, tc::k_embed_defl, W, R, L, (int)n, k, Mpad);
     MG_LAUNCHED();
 }
 
 void launch_deflation_tau_bf16(double2* t, const double2* R, const double2* L, long long n, int k, cudaStream_t s) {
-    tc::k_defl_tau<<<k, 256, 0, s>>>(t, R, L, (int)n, k);
+    MG_LAUNCH(k, 256, 0, s, tc::k_defl_tau, t, R, L, (int)n, k);
     MG_LAUNCHED();
 }
 
@@ -455,10 +463,10 @@ void launch_deflation_correction_bf16(double2* smp, const double2* X, const __nv
     __nv_bfloat16* Bt = reinterpret_cast<__nv_bfloat16*>(scratch);
     float* Yp = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(scratch) + (size_t)Ncols * n * 2);
     dim3 g((Ncols + 31) / 32, (unsigned)((n + 31) / 32));
-    tc::k_pack_x_real<<<g, dim3(32, 8), 0, s>>>(Bt, X, (int)n, N, Ncols, NT);
+    MG_LAUNCH(g, dim3(32, 8), 0, s, tc::k_pack_x_real, Bt, X, (int)n, N, Ncols, NT);
     MG_LAUNCHED();
     launch_tc(NT, Yp, W, Bt, Mpad, (int)n, Ncols, S, err, s);
-    tc::k_defl_correction_tc<<<N, 256, 0, s>>>(smp, Yp, a, k, Mpad, Ncols, S);
+    MG_LAUNCH(N, 256, 0, s, tc::k_defl_correction_tc, smp, Yp, a, k, Mpad, Ncols, S);
     MG_LAUNCHED();
 }
 
@@ -519,6 +527,7 @@ __device__ __forceinline__ int dir_of(int o) { return o == 4 ? 0 : o + 1; }
 // B(s, dir) for every site: E[(s * 5 + dir) * 1024 + off / 2], element (n = output
 // real, k = input real) of the real form of A(s, dir)^T.
 __global__ void k_embed_stencil(__nv_bfloat16* __restrict__ E, const float2* __restrict__ A, int nsites) {
+    if (grid_dependency()) return;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= (long long)nsites * 5 * KD * KD) return;
     const long long sd = e / (KD * KD);
@@ -534,6 +543,7 @@ __global__ void k_embed_stencil(__nv_bfloat16* __restrict__ E, const float2* __r
 // Thread = (site, component group of 4, rhs): four FP32 loads, one 16-byte store.
 // Grid: x = (site, component group), y = 128-rhs tile.
 __global__ void k_pack_tiles(__nv_bfloat16* __restrict__ rt, const float2* __restrict__ x, int nsites, int N) {
+    if (grid_dependency()) return;
     const int T = gridDim.y, tt = blockIdx.y;
     const int j = tt * CH + threadIdx.x;
     const int site = blockIdx.x >> 2, cg = blockIdx.x & 3;
@@ -557,6 +567,7 @@ __global__ void k_pack_tiles(__nv_bfloat16* __restrict__ rt, const float2* __res
 __global__ void __launch_bounds__(CH) k_mr_update_tc(float2* __restrict__ yh, float2* __restrict__ r,
                                                     const float2* __restrict__ p, const float2* __restrict__ alpha,
                                                     int N, bool first, __nv_bfloat16* __restrict__ rt) {
+    if (grid_dependency()) return;
     const int T = gridDim.y, tt = blockIdx.y;     // grid: x = site, y = 128-rhs tile
     const int j = tt * CH + threadIdx.x;
     const int site = blockIdx.x;
@@ -609,6 +620,7 @@ __global__ void __launch_bounds__(CH) k_mr_update_tc(float2* __restrict__ yh, fl
 __global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* __restrict__ rn, const uint4* __restrict__ r,
                                                          const uint4* __restrict__ p,
                                                          const float2* __restrict__ alpha, int nsites, int N, int T) {
+    if (grid_dependency()) return;
     constexpr int U = 4;
     const int lane = threadIdx.x & 31;
     const int G8 = (N + 7) >> 3;                  // row groups of a site
@@ -651,6 +663,7 @@ __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e,
                                                          size_t slot, int K, const float2* __restrict__ alpha,
                                                          const float2* __restrict__ Minv, int nsites, int N, int T,
                                                          bool accumulate) {
+    if (grid_dependency()) return;
     __shared__ float2 Ms[D * D];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     for (int site = blockIdx.y; site < nsites; site += gridDim.y) {
@@ -699,6 +712,7 @@ __global__ void __launch_bounds__(THREADS, kCtasPerSm)
     k_block_stencil_tc(float2* __restrict__ y, __nv_bfloat16* __restrict__ yt, const float2* __restrict__ b,
                        const __nv_bfloat16* __restrict__ xt, const __nv_bfloat16* __restrict__ E, int lx, int lt, int N,
                        double2* __restrict__ part, int* __restrict__ err) {
+    if (grid_dependency()) return;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[NSTG], empty[NSTG], afull[2], aempty[2];
     __shared__ uint32_t tmem_holder;
@@ -884,7 +898,7 @@ bool tc_stencil_supported(int d, int N) { return d == tc::tcs::D && N >= 1 && N 
 
 void launch_embed_stencil_bf16(__nv_bfloat16* E, const float2* A, int nsites, cudaStream_t s) {
     const long long tot = (long long)nsites * 5 * tc::tcs::KD * tc::tcs::KD;
-    tc::tcs::k_embed_stencil<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(E, A, nsites);
+    MG_LAUNCH((unsigned)((tot + 255) / 256), 256, 0, s, tc::tcs::k_embed_stencil, E, A, nsites);
     MG_LAUNCHED();
 }
 
@@ -894,14 +908,14 @@ size_t tc_tiles_bytes(int nsites, int N) { return (size_t)nsites * tc_tiles(N) *
 
 void launch_pack_tiles_bf16(__nv_bfloat16* rt, const float2* x, int nsites, int N, cudaStream_t s) {
     MG_REQUIRE(nsites >= 1 && nsites <= (1 << 28) && tc_tiles(N) <= 65535, MGMLMC_EINVAL, "BF16 tiles: size");
-    tc::tcs::k_pack_tiles<<<dim3(4 * nsites, tc_tiles(N)), tc::tcs::CH, 0, s>>>(rt, x, nsites, N);
+    MG_LAUNCH(dim3(4 * nsites, tc_tiles(N)), tc::tcs::CH, 0, s, tc::tcs::k_pack_tiles, rt, x, nsites, N);
     MG_LAUNCHED();
 }
 
 void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const float2* alpha, int nsites, int N, bool first,
                          __nv_bfloat16* rt, cudaStream_t s) {
     MG_REQUIRE(nsites >= 1 && nsites <= (1 << 30) && tc_tiles(N) <= 65535, MGMLMC_EINVAL, "BF16 tiles: size");
-    tc::tcs::k_mr_update_tc<<<dim3(nsites, tc_tiles(N)), tc::tcs::CH, 0, s>>>(yh, r, p, alpha, N, first, rt);
+    MG_LAUNCH(dim3(nsites, tc_tiles(N)), tc::tcs::CH, 0, s, tc::tcs::k_mr_update_tc, yh, r, p, alpha, N, first, rt);
     MG_LAUNCHED();
 }
 
@@ -919,7 +933,7 @@ static void bstc_launch(float2* y, __nv_bfloat16* yt, const float2* b, const __n
     MG_CUDA(cudaFuncSetAttribute(tc::tcs::k_block_stencil_tc<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::tcs::SMEM));
     dim3 g(groups, tc_tiles(N));
-    tc::tcs::k_block_stencil_tc<FORM><<<g, tc::tcs::THREADS, tc::tcs::SMEM, s>>>(y, yt, b, xt, E, lx, lt, N, part, err);
+    MG_LAUNCH(g, tc::tcs::THREADS, tc::tcs::SMEM, s, (tc::tcs::k_block_stencil_tc<FORM>), y, yt, b, xt, E, lx, lt, N, part, err);
     MG_LAUNCHED();
 }
 
@@ -943,7 +957,7 @@ void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __n
     const long long chunks = (long long)nsites * ((N + 7) / 8);
     const long long need = (chunks + 31) / 32;    // 8 warps x 4 chunks per CTA
     const int g = (int)(need < 6LL * kNumSM ? need : 6LL * kNumSM);
-    tc::tcs::k_mr_update_tiles<<<g, 256, 0, s>>>(reinterpret_cast<uint4*>(rn), reinterpret_cast<const uint4*>(r),
+    MG_LAUNCH(g, 256, 0, s, tc::tcs::k_mr_update_tiles, reinterpret_cast<uint4*>(rn), reinterpret_cast<const uint4*>(r),
                                                  reinterpret_cast<const uint4*>(p), alpha, nsites, N, tc_tiles(N));
     MG_LAUNCHED();
 }
@@ -955,7 +969,7 @@ void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const fl
     int G = 16 * kNumSM / tiles;
     if (G > nsites) G = nsites;
     if (G < 1) G = 1;
-    tc::tcs::k_block_diag_tiles<<<dim3(tiles, G), th, 0, s>>>(e, reinterpret_cast<const uint8_t*>(rt),
+    MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles, e, reinterpret_cast<const uint8_t*>(rt),
                                                               tc_tiles_bytes(nsites, N), K, alpha, Minv, nsites, N,
                                                               tc_tiles(N), accumulate);
     MG_LAUNCHED();

@@ -17,6 +17,7 @@ __device__ __forceinline__ uint64_t sm64(uint64_t z) {
 
 template <typename C>
 __global__ void k_noise(C* __restrict__ x, long long n, int N, uint64_t seed, uint64_t term, int64_t first) {
+    if (grid_dependency()) return;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
     const uint64_t ks = sm64(sm64(seed ^ term) ^ (uint64_t)(first + j));
@@ -32,6 +33,7 @@ __global__ void k_noise(C* __restrict__ x, long long n, int N, uint64_t seed, ui
 
 template <typename C>
 __global__ void k_probes(C* __restrict__ x, const int8_t* __restrict__ p, long long n, int N) {
+    if (grid_dependency()) return;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
     for (long long i = (long long)blockIdx.y * kRowLanes + threadIdx.y; i < n;
@@ -45,6 +47,7 @@ __global__ void k_probes(C* __restrict__ x, const int8_t* __restrict__ p, long l
 
 template <typename Cout, typename Cin>
 __global__ void k_convert(Cout* __restrict__ y, const Cin* __restrict__ x, long long count) {
+    if (grid_dependency()) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x)
         y[i] = cvtc(x[i], Cout());
@@ -52,6 +55,7 @@ __global__ void k_convert(Cout* __restrict__ y, const Cin* __restrict__ x, long 
 
 template <typename C>
 __global__ void k_zero(C* __restrict__ x, long long count) {
+    if (grid_dependency()) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x)
         x[i] = czero<C>();
@@ -60,6 +64,7 @@ __global__ void k_zero(C* __restrict__ x, long long count) {
 template <typename Cy, typename Cx_>
 __global__ void k_scale_rhs(Cy* __restrict__ y, const Cx_* __restrict__ x, const double* __restrict__ scale,
                             bool invert, long long n, int N) {
+    if (grid_dependency()) return;
     using R = re_t<Cy>;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
@@ -76,6 +81,7 @@ __global__ void k_scale_rhs(Cy* __restrict__ y, const Cx_* __restrict__ x, const
 template <typename Cy, typename Cx_>
 __global__ void k_axpy_rhs(Cy* __restrict__ y, const double2* __restrict__ alpha, const double* __restrict__ beta,
                            double sign, const Cx_* __restrict__ x, long long n, int N) {
+    if (grid_dependency()) return;
     using R = re_t<Cy>;
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
     if (j >= N) return;
@@ -94,6 +100,7 @@ __global__ void k_axpy_rhs(Cy* __restrict__ y, const double2* __restrict__ alpha
 template <typename Cx_, typename Cy>
 __global__ void k_dot(double2* __restrict__ part, const Cx_* __restrict__ x, const Cy* __restrict__ y,
                       long long n, int N) {
+    if (grid_dependency()) return;
     using R = re_t<Cx_>;
     __shared__ double2 sh[kRowLanes][kRhsTile + 1];
     const int j = blockIdx.x * kRhsTile + threadIdx.x;
@@ -119,6 +126,7 @@ __global__ void k_dot(double2* __restrict__ part, const Cx_* __restrict__ x, con
 // block: 10 us for 608 groups).
 __global__ void __launch_bounds__(256) k_finalize(double2* __restrict__ out, const double2* __restrict__ part,
                                                   int groups, int count) {
+    if (grid_dependency()) return;
     __shared__ double2 sh[32][9];
     const int j = blockIdx.x * 8 + threadIdx.x;
     double2 acc = make_double2(0.0, 0.0);
@@ -140,12 +148,12 @@ static inline dim3 blk() { return dim3(kRhsTile, kRowLanes); }
 
 template <typename C>
 void launch_noise(C* x, long long n, int N, uint64_t seed, uint64_t term, int64_t first, cudaStream_t s) {
-    k_noise<C><<<dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s>>>(x, n, N, seed, term, first);
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, (k_noise<C>), x, n, N, seed, term, first);
     MG_LAUNCHED();
 }
 template <typename C>
 void launch_probes(C* x, const int8_t* p, long long n, int N, cudaStream_t s) {
-    k_probes<C><<<dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s>>>(x, p, n, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, (k_probes<C>), x, p, n, N);
     MG_LAUNCHED();
 }
 template <typename Cout, typename Cin>
@@ -153,7 +161,7 @@ void launch_convert(Cout* y, const Cin* x, long long count, cudaStream_t s) {
     if (count <= 0) return;
     long long b = (count + 255) / 256;
     if (b > kNumSM * 16) b = kNumSM * 16;
-    k_convert<Cout, Cin><<<(int)b, 256, 0, s>>>(y, x, count);
+    MG_LAUNCH((int)b, 256, 0, s, (k_convert<Cout, Cin>), y, x, count);
     MG_LAUNCHED();
 }
 template <typename C>
@@ -161,18 +169,18 @@ void launch_zero(C* x, long long count, cudaStream_t s) {
     if (count <= 0) return;
     long long b = (count + 255) / 256;
     if (b > kNumSM * 16) b = kNumSM * 16;
-    k_zero<C><<<(int)b, 256, 0, s>>>(x, count);
+    MG_LAUNCH((int)b, 256, 0, s, (k_zero<C>), x, count);
     MG_LAUNCHED();
 }
 template <typename Cy, typename Cx_>
 void launch_scale_rhs(Cy* y, const Cx_* x, const double* scale, bool invert, long long n, int N, cudaStream_t s) {
-    k_scale_rhs<Cy, Cx_><<<dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s>>>(y, x, scale, invert, n, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, (k_scale_rhs<Cy, Cx_>), y, x, scale, invert, n, N);
     MG_LAUNCHED();
 }
 template <typename Cy, typename Cx_>
 void launch_axpy_rhs(Cy* y, const double2* alpha, const double* beta, double sign, const Cx_* x, long long n, int N,
                      cudaStream_t s) {
-    k_axpy_rhs<Cy, Cx_><<<dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s>>>(y, alpha, beta, sign, x, n, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, (k_axpy_rhs<Cy, Cx_>), y, alpha, beta, sign, x, n, N);
     MG_LAUNCHED();
 }
 
@@ -185,6 +193,7 @@ int reduce_groups(long long n, int N) { return row_groups(n, N, 4); }
 template <typename C>
 __global__ void __launch_bounds__(128) k_finalize_alpha(C* __restrict__ alpha, const double2* __restrict__ part,
                                                         int groups, int N) {
+    if (grid_dependency()) return;
     __shared__ double sh[3][4];
     const int j = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double2* r0 = part + (long long)j * groups;
@@ -215,21 +224,21 @@ __global__ void __launch_bounds__(128) k_finalize_alpha(C* __restrict__ alpha, c
 
 template <typename C>
 void launch_finalize_alpha(C* alpha, const double2* part, int groups, int N, cudaStream_t s) {
-    k_finalize_alpha<C><<<N, 128, 0, s>>>(alpha, part, groups, N);
+    MG_LAUNCH(N, 128, 0, s, (k_finalize_alpha<C>), alpha, part, groups, N);
     MG_LAUNCHED();
 }
 template void launch_finalize_alpha<double2>(double2*, const double2*, int, int, cudaStream_t);
 template void launch_finalize_alpha<float2>(float2*, const double2*, int, int, cudaStream_t);
 
 void launch_finalize(double2* out, const double2* part, int groups, int count, cudaStream_t s) {
-    k_finalize<<<(count + 7) / 8, dim3(8, 32), 0, s>>>(out, part, groups, count);
+    MG_LAUNCH((count + 7) / 8, dim3(8, 32), 0, s, k_finalize, out, part, groups, count);
     MG_LAUNCHED();
 }
 
 template <typename Cx_, typename Cy>
 void launch_dot(double2* out, const Cx_* x, const Cy* y, long long n, int N, double2* part, cudaStream_t s) {
     const int G = reduce_groups(n, N);
-    k_dot<Cx_, Cy><<<dim3(rhs_tiles(N), G), blk(), 0, s>>>(part, x, y, n, N);
+    MG_LAUNCH(dim3(rhs_tiles(N), G), blk(), 0, s, (k_dot<Cx_, Cy>), part, x, y, n, N);
     MG_LAUNCHED();
     launch_finalize(out, part, G, N, s);
 }
@@ -259,6 +268,7 @@ template void launch_dot<float2, float2>(double2*, const float2*, const float2*,
 namespace mg {
 // out[c][r] = in[r][c] for a rows x cols complex matrix (32 x 32 tiles).
 __global__ void k_transpose(double2* __restrict__ out, const double2* __restrict__ in, long long rows, int cols) {
+    if (grid_dependency()) return;
     __shared__ double2 t[32][33];
     const int c0 = blockIdx.x * 32;
     const long long nrb = (rows + 31) / 32;
@@ -281,7 +291,7 @@ __global__ void k_transpose(double2* __restrict__ out, const double2* __restrict
 void launch_transpose(double2* out, const double2* in, long long rows, int cols, cudaStream_t s) {
     const long long nrb = (rows + 31) / 32;
     dim3 g((cols + 31) / 32, (unsigned)(nrb < 65535 ? nrb : 65535));
-    k_transpose<<<g, dim3(32, 8), 0, s>>>(out, in, rows, cols);
+    MG_LAUNCH(g, dim3(32, 8), 0, s, k_transpose, out, in, rows, cols);
     MG_LAUNCHED();
 }
 }  // namespace mg
