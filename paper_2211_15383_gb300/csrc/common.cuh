@@ -47,17 +47,20 @@ std::atomic<long long>& launch_counter();   // all contexts, thread-safe
     } while (0)
 
 // ---- programmatic dependent launch
-// Kernels of the solver's chain are launched so that a kernel may be set up while the one
-// before it in the stream still runs: without it each launch starts about 2 us after the end
-// of its predecessor, as long as many of these kernels run.  Every kernel launched by
-// MG_LAUNCH begins with `if (grid_dependency()) return;`: it waits until the kernels before it
-// have completed and their writes are visible (so a chain orders as plain launches do), then
-// lets the next one be set up.  The result is always false; the branch on it keeps the
-// compiler from moving reads through const __restrict__ pointers, which it takes for
-// invariant, above the wait.
+// Kernels of the solver's chain are launched so that a kernel is set up while the one before
+// it in the stream still runs: without it each launch starts about 2 us after the end of its
+// predecessor, as long as many of these kernels run.  Every kernel launched by MG_LAUNCH begins
+// with `if (grid_dependency()) return;`: it waits until the kernels before it have completed
+// and their writes are visible, so a chain orders as plain launches do.  No kernel lets its
+// successor's CTAs in early (griddepcontrol.launch_dependents): they took the places of the
+// CTAs that finished first, which left the grids sized to one even wave unevenly spread
+// (512^2 step: 273 ms with it, 263 without dependent launches, 252 as it is; pilot draw at
+// 64^2: 8.6, 12.0, 8.1).  The result is always false; the branch on it keeps the compiler from
+// moving reads through const __restrict__ pointers, which it takes for invariant, above the
+// wait.
 __device__ __forceinline__ bool grid_dependency() {
     int z;
-    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n mov.u32 %0, 0;" : "=r"(z)::"memory");
+    asm volatile("griddepcontrol.wait;\n mov.u32 %0, 0;" : "=r"(z)::"memory");
     return z != 0;
 }
 
