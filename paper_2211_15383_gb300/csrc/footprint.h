@@ -60,7 +60,7 @@ inline size_t footprint_bytes(const Shape& s) {
             if (bf16) b += st * d * d * 80;                                  // BF16 operand tiles
         }
         const bool digits = l > 0 && s.d[l] == 16;                           // FP64 products on the tensor cores
-        if (digits) b += st * 5 * 16384 * (f64 && l + 1 < L ? 2 : 1) + st * std::ceil(N / 128) * 57344;
+        if (digits) b += st * 5 * 16384 * (f64 && l + 1 < L ? 2 : 1) + st * std::ceil(N / 128) * 65536;
         if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * (digits ? std::min(N, 16.0) : N) * 16;   // FP64 Galerkin apply
         if (l + 1 < L) {
             const double K = smoother_slots(s.nu);
@@ -76,7 +76,7 @@ inline size_t footprint_bytes(const Shape& s) {
     b += 2.0 * n0 * nvmax * 16;                                              // setup blocks
     b += nL * nL * 44 + nL * N * 136;                                        // dense coarsest inverse, BF16 solve
     if (f64 && f64_dense_inverse(s.n[L - 1]))                                // its digits; x digits, partial sums
-        b += nL * nL * 64 + nL / 16 * std::ceil(N / 128) * 57344 + std::ceil(nL / 96) * nL * N * 16;
+        b += nL * nL * 64 + nL / 16 * std::ceil(N / 128) * 65536 + std::ceil(nL / 96) * nL * N * 16;
     b += (2 * m + 1) * n0 * (N * sz + nvmax * 16);                           // FGMRES bases
     b += G * (m + 1) * N * 16 + N * (m + 1) * (m + 4) * 16;                  // Gram-Schmidt partials, Hessenberg
     b += n0 * N * 56;                                                        // refinement blocks

@@ -6,31 +6,35 @@
 // T. Ogita, S. Oishi, S. M. Rump, "Error-free transformations of matrix multiplication by
 // using fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
 //
-//  * every rhs of x is scaled by a power of two 2^-ex with |x| < 2^ex (its largest entry) and
-//    rounded to 55 bits, x = 2^ex sum_{j<7} d_j 2^{-6-8j}; the matrix by one power of two,
-//    63 bits, a = 2^ea sum_{i<8} c_i 2^{-6-8i}; all digits are integers in [-128, 127], exact
-//    in BF16.  So x moves by at most 2^-55 of its column's largest entry (FP64 itself keeps
-//    2^-53 of an entry) and a by 2^-63;
-//  * G_g = sum_{i+j=g} sum_k c_i d_j for g = 0..7: products of digits are below 2^14, sums of
+//  * every rhs of x is scaled by a power of two 2^-ex with |x| < 2^ex (its largest entry), the
+//    matrix by one power of two, and both are rounded to 63 bits, x = 2^ex sum_{j<8} d_j 2^{-6-8j},
+//    a = 2^ea sum_{i<8} c_i 2^{-6-8i}; all digits are integers in [-128, 127], exact in BF16;
+//  * G_g = sum_{i+j=g} sum_k c_i d_j for g = 0..8: products of digits are below 2^14, sums of
 //    at most 192 k and 5 pairs below 2^24, so the FP32 accumulation in TMEM is exact for the
 //    groups g <= 4 (the others weigh at most 2^-40, and their sums can only leave the
-//    exact range by rounding their last place); the dropped pairs i + j > 7 weigh 2^-64;
+//    exact range by rounding their last place); the dropped pairs i + j > 8 weigh 2^-72;
 //  * sum_g G_g 2^-8g is formed in 128-bit integers and rounded to FP64 once.
-// A product of 160 terms is then closer to the exact one than 160 FP64 FMAs are.
+// The error of an entry is 2^-53 of itself from that rounding, and about 2^-63 of the rhs' largest
+// entry; 160 FP64 FMAs leave about 2^-51 of the entries around it.  In the norm the product is
+// closer to the exact one also where a rhs is concentrated on a few sites of the lattice (the
+// second part is spread over n entries: it stays below as long as n < 2^21 of the sites the rhs
+// is concentrated on).  With 7 digits of x and 8 groups (2^-55) that was not so: residuals
+// of near-critical 1024^2 solves, dominated by localised modes, stood at 1.9e-12.
 //
 // Layout: the rhs are the MMA's M (128 rows of x digits, K = 32 reals of a site), the digits
 // of the block are its N: the 8 x 32 rows (i, output real) of a block's tile lie one after
-// another, so digit slice j of x times rows 0 .. 255 - 32j lands on the columns 32j .. 255,
-// which is exactly where G_{i+j} belongs: 7 MMAs (N = 256, 224, ..., 64) per K step, 1120
-// columns for the 35 pairs.  A job is one block of 16 output rows for 128 rhs (5 blocks of
-// the stencil, or up to 6 of a row of the dense matrix); x digits (56 KB) and block digits
-// (16 KB) of each K block move by bulk copies through a 3-stage ring, two 256-column
-// accumulators alternate, eight epilogue warps turn them into FP64.  One CTA per SM (216 KB).
-// Bound: L2 and HBM reads of the digit tiles (72 KB per K block; the MMAs of a stencil job
-// are 5600 cycles, a job takes about 16000).  Measured: D_3 x at 32^2 sites x 512 rhs
-// 4329 -> 217 us, D_2 x at 128^2 sites x 128 rhs (then by P^H D_1 P) 9.4 -> 0.9 ms, the
-// inverse of 1024 unknowns times 64 rhs 2205 -> 33 us; the two passes that scale and slice
-// x move 30 B per real more.
+// another, so digit slice j of x times the first rows of the tile lands on the columns from
+// 32j on, which is exactly where G_{i+j} belongs: 8 MMAs (N = 256, 256, 224, ..., 64) per K
+// step, 1376 columns for the 43 pairs.  A job is one block of 16 output rows for 128 rhs (5
+// blocks of the stencil, or up to 6 of a row of the dense matrix); x digits (64 KB, in two
+// halves) and block digits (16 KB) of each K block move by bulk copies through rings of 5
+// halves and 4 blocks; the 288 columns of a job's accumulator are drained into the registers of
+// eight epilogue warps, which form the FP64 results while the next job's MMAs run.  One CTA
+// per SM (224 KB).
+// Bound: L2 and HBM reads of the digit tiles (80 KB per K block).
+// Measured: D_3 x at 32^2 sites x 512 rhs 4329 -> 230 us, D_2 x at 128^2 sites x 128 rhs (before, by
+// P^H D_1 P) 9.4 -> 0.9 ms, the inverse of 1024 unknowns times 64 rhs 2205 -> 40 us; the two
+// passes that scale and slice x move 32 B per real more.
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -40,14 +44,14 @@ namespace mg {
 namespace tc {
 namespace f64 {
 constexpr int D = 16, KD = 32;             // block size, reals of a block
-constexpr int NX = 7, NA = 8;              // digit slices of x and of the matrix
+constexpr int NX = 8, NA = 8, NG = 9;      // digit slices of x and of the matrix, groups
 constexpr int XS = 128 * KD * 2;           // 8 KB: one digit slice of a 128-rhs tile
-constexpr int XT = NX * XS;                // 56 KB
+constexpr int XT = NX * XS;                // 64 KB
 constexpr int AT = NA * KD * KD * 2;       // 16 KB: the digits of one block
-constexpr int NSTG = 3;
-constexpr int STAGE = XT + AT;
-constexpr int SMEM = NSTG * STAGE;         // 216 KB
-constexpr int ACC = NA * KD;               // 256 columns per accumulator
+constexpr int XH = XT / 2;                 // 32 KB: four digit slices
+constexpr int NXH = 5, NAS = 4;            // ring slots of x halves and of blocks
+constexpr int SMEM = NXH * XH + NAS * AT;  // 224 KB
+constexpr int TCOLS = 512;                 // 288 accumulator columns, allocated as 512
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr int KSPLIT = 6;                  // K blocks of a dense job (exact sums, see above)
@@ -55,14 +59,13 @@ constexpr int KSPLIT = 6;                  // K blocks of a dense job (exact sum
 using u64 = unsigned long long;
 using i64 = long long;
 
-// round(v 2^(BITS - e)) for the biased exponent E of the largest entry (|v| < 2^(E - 1022)).
-template <int BITS>
+// round(v 2^(62 - e)), |v| < 2^e, e = E - 1022 for the biased exponent E of the largest entry.
 __device__ __forceinline__ i64 fixed_point(double v, int E) {
     const u64 b = (u64)__double_as_longlong(v);
     const int eb = (int)((b >> 52) & 0x7ff);
     const u64 m = (b & 0xFFFFFFFFFFFFFull) | (eb ? 1ull << 52 : 0ull);
     // v = m 2^(max(eb, 1) - 1075); q = m 2^sh
-    const int sh = (eb > 0 ? eb : 1) - 1075 + BITS - (E - 1022);
+    const int sh = (eb > 0 ? eb : 1) - 1075 + 62 - (E - 1022);
     u64 q;
     if (sh >= 0) q = m << sh;
     else if (sh < -54) q = 0;
@@ -107,8 +110,8 @@ __global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, cons
     if (threadIdx.y == 0 && j < N && sh[threadIdx.x] != 0) atomicMax(out + j, sh[threadIdx.x]);
 }
 
-// Digit tiles of x: per (site, 128-rhs tile) 7 K-major slices of 8 KB.  Thread = (site,
-// group of 4 components, rhs): four 16-byte loads, seven 16-byte stores.  The rows of a
+// Digit tiles of x: per (site, 128-rhs tile) 8 K-major slices of 8 KB.  Thread = (site,
+// group of 4 components, rhs): four 16-byte loads, eight 16-byte stores.  The rows of a
 // tile beyond the rhs are not written (they only reach the same rows of the product).
 __global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const double2* __restrict__ x,
                                                  const u64* __restrict__ mx, int nblk, int N, int T) {
@@ -124,8 +127,8 @@ __global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const
     u64 qr[4], qi[4];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-        qr[p] = (u64)fixed_point<54>(v[p].x, E) + 0x0080808080808080ull;
-        qi[p] = (u64)fixed_point<54>(v[p].y, E) + 0x0080808080808080ull;
+        qr[p] = (u64)fixed_point(v[p].x, E) + 0x8080808080808080ull;
+        qi[p] = (u64)fixed_point(v[p].y, E) + 0x8080808080808080ull;
     }
     uint8_t* tile = xs + ((size_t)site * T + t) * XT + kmaj32_off(row, 8 * cg);
 #pragma unroll
@@ -155,8 +158,8 @@ __global__ void __launch_bounds__(128) k_slice_a(uint8_t* __restrict__ as, const
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
         const double2 a = blk[(long long)co * ld + 4 * kg + p];
-        u[2 * p] = (u64)fixed_point<62>(to ? a.y : a.x, E) + 0x8080808080808080ull;        // times Re x
-        u[2 * p + 1] = (u64)fixed_point<62>(to ? a.x : -a.y, E) + 0x8080808080808080ull;   // times Im x
+        u[2 * p] = (u64)fixed_point(to ? a.y : a.x, E) + 0x8080808080808080ull;        // times Re x
+        u[2 * p + 1] = (u64)fixed_point(to ? a.x : -a.y, E) + 0x8080808080808080ull;   // times Im x
     }
     uint8_t* tile = as + (size_t)q * AT;
 #pragma unroll
@@ -168,10 +171,11 @@ __global__ void __launch_bounds__(128) k_slice_a(uint8_t* __restrict__ as, const
     }
 }
 
-// 2^s sum_{g<8} G_g 2^(8 (7 - g)) rounded to FP64 once.  |G_g| < 2^25.
+// 2^s sum_{g<9} G_g 2^(8 (7 - g)) rounded to FP64 once (the last group to its integer part:
+// 2^-69 of the scale).  |G_g| < 2^25.
 __device__ __forceinline__ double combine(const int* G, int s) {
     i64 hi = (((i64)G[0] * 256 + G[1]) * 256 + G[2]) * 256 + G[3];
-    const i64 lo = (((i64)G[4] * 256 + G[5]) * 256 + G[6]) * 256 + G[7];
+    const i64 lo = (((i64)G[4] * 256 + G[5]) * 256 + G[6]) * 256 + G[7] + ((G[8] + 128) >> 8);
     hi += lo >> 32;                               // T = hi 2^32 + l, 0 <= l < 2^32
     u64 l = (u64)lo & 0xFFFFFFFFull;
     const bool neg = hi < 0;
@@ -209,9 +213,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 int* __restrict__ err) {
     if (grid_dependency()) return;
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t full[NSTG], empty[NSTG], afull[2], aempty[2];
+    __shared__ __align__(8) uint64_t xfull[NXH], xempty[NXH], bfull[NAS], bempty[NAS], afull, aempty;
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
+    uint8_t* xring = smem;
+    uint8_t* bring = smem + NXH * XH;
     volatile int* abrt = &abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = gridDim.x, T = gridDim.y, t = blockIdx.y;
@@ -222,18 +228,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(2 * ACC));
+                     "r"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int q = 0; q < NSTG; ++q) {
-            mbar_init(&full[q], 1);
-            mbar_init(&empty[q], 1);
+        for (int q = 0; q < NXH; ++q) {
+            mbar_init(&xfull[q], 1);
+            mbar_init(&xempty[q], 1);
         }
-        for (int q = 0; q < 2; ++q) {
-            mbar_init(&afull[q], 1);
-            mbar_init(&aempty[q], EPI_WARPS);
+        for (int q = 0; q < NAS; ++q) {
+            mbar_init(&bfull[q], 1);
+            mbar_init(&bempty[q], 1);
         }
+        mbar_init(&afull, 1);
+        mbar_init(&aempty, EPI_WARPS);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
@@ -246,17 +254,12 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {
             // producer: a tile narrower than 128 rhs moves only its own 8-row groups
             const uint32_t slice = (uint32_t)((rows + 7) / 8) * 512u;
-            int q = 0;
+            int q = 0, hq = 0;                   // K blocks and x halves issued
             bool ok = true;
             for (int i = 0; i < njob && ok; ++i) {
                 const int job = blockIdx.x + i * G;
                 const int kb = kblocks(job);
-                for (int o = 0; o < kb; ++o, ++q) {
-                    const int slot = q % NSTG;
-                    if (q >= NSTG && !mbar_wait_ab(&empty[slot], (unsigned)((q / NSTG - 1) & 1), abrt)) {
-                        ok = false;
-                        break;
-                    }
+                for (int o = 0; o < kb && ok; ++o) {
                     long long xb, ab;
                     if (MODE == 4) {
                         xb = (job % splits) * KSPLIT + o;
@@ -265,50 +268,91 @@ __global__ void __launch_bounds__(THREADS, 1)
                         xb = nbr_site(job, o, lx, lt);
                         ab = (long long)job * 5 + o;
                     }
-                    uint8_t* st = smem + slot * STAGE;
-                    const uint8_t* xsrc = xs + ((size_t)xb * T + t) * XT;
-                    mbar_expect_tx(&full[slot], slice * NX + AT);
-                    if (slice == (uint32_t)XS) {
-                        bulk_g2s(st, xsrc, XT, &full[slot]);
-                    } else {
-                        for (int s = 0; s < NX; ++s) bulk_g2s(st + s * XS, xsrc + s * XS, slice, &full[slot]);
-                    }
-                    bulk_g2s(st + XT, as + (size_t)ab * AT, AT, &full[slot]);
-                }
-            }
-            if (*abrt)
-                // copies still in flight land before the shared memory goes back
-                for (int q2 = max(0, q - NSTG); q2 < q; ++q2) mbar_wait(&full[q2 % NSTG], (unsigned)((q2 / NSTG) & 1));
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            int q = 0, last = -1;
-            bool ok = true;
-            for (int i = 0; i < njob && ok; ++i) {
-                const int as2 = i & 1, kb = kblocks(blockIdx.x + i * G);
-                if (i >= 2 && !mbar_wait_ab(&aempty[as2], (unsigned)(((i >> 1) - 1) & 1), abrt)) break;
-                for (int o = 0; o < kb; ++o, ++q) {
-                    const int slot = q % NSTG;
-                    if (!mbar_wait_ab(&full[slot], (unsigned)((q / NSTG) & 1), abrt)) {
+                    const int bs = q % NAS;
+                    if (q >= NAS && !mbar_wait_ab(&bempty[bs], (unsigned)((q / NAS - 1) & 1), abrt)) {
                         ok = false;
                         break;
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint32_t sx = smem_u32(smem + slot * STAGE), sa = sx + XT;
-#pragma unroll
-                    for (int j = 0; j < NX; ++j)
-#pragma unroll
-                        for (int ks = 0; ks < 2; ++ks)
-                            mma_bf16(tmem + as2 * ACC + KD * j, smem_desc(sx + j * XS + ks * 256, 128, 512),
-                                     smem_desc(sa + ks * 256, 128, 512), instr_desc(128, ACC - KD * j),
-                                     (o > 0 || j > 0 || ks > 0) ? 1u : 0u);
-                    mma_commit(&empty[slot]);
-                    if (o + 1 == kb) mma_commit(&afull[as2]);
-                    last = q;
+                    mbar_expect_tx(&bfull[bs], AT);
+                    bulk_g2s(bring + bs * AT, as + (size_t)ab * AT, AT, &bfull[bs]);
+                    ++q;
+                    const uint8_t* xsrc = xs + ((size_t)xb * T + t) * XT;
+                    for (int h = 0; h < 2; ++h) {
+                        const int xslot = hq % NXH;
+                        if (hq >= NXH && !mbar_wait_ab(&xempty[xslot], (unsigned)((hq / NXH - 1) & 1), abrt)) {
+                            ok = false;
+                            break;
+                        }
+                        uint8_t* st = xring + xslot * XH;
+                        mbar_expect_tx(&xfull[xslot], slice * (NX / 2));
+                        if (slice == (uint32_t)XS) {
+                            bulk_g2s(st, xsrc + h * XH, XH, &xfull[xslot]);
+                        } else {
+                            for (int s = 0; s < NX / 2; ++s)
+                                bulk_g2s(st + s * XS, xsrc + h * XH + s * XS, slice, &xfull[xslot]);
+                        }
+                        ++hq;
+                    }
                 }
             }
+            if (*abrt) {
+                // copies still in flight land before the shared memory goes back
+                for (int q2 = max(0, q - NAS); q2 < q; ++q2) mbar_wait(&bfull[q2 % NAS], (unsigned)((q2 / NAS) & 1));
+                for (int q2 = max(0, hq - NXH); q2 < hq; ++q2) mbar_wait(&xfull[q2 % NXH], (unsigned)((q2 / NXH) & 1));
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int q = 0, hq = 0;
+            bool ok = true;
+            for (int i = 0; i < njob && ok; ++i) {
+                const int kb = kblocks(blockIdx.x + i * G);
+                if (i >= 1 && !mbar_wait_ab(&aempty, (unsigned)((i - 1) & 1), abrt)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                for (int o = 0; o < kb && ok; ++o, ++q) {
+                    const int bs = q % NAS;
+                    if (!mbar_wait_ab(&bfull[bs], (unsigned)((q / NAS) & 1), abrt)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t sa = smem_u32(bring + bs * AT);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int xslot = hq % NXH;
+                        if (!mbar_wait_ab(&xfull[xslot], (unsigned)((hq / NXH) & 1), abrt)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;");
+                        const uint32_t sx = smem_u32(xring + xslot * XH);
+#pragma unroll
+                        for (int jj = 0; jj < NX / 2; ++jj) {
+                            const int j = h * (NX / 2) + jj;
+                            const int cols = KD * (j == 0 ? NA : NG - j);      // groups j .. min(j + 7, 8)
+#pragma unroll
+                            for (int ks = 0; ks < 2; ++ks) {
+                                // columns 256 .. 287 are first written by j = 1 of the first K step: its
+                                // rows i < 7 accumulate, the last group starts there
+                                const uint64_t xd = smem_desc(sx + jj * XS + ks * 256, 128, 512);
+                                if (j == 1 && o == 0 && ks == 0) {
+                                    mma_bf16(tmem + KD, xd, smem_desc(sa, 128, 512), instr_desc(128, KD * 7), 1u);
+                                    mma_bf16(tmem + KD * 8, xd, smem_desc(sa + 7 * KD * 64, 128, 512),
+                                             instr_desc(128, KD), 0u);
+                                } else {
+                                    mma_bf16(tmem + KD * j, xd, smem_desc(sa + ks * 256, 128, 512),
+                                             instr_desc(128, cols), (o > 0 || j > 0 || ks > 0) ? 1u : 0u);
+                                }
+                            }
+                        }
+                        mma_commit(&xempty[xslot]);
+                        ++hq;
+                    }
+                    if (ok) mma_commit(&bempty[bs]);
+                }
+                if (ok) mma_commit(&afull);
+            }
             // MMAs in flight complete before the TMEM and shared memory go back
-            if (*abrt && last >= 0) mbar_wait(&empty[last % NSTG], (unsigned)((last / NSTG) & 1));
+            if (*abrt && hq > 0) mbar_wait(&xempty[(hq - 1) % NXH], (unsigned)(((hq - 1) / NXH) & 1));
         }
     } else {
         // epilogue: two warps per TMEM lane quarter, 16 of the 32 output reals each
@@ -321,8 +365,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         double dyy = 0.0;
         bool ok = true;
         for (int i = 0; i < njob; ++i) {
-            const int as2 = i & 1;
-            if (!mbar_wait_ab(&afull[as2], (unsigned)((i >> 1) & 1), abrt)) {
+            if (!mbar_wait_ab(&afull, (unsigned)(i & 1), abrt)) {
                 ok = false;
                 break;
             }
@@ -330,46 +373,45 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int job = blockIdx.x + i * G;
             const long long row0 = (long long)(MODE == 4 ? job / splits : job) * D;
             double2* yo = MODE == 4 ? y + (long long)(job % splits) * nblk * D * N : y;
-            const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(as2 * ACC + half * 16);
-#pragma unroll 1
-            for (int c = 0; c < 16; c += 4) {
-                uint32_t r[NA][4];
+            const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 16);
+            uint32_t r[NG][16];
 #pragma unroll
-                for (int g = 0; g < NA; ++g)
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3])
-                                 : "r"(base + (uint32_t)(g * KD + c)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (c == 12) {
-                    asm volatile("tcgen05.fence::before_thread_sync;");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&aempty[as2]);      // accumulator may be overwritten
-                }
-                if (j < N) {
-                    double v[4];
+            for (int g = 0; g < NG; ++g)
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                    "%13, %14, %15}, [%16];"
+                    : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
+                      "=r"(r[g][6]), "=r"(r[g][7]), "=r"(r[g][8]), "=r"(r[g][9]), "=r"(r[g][10]), "=r"(r[g][11]),
+                      "=r"(r[g][12]), "=r"(r[g][13]), "=r"(r[g][14]), "=r"(r[g][15])
+                    : "r"(base + (uint32_t)(g * KD)));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&aempty);               // the accumulator may be overwritten
+            if (j < N) {
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                        int Gi[NA];
+                for (int p = 0; p < 8; ++p) {
+                    double v[2];
 #pragma unroll
-                        for (int g = 0; g < NA; ++g) Gi[g] = __float2int_rn(__uint_as_float(r[g][p]));
-                        v[p] = finite ? combine(Gi, sc) : __longlong_as_double(0x7ff8000000000000ll);
+                    for (int u = 0; u < 2; ++u) {
+                        int Gi[NG];
+#pragma unroll
+                        for (int g = 0; g < NG; ++g) Gi[g] = __float2int_rn(__uint_as_float(r[g][2 * p + u]));
+                        v[u] = finite ? combine(Gi, sc) : __longlong_as_double(0x7ff8000000000000ll);
                     }
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        const long long idx = (row0 + half * 8 + (c >> 1) + p) * N + j;
-                        double2 o = make_double2(v[2 * p], v[2 * p + 1]);
-                        if (MODE == 1) o = csub(b[idx], o);
-                        if (MODE != 3) yo[idx] = o;
-                        if (MODE == 2 || MODE == 3) {
-                            cfmac(dyx, o, x[idx]);
-                            dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
-                        }
+                    const long long idx = (row0 + half * 8 + p) * N + j;
+                    double2 o = make_double2(v[0], v[1]);
+                    if (MODE == 1) o = csub(b[idx], o);
+                    if (MODE != 3) yo[idx] = o;
+                    if (MODE == 2 || MODE == 3) {
+                        cfmac(dyx, o, x[idx]);
+                        dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
                     }
                 }
             }
         }
         if (MODE == 2 || MODE == 3) {
-            // the two halves of a rhs meet in shared memory (the stages are free: every copy
+            // the two halves of a rhs meet in shared memory (the rings are free: every copy
             // has landed and every MMA has completed once the last accumulator was read)
             double* red = reinterpret_cast<double*>(smem);
             asm volatile("bar.sync 1, %0;" ::"r"(32 * EPI_WARPS));
@@ -388,7 +430,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (tid == 0 && abort_flag) atomicExch(err, 1);
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * ACC));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
 }
 
 // y = sum over the splits of a dense product, in order.
