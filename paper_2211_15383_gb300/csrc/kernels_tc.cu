@@ -17,6 +17,8 @@
 // Split-K partials are added in a fixed order by a second kernel.  Every
 // mbarrier wait is bounded: on timeout the CTA records an error flag, frees TMEM
 // and returns.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "tcgen05.cuh"
 
@@ -658,48 +660,66 @@ __global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* __restrict__ rn,
 }
 
 // e (=|+=) M^{-1} sum_{s < K} alpha_s r_s with the residuals r_s as BF16 tiles (slots of
-// `slot` bytes): thread = (site, rhs), M^{-1} of the site in shared memory.
+// `slot` bytes): thread = (site, RPT adjacent rhs), M^{-1} of the site in shared memory,
+// transposed.  The sum over the steps is formed component by component (four per 16-byte
+// piece of a tile row) and goes straight into the 16 outputs of each rhs, so that a
+// coefficient read serves RPT rhs and only the outputs stay in registers.
+template <int RPT>
 __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e, const uint8_t* __restrict__ rt,
                                                          size_t slot, int K, const float2* __restrict__ alpha,
                                                          const float2* __restrict__ Minv, int nsites, int N, int T,
                                                          bool accumulate) {
     if (grid_dependency()) return;
-    __shared__ float2 Ms[D * D];
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    struct alignas(8 * RPT) Rhs { float2 v[RPT]; };
+    __shared__ float2 Mt[D * D];                                // [input][output]
+    const int j = RPT * (blockIdx.x * blockDim.x + threadIdx.x);
     for (int site = blockIdx.y; site < nsites; site += gridDim.y) {
         __syncthreads();
-        for (int q = threadIdx.x; q < D * D; q += blockDim.x) Ms[q] = Minv[(size_t)site * D * D + q];
+        for (int q = threadIdx.x; q < D * D; q += blockDim.x) Mt[(q % D) * D + q / D] = Minv[(size_t)site * D * D + q];
         __syncthreads();
         if (j >= N) continue;
         const uint8_t* row = rt + ((size_t)site * T + (j >> 7)) * TILE_A + kmaj32_off(j & 127, 0);
-        const size_t base = (size_t)site * D * N + j;
-        float2 v[D], acc[D];
+        float2* out = e + (size_t)site * D * N + j;
+        Rhs acc[D];
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-            v[c] = make_float2(0.f, 0.f);
-            acc[c] = accumulate ? e[base + (size_t)c * N] : make_float2(0.f, 0.f);
+            if (accumulate) acc[c] = *reinterpret_cast<const Rhs*>(out + (size_t)c * N);
+            else
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) acc[c].v[r] = make_float2(0.f, 0.f);
         }
-#pragma unroll 2
-        for (int s = 0; s < K; ++s) {
-            const float2 a = alpha[s * N + j];
-            uint4 w[4];
 #pragma unroll
-            for (int cg = 0; cg < 4; ++cg) w[cg] = *reinterpret_cast<const uint4*>(row + s * slot + cg * 128);
+        for (int cg = 0; cg < 4; ++cg) {
+            float2 v[4][RPT];
 #pragma unroll
-            for (int cg = 0; cg < 4; ++cg) {
-                const uint32_t x[4] = {w[cg].x, w[cg].y, w[cg].z, w[cg].w};
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    cfma(v[4 * cg + q], a,
-                         make_float2(__uint_as_float(x[q] << 16), __uint_as_float(x[q] & 0xFFFF0000u)));
+                for (int r = 0; r < RPT; ++r) v[q][r] = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int s = 0; s < K; ++s) {
+                const Rhs a = *reinterpret_cast<const Rhs*>(alpha + s * N + j);
+                uint4 w[RPT];
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) w[r] = *reinterpret_cast<const uint4*>(row + s * slot + cg * 128 + r * 16);
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const uint32_t x[4] = {w[r].x, w[r].y, w[r].z, w[r].w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        cfma(v[q][r], a.v[r], make_float2(__uint_as_float(x[q] << 16), __uint_as_float(x[q] & 0xFFFF0000u)));
+                }
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int c = 0; c < D; ++c) {
+                    const float2 m = Mt[(4 * cg + q) * D + c];
+#pragma unroll
+                    for (int r = 0; r < RPT; ++r) cfma(acc[c].v[r], m, v[q][r]);
+                }
         }
 #pragma unroll
-        for (int c = 0; c < D; ++c) {
-#pragma unroll
-            for (int q = 0; q < D; ++q) cfma(acc[c], Ms[c * D + q], v[q]);
-            e[base + (size_t)c * N] = acc[c];
-        }
+        for (int c = 0; c < D; ++c) *reinterpret_cast<Rhs*>(out + (size_t)c * N) = acc[c];
     }
 }
 
@@ -964,14 +984,19 @@ void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __n
 
 void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const float2* alpha, const float2* Minv,
                              int nsites, int N, bool accumulate, cudaStream_t s) {
-    const int th = N >= 128 ? 128 : (N + 31) / 32 * 32;
-    const int tiles = (N + th - 1) / th;
-    int G = 16 * kNumSM / tiles;
-    if (G > nsites) G = nsites;
-    if (G < 1) G = 1;
-    MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles, e, reinterpret_cast<const uint8_t*>(rt),
-                                                              tc_tiles_bytes(nsites, N), K, alpha, Minv, nsites, N,
-                                                              tc_tiles(N), accumulate);
+    // two rhs per thread where N is even (16-byte accesses to e and alpha)
+    const int rpt = N % 2 == 0 ? 2 : 1;
+    const int th = std::min(128 / rpt, (N / rpt + 31) / 32 * 32);
+    const int tiles = (N + rpt * th - 1) / (rpt * th);
+    const int G = std::max(1, std::min(nsites, 16 * kNumSM / tiles));
+    const uint8_t* r = reinterpret_cast<const uint8_t*>(rt);
+    const size_t slot = tc_tiles_bytes(nsites, N);
+    if (rpt == 2)
+        MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles<2>, e, r, slot, K, alpha, Minv, nsites, N,
+                  tc_tiles(N), accumulate);
+    else
+        MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles<1>, e, r, slot, K, alpha, Minv, nsites, N,
+                  tc_tiles(N), accumulate);
     MG_LAUNCHED();
 }
 
