@@ -167,6 +167,8 @@ void launch_gamma5(C* y, const C* x, long long nsites, int d, int N, cudaStream_
 // C[M][Nc] = A[M][K] * B[K][Nc] (+ C if accumulate), complex, row-major.
 template <typename C>
 void launch_gemm_nn(C* Cm, const C* A, const C* B, int M, int K, int Nc, bool accumulate, cudaStream_t s);
+// y = A x, A n x n, N <= 32 columns, FP32.
+void launch_gemm_few(float2* y, const float2* A, const float2* x, int n, int N, cudaStream_t s);
 // C[ka][kb] = A^H B for A [n][ka], B [n][kb] (reduction over n, deterministic two-pass).
 template <typename C>
 void launch_gemm_hn(double2* Cm, const C* A, const C* B, long long n, int ka, int kb, double2* part,

@@ -97,6 +97,66 @@ __global__ void __launch_bounds__(128) k_gemm_nn8(C* __restrict__ Cm, const C* _
     }
 }
 
+// y = A x for a dense n x n matrix and few columns (N <= 32), FP32: a CTA per kFewRows rows,
+// lanes over the columns and (the rest of them, and the warps) over K; the slices are added in
+// order.  Bound by reading A once from L2 or HBM; for few columns
+// the tensor-core form takes three launches (pack, product, sum of splits: 12 us) for this one
+// (4 us at n = 256, 8 us at n = 1024).
+constexpr int kFewRows = 4;
+__global__ void __launch_bounds__(256) k_gemm_few(float2* __restrict__ y, const float2* __restrict__ A,
+                                                  const float2* __restrict__ x, int n, int N, int cols) {
+    if (grid_dependency()) return;
+    __shared__ float2 sh[8][kFewRows][33];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int j = lane % cols, kl = lane / cols, kp = 32 / cols;   // cols: power of two >= N
+    const int row0 = blockIdx.x * kFewRows;
+    float2 acc[kFewRows];
+#pragma unroll
+    for (int r = 0; r < kFewRows; ++r) acc[r] = make_float2(0.f, 0.f);
+    // warp w takes k = w kp + kl, + 8 kp, ...: U of them at a time, their loads first
+    constexpr int U = 8;
+    const int step = 8 * kp;
+    const bool full = row0 + kFewRows <= n;
+    for (int k0 = wid * kp + kl; k0 < n; k0 += U * step) {
+        float2 xv[U], av[U][kFewRows];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int k = k0 + u * step;
+            xv[u] = (k < n && j < N) ? x[(long long)k * N + j] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < kFewRows; ++r)
+                av[u][r] = (k < n && (full || row0 + r < n)) ? A[(long long)(row0 + r) * n + k] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int r = 0; r < kFewRows; ++r) cfma(acc[r], av[u][r], xv[u]);
+    }
+#pragma unroll
+    for (int r = 0; r < kFewRows; ++r) {
+        for (int o = 16; o >= cols; o >>= 1) {
+            acc[r].x += __shfl_down_sync(0xffffffffu, acc[r].x, o);
+            acc[r].y += __shfl_down_sync(0xffffffffu, acc[r].y, o);
+        }
+        if (kl == 0) sh[wid][r][j] = acc[r];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kFewRows * cols; e += 256) {
+        const int r = e / cols, c = e % cols;
+        if (c >= N || row0 + r >= n) continue;
+        float2 s = sh[0][r][c];
+        for (int w = 1; w < 8; ++w) s = cadd(s, sh[w][r][c]);
+        y[(long long)(row0 + r) * N + c] = s;
+    }
+}
+void launch_gemm_few(float2* y, const float2* A, const float2* x, int n, int N, cudaStream_t s) {
+    MG_REQUIRE(N >= 1 && N <= 32, MGMLMC_EINVAL, "few-column product: N <= 32");
+    int cols = 1;
+    while (cols < N) cols *= 2;
+    MG_LAUNCH(dim3((n + kFewRows - 1) / kFewRows), dim3(256), 0, s, k_gemm_few, y, A, x, n, N, cols);
+    MG_LAUNCHED();
+}
+
 template <typename S, typename C>
 static void gemm_nn(S* Cm, const S* A, const S* B, int M, int K, int Nc, bool accumulate, cudaStream_t s) {
     const int gx = (Nc + GN - 1) / GN;

@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
                                                                 int lx, int lt, int N, double2* __restrict__ part) {
     if (grid_dependency()) return;
     using R = re_t<C>;
-    __shared__ C As[5 * D * D];
+    __shared__ C As[5 * D * (D + 1)];             // rows padded: the four rows of a warp in different banks
     __shared__ double2 red[2][D][8];
     const int tx = threadIdx.x, c = threadIdx.y, tid = c * 8 + tx;
     const int j = blockIdx.x * 8 + tx;
@@ -443,17 +443,32 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
     C dyx = czero<C>();
     R dyy = 0;
     for (int site = blockIdx.y; site < V; site += gridDim.y) {
+        // FP32: the five neighbours' rows all in flight while the blocks are staged (one after
+        // another they were five round trips: 9 us a launch, 3 now)
+        constexpr int PRE = sizeof(C) == 8 ? 5 : 1;
+        C xv[PRE][D];
+        if (PRE == 5 && j < N)
+#pragma unroll
+            for (int dir = 0; dir < PRE; ++dir) {
+                const C* xn = x + (long long)nbr_site(site, dir, lx, lt) * D * N + j;
+#pragma unroll
+                for (int bc = 0; bc < D; ++bc) xv[dir][bc] = xn[(long long)bc * N];
+            }
         __syncthreads();
-        for (int e = tid; e < 5 * D * D; e += 8 * D) As[e] = A[(long long)site * 5 * D * D + e];
+        for (int e = tid; e < 5 * D * D; e += 8 * D) As[(e / D) * (D + 1) + e % D] = A[(long long)site * 5 * D * D + e];
         __syncthreads();
         if (j < N) {
             C acc = czero<C>();
-            for (int dir = 0; dir < 5; ++dir) {
-                const int nb = nbr_site(site, dir, lx, lt);
-                const C* xn = x + (long long)nb * D * N + j;
-                const C* Ar = As + (dir * D + c) * D;
 #pragma unroll
-                for (int bc = 0; bc < D; ++bc) cfma(acc, Ar[bc], xn[(long long)bc * N]);
+            for (int dir = 0; dir < 5; ++dir) {
+                const C* Ar = As + (dir * D + c) * (D + 1);
+                if (PRE == 1) {
+                    const C* xn = x + (long long)nbr_site(site, dir, lx, lt) * D * N + j;
+#pragma unroll
+                    for (int bc = 0; bc < D; ++bc) xv[0][bc] = xn[(long long)bc * N];
+                }
+#pragma unroll
+                for (int bc = 0; bc < D; ++bc) cfma(acc, Ar[bc], xv[PRE == 5 ? dir : 0][bc]);
             }
             const long long idx = ((long long)site * D + c) * N + j;
             if (MODE == 1) acc = csub(b[idx], acc);
@@ -723,40 +738,48 @@ __device__ __forceinline__ void store_bf16_row(uint8_t* xt, int site, int j, int
 }
 
 // The same two operators with the dofs per fine site (D) fixed at compile time: the
-// loads of QB aggregate sites (QB * D values per thread) are issued together before
-// the FMAs, instead of one load per loop trip.
-template <typename C, int NV, int D, int QB>
+// loads of QB aggregate sites (QB * D values per rhs) are issued together before the FMAs,
+// instead of one load per loop trip.  V adjacent rhs per thread (FP32: 2 where N is even, in
+// 16-byte accesses): each value takes NV coefficients from shared memory, and with one rhs a
+// read that pipe, not HBM, set the time (restriction of a d = 16 level of 128^2 sites x 128 rhs:
+// 55 us of reads against 42 us of HBM).
+template <typename C, int V> struct alignas(sizeof(C) * V) RhsOf { C v[V]; };
+
+template <typename C, int NV, int D, int QB, int V>
 __global__ void __launch_bounds__(128) k_restrict_nvd(C* __restrict__ xc, const C* __restrict__ x,
                                                       const C* __restrict__ P, int lx, int lt, int ax, int at, int N) {
     if (grid_dependency()) return;
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     constexpr int HD = D / 2;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    using X = RhsOf<C, V>;
+    const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
     const int cx = lx / ax, ct = lt / at, na = ax * at;
     const int nP = na * D * NV;
     for (int S = blockIdx.y; S < cx * ct; S += gridDim.y) {
-        const int X = S % cx, T = S / cx;
+        const int Xc = S % cx, T = S / cx;
         __syncthreads();
         for (int e = threadIdx.x; e < nP; e += blockDim.x) {
             const int q = e / (D * NV), r = e % (D * NV);
-            const int site = (X * ax + q % ax) + lx * (T * at + q / ax);
+            const int site = (Xc * ax + q % ax) + lx * (T * at + q / ax);
             Ps[e] = P[(long long)site * D * NV + r];
         }
         __syncthreads();
         if (j >= N) continue;
-        C acc[2 * NV];
+        X acc[2 * NV];
 #pragma unroll
-        for (int o = 0; o < 2 * NV; ++o) acc[o] = czero<C>();
+        for (int o = 0; o < 2 * NV; ++o)
+#pragma unroll
+            for (int u = 0; u < V; ++u) acc[o].v[u] = czero<C>();
         for (int q0 = 0; q0 < na; q0 += QB) {
-            C xv[QB][D];
+            X xv[QB][D];
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
                 const int q = q0 + qq;
-                const int site = (X * ax + q % ax) + lx * (T * at + q / ax);
+                const int site = (Xc * ax + q % ax) + lx * (T * at + q / ax);
 #pragma unroll
                 for (int a = 0; a < D; ++a)
-                    xv[qq][a] = q < na ? x[((long long)site * D + a) * N + j] : czero<C>();
+                    if (q < na) xv[qq][a] = *reinterpret_cast<const X*>(x + ((long long)site * D + a) * N + j);
             }
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
@@ -765,17 +788,21 @@ __global__ void __launch_bounds__(128) k_restrict_nvd(C* __restrict__ xc, const 
 #pragma unroll
                 for (int a = 0; a < D; ++a)
 #pragma unroll
-                    for (int jv = 0; jv < NV; ++jv) cfmac(acc[(a < HD ? 0 : NV) + jv], Pq[a * NV + jv], xv[qq][a]);
+                    for (int jv = 0; jv < NV; ++jv) {
+                        const C p = Pq[a * NV + jv];
+#pragma unroll
+                        for (int u = 0; u < V; ++u) cfmac(acc[(a < HD ? 0 : NV) + jv].v[u], p, xv[qq][a].v[u]);
+                    }
             }
         }
 #pragma unroll
-        for (int o = 0; o < 2 * NV; ++o) xc[((long long)S * 2 * NV + o) * N + j] = acc[o];
+        for (int o = 0; o < 2 * NV; ++o) *reinterpret_cast<X*>(xc + ((long long)S * 2 * NV + o) * N + j) = acc[o];
     }
 }
 
 // xt (FP32, D = 16; may be null): the BF16 operand tiles of the result as well (the
 // tensor-core residual reads them), so that no pass over x packs them later.
-template <typename C, int NV, int D, int QB>
+template <typename C, int NV, int D, int QB, int V>
 __global__ void __launch_bounds__(128) k_prolong_nvd(C* __restrict__ x, const C* __restrict__ xc,
                                                      const C* __restrict__ P, int lx, int lt, int ax, int at, int N,
                                                      bool accumulate, uint8_t* __restrict__ xt) {
@@ -783,46 +810,63 @@ __global__ void __launch_bounds__(128) k_prolong_nvd(C* __restrict__ x, const C*
     extern __shared__ __align__(16) unsigned char smem_rp[];
     C* Ps = reinterpret_cast<C*>(smem_rp);
     constexpr int HD = D / 2;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    using X = RhsOf<C, V>;
+    const int j = V * (blockIdx.x * blockDim.x + threadIdx.x);
     const int cx = lx / ax, ct = lt / at, na = ax * at;
     const int nP = na * D * NV;
     for (int S = blockIdx.y; S < cx * ct; S += gridDim.y) {
-        const int X = S % cx, T = S / cx;
+        const int Xc = S % cx, T = S / cx;
         __syncthreads();
         for (int e = threadIdx.x; e < nP; e += blockDim.x) {
             const int q = e / (D * NV), r = e % (D * NV);
-            const int site = (X * ax + q % ax) + lx * (T * at + q / ax);
+            const int site = (Xc * ax + q % ax) + lx * (T * at + q / ax);
             Ps[e] = P[(long long)site * D * NV + r];
         }
         __syncthreads();
         if (j >= N) continue;
-        C cv[2 * NV];
+        X cv[2 * NV];
 #pragma unroll
-        for (int o = 0; o < 2 * NV; ++o) cv[o] = xc[((long long)S * 2 * NV + o) * N + j];
+        for (int o = 0; o < 2 * NV; ++o) cv[o] = *reinterpret_cast<const X*>(xc + ((long long)S * 2 * NV + o) * N + j);
         for (int q0 = 0; q0 < na; q0 += QB) {
-            C ov[QB][D];
+            X ov[QB][D];
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
                 const int q = q0 + qq;
-                const int site = (X * ax + q % ax) + lx * (T * at + q / ax);
+                const int site = (Xc * ax + q % ax) + lx * (T * at + q / ax);
 #pragma unroll
-                for (int a = 0; a < D; ++a)
-                    ov[qq][a] = (accumulate && q < na) ? x[((long long)site * D + a) * N + j] : czero<C>();
+                for (int a = 0; a < D; ++a) {
+                    if (accumulate && q < na)
+                        ov[qq][a] = *reinterpret_cast<const X*>(x + ((long long)site * D + a) * N + j);
+                    else
+#pragma unroll
+                        for (int u = 0; u < V; ++u) ov[qq][a].v[u] = czero<C>();
+                }
             }
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
                 const int q = q0 + qq;
                 if (q >= na) break;
-                const int site = (X * ax + q % ax) + lx * (T * at + q / ax);
+                const int site = (Xc * ax + q % ax) + lx * (T * at + q / ax);
                 const C* Pq = Ps + q * D * NV;
 #pragma unroll
                 for (int a = 0; a < D; ++a) {
 #pragma unroll
-                    for (int jv = 0; jv < NV; ++jv) cfma(ov[qq][a], Pq[a * NV + jv], cv[(a < HD ? 0 : NV) + jv]);
-                    x[((long long)site * D + a) * N + j] = ov[qq][a];
+                    for (int jv = 0; jv < NV; ++jv) {
+                        const C p = Pq[a * NV + jv];
+#pragma unroll
+                        for (int u = 0; u < V; ++u) cfma(ov[qq][a].v[u], p, cv[(a < HD ? 0 : NV) + jv].v[u]);
+                    }
+                    *reinterpret_cast<X*>(x + ((long long)site * D + a) * N + j) = ov[qq][a];
                 }
                 if constexpr (sizeof(C) == 8 && D == 16) {
-                    if (xt) store_bf16_row(xt, site, j, N, ov[qq]);
+                    if (xt)
+#pragma unroll
+                        for (int u = 0; u < V; ++u) {
+                            float2 row[D];
+#pragma unroll
+                            for (int a = 0; a < D; ++a) row[a] = ov[qq][a].v[u];
+                            store_bf16_row(xt, site, j + u, N, row);
+                        }
                 }
             }
         }
@@ -1406,28 +1450,100 @@ void launch_block_stencil(C* y, const C* x, const C* b, const C* A, int lx, int 
     else bs_dispatch<C, 8>(y, x, b, A, lx, lt, d, N, mode, part, groups, s);
 }
 
+// Restriction of a d = 16 level for few rhs (N <= 32): thread = (rhs, coarse value), a CTA per
+// coarse site and spin block.  With a thread per rhs a CTA is one half-empty warp whose 2 NV sums
+// run one after another (10 us for 64 coarse sites x 16 rhs, this takes 5).
+template <int NV>
+__global__ void __launch_bounds__(32 * NV) k_restrict_few(float2* __restrict__ xc, const float2* __restrict__ x,
+                                                          const float2* __restrict__ P, int lx, int lt, int ax, int at,
+                                                          int N) {
+    if (grid_dependency()) return;
+    constexpr int D = 16, HD = 8;
+    extern __shared__ __align__(16) unsigned char smem_rp[];
+    float2* Ps = reinterpret_cast<float2*>(smem_rp);            // [aggregate site][a of the spin block][jv]
+    const int j = threadIdx.x, jv = threadIdx.y, tid = jv * 32 + j;
+    const int cx = lx / ax, na = ax * at;
+    const int S = blockIdx.x >> 1, sp = blockIdx.x & 1;
+    const int Xc = S % cx, T = S / cx;
+    auto site_of = [&](int q) { return (Xc * ax + q % ax) + lx * (T * at + q / ax); };
+    for (int e = tid; e < na * HD * NV; e += 32 * NV) {
+        const int q = e / (HD * NV), r = e % (HD * NV);
+        Ps[e] = P[((long long)site_of(q) * D + sp * HD) * NV + r];
+    }
+    __syncthreads();
+    if (j >= N) return;
+    float2 acc = make_float2(0.f, 0.f);
+    constexpr int QB = 4;                                       // sites whose loads are issued together
+    for (int q0 = 0; q0 < na; q0 += QB) {
+        float2 xv[QB][HD];
+#pragma unroll
+        for (int u = 0; u < QB; ++u) {
+            const float2* xs = x + ((long long)site_of(min(q0 + u, na - 1)) * D + sp * HD) * N + j;
+#pragma unroll
+            for (int a = 0; a < HD; ++a) xv[u][a] = xs[(long long)a * N];
+        }
+#pragma unroll
+        for (int u = 0; u < QB; ++u) {
+            if (q0 + u >= na) break;
+#pragma unroll
+            for (int a = 0; a < HD; ++a) cfmac(acc, Ps[((q0 + u) * HD + a) * NV + jv], xv[u][a]);
+        }
+    }
+    xc[((long long)S * 2 * NV + sp * NV + jv) * N + j] = acc;
+}
+
+template <typename C, int NV>
+static bool restrict_few(C* xc, const C* x, const C* P, int lx, int lt, int d, int ax, int at, int N, cudaStream_t s) {
+    if constexpr (sizeof(C) == 8) {
+        if (d != 16 || N > 32) return false;
+        const size_t sm = (size_t)ax * at * 8 * NV * sizeof(C);
+        MG_LAUNCH(dim3(2 * (lx / ax) * (lt / at)), dim3(32, NV), sm, s, k_restrict_few<NV>, xc, x, P, lx, lt, ax, at, N);
+        MG_LAUNCHED();
+        return true;
+    }
+    return false;
+}
+
+template <typename C, int NV, int D, int QB, int V>
+static void rp_nvd(bool restrict_op, C* out, const C* in, const C* P, int lx, int lt, int ax, int at, int N,
+                   bool accumulate, uint8_t* xt, cudaStream_t s) {
+    const int ncs = (lx / ax) * (lt / at);
+    const int cols = (N + V - 1) / V;
+    const int th = std::min(128 / V, (cols + 31) / 32 * 32);
+    const int tiles = (cols + th - 1) / th;
+    const int G = std::max(1, std::min(ncs, 16 * kNumSM / tiles));
+    const size_t sm = (size_t)ax * at * D * NV * sizeof(C);
+    if (restrict_op)
+        MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nvd<C, NV, D, QB, V>), out, in, P, lx, lt, ax, at, N);
+    else
+        MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nvd<C, NV, D, QB, V>), out, in, P, lx, lt, ax, at, N, accumulate,
+                  xt);
+    MG_LAUNCHED();
+}
+
 template <typename C, int NV>
 static void rp_launch(bool restrict_op, C* xc_or_x, const C* in, const C* P, int lx, int lt, int d, int ax, int at,
                       int N, bool accumulate, uint8_t* xt, cudaStream_t s) {
-    const int ncs = (lx / ax) * (lt / at);
-    const int th = cta_threads(N);
-    const int tiles = (N + th - 1) / th;
-    int G = 16 * kNumSM / tiles;
-    if (G > ncs) G = ncs;
-    if (G < 1) G = 1;
-    const size_t sm = (size_t)ax * at * d * NV * sizeof(C);
+    constexpr int W = sizeof(C) == 8 ? 2 : 1;
+    // two rhs per thread from 64 rhs on (below, they leave lanes idle), except in the d = 16
+    // prolongation, which also writes the BF16 tiles (39 us with one, 47 with two)
+    const bool two = W == 2 && N % 2 == 0 && N >= 64 && !(d == 16 && !restrict_op);
+    if (restrict_op && restrict_few<C, NV>(xc_or_x, in, P, lx, lt, d, ax, at, N, s)) return;
     if (d == 2) {
-        if (restrict_op) MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nvd<C, NV, 2, 4>), xc_or_x, in, P, lx, lt, ax, at, N);
-        else MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nvd<C, NV, 2, 4>), xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr);
-        MG_LAUNCHED();
+        if (two) rp_nvd<C, NV, 2, 4, W>(restrict_op, xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr, s);
+        else rp_nvd<C, NV, 2, 4, 1>(restrict_op, xc_or_x, in, P, lx, lt, ax, at, N, accumulate, nullptr, s);
         return;
     }
     if (d == 16) {
-        if (restrict_op) MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nvd<C, NV, 16, 1>), xc_or_x, in, P, lx, lt, ax, at, N);
-        else MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_prolong_nvd<C, NV, 16, 1>), xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt);
-        MG_LAUNCHED();
+        if (two) rp_nvd<C, NV, 16, 1, W>(true, xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt, s);
+        else rp_nvd<C, NV, 16, 1, 1>(restrict_op, xc_or_x, in, P, lx, lt, ax, at, N, accumulate, xt, s);
         return;
     }
+    const int ncs = (lx / ax) * (lt / at);
+    const int th = cta_threads(N);
+    const int tiles = (N + th - 1) / th;
+    const int G = std::max(1, std::min(ncs, 16 * kNumSM / tiles));
+    const size_t sm = (size_t)ax * at * d * NV * sizeof(C);
     if (restrict_op)
         MG_LAUNCH(dim3(tiles, G), th, sm, s, (k_restrict_nv<C, NV>), xc_or_x, in, P, lx, lt, d, ax, at, N);
     else

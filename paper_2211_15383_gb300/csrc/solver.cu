@@ -223,6 +223,7 @@ bool apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate, voi
     return launch_prolong<C>(x, xc, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, accumulate, c.stream, xt);
 }
 
+constexpr int kFewRhs = 32, kFewRhsUnknowns = 1024;
 template <typename C> static void coarsest_apply(Ctx& c, C* e, const C* r, int N);
 static double dinv_bytes(const Level& L, int N, double s) { return (double)L.n * L.n * s + 2.0 * L.n * N * s; }
 static double dinv_flops(const Level& L, int N) { return 8.0 * (double)L.n * L.n * N; }
@@ -238,6 +239,14 @@ template <> void coarsest_apply<double2>(Ctx& c, double2* e, const double2* r, i
 }
 template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int N) {
     const Level& L = c.lev[c.L - 1];
+    // few right-hand sides of a small level: the FP32 inverse in one launch (4 us at n = 256,
+    // 9 us at n = 1024, against 12 us of the tensor-core form's three; at twice that size
+    // reading four times the FP32 inverse takes longer)
+    if (N < kFewRhs && L.n <= kFewRhsUnknowns) {
+        ProfScope ps(c, "Dinv.f32", dinv_bytes(L, N, 8), dinv_flops(L, N));
+        launch_gemm_few(e, L.Dinv32, r, (int)L.n, N, c.stream);
+        return;
+    }
     if (L.Dinv16) {
         // BF16 inverse on the tensor cores; algorithmic bytes: the BF16 matrix once + FP32 in/out
         ProfScope ps(c, "Dinv.bf16", (double)L.n * 2 * L.n * 2 + 2.0 * L.n * N * 8, dinv_flops(L, N));
