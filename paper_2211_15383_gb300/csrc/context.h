@@ -98,6 +98,15 @@ struct Profiler {
     ~Profiler();
 };
 
+// Name of a kernel class, put together only when the profiler is on: a l b c (l < 0: none).
+struct ProfKey {
+    const char* a;
+    int l;
+    const char *b, *c;
+    ProfKey(const char* a_, int l_ = -1, const char* b_ = "", const char* c_ = "") : a(a_), l(l_), b(b_), c(c_) {}
+    std::string str() const { return std::string(a) + (l < 0 ? std::string() : std::to_string(l)) + b + c; }
+};
+
 struct Ctx;
 // Brackets the launches issued during its lifetime with events (when enabled);
 // the entry joins the profiler's pending list only once both events are
@@ -107,7 +116,7 @@ struct ProfScope {
     bool active;
     Profiler::Pending p;
     // impl_bytes < 0: the implementation moves the algorithmic bytes
-    ProfScope(Ctx& ctx, const std::string& key, double bytes, double flops, double impl_bytes = -1);
+    ProfScope(Ctx& ctx, const ProfKey& key, double bytes, double flops, double impl_bytes = -1);
     ~ProfScope();
 };
 
@@ -151,7 +160,7 @@ struct Ctx {
 
     // ---- memory
     struct Buf { void* p = nullptr; size_t bytes = 0; };
-    std::map<std::string, Buf> ws;
+    std::unordered_map<std::string, Buf> ws;
     std::unordered_map<void*, size_t> owned;   // device allocations and their sizes
     size_t live_bytes = 0, peak_bytes = 0;     // device bytes held now and at most
 

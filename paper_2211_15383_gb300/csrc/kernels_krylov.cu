@@ -452,15 +452,16 @@ __global__ void __launch_bounds__(256) k_scale_cols_if(C* __restrict__ w, const 
 __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const double* __restrict__ hsub,
                                                double* __restrict__ cs, double2* __restrict__ sn,
                                                double2* __restrict__ g, double2* __restrict__ irr,
-                                               const double* __restrict__ bnorm, u64* max, u64* clear, int j0, int j1,
-                                               int m, int N) {
+                                               const double* __restrict__ bnorm, u64* max, u64* clear, double* host, int j0,
+                                               int j1, int m, int N) {
     if (grid_dependency()) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (clear && r == 0) *clear = 0;
-    if (r >= N) return;
-    double2 gj = g[(long long)j0 * N + r];
+    const bool in = r < N;
+    if (!in && !host) return;
+    double2 gj = in ? g[(long long)j0 * N + r] : make_double2(0.0, 0.0);
     double resid = 0.0;
-    for (int j = j0; j <= j1; ++j) {
+    for (int j = j0; in && j <= j1; ++j) {
         double2* col = H + (long long)j * (m + 1) * N + r;
         double2 a = col[0];
 #pragma unroll 4
@@ -501,9 +502,20 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
         g[(long long)(j + 1) * N + r] = gj;
         if (!(t == t)) resid = t;
     }
-    if (max) {
-        const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid, bn = bnorm[r];
-        atomic_max_double(max, bn > 0.0 ? rs / bn : 0.0);
+    if (max || host) {
+        const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid, bn = in ? bnorm[r] : 0.0;
+        const double v = bn > 0.0 ? rs / bn : 0.0;
+        if (host) {
+            u64 m8 = (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const u64 w = __shfl_xor_sync(0xffffffffu, m8, o);
+                m8 = w > m8 ? w : m8;
+            }
+            if (threadIdx.x == 0) *host = __longlong_as_double((long long)m8);
+        } else {
+            atomic_max_double(max, v);
+        }
     }
 }
 
@@ -676,9 +688,10 @@ void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_
 }
 
 void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,
-                   const double* bnorm, unsigned long long* max, unsigned long long* clear, int j0, int j1, int m, int N,
-                   cudaStream_t s) {
-    MG_LAUNCH((N + 31) / 32, 32, 0, s, k_rotate, H, hsub, cs, sn, g, irr, bnorm, max, clear, j0, j1, m, N);
+                   const double* bnorm, unsigned long long* max, unsigned long long* clear, double* host, int j0, int j1,
+                   int m, int N, cudaStream_t s) {
+    MG_REQUIRE(!host || N <= kRotateWarp, MGMLMC_EINVAL, "rotations: one warp writes to the host");
+    MG_LAUNCH((N + 31) / 32, 32, 0, s, k_rotate, H, hsub, cs, sn, g, irr, bnorm, max, clear, host, j0, j1, m, N);
     MG_LAUNCHED();
 }
 

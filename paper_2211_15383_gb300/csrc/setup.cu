@@ -167,10 +167,10 @@ Profiler::~Profiler() {
     }
     for (auto e : pool) cudaEventDestroy(e);
 }
-ProfScope::ProfScope(Ctx& ctx, const std::string& key, double bytes, double flops, double impl_bytes)
+ProfScope::ProfScope(Ctx& ctx, const ProfKey& key, double bytes, double flops, double impl_bytes)
     : c(&ctx), active(ctx.prof.on) {
     if (!active) return;
-    p = Profiler::Pending{key, c->prof.take(), c->prof.take(), bytes, flops, impl_bytes < 0 ? bytes : impl_bytes};
+    p = Profiler::Pending{key.str(), c->prof.take(), c->prof.take(), bytes, flops, impl_bytes < 0 ? bytes : impl_bytes};
     MG_CUDA(cudaEventRecord(p.a, c->stream));
 }
 ProfScope::~ProfScope() {

@@ -31,7 +31,13 @@ template <> const double2* prol<double2>(const Level& L) { return L.P64; }
 template <> const float2* prol<float2>(const Level& L) { return L.P32; }
 
 static std::string nm(const char* base, int l, size_t sz) {
-    return std::string(base) + "_" + std::to_string(l) + "_" + std::to_string(sz);
+    std::string s(base);
+    s += '_';
+    s += (char)('0' + l);
+    s += '_';
+    if (sz >= 10) s += '1';
+    s += (char)('0' + sz % 10);
+    return s;
 }
 
 static const char* prec_tag(size_t sz) { return sz == sizeof(double2) ? "f64" : "f32"; }
@@ -115,7 +121,7 @@ void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* al
     double2* part = nullptr;
     if (mode >= 2) part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
     {
-        ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)), bytes, flops);
+        ProfScope ps(c, {"D", l + 1, ".", prec_tag(sizeof(C))}, bytes, flops);
         if (l == 0)
             launch_wilson<C>(y, x, b, links<C>(c), c.m0, L.lx, L.lt, N, mode, part, groups, c.stream);
         else if (!f64_stencil<C>(c, L, y, x, b, L.A64t, N, mode, part, groups))
@@ -154,7 +160,7 @@ static void apply_Dhat_tc(Ctx& c, int l, float2* y, __nv_bfloat16* yt, const __n
     {
         // algorithmic traffic: BF16 x (4 B per complex) and y (FP32 8 B or BF16 4 B) once,
         // the BF16 operands once
-        ProfScope ps(c, "D" + std::to_string(l + 1) + ".bf16",
+        ProfScope ps(c, {"D", l + 1, ".bf16"},
                      (double)L.n * N * (4 + (yt ? 4 : y ? 8 : 0)) + 5.0 * L.nsites * 8.0 * L.d * L.d,
                      40.0 * L.d * L.d * (double)L.nsites * N);
         launch_block_stencil_tc(y, yt, nullptr, xt, L.Ahat16, L.lx, L.lt, N, part, groups, device_error_flag(c),
@@ -165,7 +171,7 @@ static void apply_Dhat_tc(Ctx& c, int l, float2* y, __nv_bfloat16* yt, const __n
 
 static void pack_tiles(Ctx& c, int l, __nv_bfloat16* xt, const float2* x, int N) {
     const Level& L = c.lev[l];
-    ProfScope ps(c, "pack" + std::to_string(l + 1) + ".bf16", (double)L.n * N * (8 + 4), 0.0);
+    ProfScope ps(c, {"pack", l + 1, ".bf16"}, (double)L.n * N * (8 + 4), 0.0);
     launch_pack_tiles_bf16(xt, x, L.nsites, N, c.stream);
 }
 
@@ -178,7 +184,7 @@ static void apply_Dhat(Ctx& c, int l, C* y, const C* x, int N, int mode, C* alph
     const double s = sizeof(C);
     double2* part = mode >= 2 ? c.scratch<double2>("part_st", (size_t)groups * 2 * N) : nullptr;
     {
-        ProfScope ps(c, "D" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
+        ProfScope ps(c, {"D", l + 1, ".", prec_tag(sizeof(C))},
                      (double)L.n * N * s * (mode == 3 ? 1 : 2) + 5.0 * L.nsites * L.d * L.d * s,
                      40.0 * L.d * L.d * (double)L.nsites * N);
         if (!f64_stencil<C>(c, L, y, x, (const C*)nullptr, L.Ahat64t, N, mode, part, groups))
@@ -207,7 +213,7 @@ template <typename C>
 void apply_restrict(Ctx& c, int l, C* xc, const C* x, int N) {
     const Level& L = c.lev[l];
     const double s = sizeof(C);
-    ProfScope ps(c, "PH" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
+    ProfScope ps(c, {"PH", l + 1, ".", prec_tag(sizeof(C))},
                  (double)L.n * N * s + (double)c.lev[l + 1].n * N * s + (double)L.n * L.nvec * s,
                  8.0 * L.nvec * (double)L.n * N);
     launch_restrict<C>(xc, x, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, c.stream);
@@ -217,7 +223,7 @@ template <typename C>
 bool apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate, void* xt) {
     const Level& L = c.lev[l];
     const double s = sizeof(C);
-    ProfScope ps(c, "P" + std::to_string(l + 1) + "." + prec_tag(sizeof(C)),
+    ProfScope ps(c, {"P", l + 1, ".", prec_tag(sizeof(C))},
                  (double)L.n * N * s * (accumulate ? 2 : 1) + (double)c.lev[l + 1].n * N * s + (double)L.n * L.nvec * s,
                  8.0 * L.nvec * (double)L.n * N);
     return launch_prolong<C>(x, xc, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, accumulate, c.stream, xt);
@@ -309,7 +315,7 @@ bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bo
     {
         const int groups = block_stencil_tc_groups(L.nsites, N);
         // algorithmic traffic: e tiles (4 B per complex) and r (8 B) read, residual tiles written (4 B)
-        ProfScope ps(c, "D" + std::to_string(l + 1) + "res.bf16",
+        ProfScope ps(c, {"D", l + 1, "res.bf16"},
                      (double)L.n * N * (4 + 8 + 4) + 5.0 * L.nsites * 8.0 * L.d * L.d,
                      40.0 * L.d * L.d * (double)L.nsites * N);
         launch_block_stencil_tc(nullptr, rt, r, et, L.A16, L.lx, L.lt, N, nullptr, groups, device_error_flag(c),
@@ -320,13 +326,13 @@ bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bo
         [&](int s, bool last) { apply_Dhat_tc(c, l, nullptr, last ? nullptr : pt, rt + s * slot, N, alpha + (size_t)s * N); },
         [&](int k, bool) {
             // traffic: the K residuals (4 B per complex) read, e read and written
-            ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".bf16", (double)L.n * N * (4 * k + 16),
+            ProfScope ps(c, {"bjac", l + 1, ".bf16"}, (double)L.n * N * (4 * k + 16),
                          8.0 * (L.d + k) * (double)L.n * N);
             launch_block_diag_tiles(e, rt, k, alpha, L.Minv32, L.nsites, N, true, c.stream);
         },
         [&](int s, int t) {
             // traffic: r and p tiles read, the next r tiles written (4 B per complex)
-            ProfScope ps(c, "mr" + std::to_string(l + 1) + ".bf16", (double)L.n * N * 12, 8.0 * L.n * N);
+            ProfScope ps(c, {"mr", l + 1, ".bf16"}, (double)L.n * N * 12, 8.0 * L.n * N);
             launch_mr_update_tiles(rt + t * slot, rt + s * slot, pt, alpha + (size_t)s * N, L.nsites, N, c.stream);
         });
     return true;
@@ -347,11 +353,11 @@ bool pre_smooth_tc<float2>(Ctx& c, int l, float2* e, float2* r, int N, int nu) {
     for (int s = 0; s < nu; ++s) {
         apply_Dhat_tc(c, l, p, nullptr, rt, N, alpha);
         const bool more = s + 1 < nu;
-        ProfScope ps(c, "mr" + std::to_string(l + 1) + ".f32", (double)L.n * N * (5 * 8 + (more ? 4 : 0)),
+        ProfScope ps(c, {"mr", l + 1, ".f32"}, (double)L.n * N * (5 * 8 + (more ? 4 : 0)),
                      16.0 * L.n * N);
         launch_mr_update_tc(yh, r, p, alpha, L.nsites, N, s == 0, more ? rt : nullptr, c.stream);
     }
-    ProfScope ps(c, "bjac" + std::to_string(l + 1) + ".f32", 3.0 * L.n * N * sizeof(float2),
+    ProfScope ps(c, {"bjac", l + 1, ".f32"}, 3.0 * L.n * N * sizeof(float2),
                  8.0 * L.d * (double)L.n * N);
     launch_block_diag_apply<float2>(e, yh, L.Minv32, L.nsites, L.d, N, false, c.stream);
     return true;
@@ -411,7 +417,6 @@ static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool
     C* p = c.scratch<C>(nm("mr_p", l, sizeof(C)), nN);
     C* alpha = c.scratch<C>(nm("mr_al", l, sizeof(C)), (size_t)kMrGroup * N);
     const bool jacobi = hat_blocks<C>(L) != nullptr;
-    const std::string tag = std::to_string(l + 1) + "." + prec_tag(sizeof(C));
     const int fin = mr_steps(
         nu, need_r,
         [&](int s, bool last) {
@@ -422,16 +427,16 @@ static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool
         [&](int k, bool first) {
             const bool zero = e_zero && first;
             if (jacobi) {
-                ProfScope ps(c, "bjac" + tag, (k + (zero ? 1.0 : 2.0)) * nN * sizeof(C), 8.0 * (L.d + k) * (double)nN);
+                ProfScope ps(c, {"bjac", l + 1, ".", prec_tag(sizeof(C))}, (k + (zero ? 1.0 : 2.0)) * nN * sizeof(C), 8.0 * (L.d + k) * (double)nN);
                 launch_block_diag_combine<C>(e, rs, nN, k, alpha, minv<C>(L), L.nsites, L.d, N, !zero, c.stream);
             } else {
-                ProfScope ps(c, "mr" + std::to_string(l + 1) + "sum." + prec_tag(sizeof(C)),
+                ProfScope ps(c, {"mr", l + 1, "sum.", prec_tag(sizeof(C))},
                              (k + (zero ? 1.0 : 2.0)) * nN * sizeof(C), 8.0 * k * (double)nN);
                 launch_mr_combine<C>(e, rs, nN, k, alpha, L.n, N, zero, c.stream);
             }
         },
         [&](int s, int t) {
-            ProfScope ps(c, "mr" + tag, 3.0 * nN * sizeof(C), 8.0 * (double)nN);
+            ProfScope ps(c, {"mr", l + 1, ".", prec_tag(sizeof(C))}, 3.0 * nN * sizeof(C), 8.0 * (double)nN);
             // with a single slot the update is in place
             launch_mr_update<C>(rs + t * nN, rs + s * nN, p, alpha + (size_t)s * N, L.n, N, c.stream);
         });
@@ -537,7 +542,7 @@ static void arnoldi_step(Ctx& c, const Basis<C>& B, int j, int passes) {
     // algorithmic bytes: the j+1 basis vectors read once per Gram-Schmidt pass; the
     // implementation reads them twice (dot products, then the update) and reads w twice and
     // writes it once per pass: (2j + 5) vectors
-    ProfScope ps(c, std::string("orth.") + prec_tag(sizeof(C)), passes * (j + 1) * nN * sz,
+    ProfScope ps(c, {"orth.", -1, prec_tag(sizeof(C))}, passes * (j + 1) * nN * sz,
                  passes * 2.0 * 8.0 * (j + 1) * nN, passes * (2 * j + 5) * nN * sz);
     C* u = B.v(j + 1);
     double2* H = B.H + (size_t)j * (B.m + 1) * B.N;
@@ -579,7 +584,7 @@ static void kcycle(Ctx& c, int l, C* e, const C* r, int N, int k) {
         apply_D<C>(c, l, B.v(j + 1), B.z(j), nullptr, N, 0, nullptr);
         arnoldi_step<C>(c, B, j, 1);
     }
-    launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, nullptr, nullptr, nullptr, 0, k - 1, k, N, c.stream);
+    launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, nullptr, nullptr, nullptr, nullptr, 0, k - 1, k, N, c.stream);
     basis_update<C>(c, B, k - 1, e, false);
 }
 
@@ -647,10 +652,19 @@ static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate
         arnoldi_step<C>(c, B, j, passes);
         ++it;
         if (j + 1 < check_from && j + 1 < m && it < maxit) continue;
-        const MaxSlot ms = take_max(c);
-        launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, ms.at, ms.clear, rotated, j, m, N, c.stream);
+        double est;
+        if (N <= kRotateWarp) {
+            // one warp: it writes the maximum to the host itself
+            launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, nullptr, nullptr, c.hbuf + kMaxSlots, rotated, j, m,
+                          N, c.stream);
+            c.sync();
+            est = c.hbuf[kMaxSlots];
+        } else {
+            const MaxSlot ms = take_max(c);
+            launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, ms.at, ms.clear, nullptr, rotated, j, m, N, c.stream);
+            est = read_max(c, ms);
+        }
         rotated = j + 1;
-        const double est = read_max(c, ms);
         if (est != est) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
         if (est <= tol || it >= maxit || j + 1 >= m) break;
     }
