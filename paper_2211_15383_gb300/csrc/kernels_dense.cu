@@ -1118,6 +1118,92 @@ __global__ void __launch_bounds__(jac::kThreads) k_cholesky_grid(double2* G, dou
     }
 }
 
+// The same for small blocks (b <= kClusterMax) by a cluster of 8 CTAs: row i of the trailing
+// matrix lives in CTA i mod 8, and a finished row of R goes to all of them through distributed
+// shared memory (packed upper triangle: 132 KB at b = 128), so a column costs one cluster
+// barrier instead of a barrier of the grid through L2, and the inverse's columns find R in
+// shared memory.  Measured on the deflation of a 64^2 lattice: 344 -> 195 us a call.
+constexpr int kClusterMax = 144;
+__host__ __device__ __forceinline__ int packed_row(int i, int b) { return i * b - i * (i - 1) / 2; }   // of (i, i)
+inline size_t cluster_smem(int b) { return ((size_t)packed_row(b, b) + 8 * (size_t)b) * sizeof(double2) + b * sizeof(double); }
+
+__global__ void __launch_bounds__(256) __cluster_dims__(8, 1, 1)
+    k_cholesky_cluster(const double2* __restrict__ G, double2* __restrict__ Rinv, int b, int* status) {
+    extern __shared__ __align__(16) unsigned char smem_ch[];
+    double2* R = reinterpret_cast<double2*>(smem_ch);          // row i from (i, i) on
+    double2* tcol = R + packed_row(b, b);                      // one column per warp
+    double* inv = reinterpret_cast<double*>(tcol + 8 * b);     // 1 / R_ii
+    __shared__ double piv[2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int rank = (int)cluster_rank();
+    for (int i = rank; i < b; i += 8)
+        for (int q = i + threadIdx.x; q < b; q += 256) R[packed_row(i, b) + q - i] = G[(long long)i * b + q];
+    cluster_barrier();   // every CTA has started before the first remote store
+    for (int j = 0; j < b; ++j) {
+        double2* Rj = R + packed_row(j, b);
+        if (j % 8 == rank) {
+            if (threadIdx.x == 0) {
+                double d = Rj[0].x;
+                if (!(d > 0.0)) {
+                    *status = 1;
+                    d = 1e-300;
+                }
+                piv[0] = sqrt(d);
+                piv[1] = 1.0 / piv[0];
+            }
+            __syncthreads();
+            const double rd = piv[0], id = piv[1];
+            // warp r sends the row to CTA r; this CTA keeps it after all warps have read it
+            for (int q = lane; q < b - j; q += 32) {
+                const double2 v = q == 0 ? make_double2(rd, 0.0) : make_double2(Rj[q].x * id, Rj[q].y * id);
+                if (wid != rank) cluster_store(cluster_map(Rj + q, wid), v);
+            }
+            if (lane == 0) cluster_store(cluster_map(inv + j, wid), id);
+            __syncthreads();
+            for (int q = threadIdx.x; q < b - j; q += 256)
+                Rj[q] = q == 0 ? make_double2(rd, 0.0) : make_double2(Rj[q].x * id, Rj[q].y * id);
+        }
+        cluster_barrier();
+        // own rows p > j: a warp per row
+        int p0 = (j + 1) / 8 * 8 + rank;
+        if (p0 <= j) p0 += 8;
+        for (int p = p0 + 8 * wid; p < b; p += 64) {
+            double2* Rp = R + packed_row(p, b);
+            const double2 gp = Rj[p - j];
+            for (int q = p + lane; q < b; q += 32) {
+                const double2 gq = Rj[q - j];
+                double2 v = Rp[q - p];
+                v.x = fma(-gp.x, gq.x, fma(-gp.y, gq.y, v.x));
+                v.y = fma(-gp.x, gq.y, fma(gp.y, gq.x, v.y));
+                Rp[q - p] = v;
+            }
+        }
+        __syncthreads();
+    }
+    // column c of R^{-1}: back substitution by one warp
+    double2* t = tcol + wid * b;
+    for (int c = wid * 8 + rank; c < b; c += 64) {
+        for (int i = c; i >= 0; --i) {
+            const double2* Ri = R + packed_row(i, b);
+            double sr = 0.0, si = 0.0;
+            for (int k = i + 1 + lane; k <= c; k += 32) {
+                const double2 r = Ri[k - i], tk = t[k];
+                sr += r.x * tk.x - r.y * tk.y;
+                si += r.x * tk.y + r.y * tk.x;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sr += __shfl_xor_sync(0xffffffffu, sr, o);
+                si += __shfl_xor_sync(0xffffffffu, si, o);
+            }
+            if (lane == 0) t[i] = make_double2(((i == c ? 1.0 : 0.0) - sr) * inv[i], -si * inv[i]);
+            __syncwarp();
+        }
+        for (int i = lane; i < b; i += 32) Rinv[(long long)i * b + c] = i <= c ? t[i] : make_double2(0.0, 0.0);
+        __syncwarp();
+    }
+}
+
 __global__ void k_flag(const jac::Sync* sy, int* err) {
     if (grid_dependency()) return;
     if (err && sy->err) *err = 1;
@@ -1128,6 +1214,14 @@ size_t cholesky_work_bytes(int b) { return 2 * (size_t)b * b * sizeof(double2) +
 
 void launch_cholesky_inv(double2* G, double2* Rinv, int b, void* work, int* status, int* err, cudaStream_t s) {
     MG_REQUIRE(b >= 1 && b <= 4096, MGMLMC_EINVAL, "cholesky: 1 <= b <= 4096");
+    // to the size whose triangle fits one SM's shared memory the cluster has the cheaper barrier
+    if (b <= chol::kClusterMax) {
+        MG_CUDA(cudaFuncSetAttribute(chol::k_cholesky_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)chol::cluster_smem(chol::kClusterMax)));
+        chol::k_cholesky_cluster<<<8, 256, chol::cluster_smem(b), s>>>(G, Rinv, b, status);
+        MG_LAUNCHED();
+        return;
+    }
     // one CTA per SM, or one per warp of the trailing update where there are fewer
     const int NB = (int)std::min((long long)jacobi_grid_size(), std::max(1LL, ((long long)b * b + 63) / 64));
     double2* R = reinterpret_cast<double2*>(work);

@@ -1,6 +1,6 @@
 """The deflation eigensolver's dense pieces at the block sizes where their work splits:
 rotations formed by every CTA (blocks of up to 128) or once for all, odd blocks, blocks of
-fewer items than SMs."""
+fewer items than SMs, the Cholesky factor in a cluster (up to 144) or over the grid."""
 import numpy as np
 import pytest
 
@@ -17,8 +17,8 @@ def pkg():
     return require_gpu()
 
 
-# the block holds max(2k, k + 16) vectors (at most n): 17, 24, 66, 128, 130, 180
-@pytest.mark.parametrize("k", [1, 8, 33, 64, 65, 90])
+# the block holds max(2k, k + 16) vectors (at most n): 17, 24, 66, 128, 130, 144, 146, 180
+@pytest.mark.parametrize("k", [1, 8, 33, 64, 65, 72, 73, 90])
 def test_triplets(pkg, k):
     agg, nvec, m0 = ((2, 2), (2, 2)), (2, 4), 0.05
     theta, sv = small_problem(32, 24, 3.0, m0, agg, nvec)
