@@ -123,6 +123,66 @@ template <typename C> __host__ __device__ __forceinline__ C ctimesi(C a) { retur
 
 __host__ __device__ __forceinline__ double2 to_d(float2 a) { return make_double2(a.x, a.y); }
 __host__ __device__ __forceinline__ double2 to_d(double2 a) { return a; }
+
+// ---- sums across threads: FP32 values as pairs, FP64 values plainly
+struct PairF {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float s = h + v, b = s - h;
+        l += (h - (s - b)) + (v - b);
+        h = s;
+    }
+    __device__ __forceinline__ void add(const PairF& o) {
+        add(o.h);
+        l += o.l;
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+struct SumD {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double a) { v += a; }
+    __device__ __forceinline__ void add(const SumD& o) { v += o.v; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <typename R> struct SumOf;
+template <> struct SumOf<float> { using T = PairF; };
+template <> struct SumOf<double> { using T = SumD; };
+template <typename C> using sum_t = typename SumOf<re_t<C>>::T;
+template <typename C> struct alignas(16) CSum { sum_t<C> re, im; };   // 16 B in both precisions
+static_assert(sizeof(CSum<float2>) == 16 && sizeof(CSum<double2>) == 16, "partials are 16 bytes");
+
+__device__ __forceinline__ void warp_sum(PairF& v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        PairF w;
+        w.h = __shfl_down_sync(0xffffffffu, v.h, o);
+        w.l = __shfl_down_sync(0xffffffffu, v.l, o);
+        v.add(w);
+    }
+}
+__device__ __forceinline__ void warp_sum(SumD& v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v.v += __shfl_down_sync(0xffffffffu, v.v, o);
+}
+
+// A thread's share of a stencil's dots as a partial of 16 bytes (FP32: CSum's layout), and
+// their sums: FP64 adds and conversions run at 1/64 of the FP32 rate, and one CTA's epilogue
+// of them took longer than its sites where the lattice is small.
+__device__ __forceinline__ float4 dot_part(float2 v) { return make_float4(v.x, 0.f, v.y, 0.f); }
+__device__ __forceinline__ double2 dot_part(double2 v) { return v; }
+__device__ __forceinline__ float4 dot_part(float v) { return make_float4(v, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ double2 dot_part(double v) { return make_double2(v, 0.0); }
+__device__ __forceinline__ float4 dot_add(float4 a, float4 b) {
+    PairF x{a.x, a.y}, y{a.z, a.w};
+    x.add(PairF{b.x, b.y});
+    y.add(PairF{b.z, b.w});
+    return make_float4(x.h, x.l, y.h, y.l);
+}
+__device__ __forceinline__ double2 dot_add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+template <typename C> using dot_t = decltype(dot_part(C()));
+template <typename C> __device__ __forceinline__ dot_t<C>* dot_parts(double2* part) {
+    return reinterpret_cast<dot_t<C>*>(part);
+}
 template <typename C> __host__ __device__ __forceinline__ C cvt(double2 a);
 template <> __host__ __device__ __forceinline__ double2 cvt<double2>(double2 a) { return a; }
 template <> __host__ __device__ __forceinline__ float2 cvt<float2>(double2 a) { return make_float2((float)a.x, (float)a.y); }

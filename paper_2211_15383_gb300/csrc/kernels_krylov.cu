@@ -24,33 +24,6 @@ namespace kr {
 
 using u64 = unsigned long long;
 
-// ---- sums across threads: FP32 values as pairs, FP64 values plainly
-struct PairF {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float s = h + v, b = s - h;
-        l += (h - (s - b)) + (v - b);
-        h = s;
-    }
-    __device__ __forceinline__ void add(const PairF& o) {
-        add(o.h);
-        l += o.l;
-    }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
-struct SumD {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double a) { v += a; }
-    __device__ __forceinline__ void add(const SumD& o) { v += o.v; }
-    __device__ __forceinline__ double value() const { return v; }
-};
-template <typename R> struct SumOf;
-template <> struct SumOf<float> { using T = PairF; };
-template <> struct SumOf<double> { using T = SumD; };
-template <typename C> using sum_t = typename SumOf<re_t<C>>::T;
-template <typename C> struct alignas(16) CSum { sum_t<C> re, im; };   // 16 B in both precisions
-static_assert(sizeof(CSum<float2>) == 16 && sizeof(CSum<double2>) == 16, "partials are 16 bytes");
-
 template <typename C, int V> struct alignas(sizeof(C) * V) Vec { C v[V]; };
 
 // A block is bx x by threads: bx (a power of two, at most 32) covers the N / V columns, by

@@ -91,14 +91,14 @@ __global__ void __launch_bounds__(256) k_wilson(C* __restrict__ y, const C* __re
         }
     }
     if (MODE >= 2) {
-        __shared__ double2 sh[2][kRowLanes][kRhsTile + 1];
-        sh[0][threadIdx.y][threadIdx.x] = to_d(dyx);
-        sh[1][threadIdx.y][threadIdx.x] = make_double2((double)dyy, 0.0);
+        __shared__ dot_t<C> sh[2][kRowLanes][kRhsTile + 1];
+        sh[0][threadIdx.y][threadIdx.x] = dot_part(dyx);
+        sh[1][threadIdx.y][threadIdx.x] = dot_part(dyy);
         __syncthreads();
         if (threadIdx.y < 2 && j < N) {
-            double2 s = sh[threadIdx.y][0][threadIdx.x];
-            for (int r = 1; r < kRowLanes; ++r) s = cadd(s, sh[threadIdx.y][r][threadIdx.x]);
-            part[((long long)threadIdx.y * N + j) * gridDim.y + blockIdx.y] = s;
+            dot_t<C> s = sh[threadIdx.y][0][threadIdx.x];
+            for (int r = 1; r < kRowLanes; ++r) s = dot_add(s, sh[threadIdx.y][r][threadIdx.x]);
+            dot_parts<C>(part)[((long long)threadIdx.y * N + j) * gridDim.y + blockIdx.y] = s;
         }
     }
 }
@@ -159,15 +159,15 @@ __global__ void __launch_bounds__(256) k_block_stencil(C* __restrict__ y, const 
     }
     if (MODE >= 2) {
         __syncthreads();
-        double2* sh = reinterpret_cast<double2*>(smem_raw);   // reuse: [2][8][33]
-        sh[(0 * kRowLanes + threadIdx.y) * (kRhsTile + 1) + threadIdx.x] = to_d(dyx);
-        sh[(1 * kRowLanes + threadIdx.y) * (kRhsTile + 1) + threadIdx.x] = make_double2((double)dyy, 0.0);
+        dot_t<C>* sh = reinterpret_cast<dot_t<C>*>(smem_raw);   // reuse: [2][8][33]
+        sh[(0 * kRowLanes + threadIdx.y) * (kRhsTile + 1) + threadIdx.x] = dot_part(dyx);
+        sh[(1 * kRowLanes + threadIdx.y) * (kRhsTile + 1) + threadIdx.x] = dot_part(dyy);
         __syncthreads();
         if (threadIdx.y < 2 && j < N) {
-            double2 s = sh[(threadIdx.y * kRowLanes) * (kRhsTile + 1) + threadIdx.x];
+            dot_t<C> s = sh[(threadIdx.y * kRowLanes) * (kRhsTile + 1) + threadIdx.x];
             for (int r = 1; r < kRowLanes; ++r)
-                s = cadd(s, sh[(threadIdx.y * kRowLanes + r) * (kRhsTile + 1) + threadIdx.x]);
-            part[((long long)threadIdx.y * N + j) * gridDim.y + blockIdx.y] = s;
+                s = dot_add(s, sh[(threadIdx.y * kRowLanes + r) * (kRhsTile + 1) + threadIdx.x]);
+            dot_parts<C>(part)[((long long)threadIdx.y * N + j) * gridDim.y + blockIdx.y] = s;
         }
     }
 }
@@ -227,8 +227,8 @@ __global__ void __launch_bounds__(128) k_block_stencil_d(C* __restrict__ y, cons
     if (MODE >= 2) {
         // per-rhs partials: one thread per rhs, no cross-thread reduction needed
         if (j < N) {
-            part[((long long)0 * N + j) * gridDim.y + blockIdx.y] = to_d(dyx);
-            part[((long long)1 * N + j) * gridDim.y + blockIdx.y] = make_double2((double)dyy, 0.0);
+            dot_parts<C>(part)[((long long)0 * N + j) * gridDim.y + blockIdx.y] = dot_part(dyx);
+            dot_parts<C>(part)[((long long)1 * N + j) * gridDim.y + blockIdx.y] = dot_part(dyy);
         }
     }
 }
@@ -303,10 +303,10 @@ __global__ void __launch_bounds__(128) k_block_stencil_f2(float2* __restrict__ y
     }
     if (MODE >= 2 && j < N) {
         const long long G = gridDim.y;
-        part[((long long)0 * N + j) * G + blockIdx.y] = to_d(dyx0);
-        part[((long long)0 * N + j + 1) * G + blockIdx.y] = to_d(dyx1);
-        part[((long long)1 * N + j) * G + blockIdx.y] = make_double2((double)dyy0, 0.0);
-        part[((long long)1 * N + j + 1) * G + blockIdx.y] = make_double2((double)dyy1, 0.0);
+        dot_parts<float2>(part)[((long long)0 * N + j) * G + blockIdx.y] = dot_part(dyx0);
+        dot_parts<float2>(part)[((long long)0 * N + j + 1) * G + blockIdx.y] = dot_part(dyx1);
+        dot_parts<float2>(part)[((long long)1 * N + j) * G + blockIdx.y] = dot_part(dyy0);
+        dot_parts<float2>(part)[((long long)1 * N + j + 1) * G + blockIdx.y] = dot_part(dyy1);
     }
 }
 
@@ -419,9 +419,9 @@ __global__ void __launch_bounds__(128) k_block_stencil_f4(float2* __restrict__ y
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const float2 s = make_float2(dyx[r].x + red[tq * 12 + 3 * r], dyx[r].y + red[tq * 12 + 3 * r + 1]);
-                part[((long long)0 * N + j + r) * G + blockIdx.y] = to_d(s);
-                part[((long long)1 * N + j + r) * G + blockIdx.y] =
-                    make_double2((double)(dyy[r] + red[tq * 12 + 3 * r + 2]), 0.0);
+                dot_parts<float2>(part)[((long long)0 * N + j + r) * G + blockIdx.y] = dot_part(s);
+                dot_parts<float2>(part)[((long long)1 * N + j + r) * G + blockIdx.y] =
+                    dot_part(dyy[r] + red[tq * 12 + 3 * r + 2]);
             }
         }
     }
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
     if (grid_dependency()) return;
     using R = re_t<C>;
     __shared__ C As[5 * D * (D + 1)];             // rows padded: the four rows of a warp in different banks
-    __shared__ double2 red[2][D][8];
+    __shared__ dot_t<C> red[2][D][8];
     const int tx = threadIdx.x, c = threadIdx.y, tid = c * 8 + tx;
     const int j = blockIdx.x * 8 + tx;
     const int V = lx * lt;
@@ -480,13 +480,13 @@ __global__ void __launch_bounds__(8 * D) k_block_stencil_narrow(C* __restrict__ 
         }
     }
     if (MODE >= 2) {
-        red[0][c][tx] = to_d(dyx);
-        red[1][c][tx] = make_double2((double)dyy, 0.0);
+        red[0][c][tx] = dot_part(dyx);
+        red[1][c][tx] = dot_part(dyy);
         __syncthreads();
         if (c < 2 && j < N) {
-            double2 s2 = red[c][0][tx];
-            for (int r = 1; r < D; ++r) s2 = cadd(s2, red[c][r][tx]);
-            part[((long long)c * N + j) * gridDim.y + blockIdx.y] = s2;
+            dot_t<C> s2 = red[c][0][tx];
+            for (int r = 1; r < D; ++r) s2 = dot_add(s2, red[c][r][tx]);
+            dot_parts<C>(part)[((long long)c * N + j) * gridDim.y + blockIdx.y] = s2;
         }
     }
 }
@@ -1131,20 +1131,20 @@ __global__ void __launch_bounds__(256) k_wilson_f2(float2* __restrict__ y, const
         }
     }
     if (MODE == 2 || MODE == 3) {
-        __shared__ double2 sh[2][kRowLanes][2 * kRhsTile + 1];
+        __shared__ float4 sh[2][kRowLanes][2 * kRhsTile + 1];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            sh[0][threadIdx.y][2 * threadIdx.x + r] = to_d(dyx[r]);
-            sh[1][threadIdx.y][2 * threadIdx.x + r] = make_double2((double)dyy[r], 0.0);
+            sh[0][threadIdx.y][2 * threadIdx.x + r] = dot_part(dyx[r]);
+            sh[1][threadIdx.y][2 * threadIdx.x + r] = dot_part(dyy[r]);
         }
         __syncthreads();
         // 64 rhs x 2 quantities: threads (x, y < 4) add the 8 row lanes of one each
         const int q = threadIdx.y >> 1, jj = 2 * threadIdx.x + (threadIdx.y & 1);
         const int jo = 2 * blockIdx.x * kRhsTile + jj;
         if (threadIdx.y < 4 && jo < N) {
-            double2 acc = sh[q][0][jj];
-            for (int r = 1; r < kRowLanes; ++r) acc = cadd(acc, sh[q][r][jj]);
-            part[((long long)q * N + jo) * gridDim.y + blockIdx.y] = acc;
+            float4 acc = sh[q][0][jj];
+            for (int r = 1; r < kRowLanes; ++r) acc = dot_add(acc, sh[q][r][jj]);
+            dot_parts<float2>(part)[((long long)q * N + jo) * gridDim.y + blockIdx.y] = acc;
         }
     }
 }
@@ -1269,11 +1269,11 @@ __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y
             }
         }
     }
-    __shared__ double2 sh[2][kRowLanes][RPT * kRhsTile + 1];
+    __shared__ float4 sh[2][kRowLanes][RPT * kRhsTile + 1];
 #pragma unroll
     for (int r = 0; r < RPT; ++r) {
-        sh[0][threadIdx.y][RPT * threadIdx.x + r] = to_d(dyx[r]);
-        sh[1][threadIdx.y][RPT * threadIdx.x + r] = make_double2((double)dyy[r], 0.0);
+        sh[0][threadIdx.y][RPT * threadIdx.x + r] = dot_part(dyx[r]);
+        sh[1][threadIdx.y][RPT * threadIdx.x + r] = dot_part(dyy[r]);
     }
     __syncthreads();
     // RPT * 32 rhs x 2 quantities: thread t < 2 * RPT * 32 adds the 8 row lanes of
@@ -1283,9 +1283,9 @@ __global__ void __launch_bounds__(256, 3) k_wilson_bf16(uint32_t* __restrict__ y
         const int q = t / (RPT * kRhsTile), jj = t % (RPT * kRhsTile);
         const int jo = RPT * blockIdx.x * kRhsTile + jj;
         if (jo < N) {
-            double2 acc = sh[q][0][jj];
-            for (int r = 1; r < kRowLanes; ++r) acc = cadd(acc, sh[q][r][jj]);
-            part[((long long)q * N + jo) * gridDim.y + blockIdx.y] = acc;
+            float4 acc = sh[q][0][jj];
+            for (int r = 1; r < kRowLanes; ++r) acc = dot_add(acc, sh[q][r][jj]);
+            dot_parts<float2>(part)[((long long)q * N + jo) * gridDim.y + blockIdx.y] = acc;
         }
     }
 }

@@ -902,8 +902,8 @@ __global__ void __launch_bounds__(THREADS, kCtasPerSm)
             }
         }
         if (FORM != 2 && ok && j < N) {
-            part[((long long)0 * N + j) * G + blockIdx.x] = make_double2((double)dyx.x, (double)dyx.y);
-            part[((long long)1 * N + j) * G + blockIdx.x] = make_double2((double)dyy, 0.0);
+            dot_parts<float2>(part)[((long long)0 * N + j) * G + blockIdx.x] = dot_part(dyx);
+            dot_parts<float2>(part)[((long long)1 * N + j) * G + blockIdx.x] = dot_part(dyy);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");

@@ -187,38 +187,56 @@ void launch_axpy_rhs(Cy* y, const double2* alpha, const double* beta, double sig
 int reduce_groups(long long n, int N) { return row_groups(n, N, 4); }
 // The minimal-residual coefficient of every rhs from the row-major partials of its two
 // dots (part[i * groups + g]): alpha_j = <y, x>_j / <y, y>_j (0 where <y, y> is 0).  One block
-// per rhs, fixed order.  The quotient is taken here, once per rhs: FP64 runs at 1/64 of the
-// FP32 rate, and a division in the prologue of every thread of the update kernels was most
-// of those kernels' time on small blocks (15 us for 4 MB, 8192 rows x 16 rhs).
+// per rhs, fixed order; FP32 dots are added as pairs, since FP64 adds run at 1/64 of the FP32
+// rate (8 rhs of a 64^2 lattice: 4.0 -> 2.7 us; the stencil before it 4.4 -> 3.3).  The quotient
+// is taken here, once per rhs: a division in the prologue of every thread of the update kernels
+// was most of those kernels' time on small blocks (15 us for 4 MB, 8192 rows x 16 rhs).
 template <typename C>
 __global__ void __launch_bounds__(128) k_finalize_alpha(C* __restrict__ alpha, const double2* __restrict__ part,
                                                         int groups, int N) {
     if (grid_dependency()) return;
-    __shared__ double sh[3][4];
+    using S = sum_t<C>;
+    __shared__ double2 sh[3][4];                       // 16-byte slots, S in each
     const int j = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const double2* r0 = part + (long long)j * groups;
-    const double2* r1 = part + (long long)(N + j) * groups;
-    double v[3] = {0.0, 0.0, 0.0};
+    const CSum<C>* r0 = reinterpret_cast<const CSum<C>*>(part) + (long long)j * groups;
+    const CSum<C>* r1 = reinterpret_cast<const CSum<C>*>(part) + (long long)(N + j) * groups;
+    constexpr int U = sizeof(C) == 8 ? 4 : 1;
+    S v[3];
 #pragma unroll 4
-    for (int g = threadIdx.x; g < groups; g += 128) {
-        const double2 a = r0[g];
-        v[0] += a.x;
-        v[1] += a.y;
-        v[2] += r1[g].x;
+    for (int g0 = threadIdx.x; g0 < groups; g0 += U * 128) {
+        CSum<C> a[U];
+        S b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (g0 + 128 * u < groups) {
+                a[u] = r0[g0 + 128 * u];
+                b[u] = r1[g0 + 128 * u].re;
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (g0 + 128 * u < groups) {
+                v[0].add(a[u].re);
+                v[1].add(a[u].im);
+                v[2].add(b[u]);
+            }
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-        if (lane == 0) sh[q][wid] = v[q];
+        warp_sum(v[q]);
+        if (lane == 0) *reinterpret_cast<S*>(&sh[q][wid]) = v[q];
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const double x = (sh[0][0] + sh[0][1]) + (sh[0][2] + sh[0][3]);
-        const double y = (sh[1][0] + sh[1][1]) + (sh[1][2] + sh[1][3]);
-        const double b = (sh[2][0] + sh[2][1]) + (sh[2][2] + sh[2][3]);
-        const double ib = b > 0.0 ? 1.0 / b : 0.0;
-        alpha[j] = cvt<C>(make_double2(x * ib, y * ib));
+        double t[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            S s = *reinterpret_cast<const S*>(&sh[q][0]);
+#pragma unroll
+            for (int w = 1; w < 4; ++w) s.add(*reinterpret_cast<const S*>(&sh[q][w]));
+            t[q] = s.value();
+        }
+        const double ib = t[2] > 0.0 ? 1.0 / t[2] : 0.0;
+        alpha[j] = cvt<C>(make_double2(t[0] * ib, t[1] * ib));
     }
 }
 
