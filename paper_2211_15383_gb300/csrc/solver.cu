@@ -245,9 +245,10 @@ template <> void coarsest_apply<double2>(Ctx& c, double2* e, const double2* r, i
 }
 template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int N) {
     const Level& L = c.lev[c.L - 1];
-    // few right-hand sides of a small level: the FP32 inverse in one launch (4 us at n = 256,
-    // 9 us at n = 1024, against 12 us of the tensor-core form's three; at twice that size
-    // reading four times the FP32 inverse takes longer)
+    // few right-hand sides of a small level: the FP32 inverse in one launch (4 us at n = 256;
+    // at n = 1024 9 us for 8 rhs and 15 for 16, against 12 us of the tensor-core form's three,
+    // whose BF16 digits cost outer iterations; at twice that size reading four times the FP32
+    // inverse takes longer)
     if (N < kFewRhs && L.n <= kFewRhsUnknowns) {
         ProfScope ps(c, "Dinv.f32", dinv_bytes(L, N, 8), dinv_flops(L, N));
         launch_gemm_few(e, L.Dinv32, r, (int)L.n, N, c.stream);
