@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
         const int r = e / B, c = e % B;
         P[e] = c < kb ? A[(long long)(row0 + r) * n + k0 + c] : czero<C>();
     }
-    __syncthreads();
+    cluster_barrier();   // the panel is loaded, and every CTA has started before the first remote store
     // the CTA's candidate (value, local row) from per-thread ones: lane 0 of every warp, then warp 0
     auto reduce = [&](T bv, int bi) {
 #pragma unroll
