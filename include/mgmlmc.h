@@ -311,7 +311,8 @@ int mgmlmc_estimate_trace_concurrent(mgmlmc_ctx* const* contexts, int n, double 
 int mgmlmc_apply(mgmlmc_ctx* ctx, int op, int level, int nrhs, const double* x, double* y);
 
 /* Solve D_l x = b for nrhs host vectors [nrhs][n_l] with the outer FGMRES to
- * opt.solve_tol; *iters (may be NULL) receives the outer iteration count. */
+ * opt.solve_tol; *iters (may be NULL) receives the outer iteration count.
+ * MGMLMC_ENAN if a right-hand side holds a NaN or an infinity. */
 int mgmlmc_solve(mgmlmc_ctx* ctx, int level, int nrhs, const double* b, double* x, int* iters);
 
 /* Test hook: the Z2 vectors of mgmlmc_estimate_level as doubles [nsamples][n_l]. */

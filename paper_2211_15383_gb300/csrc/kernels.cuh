@@ -54,7 +54,7 @@ void launch_dot(double2* out, const Cx_* x, const Cy* y, long long n, int N, dou
 // What a norm's reduction writes besides, per rhs (any pointer may be null).
 struct NormOut {
     double* norm = nullptr;                  // the norm
-    // *max = max(*max, norm mul / den) over the rhs with den > 0 (den null: norm / norm), as the
+    // *max = max(*max, norm mul / den) over the rhs with den != 0 (den null: norm / norm), as the
     // bits of a double (NaN is the largest); *clear = 0 for a later use
     unsigned long long* max = nullptr;
     unsigned long long* clear = nullptr;

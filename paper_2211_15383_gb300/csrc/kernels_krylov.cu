@@ -381,7 +381,8 @@ __global__ void __launch_bounds__(256) k_finalize_norm(NormOut o, const S* __res
     if (o.norm) o.norm[r] = v;
     if (o.max) {
         const double d = o.den ? o.den[r] : v;
-        atomic_max_double(o.max, d > 0.0 ? (o.mul ? v * o.mul[r] : v) / d : 0.0);
+        // a zero right-hand side is solved; a NaN on either side is the maximum
+        atomic_max_double(o.max, d == 0.0 ? 0.0 : (o.mul ? v * o.mul[r] : v) / d);
     }
     if (o.eta) {
         double en = v;
@@ -477,7 +478,7 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
     }
     if (max || host) {
         const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid, bn = in ? bnorm[r] : 0.0;
-        const double v = bn > 0.0 ? rs / bn : 0.0;
+        const double v = bn == 0.0 ? 0.0 : rs / bn;
         if (host) {
             u64 m8 = (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 #pragma unroll
