@@ -728,9 +728,12 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
             } else {
                 float2* x32 = c.scratch<float2>("ap_x32", (size_t)nin * nrhs);
                 float2* y32 = c.scratch<float2>("ap_y32", (size_t)nout * nrhs);
-                mg::launch_convert<float2, double2>(x32, xt, nin * nrhs, c.stream);
+                // the cycle's FP32 sums of squares have FP32's range: columns of unit scale
+                auto* mx = c.scratch<unsigned long long>("unit_mx", nrhs);
+                mg::launch_absmax_cols(mx, xt, nin, nrhs, c.stream);
+                mg::launch_to_unit(x32, xt, mx, nin, nrhs, c.stream);
                 mg::mg_cycle<float2>(c, l, y32, x32, nrhs);
-                mg::launch_convert<double2, float2>(yt, y32, nout * nrhs, c.stream);
+                mg::launch_from_unit(yt, y32, mx, nout, nrhs, c.stream);
             }
     }
     mg::check_device_error(c);

@@ -39,6 +39,11 @@ void launch_scale_rhs(Cy* y, const Cx_* x, const double* scale, bool invert, lon
 template <typename Cy, typename Cx_>
 void launch_axpy_rhs(Cy* y, const double2* alpha, const double* beta, double sign, const Cx_* x,
                      long long n, int N, cudaStream_t s);
+// out[j] = bits of the largest |re|, |im| of column j; and between FP64 blocks of any scale and
+// FP32 blocks whose columns have that entry in [1/2, 1): y = 2^-e_j x and y = 2^e_j x, exact.
+void launch_absmax_cols(unsigned long long* out, const double2* x, long long n, int N, cudaStream_t s);
+void launch_to_unit(float2* y, const double2* x, const unsigned long long* mx, long long n, int N, cudaStream_t s);
+void launch_from_unit(double2* y, const float2* x, const unsigned long long* mx, long long n, int N, cudaStream_t s);
 template <typename C>
 void launch_zero(C* x, long long count, cudaStream_t s);
 // out[c][r] = in[r][c] (rows x cols complex, row-major)

@@ -81,9 +81,8 @@ __device__ __forceinline__ uint32_t pack_exact(float lo, float hi) {
     return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-// Largest |re|, |im| per rhs (cols > 1) or of everything (cols == 1: count values of a flat
-// array), as the bit pattern of the double: non-negative doubles order like integers, NaN
-// above all, so the atomic maximum does not depend on the order.
+// Largest |re|, |im| per column, as the bit pattern of the double: non-negative doubles order
+// like integers, NaN above all, so the atomic maximum does not depend on the order.
 __global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, const double2* __restrict__ x,
                                                      long long n, int N) {
     if (grid_dependency()) return;
@@ -458,7 +457,7 @@ size_t f64_tc_scratch_bytes(long long nblk, int N) {
 }
 int f64_dense_splits(int n) { return (n / D + KSPLIT - 1) / KSPLIT; }
 
-static void absmax(u64* out, const double2* x, long long n, int N, cudaStream_t s) {
+void launch_absmax_cols(u64* out, const double2* x, long long n, int N, cudaStream_t s) {
     MG_CUDA(cudaMemsetAsync(out, 0, sizeof(u64) * N, s));
     int bx = 1;
     while (bx < N && bx < 32) bx *= 2;
@@ -478,7 +477,7 @@ void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int 
     MG_REQUIRE(nblk >= 1 && nblk <= (1LL << 31) - 1, MGMLMC_EINVAL, "FP64 operand: size");
     u64* mx = const_cast<u64*>(operand_max(op, nblk));
     // a flat array as 32 columns: the maximum of its 32 column maxima is taken below
-    absmax(mx, A, nblk * (D * D) / 32, 32, s);
+    launch_absmax_cols(mx, A, nblk * (D * D) / 32, 32, s);
     MG_LAUNCH(1, dim3(1, 32), 0, s, tc::f64::k_absmax_cols, mx, reinterpret_cast<const double2*>(mx), 16, 1);
     MG_LAUNCHED();
     MG_LAUNCH((unsigned)nblk, 128, 0, s, k_slice_a, reinterpret_cast<uint8_t*>(op), A, mx, nblk, nb, nb ? ld : D);
@@ -489,7 +488,7 @@ void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int 
 static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N, cudaStream_t s) {
     const int T = f64_tiles(N);
     u64* mx = reinterpret_cast<u64*>(reinterpret_cast<uint8_t*>(scratch) + (size_t)nblk * T * XT);
-    absmax(mx, x, nblk * D, N, s);
+    launch_absmax_cols(mx, x, nblk * D, N, s);
     int bx = 8;
     while (bx < N && bx < 128) bx *= 2;
     const int by = 128 / bx;

@@ -53,6 +53,34 @@ __global__ void k_convert(Cout* __restrict__ y, const Cin* __restrict__ x, long 
         y[i] = cvtc(x[i], Cout());
 }
 
+// Exponent e of a column's largest entry (in [2^(e-1), 2^e)); 0 for a zero or non-finite one.
+__device__ __forceinline__ int unit_exponent(unsigned long long mx) {
+    const int E = (int)(mx >> 52);
+    return (mx == 0 || E == 0x7ff) ? 0 : E - 1022;
+}
+__global__ void k_to_unit(float2* __restrict__ y, const double2* __restrict__ x, const unsigned long long* __restrict__ mx,
+                          long long n, int N) {
+    if (grid_dependency()) return;
+    const int j = blockIdx.x * kRhsTile + threadIdx.x;
+    if (j >= N) return;
+    const int e = unit_exponent(mx[j]);
+    for (long long i = (long long)blockIdx.y * kRowLanes + threadIdx.y; i < n; i += (long long)gridDim.y * kRowLanes) {
+        const double2 v = x[i * N + j];
+        y[i * N + j] = make_float2((float)ldexp(v.x, -e), (float)ldexp(v.y, -e));
+    }
+}
+__global__ void k_from_unit(double2* __restrict__ y, const float2* __restrict__ x,
+                            const unsigned long long* __restrict__ mx, long long n, int N) {
+    if (grid_dependency()) return;
+    const int j = blockIdx.x * kRhsTile + threadIdx.x;
+    if (j >= N) return;
+    const int e = unit_exponent(mx[j]);
+    for (long long i = (long long)blockIdx.y * kRowLanes + threadIdx.y; i < n; i += (long long)gridDim.y * kRowLanes) {
+        const float2 v = x[i * N + j];
+        y[i * N + j] = make_double2(ldexp((double)v.x, e), ldexp((double)v.y, e));
+    }
+}
+
 template <typename C>
 __global__ void k_zero(C* __restrict__ x, long long count) {
     if (grid_dependency()) return;
@@ -162,6 +190,14 @@ void launch_convert(Cout* y, const Cin* x, long long count, cudaStream_t s) {
     long long b = (count + 255) / 256;
     if (b > kNumSM * 16) b = kNumSM * 16;
     MG_LAUNCH((int)b, 256, 0, s, (k_convert<Cout, Cin>), y, x, count);
+    MG_LAUNCHED();
+}
+void launch_to_unit(float2* y, const double2* x, const unsigned long long* mx, long long n, int N, cudaStream_t s) {
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, k_to_unit, y, x, mx, n, N);
+    MG_LAUNCHED();
+}
+void launch_from_unit(double2* y, const float2* x, const unsigned long long* mx, long long n, int N, cudaStream_t s) {
+    MG_LAUNCH(dim3(rhs_tiles(N), row_groups(n, N)), blk(), 0, s, k_from_unit, y, x, mx, n, N);
     MG_LAUNCHED();
 }
 template <typename C>

@@ -937,8 +937,11 @@ void approx_inverse(Ctx& c, int l, const double2* b, double2* x, int N) {
     const size_t nN = (size_t)c.lev[l].n * N;
     float2* b32 = c.scratch<float2>("ai_b32", nN);
     float2* x32 = c.scratch<float2>("ai_x32", nN);
-    launch_convert<float2, double2>(b32, b, (long long)nN, c.stream);
+    unsigned long long* mx = c.scratch<unsigned long long>("unit_mx", N);
+    const long long n = c.lev[l].n;
+    launch_absmax_cols(mx, b, n, N, c.stream);
+    launch_to_unit(b32, b, mx, n, N, c.stream);
     fgmres<float2>(c, l, b32, x32, N, 1e-6, c.opt.fgmres_restart, true, &ok, 1);
-    launch_convert<double2, float2>(x, x32, (long long)nN, c.stream);
+    launch_from_unit(x, x32, mx, n, N, c.stream);
 }
 }  // namespace mg
