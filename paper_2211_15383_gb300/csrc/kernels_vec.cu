@@ -271,7 +271,13 @@ __global__ void __launch_bounds__(128) k_finalize_alpha(C* __restrict__ alpha, c
             for (int w = 1; w < 4; ++w) s.add(*reinterpret_cast<const S*>(&sh[q][w]));
             t[q] = s.value();
         }
-        const double ib = t[2] > 0.0 ? 1.0 / t[2] : 0.0;
+        double ib = t[2] > 0.0 ? 1.0 / t[2] : 0.0;
+        if (sizeof(C) == 16 && t[2] > 0.0 && t[2] < 0x1p-1022) {
+            // FP64 vectors of norm 2^-511 and below: 1 / t overflows
+            t[0] *= 0x1p100;
+            t[1] *= 0x1p100;
+            ib = 1.0 / (t[2] * 0x1p100);
+        }
         alpha[j] = cvt<C>(make_double2(t[0] * ib, t[1] * ib));
     }
 }

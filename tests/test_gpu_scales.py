@@ -40,3 +40,17 @@ def test_start_vectors(pkg, prec):
     # each solve of the inverse iteration to 1e-13, its start only scaled
     for a, b in zip(*out):
         assert np.abs(a - b).max() < 1e-11 * np.abs(a).max()
+
+
+# |D r|^2 of a few hundred entries of 2^e: its reciprocal overflows, its own digits are few
+@pytest.mark.parametrize("e", [-508, -516, -520, -524])
+def test_fp64_cycle_of_tiny_vectors(pkg, e):
+    theta, sv = small_problem(16, 16, 3.0, M0, AGG, NVEC)
+    x = rand_complex(np.random.default_rng(3), (3, 512))
+    with make_ctx(pkg, theta, M0, AGG, NVEC, sv, 0, mg_precision=64) as ctx:
+        ref = ctx.apply(pkg.OP_PREC, 1, x, 512)
+        got = ctx.apply(pkg.OP_PREC, 1, np.ldexp(x.real, e) + 1j * np.ldexp(x.imag, e), 512)
+    got = np.ldexp(got.real, -e) + 1j * np.ldexp(got.imag, -e)
+    # squares of 2^(2e) on a grid of 2^-1074, a step down in scale per smoothing step
+    tol = max(1e-12, 64 * 2.0 ** (-1074 - 2 * e + 4))
+    assert np.abs(got - ref).max() <= tol * np.abs(ref).max()
