@@ -60,7 +60,7 @@ inline size_t footprint_bytes(const Shape& s) {
             if (bf16) b += st * d * d * 80;                                  // BF16 operand tiles
         }
         const bool digits = l > 0 && s.d[l] == 16;                           // FP64 products on the tensor cores
-        if (digits) b += st * 5 * 16384 * (f64 && l + 1 < L ? 2 : 1) + st * std::ceil(N / 128) * 65536;
+        if (digits) b += st * (5 * 16384 + 32) * (f64 && l + 1 < L ? 2 : 1) + st * (std::ceil(N / 128) * 65536 + N * 2);
         if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * (digits ? std::min(N, 16.0) : N) * 16;   // FP64 Galerkin apply
         if (l + 1 < L) {
             const double K = smoother_slots(s.nu);

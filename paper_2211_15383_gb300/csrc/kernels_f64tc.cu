@@ -6,8 +6,8 @@
 // T. Ogita, S. Oishi, S. M. Rump, "Error-free transformations of matrix multiplication by
 // using fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
 //
-//  * every rhs of x is scaled by a power of two 2^-ex with |x| < 2^ex (its largest entry), the
-//    matrix by one power of two, and both are rounded to 63 bits, x = 2^ex sum_{j<8} d_j 2^{-6-8j},
+//  * every rhs of x is scaled by a power of two 2^-ex with |x| < 2^ex (its largest entry), every
+//    row of the matrix likewise, and both are rounded to 63 bits, x = 2^ex sum_{j<8} d_j 2^{-6-8j},
 //    a = 2^ea sum_{i<8} c_i 2^{-6-8i}; all digits are integers in [-128, 127], exact in BF16;
 //  * G_g = sum_{i+j=g} sum_k c_i d_j for g = 0..8: products of digits are below 2^14, sums of
 //    at most 192 k and 5 pairs below 2^24, so the FP32 accumulation in TMEM is exact for the
@@ -15,11 +15,11 @@
 //    exact range by rounding their last place); the dropped pairs i + j > 8 weigh 2^-72;
 //  * sum_g G_g 2^-8g is formed in 128-bit integers and rounded to FP64 once.
 // The error of an entry is 2^-53 of itself from that rounding, and about 2^-63 of the rhs' largest
-// entry; 160 FP64 FMAs leave about 2^-51 of the entries around it.  In the norm the product is
-// closer to the exact one also where a rhs is concentrated on a few sites of the lattice (the
-// second part is spread over n entries: it stays below as long as n < 2^21 of the sites the rhs
-// is concentrated on).  With 7 digits of x and 8 groups (2^-55) that was not so: residuals
-// of near-critical 1024^2 solves, dominated by localised modes, stood at 1.9e-12.
+// entry; 160 FP64 FMAs leave about 2^-51 of the entries around it.  A site of the stencil whose
+// inputs all lie more than 2^8 below the rhs' largest entry would lose by that: its rows
+// are summed in FP64 (so are those next to an infinity or NaN, which stays where it is), and the
+// stencil is as accurate entry by entry as FP64 sums are.  With 7 digits of x and 8 groups
+// (2^-55) residuals of near-critical 1024^2 solves, dominated by localised modes, stood at 1.9e-12.
 //
 // Layout: the rhs are the MMA's M (128 rows of x digits, K = 32 reals of a site), the digits
 // of the block are its N: the 8 x 32 rows (i, output real) of a block's tile lie one after
@@ -59,10 +59,14 @@ constexpr int KSPLIT = 6;                  // K blocks of a dense job (exact sum
 using u64 = unsigned long long;
 using i64 = long long;
 
-// round(v 2^(62 - e)), |v| < 2^e, e = E - 1022 for the biased exponent E of the largest entry.
+constexpr u64 kNonFinite = 0x7FFull << 52;
+
+// round(v 2^(62 - e)), |v| < 2^e, e = E - 1022 for the biased exponent E of the largest entry; 0
+// for an infinity or NaN.
 __device__ __forceinline__ i64 fixed_point(double v, int E) {
     const u64 b = (u64)__double_as_longlong(v);
     const int eb = (int)((b >> 52) & 0x7ff);
+    if (eb > E && eb == 0x7ff) return 0;
     const u64 m = (b & 0xFFFFFFFFFFFFFull) | (eb ? 1ull << 52 : 0ull);
     // v = m 2^(max(eb, 1) - 1075); q = m 2^sh
     const int sh = (eb > 0 ? eb : 1) - 1075 + 62 - (E - 1022);
@@ -109,6 +113,90 @@ __global__ void __launch_bounds__(256) k_absmax_cols(u64* __restrict__ out, cons
     if (threadIdx.y == 0 && j < N && sh[threadIdx.x] != 0) atomicMax(out + j, sh[threadIdx.x]);
 }
 
+// The same over the finite entries of a stencil's input, and the exponent (biased) of the largest
+// entry of every site and rhs: 0 for zeros, 0x7ff where an entry is not finite.  Four threads
+// (threadIdx.y) per site and rhs.
+__global__ void __launch_bounds__(256) k_absmax_sites(u64* __restrict__ out, uint16_t* __restrict__ xe,
+                                                      const double2* __restrict__ x, int nsites, int N) {
+    if (grid_dependency()) return;
+    __shared__ u64 sh[256];
+    const int bx = blockDim.x, tid = threadIdx.y * bx + threadIdx.x, cg = threadIdx.y & 3;
+    const int j = blockIdx.x * bx + threadIdx.x;
+    const int per = blockDim.y / 4;                      // sites of a CTA at a time
+    u64 m = 0;
+    for (int s0 = blockIdx.y * per; s0 < nsites; s0 += gridDim.y * per) {
+        const int site = s0 + (threadIdx.y >> 2);
+        u64 s = 0;
+        if (j < N && site < nsites) {
+            double2 v[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[c] = x[((size_t)site * D + 4 * cg + c) * N + j];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                s = max(s, (u64)__double_as_longlong(v[c].x) & 0x7FFFFFFFFFFFFFFFull);
+                s = max(s, (u64)__double_as_longlong(v[c].y) & 0x7FFFFFFFFFFFFFFFull);
+            }
+            if (s >= kNonFinite) {
+                u64 f = 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const u64 a = (u64)__double_as_longlong(v[c].x) & 0x7FFFFFFFFFFFFFFFull;
+                    const u64 b = (u64)__double_as_longlong(v[c].y) & 0x7FFFFFFFFFFFFFFFull;
+                    f = max(f, max(a < kNonFinite ? a : 0, b < kNonFinite ? b : 0));
+                }
+                m = max(m, f);
+                s = kNonFinite;
+            } else {
+                m = max(m, s);
+            }
+        }
+        __syncthreads();
+        sh[tid] = s;
+        __syncthreads();
+        if (cg == 0 && j < N && site < nsites) {
+#pragma unroll
+            for (int q = 1; q < 4; ++q) s = max(s, sh[tid + q * bx]);
+            xe[(size_t)site * N + j] = (uint16_t)(s == 0 ? 0 : max((int)(s >> 52), 1));
+        }
+    }
+    __syncthreads();
+    sh[tid] = m;
+    __syncthreads();
+    for (int st = blockDim.y / 2; st > 0; st >>= 1) {
+        if ((int)threadIdx.y < st) sh[tid] = max(sh[tid], sh[tid + st * bx]);
+        __syncthreads();
+    }
+    if (threadIdx.y == 0 && j < N && sh[threadIdx.x] != 0) atomicMax(out + j, sh[threadIdx.x]);
+}
+
+// Exponent (biased) of the largest |re|, |im| of every row of a job's blocks: row c of the five
+// blocks of a site (nb = 0, rows of D), or of K blocks 6z .. of block row R of a dense matrix (nb
+// blocks per row, rows ld apart, job = R splits + z).  Eight lanes per row.
+__global__ void __launch_bounds__(128) k_row_exponents(uint16_t* __restrict__ re, const double2* __restrict__ A, int nb,
+                                                       int splits, int ld) {
+    if (grid_dependency()) return;
+    const long long job = blockIdx.x;
+    const int c = threadIdx.x >> 3, l = threadIdx.x & 7;
+    int count = 5;                                       // blocks
+    const double2* row = A + job * (5 * D * D) + c * D;
+    size_t step = D * D;                                 // from a block to the next
+    if (nb) {
+        const int z = (int)(job % splits);
+        count = min(KSPLIT, nb - z * KSPLIT);
+        row = A + ((job / splits) * D + c) * (long long)ld + (long long)z * KSPLIT * D;
+        step = D;
+    }
+    u64 m = 0;
+    for (int e = l; e < count * D; e += 8) {
+        const double2 a = row[(e / D) * step + e % D];
+        m = max(m, max((u64)__double_as_longlong(a.x) & 0x7FFFFFFFFFFFFFFFull,
+                       (u64)__double_as_longlong(a.y) & 0x7FFFFFFFFFFFFFFFull));
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (l == 0) re[job * D + c] = (uint16_t)(m >> 52);
+}
+
 // Digit tiles of x: per (site, 128-rhs tile) 8 K-major slices of 8 KB.  Thread = (site,
 // group of 4 components, rhs): four 16-byte loads, eight 16-byte stores.  The rows of a
 // tile beyond the rhs are not written (they only reach the same rows of the product).
@@ -143,15 +231,18 @@ __global__ void __launch_bounds__(128) k_slice_x(uint8_t* __restrict__ xs, const
 // input real; the form of the BF16 stencil operands).  Block q starts at A + base(q) with
 // rows ld apart: the stencil's blocks lie one after another (ld = 16, nb = 0), block (R, C)
 // of a dense n x n matrix starts at (16 R) n + 16 C (nb = n / 16 blocks per row, ld = n).
-// Thread = (block, output real, 8 input reals).
+// Each row relative to its own largest entry (k_row_exponents).  Thread = (block, output real, 8
+// input reals).
 __global__ void __launch_bounds__(128) k_slice_a(uint8_t* __restrict__ as, const double2* __restrict__ A,
-                                                 const u64* __restrict__ mx, long long nblk, int nb, int ld) {
+                                                 const uint16_t* __restrict__ re, long long nblk, int nb, int splits,
+                                                 int ld) {
     if (grid_dependency()) return;
     const long long q = blockIdx.x;
     if (q >= nblk) return;
     const int n = threadIdx.x >> 2, kg = threadIdx.x & 3;
     const int co = n >> 1, to = n & 1;
-    const int E = (int)(*mx >> 52);
+    const long long job = nb ? (q / nb) * splits + (q % nb) / KSPLIT : q / 5;
+    const int E = re[job * D + co];
     const double2* blk = nb ? A + (q / nb) * D * (long long)ld + (q % nb) * D : A + q * (D * D);
     u64 u[8];
 #pragma unroll
@@ -201,14 +292,42 @@ __device__ __forceinline__ double combine(const int* G, int s) {
     return neg ? -v : v;
 }
 
+// Rows c0 .. c0 + 7 of a site's product by FP64 sums, in the order of the FP64 block stencils; the
+// 16 inputs of a neighbour are loaded together.
+__device__ __noinline__ void rows_by_fp64(double2* v, const double2* __restrict__ A, const double2* __restrict__ x,
+                                          int site, int c0, int lx, int lt, int N, int j) {
+    double2 acc[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = czero<double2>();
+#pragma unroll 1
+    for (int dir = 0; dir < 5; ++dir) {
+        const double2* xn = x + (size_t)nbr_site(site, dir, lx, lt) * D * N + j;
+        const double2* Ar = A + (((size_t)site * 5 + dir) * D + c0) * D;
+        double2 xv[D];
+#pragma unroll
+        for (int bc = 0; bc < D; ++bc) xv[bc] = xn[(size_t)bc * N];
+#pragma unroll
+        for (int bc = 0; bc < D; ++bc)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) cfma(acc[c], Ar[c * D + bc], xv[bc]);
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = acc[c];
+}
+
 // MODE 0: y = A x; 1: y = b - A x; 2: y = A x with the per-rhs dots <y, x>, <y, y>; 3: the
 // dots only; 4: job (R, z) of a dense product, y[z] = its partial sum over K blocks
 // 6z .. 6z + 5.  nblk: sites of the stencil (lx x lt) or block rows of the dense matrix.
+// The stencil's results are also right entry by entry: where all of a site's inputs lie more than
+// 2^kSpread below the rhs' largest entry, whose scale the digits share, or one of them is not
+// finite, its rows are summed in FP64 instead.
+constexpr int kSpread = 8;
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
     k_block_f64(double2* __restrict__ y, const double2* __restrict__ b, const double2* __restrict__ x,
                 const uint8_t* __restrict__ xs, const uint8_t* __restrict__ as, const u64* __restrict__ mxx,
-                const u64* __restrict__ mxa, int lx, int lt, int nblk, int splits, int N, double2* __restrict__ part,
+                const uint16_t* __restrict__ xe, const uint16_t* __restrict__ re, const double2* __restrict__ A, int lx,
+                int lt, int nblk, int splits, int N, double2* __restrict__ part,
                 int* __restrict__ err) {
     if (grid_dependency()) return;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -357,19 +476,31 @@ __global__ void __launch_bounds__(THREADS, 1)
         // epilogue: two warps per TMEM lane quarter, 16 of the 32 output reals each
         const int quarter = warp & 3, half = (warp - 2) >> 2;
         const int jl = quarter * 32 + lane, j = 128 * t + jl;
-        const int ex = j < N ? (int)(mxx[j] >> 52) : 0, ea = (int)(*mxa >> 52);
-        const bool finite = ex != 0x7ff && ea != 0x7ff;
-        const int sc = (ex - 1022) + (ea - 1022) - 68;
+        const int ex = j < N ? (int)(mxx[j] >> 52) : 0;
         double2 dyx = make_double2(0.0, 0.0);
         double dyy = 0.0;
         bool ok = true;
         for (int i = 0; i < njob; ++i) {
+            const int job = blockIdx.x + i * G;
+            // exponents of the eight rows, two a word
+            const uint4 ew = *reinterpret_cast<const uint4*>(re + (long long)job * D + half * 8);
+            const uint32_t ea[4] = {ew.x, ew.y, ew.z, ew.w};
+            // (no infinity or NaN among the column and the rows)
+            bool by_sums = ex == 0x7ff;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) by_sums = by_sums || ((ea[p / 2] >> (16 * (p & 1))) & 0xFFFF) == 0x7ff;
+            if (MODE != 4 && j < N) {
+                int near = 0;
+#pragma unroll
+                for (int dir = 0; dir < 5; ++dir)
+                    near = max(near, (int)xe[(size_t)nbr_site(job, dir, lx, lt) * N + j]);
+                by_sums = by_sums || (near > 0 && (near == 0x7ff || near + kSpread < ex));
+            }
             if (!mbar_wait_ab(&afull, (unsigned)(i & 1), abrt)) {
                 ok = false;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const int job = blockIdx.x + i * G;
             const long long row0 = (long long)(MODE == 4 ? job / splits : job) * D;
             double2* yo = MODE == 4 ? y + (long long)(job % splits) * nblk * D * N : y;
             const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 16);
@@ -387,16 +518,31 @@ __global__ void __launch_bounds__(THREADS, 1)
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
             if (lane == 0) mbar_arrive(&aempty);               // the accumulator may be overwritten
-            if (j < N) {
+            if (by_sums && j < N) {
+                double2 s[8];
+                if (MODE != 4) rows_by_fp64(s, A, x, job, half * 8, lx, lt, N, j);
+#pragma unroll 1
+                for (int p = 0; p < 8; ++p) {
+                    const long long idx = (row0 + half * 8 + p) * N + j;
+                    double2 o = MODE == 4 ? make_double2(NAN, NAN) : s[p];
+                    if (MODE == 1) o = csub(b[idx], o);
+                    if (MODE != 3) yo[idx] = o;
+                    if (MODE == 2 || MODE == 3) {
+                        cfmac(dyx, o, x[idx]);
+                        dyy = fma(o.x, o.x, fma(o.y, o.y, dyy));
+                    }
+                }
+            } else if (j < N) {
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
+                    const int sc = ex + (int)((ea[p / 2] >> (16 * (p & 1))) & 0xFFFF) - (2 * 1022 + 68);
                     double v[2];
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         int Gi[NG];
 #pragma unroll
                         for (int g = 0; g < NG; ++g) Gi[g] = __float2int_rn(__uint_as_float(r[g][2 * p + u]));
-                        v[u] = finite ? combine(Gi, sc) : __longlong_as_double(0x7ff8000000000000ll);
+                        v[u] = combine(Gi, sc);
                     }
                     const long long idx = (row0 + half * 8 + p) * N + j;
                     double2 o = make_double2(v[0], v[1]);
@@ -451,11 +597,15 @@ using namespace tc::f64;
 static int f64_tiles(int N) { return (N + 127) / 128; }
 
 bool f64_tc_supported(int d, int N) { return d == D && f64_tiles(N) <= 65535; }
-size_t f64_tc_operand_bytes(long long nblk) { return (size_t)nblk * AT + 256; }
-size_t f64_tc_scratch_bytes(long long nblk, int N) {
-    return (size_t)nblk * f64_tiles(N) * XT + ((size_t)N * sizeof(u64) + 255) / 256 * 256;
-}
 int f64_dense_splits(int n) { return (n / D + KSPLIT - 1) / KSPLIT; }
+static long long operand_jobs(long long nblk, int nb) { return nb ? (long long)nb * f64_dense_splits(nb * D) : nblk / 5; }
+size_t f64_tc_operand_bytes(long long nblk, int nb) {
+    return (size_t)nblk * AT + (size_t)operand_jobs(nblk, nb) * D * sizeof(uint16_t);
+}
+static size_t max_bytes(int N) { return ((size_t)N * sizeof(u64) + 255) / 256 * 256; }
+size_t f64_tc_scratch_bytes(long long nblk, int N) {
+    return (size_t)nblk * f64_tiles(N) * XT + max_bytes(N) + ((size_t)nblk * N * sizeof(uint16_t) + 255) / 256 * 256;
+}
 
 void launch_absmax_cols(u64* out, const double2* x, long long n, int N, cudaStream_t s) {
     MG_CUDA(cudaMemsetAsync(out, 0, sizeof(u64) * N, s));
@@ -468,27 +618,41 @@ void launch_absmax_cols(u64* out, const double2* x, long long n, int N, cudaStre
     MG_LAUNCHED();
 }
 
-// Operand: the digit tiles, then (256-byte aligned) the bits of the largest entry.
-static const u64* operand_max(const void* op, long long nblk) {
-    return reinterpret_cast<const u64*>(reinterpret_cast<const uint8_t*>(op) + (size_t)nblk * AT);
+// Operand: the digit tiles, then the exponents of the rows of every job.
+static const uint16_t* operand_rows(const void* op, long long nblk) {
+    return reinterpret_cast<const uint16_t*>(reinterpret_cast<const uint8_t*>(op) + (size_t)nblk * AT);
 }
 
 void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int ld, cudaStream_t s) {
     MG_REQUIRE(nblk >= 1 && nblk <= (1LL << 31) - 1, MGMLMC_EINVAL, "FP64 operand: size");
-    u64* mx = const_cast<u64*>(operand_max(op, nblk));
-    // a flat array as 32 columns: the maximum of its 32 column maxima is taken below
-    launch_absmax_cols(mx, A, nblk * (D * D) / 32, 32, s);
-    MG_LAUNCH(1, dim3(1, 32), 0, s, tc::f64::k_absmax_cols, mx, reinterpret_cast<const double2*>(mx), 16, 1);
+    uint16_t* re = const_cast<uint16_t*>(operand_rows(op, nblk));
+    const int splits = nb ? f64_dense_splits(nb * D) : 1;
+    MG_LAUNCH((unsigned)operand_jobs(nblk, nb), 128, 0, s, k_row_exponents, re, A, nb, splits, nb ? ld : D);
     MG_LAUNCHED();
-    MG_LAUNCH((unsigned)nblk, 128, 0, s, k_slice_a, reinterpret_cast<uint8_t*>(op), A, mx, nblk, nb, nb ? ld : D);
+    MG_LAUNCH((unsigned)nblk, 128, 0, s, k_slice_a, reinterpret_cast<uint8_t*>(op), A, re, nblk, nb, splits, nb ? ld : D);
     MG_LAUNCHED();
 }
 
-// Slices x into the scratch: digit tiles, then the largest entry per rhs.
-static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N, cudaStream_t s) {
+// Slices x into the scratch: digit tiles, then the largest entry per rhs and (for the stencil) the
+// exponents per site and rhs.
+static const uint16_t* site_exponents(const u64* mx, int N) {
+    return reinterpret_cast<const uint16_t*>(reinterpret_cast<const uint8_t*>(mx) + max_bytes(N));
+}
+static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N, bool sites, cudaStream_t s) {
     const int T = f64_tiles(N);
     u64* mx = reinterpret_cast<u64*>(reinterpret_cast<uint8_t*>(scratch) + (size_t)nblk * T * XT);
-    launch_absmax_cols(mx, x, nblk * D, N, s);
+    if (sites) {
+        MG_CUDA(cudaMemsetAsync(mx, 0, sizeof(u64) * N, s));
+        int cx = 1;
+        while (cx < N && cx < 32) cx *= 2;
+        const int cy = 256 / cx, gx = (N + cx - 1) / cx;
+        const int gy = (int)std::max(1LL, std::min((4 * nblk + cy - 1) / cy, 8LL * kNumSM / gx));
+        MG_LAUNCH(dim3(gx, gy), dim3(cx, cy), 0, s, k_absmax_sites, mx, const_cast<uint16_t*>(site_exponents(mx, N)), x,
+                  (int)nblk, N);
+        MG_LAUNCHED();
+    } else {
+        launch_absmax_cols(mx, x, nblk * D, N, s);
+    }
     int bx = 8;
     while (bx < N && bx < 128) bx *= 2;
     const int by = 128 / bx;
@@ -499,11 +663,11 @@ static const u64* slice_x(void* scratch, const double2* x, long long nblk, int N
 
 template <int MODE>
 static void f64_launch(double2* y, const double2* b, const double2* x, const void* scratch, const void* op,
-                       const u64* mxx, const u64* mxa, int lx, int lt, int nblk, int splits, int N, double2* part,
-                       int groups, int* err, cudaStream_t s) {
+                       const u64* mxx, const uint16_t* xe, const uint16_t* re, const double2* A, int lx, int lt, int nblk,
+                       int splits, int N, double2* part, int groups, int* err, cudaStream_t s) {
     MG_CUDA(cudaFuncSetAttribute(k_block_f64<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-    MG_LAUNCH(dim3(groups, f64_tiles(N)), THREADS, SMEM, s, (k_block_f64<MODE>), y, b, x, reinterpret_cast<const uint8_t*>(scratch), reinterpret_cast<const uint8_t*>(op), mxx, mxa, lx, lt,
-        nblk, splits, N, part, err);
+    MG_LAUNCH(dim3(groups, f64_tiles(N)), THREADS, SMEM, s, (k_block_f64<MODE>), y, b, x, reinterpret_cast<const uint8_t*>(scratch), reinterpret_cast<const uint8_t*>(op), mxx, xe, re, A, lx,
+              lt, nblk, splits, N, part, err);
     MG_LAUNCHED();
 }
 
@@ -511,17 +675,18 @@ int block_stencil_f64_groups(int nsites, int N) {
     return std::max(1, std::min(nsites, kNumSM / f64_tiles(N)));
 }
 
-void launch_block_stencil_f64(double2* y, const double2* x, const double2* b, const void* op, int lx, int lt, int N,
-                              int mode, void* scratch, double2* part, int groups, int* err, cudaStream_t s) {
+void launch_block_stencil_f64(double2* y, const double2* x, const double2* b, const void* op, const double2* A, int lx,
+                              int lt, int N, int mode, void* scratch, double2* part, int groups, int* err, cudaStream_t s) {
     const int V = lx * lt;
     MG_REQUIRE(f64_tc_supported(D, N) && groups >= 1 && groups <= V, MGMLMC_EINVAL, "FP64 stencil: size");
-    const u64* mxx = slice_x(scratch, x, V, N, s);
-    const u64* mxa = operand_max(op, 5LL * V);
+    const u64* mxx = slice_x(scratch, x, V, N, true, s);
+    const uint16_t* xe = site_exponents(mxx, N);
+    const uint16_t* re = operand_rows(op, 5LL * V);
     switch (mode) {
-        case 0: f64_launch<0>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
-        case 1: f64_launch<1>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
-        case 2: f64_launch<2>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
-        default: f64_launch<3>(y, b, x, scratch, op, mxx, mxa, lx, lt, V, 1, N, part, groups, err, s); break;
+        case 0: f64_launch<0>(y, b, x, scratch, op, mxx, xe, re, A, lx, lt, V, 1, N, part, groups, err, s); break;
+        case 1: f64_launch<1>(y, b, x, scratch, op, mxx, xe, re, A, lx, lt, V, 1, N, part, groups, err, s); break;
+        case 2: f64_launch<2>(y, b, x, scratch, op, mxx, xe, re, A, lx, lt, V, 1, N, part, groups, err, s); break;
+        default: f64_launch<3>(y, b, x, scratch, op, mxx, xe, re, A, lx, lt, V, 1, N, part, groups, err, s); break;
     }
 }
 
@@ -534,13 +699,13 @@ void launch_dense_f64(double2* y, const double2* x, const void* op, int n, int N
                       cudaStream_t s) {
     const int nb = n / D, S = f64_dense_splits(n);
     MG_REQUIRE(n % D == 0 && f64_tc_supported(D, N), MGMLMC_EINVAL, "FP64 dense product: n % 16 == 0");
-    const u64* mxx = slice_x(scratch, x, nb, N, s);
+    const u64* mxx = slice_x(scratch, x, nb, N, false, s);
     double2* p = reinterpret_cast<double2*>(reinterpret_cast<uint8_t*>(scratch) +
                                             (f64_tc_scratch_bytes(nb, N) + 255) / 256 * 256);
     const long long jobs = (long long)nb * S;
     const int G = (int)std::max(1LL, std::min(jobs, (long long)kNumSM / f64_tiles(N)));
-    f64_launch<4>(S == 1 ? y : p, nullptr, nullptr, scratch, op, mxx, operand_max(op, (long long)nb * nb), 0, 0, nb, S,
-                  N, nullptr, G, err, s);
+    f64_launch<4>(S == 1 ? y : p, nullptr, nullptr, scratch, op, mxx, nullptr, operand_rows(op, (long long)nb * nb),
+                  nullptr, 0, 0, nb, S, N, nullptr, G, err, s);
     if (S > 1) {
         const long long cnt = (long long)n * N;
         MG_LAUNCH((int)std::min((cnt + 255) / 256, 16LL * kNumSM), 256, 0, s, k_sum_splits, y, p, cnt, S);

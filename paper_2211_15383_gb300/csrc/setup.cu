@@ -237,12 +237,12 @@ void copy_state(Ctx& d, Ctx& s) {
         const size_t nb = (size_t)b.nsites * b.d * b.d;
         a.A64 = dup(d, b.A64, 5 * nb);
         a.A32 = dup(d, b.A32, 5 * nb);
-        auto dup_digits = [&](const void* p, long long nblk) -> void* {
-            return dup(d, reinterpret_cast<const char*>(p), f64_tc_operand_bytes(nblk));
+        auto dup_digits = [&](const void* p, long long nblk, int nb) -> void* {
+            return dup(d, reinterpret_cast<const char*>(p), f64_tc_operand_bytes(nblk, nb));
         };
-        a.A64t = dup_digits(b.A64t, 5LL * b.nsites);
-        a.Ahat64t = dup_digits(b.Ahat64t, 5LL * b.nsites);
-        a.Dinv64t = dup_digits(b.Dinv64t, (b.n / 16) * (b.n / 16));
+        a.A64t = dup_digits(b.A64t, 5LL * b.nsites, 0);
+        a.Ahat64t = dup_digits(b.Ahat64t, 5LL * b.nsites, 0);
+        a.Dinv64t = dup_digits(b.Dinv64t, (b.n / 16) * (b.n / 16), (int)(b.n / 16));
         a.Minv64 = dup(d, b.Minv64, nb);
         a.Minv32 = dup(d, b.Minv32, nb);
         a.Ahat64 = dup(d, b.Ahat64, 5 * nb);
@@ -381,7 +381,7 @@ static void coarsest_inverse(Ctx& c) {
         }
         if (f64_dense_inverse(n)) {
             const long long nb = n / 16;
-            if (!L.Dinv64t) L.Dinv64t = c.dev_alloc(f64_tc_operand_bytes(nb * nb));
+            if (!L.Dinv64t) L.Dinv64t = c.dev_alloc(f64_tc_operand_bytes(nb * nb, (int)nb));
             launch_f64_operand(L.Dinv64t, L.Dinv64, nb * nb, (int)nb, (int)n, c.stream);
         }
     } else {
@@ -403,7 +403,7 @@ static void coarsest_inverse(Ctx& c) {
 // Digits of a level's stencil blocks for the FP64 products on the tensor cores.
 static void f64_stencil_operand(Ctx& c, void*& op, const double2* A, const Level& L) {
     if (!f64_tc_supported(L.d, 1)) return;
-    if (!op) op = c.dev_alloc(f64_tc_operand_bytes(5LL * L.nsites));
+    if (!op) op = c.dev_alloc(f64_tc_operand_bytes(5LL * L.nsites, 0));
     launch_f64_operand(op, A, 5LL * L.nsites, 0, 0, c.stream);
 }
 

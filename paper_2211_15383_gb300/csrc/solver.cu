@@ -59,17 +59,17 @@ static bool galerkin_form_cheaper(const Ctx& c, int l) {
 // three extra launches cost more than the FP64 pipe saves.
 constexpr int kF64TcMinRhs = 16;
 template <typename C>
-static bool f64_stencil(Ctx&, const Level&, C*, const C*, const C*, const void*, int, int, double2*, int) {
+static bool f64_stencil(Ctx&, const Level&, C*, const C*, const C*, const void*, const C*, int, int, double2*, int) {
     return false;
 }
 static bool f64_stencil_used(const Level& L, const void* op, int N) {
     return op && N >= kF64TcMinRhs && f64_tc_supported(L.d, N);
 }
 template <>
-bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, const double2* b, const void* op, int N,
-                          int mode, double2* part, int groups) {
+bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, const double2* b, const void* op,
+                          const double2* A, int N, int mode, double2* part, int groups) {
     if (!f64_stencil_used(L, op, N)) return false;
-    launch_block_stencil_f64(y, x, b, op, L.lx, L.lt, N, mode,
+    launch_block_stencil_f64(y, x, b, op, A, L.lx, L.lt, N, mode,
                              c.scratch_bytes("f64_tc", f64_tc_scratch_bytes(L.nsites, N)), part, groups,
                              device_error_flag(c), c.stream);
     return true;
@@ -124,7 +124,7 @@ void apply_D(Ctx& c, int l, C* y, const C* x, const C* b, int N, int mode, C* al
         ProfScope ps(c, {"D", l + 1, ".", prec_tag(sizeof(C))}, bytes, flops);
         if (l == 0)
             launch_wilson<C>(y, x, b, links<C>(c), c.m0, L.lx, L.lt, N, mode, part, groups, c.stream);
-        else if (!f64_stencil<C>(c, L, y, x, b, L.A64t, N, mode, part, groups))
+        else if (!f64_stencil<C>(c, L, y, x, b, L.A64t, blocks<C>(L), N, mode, part, groups))
             launch_block_stencil<C>(y, x, b, blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
     if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
@@ -187,7 +187,7 @@ static void apply_Dhat(Ctx& c, int l, C* y, const C* x, int N, int mode, C* alph
         ProfScope ps(c, {"D", l + 1, ".", prec_tag(sizeof(C))},
                      (double)L.n * N * s * (mode == 3 ? 1 : 2) + 5.0 * L.nsites * L.d * L.d * s,
                      40.0 * L.d * L.d * (double)L.nsites * N);
-        if (!f64_stencil<C>(c, L, y, x, (const C*)nullptr, L.Ahat64t, N, mode, part, groups))
+        if (!f64_stencil<C>(c, L, y, x, (const C*)nullptr, L.Ahat64t, hat_blocks<C>(L), N, mode, part, groups))
             launch_block_stencil<C>(y, x, nullptr, hat_blocks<C>(L), L.lx, L.lt, L.d, N, mode, part, groups, c.stream);
     }
     if (mode >= 2) mr_alpha<C>(c, alpha, part, groups, N);
