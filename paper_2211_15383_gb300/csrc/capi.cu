@@ -723,7 +723,11 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
             }
             break;
         default:
-            if (c.opt.mg_precision == 64) {
+            if (c.opt.mg_precision == 64 && op == MGMLMC_OP_DINV_C) {
+                // FP64 sums, also where the cycle takes digit products: those are accurate
+                // relative to a column's largest entry, not entry by entry
+                mg::launch_gemm_nn<double2>(yt, c.lev[l].Dinv64, xt, (int)nin, (int)nin, nrhs, false, c.stream);
+            } else if (c.opt.mg_precision == 64) {
                 mg::mg_cycle<double2>(c, l, yt, xt, nrhs);
             } else {
                 float2* x32 = c.scratch<float2>("ap_x32", (size_t)nin * nrhs);

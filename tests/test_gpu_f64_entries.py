@@ -77,3 +77,24 @@ def test_rows_of_every_scale(pkg):
         rows = A.max(axis=0)
         assert rows.max() > 2.0 ** 18 * np.median(rows)
         check(ctx, pkg.OP_SMOOTH, 2, x)
+
+
+def gemm_check(ctx, op, level, x):
+    """As check for a dense operator of n unknowns: n complex products an entry."""
+    n = x.shape[1]
+    A = np.abs(by_sums(ctx, op, level, np.eye(n, dtype=np.complex128)))
+    got, ref = ctx.apply(op, level, x, n), by_sums(ctx, op, level, x)
+    assert np.all(np.abs(got - ref) <= 2 * 4 * n * U * (np.abs(x) @ A))
+
+
+def test_inverse(pkg):
+    """A heavy mass: the inverse decays with the distance, and so do its rows' products with a
+    right-hand side of one large entry."""
+    agg, nvec = ((2, 2),), (4,)
+    theta, sv = small_problem(32, 32, 3.0, 6.0, agg, nvec)
+    with make_ctx(pkg, theta, 6.0, agg, nvec, sv, 0, mg_precision=64) as ctx:
+        n = ctx.level_info(2)[3]
+        rng = np.random.default_rng(7)
+        x = scaled(rng, 18, n, d=8)
+        x[:, 100] = 1.0                            # far above the rest
+        gemm_check(ctx, pkg.OP_DINV_C, 2, x)
