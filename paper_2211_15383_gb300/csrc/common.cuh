@@ -127,27 +127,49 @@ __host__ __device__ __forceinline__ double2 to_d(double2 a) { return a; }
 // ---- sums across threads: FP32 values as pairs, FP64 values plainly
 struct PairF {
     float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float v) {
+    __host__ __device__ __forceinline__ void add(float v) {
         const float s = h + v, b = s - h;
         l += (h - (s - b)) + (v - b);
         h = s;
     }
-    __device__ __forceinline__ void add(const PairF& o) {
+    __host__ __device__ __forceinline__ void add(const PairF& o) {
         add(o.h);
         l += o.l;
     }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+    __host__ __device__ __forceinline__ double value() const { return (double)h + (double)l; }
 };
 struct SumD {
     double v = 0.0;
-    __device__ __forceinline__ void add(double a) { v += a; }
-    __device__ __forceinline__ void add(const SumD& o) { v += o.v; }
-    __device__ __forceinline__ double value() const { return v; }
+    __host__ __device__ __forceinline__ void add(double a) { v += a; }
+    __host__ __device__ __forceinline__ void add(const SumD& o) { v += o.v; }
+    __host__ __device__ __forceinline__ double value() const { return v; }
 };
 template <typename R> struct SumOf;
 template <> struct SumOf<float> { using T = PairF; };
 template <> struct SumOf<double> { using T = SumD; };
 template <typename C> using sum_t = typename SumOf<re_t<C>>::T;
+
+// Squares of V rhs over the rows of a thread.  FP32: plain accumulators, folded into the sums every
+// kRowsPerSum rows, so that their error does not grow with the rows that a grid leaves a thread
+// (a thread of a 2097152 x 128 block has 862).
+constexpr int kRowsPerSum = 64;
+template <typename R, int V> struct SquareSums {
+    typename SumOf<R>::T total[V];
+    R part[V] = {};
+    int rows = 0;
+    __host__ __device__ __forceinline__ void add(int q, R x, R y) { part[q] = fma(x, x, fma(y, y, part[q])); }
+    __host__ __device__ __forceinline__ void end_row() {
+        if (sizeof(R) == 4 && ++rows >= kRowsPerSum) fold();
+    }
+    __host__ __device__ __forceinline__ void fold() {
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            total[q].add(part[q]);
+            part[q] = 0;
+        }
+        rows = 0;
+    }
+};
 template <typename C> struct alignas(16) CSum { sum_t<C> re, im; };   // 16 B in both precisions
 static_assert(sizeof(CSum<float2>) == 16 && sizeof(CSum<double2>) == 16, "partials are 16 bytes");
 

@@ -194,12 +194,10 @@ __global__ void __launch_bounds__(256, 4) k_multiaxpy(C* __restrict__ w, const C
         if (j < N)
             cs[k * blockDim.x + threadIdx.x] = *reinterpret_cast<const Vec<C, V>*>(cf + (long long)k * N + j);
     __syncthreads();
-    R ns[V], nrm[V];
+    R ns[V];
+    SquareSums<R, V> nrm;
 #pragma unroll
-    for (int q = 0; q < V; ++q) {
-        ns[q] = (nscale && j < N && nscale[j + q] != 0.0) ? (R)nscale[j + q] : (R)1;
-        nrm[q] = 0;
-    }
+    for (int q = 0; q < V; ++q) ns[q] = (nscale && j < N && nscale[j + q] != 0.0) ? (R)nscale[j + q] : (R)1;
     if (j < N)
         for (long long t = (long long)blockIdx.y * blockDim.y + threadIdx.y; t < n;
              t += (long long)gridDim.y * blockDim.y) {
@@ -224,17 +222,14 @@ __global__ void __launch_bounds__(256, 4) k_multiaxpy(C* __restrict__ w, const C
             }
             *reinterpret_cast<Vec<C, V>*>(w + i * N + j) = acc;
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const R ax = acc.v[q].x * ns[q], ay = acc.v[q].y * ns[q];
-                nrm[q] = fma(ax, ax, fma(ay, ay, nrm[q]));
-            }
+            for (int q = 0; q < V; ++q) nrm.add(q, acc.v[q].x * ns[q], acc.v[q].y * ns[q]);
+            nrm.end_row();
         }
     if (npart) {
+        nrm.fold();
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            sum_t<C> s;
-            s.add(nrm[q]);
-            s = block_rows_sum(s, sh);
+            const sum_t<C> s = block_rows_sum(nrm.total[q], sh);
             if (threadIdx.y == 0 && j < N) npart[(long long)blockIdx.y * N + j + q] = s;
         }
     }
@@ -543,8 +538,8 @@ static int dot_groups(long long n, int N) { return groups_of(n, N, 1, 4); }
 size_t dot_part_bytes(long long n, int N, int m) {
     return (size_t)std::max(groups_of(n, N, 1, 4), groups_of(n, N, 2, 4)) * m * N * 16;
 }
-// The updates of Gram-Schmidt stream m + 2 vectors with few loads per row: more blocks per
-// SM keep more of them in flight.
+// The updates of Gram-Schmidt stream m + 2 vectors with few loads per row: two waves of the four
+// blocks that an SM holds.
 static int axpy_groups(long long n, int N) { return groups_of(n, N, 1, 8); }
 size_t norm_part_bytes(long long n, int N) { return (size_t)axpy_groups(n, N) * N * 8; }
 
