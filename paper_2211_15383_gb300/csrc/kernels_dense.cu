@@ -410,8 +410,9 @@ __global__ void __launch_bounds__(32 * kGJRowsPerCTA) k_gj_eliminate(C* A, int n
 // its shared memory (at most 6144 rows: 768 rows x 256 B a CTA).  Per column every CTA sends
 // its pivot candidate with that candidate's panel row, and the owner row k, to all CTAs
 // through distributed shared memory; after one cluster barrier each CTA knows the pivot
-// (largest max(|Re|, |Im|), ties to the smallest row), scales its own copy of the pivot row
-// and eliminates its rows, which also gives the candidates of the next column.  What a
+// (largest |A[i][k]|^2 in FP64, ties to the smallest row), scales its own copy of the pivot row by
+// its reciprocal (rounded once) and eliminates its rows, which also gives the candidates of the
+// next column: the same arithmetic as k_gj_pivot's and k_gj_eliminate's.  What a
 // column costs is that chain (exchange, barrier, scale, eliminate: about 2 us), where the two
 // launches per column of k_gj_pivot and k_gj_eliminate cost 17 us at n = 1024 and 23 us at
 // n = 4096; larger matrices keep those.
@@ -439,38 +440,54 @@ __device__ __forceinline__ void cluster_store(uint32_t a, double2 v) {
 __device__ __forceinline__ void cluster_store(uint32_t a, int v) {
     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ void cluster_store(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
 __device__ __forceinline__ void cluster_store(uint32_t a, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
-template <typename C> __device__ __forceinline__ re_t<C> gj_size(C v) { return fmax(fabs(v.x), fabs(v.y)); }
-
-// 1 / p.  FP32: scaled by the larger part, then one Newton step, which leaves the rounding of
-// the last operation.
+__device__ __forceinline__ void cluster_store(uint32_t a, long long v) {
+    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+// 1 / p.  FP32: to about 2^-45 in pairs of FP32, then rounded once, which is the FP64 quotient's
+// rounding but for one case in 2^20 (formed in FP64 it took 0.4 us of a column's chain); p is
+// scaled by a power of two to between 1 and 2, which is exact.
 __device__ __forceinline__ float2 gj_reciprocal(float2 p) {
-    const float m = 1.f / fmaxf(fabsf(p.x), fabsf(p.y));
-    const float x = p.x * m, y = p.y * m;
-    const float q = m / fmaf(x, x, y * y);
-    float2 r = mk(x * q, -y * q);
-    const float ex = fmaf(-p.x, r.x, fmaf(p.y, r.y, 1.f)), ey = fmaf(-p.x, r.y, -p.y * r.x);
-    return mk(fmaf(r.x, ex, fmaf(-r.y, ey, r.x)), fmaf(r.x, ey, fmaf(r.y, ex, r.y)));
+    const float m = fmaxf(fabsf(p.x), fabsf(p.y));
+    const int e = (int)(__float_as_uint(m) >> 23) - 127;
+    if (e < -100 || e > 100) {
+        const double x = p.x, y = p.y, ir = 1.0 / (x * x + y * y);
+        return mk((float)(x * ir), (float)(-y * ir));
+    }
+    const float f = __uint_as_float((uint32_t)(127 - e) << 23);
+    const float x = p.x * f, y = p.y * f;
+    const float xx = x * x, yy = y * y;
+    float dh = xx + yy;                                          // |p|^2 = dh + dl
+    const float b = dh - xx;
+    float dl = (xx - (dh - b)) + (yy - b) + (fmaf(x, x, -xx) + fmaf(y, y, -yy));
+    const float q = 1.f / dh;
+    const float ql = q * (fmaf(-dh, q, 1.f) - dl * q);           // 1 / |p|^2 = q + ql
+    const float rx = x * q, ry = y * q;
+    return mk((rx + (fmaf(x, q, -rx) + x * ql)) * f, -(ry + (fmaf(y, q, -ry) + y * ql)) * f);
 }
 __device__ __forceinline__ double2 gj_reciprocal(double2 p) {
     const double den = p.x * p.x + p.y * p.y;
     return mk(p.x / den, -p.y / den);
 }
 
+// |v|^2 in FP64 as its bit pattern: non-negative doubles order like integers, whose comparisons
+// run on the integer pipe (in FP64 those of the reductions took 2 us a column); -1 for NaN.
+template <typename C> __device__ __forceinline__ long long gj_key(C v) {
+    const long long b = __double_as_longlong(gj_mag2(v));
+    return b <= (0x7FFLL << 52) ? b : -1;
+}
 template <typename C>
 __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 1, 1)
     k_gj_panel(C* A, int n, int k0, int kb, int R, GJWork w) {
-    using T = re_t<C>;
+    using T = long long;                         // sizes of the candidates (gj_key)
     constexpr int B = GJPanel<C>::B;             // columns of a panel row: 256 bytes
     constexpr int U = 16 / (int)sizeof(C);       // columns per 16 bytes
     struct alignas(16) Unit { C v[U]; };
     extern __shared__ __align__(16) unsigned char smem_gj[];
     C* P = reinterpret_cast<C*>(smem_gj);        // this CTA's rows
+    C* col = P + (size_t)R * B;                  // their entries in the next column
     __shared__ __align__(16) C xrow[2][kGJCluster][B], krow[2][B];
     __shared__ T xval[2][kGJCluster];
     __shared__ int xidx[2][kGJCluster];
@@ -486,7 +503,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
     }
     cluster_barrier();   // the panel is loaded, and every CTA has started before the first remote store
     // the CTA's candidate (value, local row) from per-thread ones: lane 0 of every warp, then warp 0
-    auto reduce = [&](T bv, int bi) {
+    auto reduce = [&](T& bv, int bi) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
@@ -509,7 +526,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
     int ci = 0x7fffffff;
     for (int r = tid; r < rows; r += kGJPanelThreads)
         if (row0 + r >= k0) {
-            const T m = gj_size(P[r * B]);
+            const T m = gj_key(P[r * B]);
             if (m > cv) { cv = m; ci = r; }
         }
     for (int c = 0; c < kb; ++c) {
@@ -523,7 +540,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
                 if (k >= row0 && k < row0 + rows) cluster_store(cluster_map(&krow[par][lane], wid), P[(k - row0) * B + lane]);
             }
             if (lane == 0) {
-                cluster_store(cluster_map(&xval[par][rank], wid), mine ? gj_size(P[bi * B + c]) : (T)-1);
+                cluster_store(cluster_map(&xval[par][rank], wid), mine ? cv : (T)-1);
                 cluster_store(cluster_map(&xidx[par][rank], wid), mine ? row0 + bi : 0x7fffffff);
             }
         }
@@ -538,7 +555,7 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
         if (wid == 0) {
             const C raw = lane < B ? xrow[par][best][lane] : czero<C>();
             C piv = mk(__shfl_sync(0xffffffffu, raw.x, c), __shfl_sync(0xffffffffu, raw.y, c));
-            if (!ok) piv = mk((T)1, (T)0);
+            if (!ok) piv = mk((re_t<C>)1, (re_t<C>)0);
             const C inv = gj_reciprocal(piv);
             const C sv = lane == c ? inv : cmul(raw, inv);
             if (lane < B) {
@@ -555,8 +572,6 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
         __syncthreads();
         // eliminate column k from the other rows: 8 threads per row
         const int sub = tid & 7;
-        cv = (T)-1;
-        ci = 0x7fffffff;
         // thread `sub` of a row's eight holds the 16-byte units sub and sub + 8
         Unit s[2];
 #pragma unroll
@@ -576,16 +591,22 @@ __global__ void __launch_bounds__(kGJPanelThreads) __cluster_dims__(kGJCluster, 
                     for (int u = 0; u < U; ++u) {
                         const int cc = (sub + 8 * q) * U + u;
                         o.v[u] = csub(cc == c ? czero<C>() : o.v[u], cmul(f, s[q].v[u]));
-                        if (cc == c + 1 && row0 + r > k) {
-                            const T m = gj_size(o.v[u]);
-                            if (m > cv) { cv = m; ci = r; }
-                        }
+                        if (cc == c + 1) col[r] = o.v[u];
                     }
                     *pu = o;
                 }
             }
         }
         __syncthreads();
+        // candidates of the next column, a thread per row: in the loop above the FP64 squares
+        // would be issued for every warp and row
+        cv = (T)-1;
+        ci = 0x7fffffff;
+        if (c + 1 < kb)
+            for (int r = max(0, k + 1 - row0) + tid; r < rows; r += kGJPanelThreads) {
+                const T m = gj_key(col[r]);
+                if (m > cv) { cv = m; ci = r; }
+            }
     }
     for (int e = tid; e < rows * B; e += kGJPanelThreads) {
         const int r = e / B, c = e % B;
@@ -737,11 +758,12 @@ void launch_gauss_jordan(C* A, int n, void* work, cudaStream_t s) {
     const int R = (n + kGJCluster - 1) / kGJCluster;             // rows per CTA of the panel cluster
     const bool cluster = R <= kGJPanelRows;
     if (cluster)
-        MG_CUDA(cudaFuncSetAttribute(k_gj_panel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGJPanelRows * 256));
+        MG_CUDA(cudaFuncSetAttribute(k_gj_panel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kGJPanelRows * (256 + (int)sizeof(C))));
     for (int k0 = 0; k0 < n; k0 += B) {
         const int kb = n - k0 < B ? n - k0 : B;
         if (cluster) {
-            k_gj_panel<C><<<kGJCluster, kGJPanelThreads, (size_t)R * 256, s>>>(A, n, k0, kb, R, w);
+            k_gj_panel<C><<<kGJCluster, kGJPanelThreads, (size_t)R * (256 + sizeof(C)), s>>>(A, n, k0, kb, R, w);
         } else {
             for (int k = k0; k < k0 + kb; ++k) {
                 MG_LAUNCH(1, 1024, 0, s, (k_gj_pivot<C>), A, n, k, k0, kb, w, k > k0 ? ncand : 0);
