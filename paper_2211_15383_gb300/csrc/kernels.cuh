@@ -100,13 +100,13 @@ void launch_refine_axpy(double2* y, const double* scale, double sign, const floa
 template <typename C>
 void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_t s);
 // Givens rotations of the Hessenberg columns j0..j1 (H[j][m + 1][N], subdiagonals hsub[j][N]):
-// rotations cs, sn [j][N], rotated right-hand side g[m + 1][N], irr[j][N] = 1 / R_jj; *max =
-// max(*max, residual / bnorm) after column j1 (max may be null), *clear = 0; for N <= kRotateWarp
-// the maximum can go to *host (pinned memory) instead.
+// rotations cs, sn [j][N], rotated right-hand side g[m + 1][N], irr[j][N] = 1 / R_jj; max[j] =
+// max(max[j], residual / bnorm) after each column j (max may be null); for N <= kRotateWarp the
+// maxima can go to host[j] (pinned memory) instead.
 constexpr int kRotateWarp = 32;
 void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,
-                   const double* bnorm, unsigned long long* max, unsigned long long* clear, double* host, int j0, int j1,
-                   int m, int N, cudaStream_t s);
+                   const double* bnorm, unsigned long long* max, double* host, int j0, int j1, int m, int N,
+                   cudaStream_t s);
 // cf[i][N] = y_i / eta_i, i <= j, with R y = g.
 template <typename C>
 void launch_back_substitute(C* cf, const double2* H, const double2* g, const double2* irr, const double* ieta, int j,

@@ -417,20 +417,21 @@ __global__ void __launch_bounds__(256) k_scale_cols_if(C* __restrict__ w, const 
 // ---- Givens rotations of the Hessenberg columns j0 .. j1, one thread per rhs.  Column j:
 // entries i <= j at H[(j (m + 1) + i) N + r] (overwritten by R), subdiagonal hsub[j N + r];
 // rotation i: (a, b) <- (c a + s b, -conj(s) a + c b).  irr = 1 / R[j][j] (0 if it is 0).
-// The residual estimate after column j1 goes to *max, divided by bnorm.
+// The residual estimate after column j, divided by bnorm, goes to max[j] (their maximum over the rhs),
+// or to host[j] where one warp holds all rhs.
 __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const double* __restrict__ hsub,
                                                double* __restrict__ cs, double2* __restrict__ sn,
                                                double2* __restrict__ g, double2* __restrict__ irr,
-                                               const double* __restrict__ bnorm, u64* max, u64* clear, double* host, int j0,
-                                               int j1, int m, int N) {
+                                               const double* __restrict__ bnorm, u64* max, double* host, int j0, int j1, int m,
+                                               int N) {
     if (grid_dependency()) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (clear && r == 0) *clear = 0;
     const bool in = r < N;
     if (!in && !host) return;
     double2 gj = in ? g[(long long)j0 * N + r] : make_double2(0.0, 0.0);
+    const double bn = in && bnorm ? bnorm[r] : 0.0;
     double resid = 0.0;
-    for (int j = j0; in && j <= j1; ++j) {
+    auto column = [&](int j) {
         double2* col = H + (long long)j * (m + 1) * N + r;
         double2 a = col[0];
 #pragma unroll 4
@@ -470,9 +471,11 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
         gj = make_double2(-sg.x, -sg.y);
         g[(long long)(j + 1) * N + r] = gj;
         if (!(t == t)) resid = t;
-    }
-    if (max || host) {
-        const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid, bn = in ? bnorm[r] : 0.0;
+    };
+    for (int j = j0; j <= j1; ++j) {
+        if (in) column(j);
+        if (!max && !host) continue;
+        const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid;
         const double v = bn == 0.0 ? 0.0 : rs / bn;
         if (host) {
             u64 m8 = (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
@@ -481,9 +484,9 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
                 const u64 w = __shfl_xor_sync(0xffffffffu, m8, o);
                 m8 = w > m8 ? w : m8;
             }
-            if (threadIdx.x == 0) *host = __longlong_as_double((long long)m8);
+            if (threadIdx.x == 0) host[j] = __longlong_as_double((long long)m8);
         } else {
-            atomic_max_double(max, v);
+            atomic_max_double(max + j, v);
         }
     }
 }
@@ -657,10 +660,10 @@ void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_
 }
 
 void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,
-                   const double* bnorm, unsigned long long* max, unsigned long long* clear, double* host, int j0, int j1,
-                   int m, int N, cudaStream_t s) {
+                   const double* bnorm, unsigned long long* max, double* host, int j0, int j1, int m, int N,
+                   cudaStream_t s) {
     MG_REQUIRE(!host || N <= kRotateWarp, MGMLMC_EINVAL, "rotations: one warp writes to the host");
-    MG_LAUNCH((N + 31) / 32, 32, 0, s, k_rotate, H, hsub, cs, sn, g, irr, bnorm, max, clear, host, j0, j1, m, N);
+    MG_LAUNCH((N + 31) / 32, 32, 0, s, k_rotate, H, hsub, cs, sn, g, irr, bnorm, max, host, j0, j1, m, N);
     MG_LAUNCHED();
 }
 

@@ -447,6 +447,7 @@ static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool
 // A maximum that the next reduction writes (NormOut::max and ::clear, or launch_rotate's) and
 // read_max returns.  Four in turn: at most two are taken between two reads.
 constexpr int kMaxSlots = 4;
+constexpr int kMaxRestart = 64;   // columns of a cycle at most
 struct MaxSlot {
     int i = 0;
     unsigned long long *at = nullptr, *clear = nullptr;
@@ -585,7 +586,7 @@ static void kcycle(Ctx& c, int l, C* e, const C* r, int N, int k) {
         apply_D<C>(c, l, B.v(j + 1), B.z(j), nullptr, N, 0, nullptr);
         arnoldi_step<C>(c, B, j, 1);
     }
-    launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, nullptr, nullptr, nullptr, nullptr, 0, k - 1, k, N, c.stream);
+    launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, nullptr, nullptr, nullptr, 0, k - 1, k, N, c.stream);
     basis_update<C>(c, B, k - 1, e, false);
 }
 
@@ -635,8 +636,10 @@ static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate
                          long long& it, long long maxit, bool inner) {
     const int N = B.N, m = B.m;
     // Inner cycles of the refinement loop converge in a repeatable number of steps per level
-    // and tolerance: the host reads the residual estimate (a round trip that leaves the GPU
-    // idle) only from two steps before the last such count on.
+    // and tolerance: the host reads the residual estimates (a round trip that leaves the GPU
+    // idle) only from two steps before the last such count on.  It reads those of every
+    // column: a cycle ends with the first that meets tol, whatever steps were taken after it, so
+    // that the counts of earlier calls change its time and nothing else.
     int* hint = nullptr;
     if (inner) {
         const int dec = std::min(15, std::max(0, (int)std::floor(-std::log10(tol))));
@@ -646,29 +649,36 @@ static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate
     // classical Gram-Schmidt: twice in FP64; once in the FP32 inner solve of the refinement
     // loop, whose FP64 residual absorbs the loss of orthogonality
     const int passes = sizeof(C) == sizeof(double2) ? 2 : 1;
+    unsigned long long* dmax = nullptr;
+    double* est = c.hbuf + kMaxSlots;            // per column
+    if (N > kRotateWarp) {
+        dmax = c.scratch<unsigned long long>("fg_est", kMaxRestart);
+        MG_CUDA(cudaMemsetAsync(dmax, 0, m * sizeof(unsigned long long), c.stream));
+    }
     int j = 0, rotated = 0;
-    for (;; ++j) {
+    for (bool done = false; !done; ++j) {
         mg_cycle<C>(c, l, B.z(j), B.v(j), N);
         apply_D<C>(c, l, B.v(j + 1), B.z(j), nullptr, N, 0, nullptr);
         arnoldi_step<C>(c, B, j, passes);
         ++it;
         if (j + 1 < check_from && j + 1 < m && it < maxit) continue;
-        double est;
-        if (N <= kRotateWarp) {
-            // one warp: it writes the maximum to the host itself
-            launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, nullptr, nullptr, c.hbuf + kMaxSlots, rotated, j, m,
-                          N, c.stream);
-            c.sync();
-            est = c.hbuf[kMaxSlots];
-        } else {
-            const MaxSlot ms = take_max(c);
-            launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, ms.at, ms.clear, nullptr, rotated, j, m, N, c.stream);
-            est = read_max(c, ms);
+        // up to 32 rhs one warp writes the maxima to the host itself
+        launch_rotate(B.H, B.hsub, B.cs, B.sn, B.g, B.irr, bnorm, dmax, dmax ? nullptr : est, rotated, j, m, N, c.stream);
+        if (dmax)
+            MG_CUDA(cudaMemcpyAsync(est + rotated, dmax + rotated, (j + 1 - rotated) * sizeof(double),
+                                    cudaMemcpyDeviceToHost, c.stream));
+        c.sync();
+        for (; rotated <= j && !done; ++rotated) {
+            if (est[rotated] != est[rotated]) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
+            done = est[rotated] <= tol;
         }
-        rotated = j + 1;
-        if (est != est) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
-        if (est <= tol || it >= maxit || j + 1 >= m) break;
+        if (done) {
+            it -= j + 1 - rotated;               // steps beyond it were not needed
+            j = rotated - 1;
+        }
+        done |= it >= maxit || j + 1 >= m;
     }
+    --j;                                         // the last column
     if (hint) *hint = j + 1;
     basis_update<C>(c, B, j, x, accumulate);
 }
