@@ -601,10 +601,11 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
     C* rc = c.scratch<C>(nm("cyc_rc", l + 1, sizeof(C)), (size_t)Lc.n * N);
     C* ec = c.scratch<C>(nm("cyc_ec", l + 1, sizeof(C)), (size_t)Lc.n * N);
     const size_t nN = (size_t)L.n * N;
-    auto residual_slots = [&](int nu) { return c.scratch<C>(nm("cyc_res", l, sizeof(C)), mr_slots(nu) * nN); };
+    auto residual_slots = [&](int slots) { return c.scratch<C>(nm("cyc_res", l, sizeof(C)), slots * nN); };
     bool e_zero = true;
     if (c.opt.nu_pre > 0) {
-        C* res = residual_slots(c.opt.nu_pre);
+        // the pre-smoother on the tensor cores keeps one residual
+        C* res = residual_slots(tc_smoother<C>(L, N) ? 1 : mr_slots(c.opt.nu_pre));
         MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C) * nN, cudaMemcpyDeviceToDevice, c.stream));
         // leaves res = r - D e
         if (!pre_smooth_tc<C>(c, l, e, res, N, c.opt.nu_pre))
@@ -623,7 +624,7 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
     const bool have_et = apply_prolong<C>(c, l, e, ec, N, !e_zero, et);
     if (c.opt.nu_post <= 0 || post_smooth_tc<C>(c, l, e, r, N, have_et) || post_smooth_fine_bf16<C>(c, l, e, r, N))
         return;
-    C* res = residual_slots(c.opt.nu_post);
+    C* res = residual_slots(mr_slots(c.opt.nu_post));
     apply_D<C>(c, l, res, e, r, N, 1, nullptr);
     mr_smooth<C>(c, l, e, res, N, c.opt.nu_post, false, false);
 }
