@@ -445,7 +445,9 @@ static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool
 }
 
 // A maximum that the next reduction writes (NormOut::max and ::clear, or launch_rotate's) and
-// read_max returns.  Four in turn: at most two are taken between two reads.
+// read_max returns.  Four in turn: at most two are taken between two reads.  Each is taken
+// right before the launch that it is for (nothing in between may fail: that launch also
+// clears the place of the turn after the next).
 constexpr int kMaxSlots = 4;
 constexpr int kMaxRestart = 64;   // columns of a cycle at most
 struct MaxSlot {
@@ -701,6 +703,7 @@ long long fgmres(Ctx& c, int l, const C* b, C* x, int N, double tol, long long m
         norms<C>(c, o, b, n, N);
     }
     for (;;) {
+        if (!x_unset) apply_D<C>(c, l, B.V, x, b, N, 1, nullptr);
         const MaxSlot ms = take_max(c);
         NormOut o = basis_start(B);
         o.max = ms.at;
@@ -710,7 +713,6 @@ long long fgmres(Ctx& c, int l, const C* b, C* x, int N, double tol, long long m
             launch_scale_norm<C, C>(o, B.V, b, nullptr, false, n, N, B.npart, c.stream);
         } else {
             o.den = bnorm;
-            apply_D<C>(c, l, B.V, x, b, N, 1, nullptr);
             launch_norm<C>(o, B.V, n, N, B.npart, c.stream);
         }
         const double ratio = read_max(c, ms);
