@@ -49,7 +49,11 @@ typedef enum {
 
 typedef struct mgmlmc_ctx mgmlmc_ctx;
 
-/* Device allocator hooks: alloc returns a device pointer (NULL = refused). */
+/* Device allocator hooks: alloc returns a device pointer (NULL = refused).  Some of
+ * a context's memory only makes it faster (digits of the FP64 operators for
+ * products of 16 and more right-hand sides, residuals that the smoother keeps).  If
+ * an allocation is refused, the context gives that memory back and asks once more;
+ * it then works without it until the next mgmlmc_set_hierarchy. */
 typedef void* (*mgmlmc_alloc_fn)(void* user, size_t bytes);
 typedef void (*mgmlmc_free_fn)(void* user, void* ptr);
 
@@ -396,8 +400,9 @@ typedef struct {
  * that fit with a restart of at most 16, then restart length (8, 16, 24), smoother
  * steps (2, 6) and, with four levels or more, the other coarse-grid correction.
  * The fastest becomes the context's setting; its work space is released.  Needs a
- * hierarchy (and the deflation, if any, already computed).  MGMLMC_ENOMEM if no
- * block width fits the budget. */
+ * hierarchy (and the deflation, if any, already computed).  If no block width fits
+ * the budget, the context gives up the memory that it can do without (see
+ * mgmlmc_alloc_fn); MGMLMC_ENOMEM if none fits then. */
 int mgmlmc_autotune(mgmlmc_ctx* ctx, size_t hbm_budget, int max_trials, mgmlmc_tune_result* out);
 
 /* Level geometry: sites per direction, dof per site, n_l. */
@@ -516,7 +521,9 @@ void mgmlmc_server_destroy(mgmlmc_server* srv);
  * for it is mgmlmc_request_footprint while no request of the same shape (lattice,
  * hierarchy, k, precision, block width, restart length) has finished, then 1.1 x
  * the largest device peak of those that have.  MGMLMC_EINVAL for a malformed
- * request, MGMLMC_ENOMEM if that footprint exceeds the whole budget. */
+ * request, MGMLMC_ENOMEM if that footprint exceeds the whole budget, also without the
+ * memory that a context can do without (see mgmlmc_alloc_fn): such a request runs
+ * without it and reserves that much less. */
 int mgmlmc_submit(mgmlmc_server* srv, const mgmlmc_request* req, uint64_t* id);
 
 /* MGMLMC_OK and *out filled once the request has finished (its own outcome is

@@ -10,7 +10,6 @@
 #include <vector>
 
 #include "context.h"
-#include "footprint.h"
 
 using mg::Ctx;
 using mg::Error;
@@ -300,6 +299,7 @@ int mgmlmc_set_options(mgmlmc_ctx* h, const mgmlmc_options* opt) {
     MG_REQUIRE(opt->mg_precision == c.opt.mg_precision, MGMLMC_EINVAL,
                "set_options: mg_precision is fixed for the life of a context");
     c.opt = *opt;
+    if (c.have_hier && c.opt.max_block_rhs >= mg::kF64TcMinRhs) mg::prepare_digits(c);
     API_END
 }
 
@@ -728,7 +728,7 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
                 // relative to a column's largest entry, not entry by entry
                 mg::launch_gemm_nn<double2>(yt, c.lev[l].Dinv64, xt, (int)nin, (int)nin, nrhs, false, c.stream);
             } else if (c.opt.mg_precision == 64) {
-                mg::mg_cycle<double2>(c, l, yt, xt, nrhs);
+                mg::with_less_memory(c, [&] { mg::mg_cycle<double2>(c, l, yt, xt, nrhs); });
             } else {
                 float2* x32 = c.scratch<float2>("ap_x32", (size_t)nin * nrhs);
                 float2* y32 = c.scratch<float2>("ap_y32", (size_t)nout * nrhs);
@@ -736,7 +736,7 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
                 auto* mx = c.scratch<unsigned long long>("unit_mx", nrhs);
                 mg::launch_absmax_cols(mx, xt, nin, nrhs, c.stream);
                 mg::launch_to_unit(x32, xt, mx, nin, nrhs, c.stream);
-                mg::mg_cycle<float2>(c, l, y32, x32, nrhs);
+                mg::with_less_memory(c, [&] { mg::mg_cycle<float2>(c, l, y32, x32, nrhs); });
                 mg::launch_from_unit(yt, y32, mx, nout, nrhs, c.stream);
             }
     }
@@ -864,6 +864,7 @@ mg::Shape context_shape(const Ctx& c) {
     }
     s.k = c.defl.k;
     s.precision = c.opt.mg_precision;
+    s.lean = c.lean;
     return s;
 }
 
@@ -932,6 +933,7 @@ extern "C" int mgmlmc_autotune(mgmlmc_ctx* h, size_t hbm_budget, int max_trials,
         // coarse-grid correction: allocated in an untimed run
         if (q.N != last_N || q.m > warm_m || q.nu > warm_nu || q.kc != warm_kc) {
             if (q.N != last_N) release_scratch(c);
+            mg::prepare_digits(c);               // where the context's own blocks were too narrow
             run_all();
             if (q.N != last_N) warm_m = warm_nu = 0;
             last_N = q.N;
@@ -975,7 +977,14 @@ extern "C" int mgmlmc_autotune(mgmlmc_ctx* h, size_t hbm_budget, int max_trials,
             Cand q{N, m1, start.nu_post, start.kcycle_iters};
             if (fits(q, nullptr)) widths.push_back(N);
         }
+        if (widths.empty()) {
+            // without the memory that a context can do without
+            base.lean = true;
+            for (int N : {1024, 512, 256, 128, 64, 32})
+                if (fits(Cand{N, m1, start.nu_post, start.kcycle_iters}, nullptr)) widths.push_back(N);
+        }
         MG_REQUIRE(!widths.empty(), MGMLMC_ENOMEM, "autotune: no block width fits the budget");
+        if (base.lean) c.set_lean();
         for (size_t i = 0; i < widths.size() && i < 3 && trials < max_trials; ++i)
             time_one(Cand{widths[i], m1, start.nu_post, start.kcycle_iters});
         // 2. restart length: 8, then 4 where 8 won; 12; 24 where 16 still leads

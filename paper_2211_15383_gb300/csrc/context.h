@@ -8,6 +8,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "footprint.h"
 #include "kernels.cuh"
 
 struct mgmlmc_ctx;
@@ -164,6 +165,19 @@ struct Ctx {
     std::unordered_map<void*, size_t> owned;   // device allocations and their sizes
     size_t live_bytes = 0, peak_bytes = 0;     // device bytes held now and at most
 
+    // Device memory that only makes things faster: the digits of the FP64 products, their work
+    // space, and more than one residual in a smoother's group.  It is asked for with try_alloc
+    // and try_scratch, and is given back when an allocation that is needed is refused, so that
+    // what fits without it still runs.  lean: do without it from the start.
+    bool lean = false;
+    int smoother_group = kSmootherGroup;       // residuals that a smoother keeps at most
+    bool extra_residuals = false;              // some smoother's space holds more than one
+    int cycles = 0;                            // running multigrid cycles (they use the residuals)
+    bool release_optional();                   // false: nothing to give back
+    void* try_alloc(size_t bytes);             // nullptr if refused
+    void* try_scratch(const std::string& name, size_t bytes);
+    void set_lean();
+
     void* dev_alloc(size_t bytes);
     void dev_free(void* p);
     template <typename T> T* alloc_n(size_t count) { return reinterpret_cast<T*>(dev_alloc(count * sizeof(T))); }
@@ -201,6 +215,15 @@ long long fgmres(Ctx& c, int l, const C* b, C* x, int N, double tol, long long m
 long long solve(Ctx& c, int l, const double2* b, double2* x, int N, double tol, int* ok);
 // One FGMRES cycle (restart length m) in the multigrid precision: x ~ D_l^{-1} b.
 void approx_inverse(Ctx& c, int l, const double2* b, double2* x, int N);
+// Runs f, and once more with the optional memory given back if it was refused memory.
+template <typename F> auto with_less_memory(Ctx& c, F f) {
+    try {
+        return f();
+    } catch (const Error& e) {
+        if (e.code != MGMLMC_ENOMEM || !c.release_optional()) throw;
+    }
+    return f();
+}
 void column_norms(Ctx& c, double* out, const double2* x, long long n, int N);
 // Throws MGMLMC_ETIMEOUT if a kernel with bounded waits recorded a timeout.
 void check_device_error(Ctx& c);
@@ -239,6 +262,9 @@ const Deflation* term_deflation(const Ctx& c, int a, int b);
 // the deflated trace over them (called whenever a deflation is stored).
 void prepare_tc_deflation(Ctx& c, Deflation& D);
 void upload_links(Ctx& c, const double* theta);
+// Digits of the FP64 products that the hierarchy does not have yet, for blocks of kF64TcMinRhs
+// right-hand sides and more (where the memory is granted).
+void prepare_digits(Ctx& c);
 
 }  // namespace mg
 

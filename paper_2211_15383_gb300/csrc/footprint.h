@@ -25,14 +25,20 @@ struct Shape {
     int precision = 64;              // mg_precision
     int kcycle = 0;                  // K-cycle steps per coarse-grid correction
     int nu = 4;                      // smoothing steps per level (the larger of pre and post)
+    bool lean = false;               // without the memory that a context can do without
 };
 
 // The FP64 coarsest inverse (mg_precision 64) is applied on the tensor cores up to this
 // size: its digits take 64 bytes an entry (1.1 GB at 4096 unknowns, 17 GB at 16384).
 inline bool f64_dense_inverse(long long n) { return n % 16 == 0 && n <= 4096; }
 
+// FP64 products run as digit products from this many right-hand sides on (below, the digits'
+// extra launches cost more than the FP64 pipe saves); contexts of narrower blocks keep none.
+constexpr int kF64TcMinRhs = 16;
+
 // Residuals that the smoother keeps at once: those of a group of at most 8 steps.
-inline int smoother_slots(int nu) { return std::min(std::max(nu, 1), 8); }
+constexpr int kSmootherGroup = 8;
+inline int smoother_slots(int nu) { return std::min(std::max(nu, 1), kSmootherGroup); }
 
 inline size_t footprint_bytes(const Shape& s) {
     const double N = std::max(1, s.N);
@@ -59,11 +65,11 @@ inline size_t footprint_bytes(const Shape& s) {
             b += st * d * d * (24 + 16) + st * 5 * d * d * 24;               // M^{-1}, D M^{-1}, work
             if (bf16) b += st * d * d * 80;                                  // BF16 operand tiles
         }
-        const bool digits = l > 0 && s.d[l] == 16;                           // FP64 products on the tensor cores
+        const bool digits = l > 0 && s.d[l] == 16 && s.N >= kF64TcMinRhs && !s.lean;   // FP64 digit products
         if (digits) b += st * (5 * 16384 + 32) * (f64 && l + 1 < L ? 2 : 1) + st * (std::ceil(N / 128) * 65536 + N * 2);
         if (l > 0) b += (2.0 * (double)s.n[l - 1] + n) * (digits ? std::min(N, 16.0) : N) * 16;   // FP64 Galerkin apply
         if (l + 1 < L) {
-            const double K = smoother_slots(s.nu);
+            const double K = s.lean ? 1 : smoother_slots(s.nu);
             const bool tiles = bf16 && l > 0 && s.d[l] == 16;                // smoothed on the tensor cores
             b += n * N * sz * (tiles ? 3 : K + 1) + 2.0 * (double)s.n[l + 1] * N * sz;   // V-cycle blocks
             if (tiles) b += (K + 2) * st * std::ceil(N / 128) * 8192 + n * N * 8;        // BF16 tiles, rhs
@@ -75,7 +81,7 @@ inline size_t footprint_bytes(const Shape& s) {
     }
     b += 2.0 * n0 * nvmax * 16;                                              // setup blocks
     b += nL * nL * 44 + nL * N * 136;                                        // dense coarsest inverse, BF16 solve
-    if (f64 && f64_dense_inverse(s.n[L - 1]))                                // its digits; x digits, partial sums
+    if (f64 && f64_dense_inverse(s.n[L - 1]) && s.N >= kF64TcMinRhs && !s.lean)   // its digits; x digits, partial sums
         b += nL * nL * 64 + nL / 16 * std::ceil(N / 128) * 65536 + std::ceil(nL / 96) * nL * N * 16;
     b += (2 * m + 1) * n0 * (N * sz + nvmax * 16);                           // FGMRES bases
     b += G * (m + 1) * N * 16 + N * (m + 1) * (m + 4) * 16;                  // Gram-Schmidt partials, Hessenberg

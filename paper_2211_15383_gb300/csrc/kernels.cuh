@@ -246,7 +246,7 @@ void launch_pack_tiles_bf16(__nv_bfloat16* rt, const float2* x, int nsites, int 
 // r.  d = 16.
 void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const float2* alpha, int nsites, int N, bool first,
                          __nv_bfloat16* rt, cudaStream_t s);
-// rn = r - alpha p as BF16 tiles (rn distinct from r), and e (=|+=) Minv sum_{s < K} alpha_s r_s over
+// rn = r - alpha p as BF16 tiles (rn may be r), and e (=|+=) Minv sum_{s < K} alpha_s r_s over
 // K consecutive sets of tiles (tc_tiles_bytes apart).
 void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __nv_bfloat16* p, const float2* alpha,
                             int nsites, int N, cudaStream_t s);

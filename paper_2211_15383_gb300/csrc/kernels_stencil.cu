@@ -11,6 +11,7 @@
 // component (e.g. (1 - sigma_1) psi = (a, -a) with a = psi_0 - psi_1).
 #include <algorithm>
 
+#include "footprint.h"
 #include "kernels.cuh"
 
 namespace mg {
@@ -920,7 +921,7 @@ __global__ void __launch_bounds__(256) k_mr_update(C* rn, const C* r, const C* _
 }
 
 // e (=|+=) sum_{s < K} alpha_s r_s
-constexpr int kMrGroup = 8;   // as in the solver's group loop
+constexpr int kMrGroup = kSmootherGroup;
 template <typename C, int V>
 __global__ void __launch_bounds__(256) k_mr_combine(C* __restrict__ e, const C* __restrict__ rs, size_t slot, int K,
                                                     const C* __restrict__ alpha, long long n, int N, bool e_is_zero) {
@@ -948,8 +949,7 @@ __global__ void __launch_bounds__(256) k_mr_combine(C* __restrict__ e, const C* 
 
 // The same two with the residuals and the image in BF16 (one bf16x2 word per complex
 // value), four rhs per thread: 16-byte accesses.  N % 4 == 0.
-__global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* __restrict__ rn,
-                                                             const uint32_t* __restrict__ r,
+__global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r,
                                                              const uint32_t* __restrict__ p,
                                                              const float2* __restrict__ alpha, long long n, int N) {
     if (grid_dependency()) return;

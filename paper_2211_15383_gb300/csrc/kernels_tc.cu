@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(CH) k_mr_update_tc(float2* __restrict__ yh, fl
 // 28, and the last one none.  One warp per 8-row group of a tile (512 contiguous bytes,
 // 16 B per lane: row lane & 7), four groups in flight; only the row groups that hold rhs
 // are touched.  Bound by HBM, or by L2 where the tiles fit it.
-__global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* __restrict__ rn, const uint4* __restrict__ r,
+__global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* rn, const uint4* r,
                                                          const uint4* __restrict__ p,
                                                          const float2* __restrict__ alpha, int nsites, int N, int T) {
     if (grid_dependency()) return;

@@ -97,8 +97,9 @@ int term_levels_of(const mgmlmc_request& r) {
 }
 
 // Device bytes a request's context holds at most (mg::footprint_bytes).
-size_t footprint_bytes(const mgmlmc_request& r, const Geometry& g) {
+size_t footprint_bytes(const mgmlmc_request& r, const Geometry& g, bool lean = false) {
     mg::Shape s;
+    s.lean = lean;
     s.L = g.L;
     s.nterm_levels = term_levels_of(r);
     for (int l = 0; l < g.L; ++l) {
@@ -134,6 +135,7 @@ struct Job {
     std::vector<std::vector<double>> start;   // start vectors of levels 1..L-1
     std::string shape;
     size_t reserved = 0;
+    bool lean = false;                        // without the memory that a context can do without
     int retries = 0;
     bool done = false;
     std::atomic<bool> cancel{false};
@@ -223,6 +225,7 @@ int run_job(Job& j, cudaStream_t stream, PoolUser* pu, std::string& msg, size_t&
     j.res.queued_s = seconds_between(j.t_submit, t0);
     step(j.cancel.load() ? MGMLMC_ECANCELLED : MGMLMC_OK, "admission");
     step(rc == MGMLMC_OK ? mgmlmc_create(&ctx, &r.opt, stream, pool_alloc, pool_free, pu) : rc, "create");
+    if (ctx && j.lean) ctx->c.set_lean();
     step(rc == MGMLMC_OK ? mgmlmc_set_gauge(ctx, r.Lx, r.Lt, j.theta.data()) : rc, "set_gauge");
     step(rc == MGMLMC_OK ? mgmlmc_set_mass(ctx, r.m0) : rc, "set_mass");
     if (rc == MGMLMC_OK) {
@@ -435,8 +438,19 @@ int mgmlmc_submit(mgmlmc_server* srv, const mgmlmc_request* req, uint64_t* id) {
     job->t_submit = Clock::now();
     std::lock_guard<std::mutex> lk(srv->mu);
     if (srv->stopping) return fail(MGMLMC_ESTATE, "submit: server stopping");
-    auto lp = srv->learned.find(job->shape);
-    const size_t bytes = lp != srv->learned.end() ? lp->second + lp->second / 10 : footprint_bytes(r, g);
+    auto bytes_of = [&](bool lean) {
+        auto lp = srv->learned.find(job->shape + (lean ? "/lean" : ""));
+        return lp != srv->learned.end() ? lp->second + lp->second / 10 : footprint_bytes(r, g, lean);
+    };
+    size_t bytes = bytes_of(false);
+    if (srv->adm->too_large(bytes)) {
+        const size_t lean = bytes_of(true);
+        if (!srv->adm->too_large(lean)) {
+            job->lean = true;
+            job->shape += "/lean";
+            bytes = lean;
+        }
+    }
     if (srv->adm->too_large(bytes))
         return fail(MGMLMC_ENOMEM, "submit: footprint " + std::to_string(bytes) + " B exceeds the budget of " +
                                        std::to_string(srv->adm->budget()) + " B");

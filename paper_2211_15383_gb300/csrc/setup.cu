@@ -8,28 +8,75 @@
 #include <vector>
 
 #include "context.h"
-#include "footprint.h"
 
 namespace mg {
 
 // ------------------------------------------------------------------ memory
-void* Ctx::dev_alloc(size_t bytes) {
+void* Ctx::try_alloc(size_t bytes) {
     if (bytes == 0) bytes = 16;
     void* p = nullptr;
     if (alloc) {
         p = alloc(alloc_user, bytes);
-        if (!p) throw Error(MGMLMC_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes refused");
-    } else {
-        cudaError_t e = cudaMalloc(&p, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            throw Error(MGMLMC_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + "): " + cudaGetErrorString(e));
-        }
+        if (!p) return nullptr;
+    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
     owned[p] = bytes;
     live_bytes += bytes;
     peak_bytes = std::max(peak_bytes, live_bytes);
     return p;
+}
+
+void* Ctx::dev_alloc(size_t bytes) {
+    void* p = try_alloc(bytes);
+    if (!p && release_optional()) p = try_alloc(bytes);
+    if (!p) throw Error(MGMLMC_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes refused");
+    return p;
+}
+
+bool Ctx::release_optional() {
+    bool any = false;
+    auto drop = [&](void*& p) {
+        if (!p) return;
+        if (!any) sync();                        // kernels in flight may read it
+        any = true;
+        dev_free(p);
+        p = nullptr;
+    };
+    for (Level& l : lev) {
+        drop(l.A64t);
+        drop(l.Ahat64t);
+        drop(l.Dinv64t);
+    }
+    for (auto& kv : ws) {
+        auto starts = [&](const char* s) { return kv.first.rfind(s, 0) == 0; };
+        const bool residuals = starts("cyc_res_") || starts("mr_rt_") || starts("mrf_rb");
+        if (starts("f64_") || (residuals && cycles == 0 && extra_residuals)) {
+            drop(kv.second.p);
+            kv.second.bytes = 0;
+        }
+    }
+    if (cycles == 0) {
+        smoother_group = 1;
+        extra_residuals = false;
+    }
+    return any;
+}
+
+void Ctx::set_lean() {
+    lean = true;
+    release_optional();
+}
+
+void* Ctx::try_scratch(const std::string& name, size_t bytes) {
+    Buf& b = ws[name];
+    if (b.p && b.bytes >= bytes) return b.p;
+    if (b.p) dev_free(b.p);
+    b.bytes = ((bytes + 255) / 256) * 256;
+    b.p = try_alloc(b.bytes);
+    if (!b.p) b.bytes = 0;
+    return b.p;
 }
 
 void Ctx::dev_free(void* p) {
@@ -117,6 +164,7 @@ void Ctx::free_hierarchy() {
     free_deflation();
     L = 0;
     have_hier = false;
+    smoother_group = lean ? 1 : kSmootherGroup;
     for (auto& s : stats) s = TermStats();
 }
 
@@ -218,6 +266,8 @@ void copy_state(Ctx& d, Ctx& s) {
     d.have_mass = s.have_mass;
     d.have_hier = s.have_hier;
     d.m0 = s.m0;
+    d.lean = s.lean;
+    d.smoother_group = s.smoother_group;
     const size_t V = (size_t)s.Lx * s.Lt;
     d.U64 = dup(d, s.U64, 2 * V);
     d.U32 = dup(d, s.U32, 2 * V);
@@ -238,7 +288,10 @@ void copy_state(Ctx& d, Ctx& s) {
         a.A64 = dup(d, b.A64, 5 * nb);
         a.A32 = dup(d, b.A32, 5 * nb);
         auto dup_digits = [&](const void* p, long long nblk, int nb) -> void* {
-            return dup(d, reinterpret_cast<const char*>(p), f64_tc_operand_bytes(nblk, nb));
+            const size_t bytes = f64_tc_operand_bytes(nblk, nb);
+            void* q = p ? d.try_alloc(bytes) : nullptr;
+            if (q) MG_CUDA(cudaMemcpyAsync(q, p, bytes, cudaMemcpyDeviceToDevice, d.stream));
+            return q;
         };
         a.A64t = dup_digits(b.A64t, 5LL * b.nsites, 0);
         a.Ahat64t = dup_digits(b.Ahat64t, 5LL * b.nsites, 0);
@@ -364,6 +417,30 @@ constexpr int kRefreshRounds = 2;
 constexpr int kRayleighRitzEvery = 4;
 
 // ------------------------------------------------------------------ hierarchy
+// Digits of a level's stencil blocks, and of the coarsest inverse, for the FP64 products on the
+// tensor cores: kept where blocks can be wide enough to use them and the memory is granted.
+static bool digits_wanted(const Ctx& c) { return !c.lean && c.opt.max_block_rhs >= kF64TcMinRhs; }
+static void f64_stencil_operand(Ctx& c, void*& op, const double2* A, const Level& L) {
+    if (!digits_wanted(c) || !f64_tc_supported(L.d, 1)) return;
+    if (!op) op = c.try_alloc(f64_tc_operand_bytes(5LL * L.nsites, 0));
+    if (op) launch_f64_operand(op, A, 5LL * L.nsites, 0, 0, c.stream);
+}
+static void f64_inverse_operand(Ctx& c) {
+    Level& L = c.lev[c.L - 1];
+    const long long nb = L.n / 16;
+    if (!digits_wanted(c) || !f64_dense_inverse(L.n)) return;
+    if (!L.Dinv64t) L.Dinv64t = c.try_alloc(f64_tc_operand_bytes(nb * nb, (int)nb));
+    if (L.Dinv64t) launch_f64_operand(L.Dinv64t, L.Dinv64, nb * nb, (int)nb, (int)L.n, c.stream);
+}
+void prepare_digits(Ctx& c) {
+    for (int l = 1; l < c.L; ++l) {
+        Level& L = c.lev[l];
+        if (!L.A64t) f64_stencil_operand(c, L.A64t, L.A64, L);
+        if (c.opt.mg_precision == 64 && l + 1 < c.L && !L.Ahat64t) f64_stencil_operand(c, L.Ahat64t, L.Ahat64, L);
+    }
+    if (c.opt.mg_precision == 64 && c.L > 0 && !c.lev[c.L - 1].Dinv64t) f64_inverse_operand(c);
+}
+
 static void coarsest_inverse(Ctx& c) {
     Level& L = c.lev[c.L - 1];
     const long long n = L.n;
@@ -379,11 +456,7 @@ static void coarsest_inverse(Ctx& c) {
             ProfScope ps(c, "setup.gauss_jordan.f64", 2.0 * n * n * 16 * std::ceil(n / 16.0), 8.0 * n * n * n);
             launch_gauss_jordan<double2>(L.Dinv64, (int)n, work, c.stream);
         }
-        if (f64_dense_inverse(n)) {
-            const long long nb = n / 16;
-            if (!L.Dinv64t) L.Dinv64t = c.dev_alloc(f64_tc_operand_bytes(nb * nb, (int)nb));
-            launch_f64_operand(L.Dinv64t, L.Dinv64, nb * nb, (int)nb, (int)n, c.stream);
-        }
+        f64_inverse_operand(c);
     } else {
         if (!L.Dinv32) L.Dinv32 = c.alloc_n<float2>((size_t)n * n);
         launch_convert<float2, double2>(L.Dinv32, Dd, n * n, c.stream);
@@ -398,13 +471,6 @@ static void coarsest_inverse(Ctx& c) {
     MG_CUDA(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     c.sync();
     MG_REQUIRE(hs == 0, MGMLMC_EINVAL, "coarsest operator is singular (zero pivot)");
-}
-
-// Digits of a level's stencil blocks for the FP64 products on the tensor cores.
-static void f64_stencil_operand(Ctx& c, void*& op, const double2* A, const Level& L) {
-    if (!f64_tc_supported(L.d, 1)) return;
-    if (!op) op = c.dev_alloc(f64_tc_operand_bytes(5LL * L.nsites, 0));
-    launch_f64_operand(op, A, 5LL * L.nsites, 0, 0, c.stream);
 }
 
 // Block-Jacobi smoother of coarse level l: M = block diagonal of D_l (the self

@@ -54,24 +54,25 @@ static bool galerkin_form_cheaper(const Ctx& c, int l) {
     return galerkin < direct;
 }
 
-// FP64 block stencils with d = 16 run on the tensor cores (exact integer digit products, at
-// least as accurate as FP64 sums) from this many right-hand sides on; below it the digits'
-// three extra launches cost more than the FP64 pipe saves.
-constexpr int kF64TcMinRhs = 16;
+// FP64 block stencils with d = 16 run on the tensor cores (exact integer digit products, as
+// accurate as FP64 sums) from kF64TcMinRhs right-hand sides on, where the level has its digits
+// and their work space is granted.  op: the level's own pointer (an allocation may take the
+// digits away).
 template <typename C>
-static bool f64_stencil(Ctx&, const Level&, C*, const C*, const C*, const void*, const C*, int, int, double2*, int) {
+static bool f64_stencil(Ctx&, const Level&, C*, const C*, const C*, void* const&, const C*, int, int, double2*, int) {
     return false;
 }
 static bool f64_stencil_used(const Level& L, const void* op, int N) {
     return op && N >= kF64TcMinRhs && f64_tc_supported(L.d, N);
 }
 template <>
-bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, const double2* b, const void* op,
+bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, const double2* b, void* const& op,
                           const double2* A, int N, int mode, double2* part, int groups) {
+    int* err = device_error_flag(c);
     if (!f64_stencil_used(L, op, N)) return false;
-    launch_block_stencil_f64(y, x, b, op, A, L.lx, L.lt, N, mode,
-                             c.scratch_bytes("f64_tc", f64_tc_scratch_bytes(L.nsites, N)), part, groups,
-                             device_error_flag(c), c.stream);
+    void* scr = c.try_scratch("f64_tc", f64_tc_scratch_bytes(L.nsites, N));
+    if (!scr) return false;
+    launch_block_stencil_f64(y, x, b, op, A, L.lx, L.lt, N, mode, scr, part, groups, err, c.stream);
     return true;
 }
 template <typename C> static int bst_groups(const Level& L, const void* op, int N) {
@@ -144,11 +145,17 @@ int* device_error_flag(Ctx& c) {
 template <typename C> static bool tc_smoother(const Level&, int) { return false; }
 template <> bool tc_smoother<float2>(const Level& L, int N) { return L.Ahat16 && tc_stencil_supported(L.d, N); }
 
-// `slots` consecutive sets of BF16 tiles of one level-l block vector.
-static __nv_bfloat16* tc_tiles(Ctx& c, const char* name, int l, int N, int slots = 1) {
-    return reinterpret_cast<__nv_bfloat16*>(
-        c.scratch_bytes(nm(name, l, 2), slots * tc_tiles_bytes(c.lev[l].nsites, N)));
+// BF16 tiles of one level-l block vector.
+static __nv_bfloat16* tc_tiles(Ctx& c, const char* name, int l, int N) {
+    return reinterpret_cast<__nv_bfloat16*>(c.scratch_bytes(nm(name, l, 2), tc_tiles_bytes(c.lev[l].nsites, N)));
 }
+
+// A multigrid cycle (or a smoother operator) is running: its residuals are in use.
+struct CycleScope {
+    Ctx& c;
+    explicit CycleScope(Ctx& ctx) : c(ctx) { ++c.cycles; }
+    ~CycleScope() { --c.cycles; }
+};
 
 // y = (D_l M_l^{-1}) x on the tensor cores, x given as its BF16 tiles xt, y as FP32 rows
 // (y) or BF16 tiles (yt), or only alpha (may be null) = <y, x> / <y, y> (against the BF16 x).
@@ -206,6 +213,7 @@ template <typename C>
 void apply_smoother_operator(Ctx& c, int l, C* y, const C* x, int N) {
     MG_REQUIRE(l >= 1 && l < c.L - 1 && hat_blocks<C>(c.lev[l]), MGMLMC_EINVAL,
                "smoother operator: only coarse levels above the coarsest");
+    const CycleScope running(c);
     if (!apply_smoother_tc<C>(c, l, y, x, N)) apply_Dhat<C>(c, l, y, x, N, 0, nullptr);
 }
 
@@ -236,10 +244,12 @@ static double dinv_flops(const Level& L, int N) { return 8.0 * (double)L.n * L.n
 template <> void coarsest_apply<double2>(Ctx& c, double2* e, const double2* r, int N) {
     const Level& L = c.lev[c.L - 1];
     ProfScope ps(c, "Dinv.f64", dinv_bytes(L, N, 16), dinv_flops(L, N));
+    int* err = device_error_flag(c);
     if (L.Dinv64t && N >= kF64TcMinRhs && f64_tc_supported(16, N)) {
-        void* scr = c.scratch_bytes("f64_dense", f64_dense_scratch_bytes((int)L.n, N));
-        launch_dense_f64(e, r, L.Dinv64t, (int)L.n, N, scr, device_error_flag(c), c.stream);
-        return;
+        if (void* scr = c.try_scratch("f64_dense", f64_dense_scratch_bytes((int)L.n, N))) {
+            launch_dense_f64(e, r, L.Dinv64t, (int)L.n, N, scr, err, c.stream);
+            return;
+        }
     }
     launch_gemm_nn<double2>(e, L.Dinv64, r, (int)L.n, (int)L.n, N, false, c.stream);
 }
@@ -265,19 +275,25 @@ template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int 
     launch_gemm_nn<float2>(e, L.Dinv32, r, (int)L.n, (int)L.n, N, false, c.stream);
 }
 
-// Minimal-residual steps are taken in groups of at most kMrGroup: the residuals of a
+// Minimal-residual steps are taken in groups of at most kSmootherGroup: the residuals of a
 // group stay in consecutive slots, and the correction takes sum_s alpha_s r_s once per
-// group.  Slots needed for nu steps:
-constexpr int kMrGroup = 8;
-static int mr_slots(int nu) { return std::min(std::max(nu, 1), kMrGroup); }
+// group.  Slots for nu steps of `bytes` each, as many as the memory allows (one at least: it is
+// updated in place); K: their number.
+static void* mr_slots(Ctx& c, const std::string& name, size_t bytes, int nu, int& K) {
+    for (K = std::min(smoother_slots(nu), c.smoother_group); K > 1; K = c.smoother_group = (K + 1) / 2)
+        if (void* p = c.try_scratch(name, K * bytes)) {
+            c.extra_residuals = true;
+            return p;
+        }
+    return c.scratch_bytes(name, bytes);
+}
 
 // The group loop, for any form of the vectors: image(s, last) forms the image of slot s and
 // its coefficient (the last step of all needs no image), flush(K, first) adds the K slots to
 // the correction, update(s, t) forms the next residual from slot s in slot t.  Returns the
 // slot of the final residual (with need_r), else -1.
 template <typename Image, typename Flush, typename Update>
-static int mr_steps(int nu, bool need_r, Image image, Flush flush, Update update) {
-    const int K = mr_slots(nu);
+static int mr_steps(int nu, int K, bool need_r, Image image, Flush flush, Update update) {
     int slot = 0;
     for (int s = 0; s < nu; ++s) {
         const bool last = s + 1 == nu && !need_r;
@@ -306,11 +322,12 @@ template <>
 bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bool have_et) {
     if (!post_smooths_tc<float2>(c, l, N)) return false;
     const Level& L = c.lev[l];
-    const int nu = c.opt.nu_post, K = mr_slots(nu);
-    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kMrGroup * N);
+    const int nu = c.opt.nu_post;
+    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kSmootherGroup * N);
     __nv_bfloat16* et = tc_tiles(c, "cyc_et", l, N);
-    __nv_bfloat16* rt = tc_tiles(c, "mr_rt", l, N, K);
     __nv_bfloat16* pt = tc_tiles(c, "mr_pt", l, N);
+    int K = 1;
+    __nv_bfloat16* rt = reinterpret_cast<__nv_bfloat16*>(mr_slots(c, nm("mr_rt", l, 2), tc_tiles_bytes(L.nsites, N), nu, K));
     const size_t slot = tc_tiles_bytes(L.nsites, N) / sizeof(__nv_bfloat16);
     if (!have_et) pack_tiles(c, l, et, e, N);
     {
@@ -323,7 +340,7 @@ bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bo
                                 c.stream);
     }
     mr_steps(
-        nu, false,
+        nu, K, false,
         [&](int s, bool last) { apply_Dhat_tc(c, l, nullptr, last ? nullptr : pt, rt + s * slot, N, alpha + (size_t)s * N); },
         [&](int k, bool) {
             // traffic: the K residuals (4 B per complex) read, e read and written
@@ -348,7 +365,7 @@ bool pre_smooth_tc<float2>(Ctx& c, int l, float2* e, float2* r, int N, int nu) {
     if (!tc_smoother<float2>(L, N)) return false;
     float2* yh = c.scratch<float2>(nm("mr_y", l, sizeof(float2)), (size_t)L.n * N);
     float2* p = c.scratch<float2>(nm("mr_p", l, sizeof(float2)), (size_t)L.n * N);
-    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kMrGroup * N);
+    float2* alpha = c.scratch<float2>(nm("mr_al", l, sizeof(float2)), (size_t)kSmootherGroup * N);
     __nv_bfloat16* rt = tc_tiles(c, "mr_rt", l, N);
     pack_tiles(c, l, rt, r, N);
     for (int s = 0; s < nu; ++s) {
@@ -374,18 +391,19 @@ bool post_smooth_fine_bf16<float2>(Ctx& c, int l, float2* e, const float2* r, in
     if (l != 0 || nu <= 0 || c.opt.mg_precision != 16 || N % 4) return false;
     const Level& L = c.lev[0];
     const size_t nN = (size_t)L.n * N;
-    uint32_t* rb = c.scratch<uint32_t>("mrf_rb", mr_slots(nu) * nN);
     uint32_t* pb = c.scratch<uint32_t>("mrf_pb", nN);
-    float2* alpha = c.scratch<float2>(nm("mr_al", 0, sizeof(float2)), (size_t)kMrGroup * N);
+    float2* alpha = c.scratch<float2>(nm("mr_al", 0, sizeof(float2)), (size_t)kSmootherGroup * N);
     const int groups = stencil_groups_bf16(L.nsites, N);
     double2* part = c.scratch<double2>("part_st", (size_t)groups * 2 * N);
+    int K = 1;
+    uint32_t* rb = reinterpret_cast<uint32_t*>(mr_slots(c, "mrf_rb", nN * sizeof(uint32_t), nu, K));
     {
         // algorithmic traffic: e and r read (8 B each), the BF16 residual written
         ProfScope ps(c, "D1res.bf16", (double)nN * 20 + 2.0 * L.nsites * 8, 60.0 * L.nsites * N);
         launch_wilson_residual_bf16(rb, e, r, c.U32, c.m0, L.lx, L.lt, N, stencil_groups(L.nsites, N), c.stream);
     }
     mr_steps(
-        nu, false,
+        nu, K, false,
         [&](int s, bool last) {
             {
                 // algorithmic traffic: BF16 x read, y written once (4 B per complex), links once
@@ -407,19 +425,19 @@ bool post_smooth_fine_bf16<float2>(Ctx& c, int l, float2* e, const float2* r, in
     return true;
 }
 
-// nu MR steps on D_l e = r0 starting from e (or 0); rs has mr_slots(nu) slots, the first
+// nu MR steps on D_l e = r0 starting from e (or 0); rs has K slots, the first
 // holding the current residual.  Returns the slot with the final residual (need_r).  On
 // coarse levels above the coarsest: block-Jacobi MR, minimal-residual steps on D M^{-1}
 // whose preconditioned correction M^{-1} sum_s alpha_s r_s goes to e.
 template <typename C>
-static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int N, int nu, bool e_zero, bool need_r) {
+static C* mr_smooth(Ctx& c, int l, C* e, C* rs, int K, int N, int nu, bool e_zero, bool need_r) {
     const Level& L = c.lev[l];
     const size_t nN = (size_t)L.n * N;
     C* p = c.scratch<C>(nm("mr_p", l, sizeof(C)), nN);
-    C* alpha = c.scratch<C>(nm("mr_al", l, sizeof(C)), (size_t)kMrGroup * N);
+    C* alpha = c.scratch<C>(nm("mr_al", l, sizeof(C)), (size_t)kSmootherGroup * N);
     const bool jacobi = hat_blocks<C>(L) != nullptr;
     const int fin = mr_steps(
-        nu, need_r,
+        nu, K, need_r,
         [&](int s, bool last) {
             const int mode = last ? 3 : 2;
             if (jacobi) apply_Dhat<C>(c, l, last ? nullptr : p, rs + s * nN, N, mode, alpha + (size_t)s * N);
@@ -598,20 +616,22 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
         coarsest_apply<C>(c, e, r, N);
         return;
     }
+    const CycleScope running(c);
     const Level& L = c.lev[l];
     const Level& Lc = c.lev[l + 1];
     C* rc = c.scratch<C>(nm("cyc_rc", l + 1, sizeof(C)), (size_t)Lc.n * N);
     C* ec = c.scratch<C>(nm("cyc_ec", l + 1, sizeof(C)), (size_t)Lc.n * N);
     const size_t nN = (size_t)L.n * N;
-    auto residual_slots = [&](int slots) { return c.scratch<C>(nm("cyc_res", l, sizeof(C)), slots * nN); };
+    int K = 1;
+    auto residual_slots = [&](int nu) { return reinterpret_cast<C*>(mr_slots(c, nm("cyc_res", l, sizeof(C)), sizeof(C) * nN, nu, K)); };
     bool e_zero = true;
     if (c.opt.nu_pre > 0) {
         // the pre-smoother on the tensor cores keeps one residual
-        C* res = residual_slots(tc_smoother<C>(L, N) ? 1 : mr_slots(c.opt.nu_pre));
+        C* res = residual_slots(tc_smoother<C>(L, N) ? 1 : c.opt.nu_pre);
         MG_CUDA(cudaMemcpyAsync(res, r, sizeof(C) * nN, cudaMemcpyDeviceToDevice, c.stream));
         // leaves res = r - D e
         if (!pre_smooth_tc<C>(c, l, e, res, N, c.opt.nu_pre))
-            res = mr_smooth<C>(c, l, e, res, N, c.opt.nu_pre, true, true);
+            res = mr_smooth<C>(c, l, e, res, K, N, c.opt.nu_pre, true, true);
         e_zero = false;
         apply_restrict<C>(c, l, rc, res, N);
     } else {
@@ -626,9 +646,9 @@ void mg_cycle(Ctx& c, int l, C* e, const C* r, int N) {
     const bool have_et = apply_prolong<C>(c, l, e, ec, N, !e_zero, et);
     if (c.opt.nu_post <= 0 || post_smooth_tc<C>(c, l, e, r, N, have_et) || post_smooth_fine_bf16<C>(c, l, e, r, N))
         return;
-    C* res = residual_slots(mr_slots(c.opt.nu_post));
+    C* res = residual_slots(c.opt.nu_post);
     apply_D<C>(c, l, res, e, r, N, 1, nullptr);
-    mr_smooth<C>(c, l, e, res, N, c.opt.nu_post, false, false);
+    mr_smooth<C>(c, l, e, res, K, N, c.opt.nu_post, false, false);
 }
 
 // One Arnoldi cycle from the started basis B (first vector, eta_0, g_0): at most B.m steps,
@@ -743,7 +763,7 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
 // column chunks of at most that width, so the Krylov work space stays bounded.
 long long solve(Ctx& c, int l, const double2* b, double2* x, int N, double tol, int* ok) {
     const int blk = c.opt.max_block_rhs;
-    if (N <= blk) return solve_block(c, l, b, x, N, tol, ok);
+    if (N <= blk) return with_less_memory(c, [&] { return solve_block(c, l, b, x, N, tol, ok); });
     const long long n = c.lev[l].n;
     double2* bb = c.scratch<double2>("sv_chunk_b", (size_t)n * blk);
     double2* xb = c.scratch<double2>("sv_chunk_x", (size_t)n * blk);
@@ -755,7 +775,7 @@ long long solve(Ctx& c, int l, const double2* b, double2* x, int N, double tol, 
         MG_CUDA(cudaMemcpy2DAsync(bb, nb * w, b + j0, (size_t)N * w, nb * w, (size_t)n, cudaMemcpyDeviceToDevice,
                                   c.stream));
         int okb = 0;
-        it += solve_block(c, l, bb, xb, nb, tol, &okb);
+        it += with_less_memory(c, [&] { return solve_block(c, l, bb, xb, nb, tol, &okb); });
         all &= okb;
         MG_CUDA(cudaMemcpy2DAsync(x + j0, (size_t)N * w, xb, nb * w, nb * w, (size_t)n, cudaMemcpyDeviceToDevice,
                                   c.stream));
@@ -944,7 +964,7 @@ void column_norms(Ctx& c, double* out, const double2* x, long long n, int N) {
 void approx_inverse(Ctx& c, int l, const double2* b, double2* x, int N) {
     int ok = 0;
     if (c.opt.mg_precision == 64) {
-        fgmres<double2>(c, l, b, x, N, 1e-14, c.opt.fgmres_restart, true, &ok, 1);
+        with_less_memory(c, [&] { return fgmres<double2>(c, l, b, x, N, 1e-14, c.opt.fgmres_restart, true, &ok, 1); });
         return;
     }
     const size_t nN = (size_t)c.lev[l].n * N;
@@ -954,7 +974,7 @@ void approx_inverse(Ctx& c, int l, const double2* b, double2* x, int N) {
     const long long n = c.lev[l].n;
     launch_absmax_cols(mx, b, n, N, c.stream);
     launch_to_unit(b32, b, mx, n, N, c.stream);
-    fgmres<float2>(c, l, b32, x32, N, 1e-6, c.opt.fgmres_restart, true, &ok, 1);
+    with_less_memory(c, [&] { return fgmres<float2>(c, l, b32, x32, N, 1e-6, c.opt.fgmres_restart, true, &ok, 1); });
     launch_from_unit(x, x32, mx, n, N, c.stream);
 }
 }  // namespace mg

@@ -1,5 +1,6 @@
 """A device allocation that is refused leaves a context as good as before: the same call, with
-the memory granted, gives what it gives on a fresh context."""
+the memory granted, gives what it gives on a fresh context, in as many iterations (to rounding:
+the context has given up the memory that it can do without)."""
 import numpy as np
 import pytest
 
@@ -67,4 +68,4 @@ def test_solve(pkg, monkeypatch, prec, n):
                 assert e.code == ENOMEM
             alloc.start()
             x, it = ctx.solve(2, b)
-            assert it == iters and np.array_equal(x, ref), i
+            assert it == iters and np.abs(x - ref).max() < 1e-10 * np.abs(ref).max(), i
