@@ -60,9 +60,10 @@ typedef void (*mgmlmc_free_fn)(void* user, void* ptr);
 typedef struct {
     int mg_precision;     /* 64: FP64 multigrid preconditioner ("plain FP64 path");
                              32: FP32 V-cycle with a BF16 tensor-core coarsest solve
-                             (mixed; FP32 for fewer than 32 rhs and at most 1024
-                             unknowns); 16: as 32, and the coarse-level smoother's
-                             block stencil (d = 16) on the tensor cores in BF16.
+                             (mixed; FP32 for few rhs of a small coarsest level,
+                             e.g. 16 of 1024 unknowns, 31 of 512); 16: as 32, and
+                             the coarse-level smoother's block stencil (d = 16) on
+                             the tensor cores in BF16.
                              The outer FGMRES, its residuals and every sample are
                              FP64 in all cases.                                [64]    */
     double solve_tol;     /* relative residual ||b - D x|| / ||b|| of every solve;

@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(128) k_gemm_nn8(C* __restrict__ Cm, const C* _
 // y = A x for a dense n x n matrix and few columns (N <= 32), FP32: a CTA per kFewRows rows,
 // lanes over the columns and (the rest of them, and the warps) over K; the slices are added in
 // order.  Bound by reading A once from L2 or HBM; for few columns
-// the tensor-core form takes three launches (pack, product, sum of splits: 12 us) for this one
-// (4 us at n = 256, 8 us at n = 1024).
+// the tensor-core form takes three launches (pack, product, sum of splits) for this one; the
+// solver's rule between the two stands there with the times of both.
 constexpr int kFewRows = 4;
 __global__ void __launch_bounds__(256) k_gemm_few(float2* __restrict__ y, const float2* __restrict__ A,
                                                   const float2* __restrict__ x, int n, int N, int cols) {

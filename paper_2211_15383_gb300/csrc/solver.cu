@@ -237,7 +237,24 @@ bool apply_prolong(Ctx& c, int l, C* x, const C* xc, int N, bool accumulate, voi
     return launch_prolong<C>(x, xc, prol<C>(L), L.lx, L.lt, L.d, L.ax, L.at, L.nvec, N, accumulate, c.stream, xt);
 }
 
-constexpr int kFewRhs = 32, kFewRhsUnknowns = 1024;
+// Few right-hand sides of a small level are solved by the FP32 inverse in one launch, whose time
+// goes with n (its dependent loads) and with the power of two of columns that N fills (each
+// matrix entry's arithmetic); the BF16 form on the tensor cores takes three launches, 15 us up
+// to n = 1024 whatever N.  Measured, us (with the launch gaps), for 2, 4, 8, 16 and 32 columns:
+//   n = 256: 8.0, 6.7, 6.5, 8.1, 10.5;  n = 512: 8.0, 7.5, 8.2, 10.2, 16.2;
+//   n = 1024: 8.2, 9.6, 12.3, 18.3, 30.6;  n = 2048: 14, 21, 33, 57, 107 (BF16: 17).
+// Solves on the levels above take the same iterations with either (16 to 19 at 64^2), those on the
+// coarsest level itself fewer with the FP32 inverse (six inverse iterations of 16 rhs at n = 1024:
+// 23 for 36 to 1e-12, 18 for 24 to 1e-7), so that 16 columns at n = 1024 pay there (deflation of
+// 64^2 182 ms, 194 with BF16; the pilot draw 7.49 and 7.42) and 32 columns, at twice the other
+// form's time, do not.  The line: columns times n.  A level without the BF16 inverse (n no multiple of 128) takes the one launch throughout (960 unknowns:
+// 8.3 to 29 us, the tiled FP32 product 43 to 66).
+constexpr long long kFewRhs = 32, kFewRhsWork = 16384, kFewRhsUnknowns = 1024;
+static bool few_rhs(const Level& L, int N) {
+    long long cols = 1;
+    while (cols < N) cols *= 2;
+    return N < kFewRhs && L.n <= kFewRhsUnknowns && (!L.Dinv16 || cols * L.n <= kFewRhsWork);
+}
 template <typename C> static void coarsest_apply(Ctx& c, C* e, const C* r, int N);
 static double dinv_bytes(const Level& L, int N, double s) { return (double)L.n * L.n * s + 2.0 * L.n * N * s; }
 static double dinv_flops(const Level& L, int N) { return 8.0 * (double)L.n * L.n * N; }
@@ -255,11 +272,7 @@ template <> void coarsest_apply<double2>(Ctx& c, double2* e, const double2* r, i
 }
 template <> void coarsest_apply<float2>(Ctx& c, float2* e, const float2* r, int N) {
     const Level& L = c.lev[c.L - 1];
-    // few right-hand sides of a small level: the FP32 inverse in one launch (4 us at n = 256;
-    // at n = 1024 9 us for 8 rhs and 15 for 16, against 12 us of the tensor-core form's three,
-    // whose BF16 digits cost outer iterations; at twice that size reading four times the FP32
-    // inverse takes longer)
-    if (N < kFewRhs && L.n <= kFewRhsUnknowns) {
+    if (few_rhs(L, N)) {
         ProfScope ps(c, "Dinv.f32", dinv_bytes(L, N, 8), dinv_flops(L, N));
         launch_gemm_few(e, L.Dinv32, r, (int)L.n, N, c.stream);
         return;
