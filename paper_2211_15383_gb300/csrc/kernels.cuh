@@ -129,7 +129,8 @@ void launch_wilson(C* y, const C* x, const C* b, const C* U, double m0, int lx, 
 // Fine-level smoother in BF16 (one bf16x2 word per complex value, [row][rhs]):
 // y = D x (y may be null) with per-rhs dots conj(y).x, |y|^2 (partials as launch_wilson
 // mode 2; N % 4 == 0), the residual b - D x rounded to BF16 (N even), and the smoother's
-// updates: rn = r - alpha p, e (=|+=) sum_{s < K} alpha_s r_s over K <= 8 slots (N % 4 == 0).
+// updates: rn = r - alpha p (rn may be r), e += sum_{s < K} alpha_s r_s over K <= kSmootherGroup
+// slots (N % 4 == 0).
 void launch_wilson_bf16(uint32_t* y, const uint32_t* x, const float2* U, double m0, int lx, int lt, int N,
                         double2* part, int groups, cudaStream_t s);
 void launch_wilson_residual_bf16(uint32_t* y, const float2* x, const float2* b, const float2* U, double m0, int lx,
@@ -137,7 +138,7 @@ void launch_wilson_residual_bf16(uint32_t* y, const float2* x, const float2* b, 
 void launch_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r, const uint32_t* p, const float2* alpha, long long n,
                                 int N, cudaStream_t s);
 void launch_mr_combine_bf16(float2* e, const uint32_t* rs, size_t slot, int K, const float2* alpha, long long n, int N,
-                            bool e_is_zero, cudaStream_t s);
+                            cudaStream_t s);
 // Coarse 5-point block stencil y_s = sum_dir A[s][dir] x_nbr(s,dir), d x d complex blocks,
 // dir = 0 self, 1 +x, 2 -x, 3 +t, 4 -t (periodic; boundary signs live in the blocks).
 template <typename C>
@@ -246,12 +247,12 @@ void launch_pack_tiles_bf16(__nv_bfloat16* rt, const float2* x, int nsites, int 
 // r.  d = 16.
 void launch_mr_update_tc(float2* yh, float2* r, const float2* p, const float2* alpha, int nsites, int N, bool first,
                          __nv_bfloat16* rt, cudaStream_t s);
-// rn = r - alpha p as BF16 tiles (rn may be r), and e (=|+=) Minv sum_{s < K} alpha_s r_s over
+// rn = r - alpha p as BF16 tiles (rn may be r), and e += Minv sum_{s < K} alpha_s r_s over
 // K consecutive sets of tiles (tc_tiles_bytes apart).
 void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __nv_bfloat16* p, const float2* alpha,
                             int nsites, int N, cudaStream_t s);
 void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const float2* alpha, const float2* Minv,
-                             int nsites, int N, bool accumulate, cudaStream_t s);
+                             int nsites, int N, cudaStream_t s);
 int block_stencil_tc_groups(int nsites, int N);
 // Output: y (FP32 rows), yt (BF16 tiles) or neither (the dots only); with b (FP32 rows,
 // yt only) the tiles receive the residual b - A x and no dots are formed.

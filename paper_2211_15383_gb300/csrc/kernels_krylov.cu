@@ -31,11 +31,10 @@ template <typename C, int V> struct alignas(sizeof(C) * V) Vec { C v[V]; };
 struct Shape2 {
     dim3 g, b;
 };
-static Shape2 shape(long long n, int N, int V, int groups) {
+static Shape2 shape(int N, int V, int groups) {
     const int cols = (N + V - 1) / V;
     int bx = 1;
     while (bx < cols && bx < 32) bx *= 2;
-    (void)n;
     return {dim3((cols + bx - 1) / bx, groups), dim3(bx, 256 / bx)};
 }
 static int groups_of(long long n, int N, int V, int per_sm) {
@@ -554,7 +553,7 @@ void launch_multidot(C* cf, double2* H, const C* V, int m, const C* w, long long
     const int W = width<C>(N);
     const int G = groups_of(n, N, W, 4);
     constexpr int W2 = sizeof(C) == 8 ? 2 : 1;   // FP64: one rhs per thread
-    const Shape2 s2 = shape(n, N, W, G), s1 = shape(n, N, 1, G);
+    const Shape2 s2 = shape(N, W, G), s1 = shape(N, 1, G);
     // at most 32 vectors a launch (their sums are registers)
     for (int k0 = 0; k0 < m; k0 += 32) {
         const int mk_ = std::min(32, m - k0);
@@ -594,10 +593,10 @@ void launch_multiaxpy(C* w, const C* cf, int m, const C* V, long long n, int N, 
     constexpr int W2 = sizeof(C) == 8 ? 2 : 1;
     const int G = axpy_groups(n, N);
     if (width<C>(N) == 2) {
-        const Shape2 sh = shape(n, N, W2, G);
+        const Shape2 sh = shape(N, W2, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_multiaxpy<C, W2>), w, cf, m, V, n, N, accumulate, np, nscale);
     } else {
-        const Shape2 sh = shape(n, N, 1, G);
+        const Shape2 sh = shape(N, 1, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_multiaxpy<C, 1>), w, cf, m, V, n, N, accumulate, np, nscale);
     }
     MG_LAUNCHED();
@@ -610,10 +609,10 @@ void launch_norm(const NormOut& o, const C* x, long long n, int N, void* part, c
     constexpr int W2 = sizeof(C) == 8 ? 2 : 1;
     const int G = dot_groups(n, N);
     if (width<C>(N) == 2) {
-        const Shape2 sh = shape(n, N, W2, G);
+        const Shape2 sh = shape(N, W2, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_norm2<C, W2>), np, x, n, N);
     } else {
-        const Shape2 sh = shape(n, N, 1, G);
+        const Shape2 sh = shape(N, 1, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_norm2<C, 1>), np, x, n, N);
     }
     MG_LAUNCHED();
@@ -627,10 +626,10 @@ void launch_scale_norm(const NormOut& o, Cy* y, const Cx_* x, const double* scal
     constexpr int W2 = sizeof(Cy) == 8 ? 2 : 1;
     const int G = dot_groups(n, N);
     if (width<Cy>(N) == 2) {
-        const Shape2 sh = shape(n, N, W2, G);
+        const Shape2 sh = shape(N, W2, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_norm<Cy, Cx_, W2>), y, x, scale, inverse, n, N, np);
     } else {
-        const Shape2 sh = shape(n, N, 1, G);
+        const Shape2 sh = shape(N, 1, G);
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_norm<Cy, Cx_, 1>), y, x, scale, inverse, n, N, np);
     }
     MG_LAUNCHED();
@@ -640,7 +639,7 @@ void launch_scale_norm(const NormOut& o, Cy* y, const Cx_* x, const double* scal
 void launch_refine_axpy(double2* y, const double* scale, double sign, const float2* x, long long n, int N,
                         bool accumulate, const NormOut* of_x, const NormOut* of_y, void* part, cudaStream_t s) {
     const int G = dot_groups(n, N);
-    const Shape2 sh = shape(n, N, 1, G);
+    const Shape2 sh = shape(N, 1, G);
     if (of_y) {
         MG_LAUNCH(sh.g, sh.b, 0, s, (k_refine_axpy<false>), y, scale, sign, x, n, N, accumulate, part);
         MG_LAUNCHED();
@@ -654,7 +653,7 @@ void launch_refine_axpy(double2* y, const double* scale, double sign, const floa
 
 template <typename C>
 void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_t s) {
-    const Shape2 sh = shape(n, N, 1, groups_of(n, N, 1, 4));
+    const Shape2 sh = shape(N, 1, groups_of(n, N, 1, 4));
     MG_LAUNCH(sh.g, sh.b, 0, s, (k_scale_cols_if<C>), w, f, n, N);
     MG_LAUNCHED();
 }

@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(256) k_mr_combine(C* __restrict__ e, const C* 
     }
 }
 
-// The same two with the residuals and the image in BF16 (one bf16x2 word per complex
+// The same two (the sum always adds to e) with the residuals and the image in BF16 (one bf16x2 word per complex
 // value), four rhs per thread: 16-byte accesses.  N % 4 == 0.
 __global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r,
                                                              const uint32_t* __restrict__ p,
@@ -984,7 +984,7 @@ __global__ void __launch_bounds__(256) k_mr_update_fine_bf16(uint32_t* rn, const
 
 __global__ void __launch_bounds__(256) k_mr_combine_bf16(float2* __restrict__ e, const uint32_t* __restrict__ rs,
                                                          size_t slot, int K, const float2* __restrict__ alpha,
-                                                         long long n, int N, bool e_is_zero) {
+                                                         long long n, int N) {
     if (grid_dependency()) return;
     const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (j >= N) return;
@@ -996,13 +996,11 @@ __global__ void __launch_bounds__(256) k_mr_combine_bf16(float2* __restrict__ e,
 #pragma unroll
         for (int s = 0; s < kMrGroup; ++s)
             if (s < K) rv[s] = *reinterpret_cast<const VecOf<uint32_t, 4>*>(rs + s * slot + i * N + j);
-        if (!e_is_zero) {
-            ev[0] = *reinterpret_cast<const VecOf<float2, 2>*>(er);
-            ev[1] = *reinterpret_cast<const VecOf<float2, 2>*>(er + 2);
-        }
+        ev[0] = *reinterpret_cast<const VecOf<float2, 2>*>(er);
+        ev[1] = *reinterpret_cast<const VecOf<float2, 2>*>(er + 2);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            float2 acc = e_is_zero ? make_float2(0.f, 0.f) : ev[q >> 1].v[q & 1];
+            float2 acc = ev[q >> 1].v[q & 1];
 #pragma unroll
             for (int s = 0; s < kMrGroup; ++s)
                 if (s < K) cfma(acc, alpha[s * N + j + q], bf2_lo(rv[s].v[q]));
@@ -1173,12 +1171,10 @@ bool wilson_f2<float2>(float2* y, const float2* x, const float2* b, const float2
 
 // ---------------------------------------------------------------------------
 // Fine-level smoother with the residual and its image held in BF16 ([row][rhs],
-// one bf16x2 per complex value): the operator y = D x with the MR dots
-// conj(y).x, |y|^2 (FP32 arithmetic, two rhs per thread, 8-byte accesses), the
-// FP32 -> BF16 packing and the MR update e (=|+=) alpha r, r -= alpha p.
-
-// Four rhs per thread: 16-byte accesses (four bf16x2 words), ten loads of a site in
-// flight per thread.  N % 4 == 0.
+// one bf16x2 per complex value): the operator y = D x with the minimal-residual dots
+// conj(y).x, |y|^2 (FP32 arithmetic, ten loads of a site in flight per thread; N % 4 == 0).
+// The first residual comes from k_wilson_f2<4>, the updates are k_mr_update_fine_bf16 and
+// k_mr_combine_bf16.
 // RPT right-hand sides per thread (4: 16-byte accesses, a warp spans 128 rhs; 2: 8-byte
 // accesses, 64 rhs, so that a block of 64 keeps every lane busy).
 // STORE = false: the dots only (the last minimal-residual step needs no image).
@@ -1642,11 +1638,11 @@ void launch_mr_update_fine_bf16(uint32_t* rn, const uint32_t* r, const uint32_t*
 }
 
 void launch_mr_combine_bf16(float2* e, const uint32_t* rs, size_t slot, int K, const float2* alpha, long long n, int N,
-                            bool e_is_zero, cudaStream_t s) {
+                            cudaStream_t s) {
     MG_REQUIRE(N % 4 == 0 && K >= 1 && K <= kMrGroup, MGMLMC_EINVAL, "BF16 MR sum: N a multiple of 4, group size");
     dim3 g, b;
     row_shape(n, N, 4, 8, g, b);
-    MG_LAUNCH(g, b, 0, s, k_mr_combine_bf16, e, rs, slot, K, alpha, n, N, e_is_zero);
+    MG_LAUNCH(g, b, 0, s, k_mr_combine_bf16, e, rs, slot, K, alpha, n, N);
     MG_LAUNCHED();
 }
 

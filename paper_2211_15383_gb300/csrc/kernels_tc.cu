@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* rn, const uint4*
     }
 }
 
-// e (=|+=) M^{-1} sum_{s < K} alpha_s r_s with the residuals r_s as BF16 tiles (slots of
+// e += M^{-1} sum_{s < K} alpha_s r_s with the residuals r_s as BF16 tiles (slots of
 // `slot` bytes): thread = (site, RPT adjacent rhs), M^{-1} of the site in shared memory,
 // transposed.  The sum over the steps is formed component by component (four per 16-byte
 // piece of a tile row) and goes straight into the 16 outputs of each rhs, so that a
@@ -667,8 +667,7 @@ __global__ void __launch_bounds__(256) k_mr_update_tiles(uint4* rn, const uint4*
 template <int RPT>
 __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e, const uint8_t* __restrict__ rt,
                                                          size_t slot, int K, const float2* __restrict__ alpha,
-                                                         const float2* __restrict__ Minv, int nsites, int N, int T,
-                                                         bool accumulate) {
+                                                         const float2* __restrict__ Minv, int nsites, int N, int T) {
     if (grid_dependency()) return;
     struct alignas(8 * RPT) Rhs { float2 v[RPT]; };
     __shared__ float2 Mt[D * D];                                // [input][output]
@@ -683,7 +682,9 @@ __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e,
         Rhs acc[D];
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-            if (accumulate) acc[c] = *reinterpret_cast<const Rhs*>(out + (size_t)c * N);
+            // K is never 0: the branch keeps the 16 loads of e together ahead of the sums
+            // (16^2 sites x 256 rhs, K = 4, without it: 50 us a launch instead of 37)
+            if (K > 0) acc[c] = *reinterpret_cast<const Rhs*>(out + (size_t)c * N);
             else
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) acc[c].v[r] = make_float2(0.f, 0.f);
@@ -983,7 +984,7 @@ void launch_mr_update_tiles(__nv_bfloat16* rn, const __nv_bfloat16* r, const __n
 }
 
 void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const float2* alpha, const float2* Minv,
-                             int nsites, int N, bool accumulate, cudaStream_t s) {
+                             int nsites, int N, cudaStream_t s) {
     // two rhs per thread where N is even (16-byte accesses to e and alpha), from 64 rhs on
     // (below, the idle lanes cost more: 7.8 against 5.2 us at 16 rhs)
     const int rpt = N % 2 == 0 && N >= 64 ? 2 : 1;
@@ -994,10 +995,10 @@ void launch_block_diag_tiles(float2* e, const __nv_bfloat16* rt, int K, const fl
     const size_t slot = tc_tiles_bytes(nsites, N);
     if (rpt == 2)
         MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles<2>, e, r, slot, K, alpha, Minv, nsites, N,
-                  tc_tiles(N), accumulate);
+                  tc_tiles(N));
     else
         MG_LAUNCH(dim3(tiles, G), th, 0, s, tc::tcs::k_block_diag_tiles<1>, e, r, slot, K, alpha, Minv, nsites, N,
-                  tc_tiles(N), accumulate);
+                  tc_tiles(N));
     MG_LAUNCHED();
 }
 

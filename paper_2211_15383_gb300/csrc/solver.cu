@@ -359,7 +359,7 @@ bool post_smooth_tc<float2>(Ctx& c, int l, float2* e, const float2* r, int N, bo
             // traffic: the K residuals (4 B per complex) read, e read and written
             ProfScope ps(c, {"bjac", l + 1, ".bf16"}, (double)L.n * N * (4 * k + 16),
                          8.0 * (L.d + k) * (double)L.n * N);
-            launch_block_diag_tiles(e, rt, k, alpha, L.Minv32, L.nsites, N, true, c.stream);
+            launch_block_diag_tiles(e, rt, k, alpha, L.Minv32, L.nsites, N, c.stream);
         },
         [&](int s, int t) {
             // traffic: r and p tiles read, the next r tiles written (4 B per complex)
@@ -428,7 +428,7 @@ bool post_smooth_fine_bf16<float2>(Ctx& c, int l, float2* e, const float2* r, in
         },
         [&](int k, bool) {
             ProfScope ps(c, "mr1sum.bf16", (double)nN * (4 * k + 16), 8.0 * k * nN);
-            launch_mr_combine_bf16(e, rb, nN, k, alpha, L.n, N, false, c.stream);
+            launch_mr_combine_bf16(e, rb, nN, k, alpha, L.n, N, c.stream);
         },
         [&](int s, int t) {
             // traffic: r and p read, the next r written (4 B each)
