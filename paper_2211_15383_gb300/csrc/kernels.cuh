@@ -161,7 +161,7 @@ template <typename C>
 bool launch_prolong(C* x, const C* xc, const C* P, int lx, int lt, int d, int ax, int at, int nvec,
                     int N, bool accumulate, cudaStream_t s, void* xt = nullptr);
 // Minimal-residual smoother: rn = r - alpha p, and e (=|+=) sum_{s < K} alpha_s r_s over the
-// K <= 8 residuals r_s in slots of rs (slot: values between them; alpha[K][N]).
+// K <= kSmootherGroup residuals r_s in slots of rs (slot: values between them; alpha[K][N]).
 template <typename C>
 void launch_mr_update(C* rn, const C* r, const C* p, const C* alpha, long long n, int N, cudaStream_t s);
 template <typename C>
