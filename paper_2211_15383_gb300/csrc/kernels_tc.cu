@@ -682,9 +682,9 @@ __global__ void __launch_bounds__(CH) k_block_diag_tiles(float2* __restrict__ e,
         Rhs acc[D];
 #pragma unroll
         for (int c = 0; c < D; ++c) {
-            // K is never 0: the branch keeps the 16 loads of e together ahead of the sums
+            // T is never 0: the branch keeps the 16 loads of e together ahead of the sums
             // (16^2 sites x 256 rhs, K = 4, without it: 50 us a launch instead of 37)
-            if (K > 0) acc[c] = *reinterpret_cast<const Rhs*>(out + (size_t)c * N);
+            if (T > 0) acc[c] = *reinterpret_cast<const Rhs*>(out + (size_t)c * N);
             else
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) acc[c].v[r] = make_float2(0.f, 0.f);
