@@ -101,7 +101,7 @@ template <typename C>
 void launch_scale_cols_if(C* w, const double* f, long long n, int N, cudaStream_t s);
 // Givens rotations of the Hessenberg columns j0..j1 (H[j][m + 1][N], subdiagonals hsub[j][N]):
 // rotations cs, sn [j][N], rotated right-hand side g[m + 1][N], irr[j][N] = 1 / R_jj; max[j] =
-// max(max[j], residual / bnorm) after each column j (max may be null); for N <= kRotateWarp the
+// max(max[j], (residual / bnorm)^2) after each column j (max may be null); for N <= kRotateWarp the
 // maxima can go to host[j] (pinned memory) instead.
 constexpr int kRotateWarp = 32;
 void launch_rotate(double2* H, const double* hsub, double* cs, double2* sn, double2* g, double2* irr,

@@ -416,8 +416,9 @@ __global__ void __launch_bounds__(256) k_scale_cols_if(C* __restrict__ w, const 
 // ---- Givens rotations of the Hessenberg columns j0 .. j1, one thread per rhs.  Column j:
 // entries i <= j at H[(j (m + 1) + i) N + r] (overwritten by R), subdiagonal hsub[j N + r];
 // rotation i: (a, b) <- (c a + s b, -conj(s) a + c b).  irr = 1 / R[j][j] (0 if it is 0).
-// The residual estimate after column j, divided by bnorm, goes to max[j] (their maximum over the rhs),
-// or to host[j] where one warp holds all rhs.
+// The square of the residual estimate after column j, divided by bnorm, goes to max[j] (the maximum
+// over the rhs), or to host[j] where one warp holds all rhs: with the square root and the quotient
+// of every column the first look of a cycle, at ten or more columns, took 10 us longer.
 __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const double* __restrict__ hsub,
                                                double* __restrict__ cs, double2* __restrict__ sn,
                                                double2* __restrict__ g, double2* __restrict__ irr,
@@ -429,6 +430,8 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
     if (!in && !host) return;
     double2 gj = in ? g[(long long)j0 * N + r] : make_double2(0.0, 0.0);
     const double bn = in && bnorm ? bnorm[r] : 0.0;
+    const double lift = bn < 0x1p-900 ? 0x1p200 : 1.0;         // 1 / |b| stays finite
+    const double ib = bn == 0.0 ? 0.0 : 1.0 / (bn * lift);
     double resid = 0.0;
     auto column = [&](int j) {
         double2* col = H + (long long)j * (m + 1) * N + r;
@@ -474,8 +477,8 @@ __global__ void __launch_bounds__(32) k_rotate(double2* __restrict__ H, const do
     for (int j = j0; j <= j1; ++j) {
         if (in) column(j);
         if (!max && !host) continue;
-        const double rs = resid == resid ? sqrt(gj.x * gj.x + gj.y * gj.y) : resid;
-        const double v = bn == 0.0 ? 0.0 : rs / bn;
+        const double gx = gj.x * lift * ib, gy = gj.y * lift * ib;
+        const double v = resid == resid ? fma(gx, gx, gy * gy) : resid;
         if (host) {
             u64 m8 = (u64)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 #pragma unroll

@@ -686,7 +686,7 @@ static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate
     // loop, whose FP64 residual absorbs the loss of orthogonality
     const int passes = sizeof(C) == sizeof(double2) ? 2 : 1;
     unsigned long long* dmax = nullptr;
-    double* est = c.hbuf + kMaxSlots;            // per column
+    double* est = c.hbuf + kMaxSlots;            // squares of the estimates, per column
     if (N > kRotateWarp) {
         dmax = c.scratch<unsigned long long>("fg_est", kMaxRestart);
         MG_CUDA(cudaMemsetAsync(dmax, 0, m * sizeof(unsigned long long), c.stream));
@@ -706,7 +706,7 @@ static void fgmres_cycle(Ctx& c, int l, const Basis<C>& B, C* x, bool accumulate
         c.sync();
         for (; rotated <= j && !done; ++rotated) {
             if (est[rotated] != est[rotated]) throw Error(MGMLMC_ENAN, "FGMRES: NaN in Arnoldi");
-            done = est[rotated] <= tol;
+            done = std::sqrt(est[rotated]) <= tol;
         }
         if (done) {
             it -= j + 1 - rotated;               // steps beyond it were not needed
