@@ -121,6 +121,17 @@ struct ProfScope {
     ~ProfScope();
 };
 
+// An inner cycle of the refinement stops at the first step that meets `margin` times the reduction
+// that is left to do, but no less than `floor` (what FP32 arithmetic can deliver).
+struct InnerTolerance {
+    double margin, floor;
+};
+constexpr InnerTolerance kInner{0.3, 2e-7};
+// The setup's test vectors carry the residuals of many solves on: its cycles aim lower (four 64^2
+// setups against 64 bits: 13, 5.4, 5.9, 8.4e-14, with the other pair 17, 7.3, 8.3, 12; at a
+// margin of 0.03 and a floor of 1e-8 no better for twice the time).
+constexpr InnerTolerance kInnerSetup{0.1, 5e-8};
+
 struct Ctx {
     mgmlmc_options opt{};
     Profiler prof;
@@ -158,6 +169,7 @@ struct Ctx {
     // the refinement loop may take its residuals from FP32 products between FP64 ones
     // (the estimator's solves: Z2 right-hand sides, no strong cancellation in D e)
     bool fp32_residual_updates = false;
+    InnerTolerance inner = kInner;
 
     // ---- memory
     struct Buf { void* p = nullptr; size_t bytes = 0; };
@@ -192,6 +204,13 @@ struct Ctx {
     void free_hierarchy();
     void free_deflation();
     void sync();
+};
+
+struct InnerScope {
+    Ctx& c;
+    const InnerTolerance keep;
+    InnerScope(Ctx& ctx, InnerTolerance t) : c(ctx), keep(ctx.inner) { c.inner = t; }
+    ~InnerScope() { c.inner = keep; }
 };
 
 // ---- solver layer (solver.cu)

@@ -568,6 +568,7 @@ void build_hierarchy(Ctx& c, int nlev, const int* ax, const int* at, const int* 
     launch_materialize_wilson(c.lev[0].A64, c.U64, c.m0, c.Lx, c.Lt, c.stream);
     rebuild_from(c, 0);
     if (setup_iters > 0) {
+        const InnerScope inner(c, kInnerSetup);
         // The setup solves run nvec right-hand sides only, so their Krylov bases are
         // small: they use a restart length of at least kSetupRestart, which keeps the
         // low modes a hierarchy built from rough vectors still misses (a short restart

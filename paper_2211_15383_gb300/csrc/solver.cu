@@ -817,9 +817,6 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
     double* rnorm = c.scratch<double>("ir_rn", N);
     double* inorm = c.scratch<double>("ir_in", N);
     void* npart = c.scratch_bytes("part_nrm", norm_part_bytes(n, N));
-    // inner tolerance: the reduction still needed this cycle (with margin), but no
-    // tighter than FP32 arithmetic can deliver
-    const double inner_floor = 2e-7;
     // In the estimator's solves (c.fp32_residual_updates) the next residual comes from an
     // FP32 product, r <- r - |r| D e, between FP64 ones.  Its error against
     // the FP64 residual b - D x is below kFp32Product ||D|| |e| |r| (rounding of the FP32
@@ -907,7 +904,7 @@ static long long solve_block(Ctx& c, int l, const double2* b, double2* x, int N,
         if (it >= maxit) break;
         // one FGMRES cycle in FP32 on r / |r|: its own FP32 residual cannot certify more than
         // ~1e-6 relative, so the FP64 residual of this loop decides on restarts
-        const double inner_tol = std::max(inner_floor, 0.3 * tol / ratio);
+        const double inner_tol = std::max(c.inner.floor, c.inner.margin * tol / ratio);
         NormOut start = basis_start(B);
         start.norm = inorm;
         launch_scale_norm<float2, double2>(start, B.V, r, rn, true, n, N, npart, c.stream);
