@@ -706,6 +706,12 @@ int mgmlmc_apply(mgmlmc_ctx* h, int op, int level, int nrhs, const double* x, do
     MG_REQUIRE(op >= 0 && op <= 6, MGMLMC_EINVAL, "apply: unknown op");
     double2* xt = upload_block(c, x, nin, nrhs, "ap_x");
     double2* yt = c.scratch<double2>("ap_y", (size_t)nout * nrhs);
+    // operators, unlike the solves' residuals, are looked at entry by entry
+    struct Entrywise {
+        Ctx& c;
+        explicit Entrywise(Ctx& ctx, bool on) : c(ctx) { c.entrywise = on; }
+        ~Entrywise() { c.entrywise = false; }
+    } entrywise{c, op == MGMLMC_OP_D || op == MGMLMC_OP_SMOOTH};
     switch (op) {
         case MGMLMC_OP_D: mg::apply_D<double2>(c, l, yt, xt, nullptr, nrhs, 0, nullptr); break;
         case MGMLMC_OP_PH: mg::apply_restrict<double2>(c, l, yt, xt, nrhs); break;

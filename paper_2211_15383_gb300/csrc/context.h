@@ -169,6 +169,8 @@ struct Ctx {
     // the refinement loop may take its residuals from FP32 products between FP64 ones
     // (the estimator's solves: Z2 right-hand sides, no strong cancellation in D e)
     bool fp32_residual_updates = false;
+    // FP64 products accurate entry by entry, not only in the norm (the operators of mgmlmc_apply)
+    bool entrywise = false;
     InnerTolerance inner = kInner;
 
     // ---- memory

@@ -265,8 +265,9 @@ void launch_block_stencil_tc(float2* y, __nv_bfloat16* yt, const float2* b, cons
 // the blocks of a d = 16 stencil one after another (nb = 0), or those of a dense matrix with
 // nb blocks per row, rows ld apart.  launch_block_stencil_f64: modes and partials as
 // launch_block_stencil; launch_dense_f64: y = A x for the dense n x n matrix (n % 16 == 0).
-// A: the blocks themselves (rows whose inputs are far below the rhs' largest entry or not finite
-// are summed in FP64).  A column of x with a non-finite entry gives NaN in the dense product.
+// A: the blocks themselves; entrywise: rows whose inputs are far below the rhs' largest entry or not
+// finite are summed in FP64 from them (else only those of columns with a non-finite entry).  A
+// column of x with a non-finite entry gives NaN in the dense product.
 // scratch: 256-byte aligned.
 bool f64_tc_supported(int d, int N);
 size_t f64_tc_operand_bytes(long long nblk, int nb);
@@ -274,7 +275,7 @@ void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int 
 size_t f64_tc_scratch_bytes(long long nsites, int N);
 int block_stencil_f64_groups(int nsites, int N);
 void launch_block_stencil_f64(double2* y, const double2* x, const double2* b, const void* op, const double2* A, int lx,
-                              int lt, int N, int mode, void* scratch, double2* part, int groups, int* err, cudaStream_t s);
+                              int lt, int N, int mode, bool entrywise, void* scratch, double2* part, int groups, int* err, cudaStream_t s);
 size_t f64_dense_scratch_bytes(int n, int N);
 void launch_dense_f64(double2* y, const double2* x, const void* op, int n, int N, void* scratch, int* err,
                       cudaStream_t s);

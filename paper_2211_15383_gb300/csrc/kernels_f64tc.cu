@@ -15,11 +15,14 @@
 //    exact range by rounding their last place); the dropped pairs i + j > 8 weigh 2^-72;
 //  * sum_g G_g 2^-8g is formed in 128-bit integers and rounded to FP64 once.
 // The error of an entry is 2^-53 of itself from that rounding, and about 2^-63 of the rhs' largest
-// entry; 160 FP64 FMAs leave about 2^-51 of the entries around it.  A site of the stencil whose
-// inputs all lie more than 2^8 below the rhs' largest entry would lose by that: its rows
-// are summed in FP64 (so are those next to an infinity or NaN, which stays where it is), and the
-// stencil is as accurate entry by entry as FP64 sums are.  With 7 digits of x and 8 groups
-// (2^-55) residuals of near-critical 1024^2 solves, dominated by localised modes, stood at 1.9e-12.
+// entry; 160 FP64 FMAs leave about 2^-51 of the entries around it.  In the norm, by which the solver
+// decides, the product is closer to the exact one also where a rhs is concentrated on a few
+// sites (the second part is spread over n entries: it stays below as long as n < 2^21 of them).  Entry
+// by entry a site loses whose inputs all lie more than 2^8 below the rhs' largest entry; where the
+// caller asks for it (the operators of mgmlmc_apply), its rows are summed in FP64 instead, and so are
+// those next to an infinity or NaN, which stays where it is.  In the solves of the near-critical 1024^2
+// lattice, dominated by localised modes, that would be most sites (189 -> 140 samples/s).  With 7
+// digits of x and 8 groups (2^-55) their residuals stood at 1.9e-12.
 //
 // Layout: the rhs are the MMA's M (128 rows of x digits, K = 32 reals of a site), the digits
 // of the block are its N: the 8 x 32 rows (i, output real) of a block's tile lie one after
@@ -321,9 +324,9 @@ __device__ __noinline__ void rows_by_fp64(double2* v, const double2* __restrict_
 // MODE 0: y = A x; 1: y = b - A x; 2: y = A x with the per-rhs dots <y, x>, <y, y>; 3: the
 // dots only; 4: job (R, z) of a dense product, y[z] = its partial sum over K blocks
 // 6z .. 6z + 5.  nblk: sites of the stencil (lx x lt) or block rows of the dense matrix.
-// The stencil's results are also right entry by entry: where all of a site's inputs lie more than
-// 2^kSpread below the rhs' largest entry, whose scale the digits share, or one of them is not
-// finite, its rows are summed in FP64 instead.
+// With xe (exponents per site and rhs) the stencil's results are also right entry by entry: where all
+// of a site's inputs lie more than 2^kSpread below the rhs' largest entry, whose scale the digits
+// share, or one of them is not finite, its rows are summed in FP64 instead.
 constexpr int kSpread = 8;
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -492,7 +495,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             bool by_sums = ex == 0x7ff;
 #pragma unroll
             for (int p = 0; p < 8; ++p) by_sums = by_sums || ((ea[p / 2] >> (16 * (p & 1))) & 0xFFFF) == 0x7ff;
-            if (MODE != 4 && j < N) {
+            if (MODE != 4 && xe && j < N) {
                 int near = 0;
 #pragma unroll
                 for (int dir = 0; dir < 5; ++dir)
@@ -636,8 +639,8 @@ void launch_f64_operand(void* op, const double2* A, long long nblk, int nb, int 
     MG_LAUNCHED();
 }
 
-// Slices x into the scratch: digit tiles, then the largest entry per rhs and (for the stencil) the
-// exponents per site and rhs.
+// Slices x into the scratch: digit tiles, then the largest entry per rhs and (sites) the exponents
+// per site and rhs, with the largest of the finite entries.
 static const uint16_t* site_exponents(const u64* mx, int N) {
     return reinterpret_cast<const uint16_t*>(reinterpret_cast<const uint8_t*>(mx) + max_bytes(N));
 }
@@ -679,11 +682,11 @@ int block_stencil_f64_groups(int nsites, int N) {
 }
 
 void launch_block_stencil_f64(double2* y, const double2* x, const double2* b, const void* op, const double2* A, int lx,
-                              int lt, int N, int mode, void* scratch, double2* part, int groups, int* err, cudaStream_t s) {
+                              int lt, int N, int mode, bool entrywise, void* scratch, double2* part, int groups, int* err, cudaStream_t s) {
     const int V = lx * lt;
     MG_REQUIRE(f64_tc_supported(D, N) && groups >= 1 && groups <= V, MGMLMC_EINVAL, "FP64 stencil: size");
-    const u64* mxx = slice_x(scratch, x, V, N, true, s);
-    const uint16_t* xe = site_exponents(mxx, N);
+    const u64* mxx = slice_x(scratch, x, V, N, entrywise, s);
+    const uint16_t* xe = entrywise ? site_exponents(mxx, N) : nullptr;
     const uint16_t* re = operand_rows(op, 5LL * V);
     switch (mode) {
         case 0: f64_launch<0>(y, b, x, scratch, op, mxx, xe, re, A, lx, lt, V, 1, N, part, groups, err, s); break;

@@ -54,8 +54,8 @@ static bool galerkin_form_cheaper(const Ctx& c, int l) {
     return galerkin < direct;
 }
 
-// FP64 block stencils with d = 16 run on the tensor cores (exact integer digit products, as
-// accurate as FP64 sums) from kF64TcMinRhs right-hand sides on, where the level has its digits
+// FP64 block stencils with d = 16 run on the tensor cores (exact integer digit products, in the
+// norm as accurate as FP64 sums, entry by entry with c.entrywise) from kF64TcMinRhs right-hand sides on, where the level has its digits
 // and their work space is granted.  op: the level's own pointer (an allocation may take the
 // digits away).
 template <typename C>
@@ -72,7 +72,7 @@ bool f64_stencil<double2>(Ctx& c, const Level& L, double2* y, const double2* x, 
     if (!f64_stencil_used(L, op, N)) return false;
     void* scr = c.try_scratch("f64_tc", f64_tc_scratch_bytes(L.nsites, N));
     if (!scr) return false;
-    launch_block_stencil_f64(y, x, b, op, A, L.lx, L.lt, N, mode, scr, part, groups, err, c.stream);
+    launch_block_stencil_f64(y, x, b, op, A, L.lx, L.lt, N, mode, c.entrywise, scr, part, groups, err, c.stream);
     return true;
 }
 template <typename C> static int bst_groups(const Level& L, const void* op, int N) {
